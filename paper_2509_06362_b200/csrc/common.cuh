@@ -18,19 +18,23 @@ constexpr long long kWaitCycles = 4000000000ll;  // bound on any device-side wai
 // 9:    block layout with 16 warps striding over up to 128 instances, state in shared memory
 // 10..18: thread mapping, by how many lanes of a warp work at a time (32, 24, 16, 12, 8, 6, 4, 2, 1:
 //        the larger the placements, the fewer fit the warp's pools)
-constexpr int kNumBuckets = 20;
+// 20..24: walking kernel, by the room a placement needs: one, 2, 4, 8, 16 times a warp's part (walk.cuh)
+constexpr int kNumBuckets = 25;
+constexpr int kWalkBucket0 = 20;
+constexpr int kWalkBuckets = 5;
+constexpr int kWalkModes = kWalkBuckets;
 constexpr int kGenericBlockBucket = 9;
 constexpr int kThreadBucket0 = 10;  // buckets 10..18: the thread mapping, by lanes per warp
 constexpr int kThreadBuckets = 9;
 constexpr int kWideBucket = 19;     // 33..128 instances under the engines of the lane-group code: one warp per placement
 constexpr int kCostBins = 256;   // bin 0 = most expensive (largest total batch cap)
-constexpr int kCounterWords = 17408;  // counters | work counters | histograms + cursors, cleared per call
+constexpr int kCounterWords = 20480;  // counters | work counters | histograms + cursors, cleared per call
 // histogram sets (rows of kCostBins words in EvalParams::hist): candidates that can only go to a lane-group
-// or block bucket, only to a thread bucket, or either way (counted once per side); then the write cursors
-constexpr int kHistOnlyG = 0, kHistBothG = 10, kHistOnlyT = 20, kHistBothT = 29, kHistWide = 38, kHistBothW = 39, kHistCursor = 40;
+// or block bucket, only to a walking or thread bucket, or either way (counted once per side); then the write cursors
+constexpr int kHistOnlyG = 0, kHistBothG = 10, kHistOnlyT = 20, kHistBothT = 34, kHistWide = 48, kHistBothW = 49, kHistCursor = 50;
 constexpr int kHistRows = kHistCursor + kNumBuckets;
 // counters beside the bucket counts (EvalParams::bucket_count[0..31])
-constexpr int kCtrBoth = 24, kCtrLoaded = 25, kCtrCut = 26, kCtrUseThreads = 27;
+constexpr int kCtrBoth = 28, kCtrLoaded = 29, kCtrCut = 30, kCtrUseThreads = 31;
 constexpr int kGroupThreads = 128;
 constexpr int kScanTile = 256;       // requests per scan tile of the thread mapping
 constexpr int kScanHdrUnits = 40;    // 16-byte units of a scan tile's header (see scan_trace_kernel)
@@ -250,6 +254,7 @@ struct EvalParams {
     const uint4* trace_scan[kMaxTraces];
     const uint64_t* trace_class_tot[kMaxTraces];  // [n_classes][2]: count, checksum sum
     uint32_t trace_n[kMaxTraces];
+    const uint4* trace_reqs[kMaxTraces];  // walking kernel: the requests as loaded
     const uint64_t* rej_hash;  // [n_req] checksum term of "request r was rejected" (same for every candidate)
     const int32_t* rows;     // [n_rows][kRowStride]
     const int32_t* devices;
@@ -269,8 +274,9 @@ struct EvalParams {
     uint32_t* work_ctr;      // [16]: next work item of the block kernels [1..4], of the thread buckets [5..13], of the wide kernel [14]
     uint32_t* hist;          // [kHistRows][kCostBins]: candidates per cost bin by set, then write cursors
     uint32_t* code;          // [n_cand] lane-group / block bucket << 8 | cost bin, 0xFFFFFFFF if none
-    uint32_t* code2;         // [n_cand] thread bucket << 8 | cost bin, 0xFFFFFFFF if none
+    uint32_t* code2;         // [n_cand] walking or thread bucket << 8 | cost bin, 0xFFFFFFFF if none
     uint32_t demand_tok_s;   // output tokens per second the trace(s) ask for
+    uint32_t walk_all;        // MAASO_MAP_AUTO: the batch goes to the walking kernel whatever its load
     uint32_t thread_min_cand; // MAASO_MAP_AUTO: fewest loaded candidates for which the thread mapping is chosen
     uint32_t group_warps;    // warps the lane-group grid keeps resident (capacity for promotions)
     uint32_t* sm_ctr;        // [n_sm] next work item of each SM's share (lane-group kernel)
@@ -278,6 +284,8 @@ struct EvalParams {
     uint32_t promote_pct;
     uint32_t thread_pool_units;  // thread mapping: 16-byte units one warp has for the cold part of its placements' state
     uint32_t thread_hot_units;   // and for the hot part (3 units per instance, shared memory)
+    uint32_t* walk_ctr;      // [kWalkBuckets]: next placement of each walking bucket
+    uint32_t walk_bytes;     // walking kernel: bytes of shared memory one warp has for a placement, 0 = not used
     long long wait_cycles;   // bound of every device-side wait
     uint32_t stall_test;     // test hook: never issue the trace copies
     int32_t* dump_row;       // [n_cand] or null

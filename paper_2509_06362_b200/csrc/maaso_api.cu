@@ -7,7 +7,7 @@
 #include <string>
 #include <vector>
 
-#include "common.cuh"
+#include "walk.cuh"
 
 namespace maaso {
 cudaError_t launch_prep(const EvalParams& P, const uint32_t* dump_idx, cudaStream_t stream, int* launches);
@@ -24,6 +24,7 @@ cudaError_t launch_eval_thread(const EvalParams& P, int grid, uint32_t pool_byte
 int occupancy_eval_thread(const EvalParams& P, uint32_t pool_bytes, uint32_t hot_bytes, bool in_smem);
 size_t thread_scratch_per_warp(uint32_t pool_bytes);
 uint32_t thread_fixed_smem(uint32_t n_models, uint32_t n_rows);
+cudaError_t launch_eval_walk(const EvalParams& P, int sm_count, cudaStream_t stream);
 cudaError_t launch_eval_wide(const EvalParams& P, int grid, cudaStream_t stream);
 int occupancy_eval_wide(const EvalParams& P);
 size_t wide_scratch_per_warp();
@@ -56,6 +57,8 @@ struct maaso_trace {
     uint64_t n;
     uint32_t n_classes;
     uint32_t max_model;
+    uint32_t max_in;  // most input tokens of a request
+    bool small_limits;  // every finite SLO limit fits the walking kernel's 32-bit times
     double tok_rate;  // output tokens per second the trace asks for (routing hint of MAASO_MAP_AUTO)
 };
 
@@ -64,6 +67,7 @@ struct maaso_ctx {
     int sm_count;
     bool has_profile;
     uint32_t n_models, n_strategies, n_rows;
+    int64_t max_step, max_pre_base, max_q16;  // largest entries of the tables
     int32_t* d_rows;
     int32_t* d_devices;
     int32_t* d_min_devices;
@@ -91,7 +95,8 @@ struct maaso_ctx {
     bool thread_blocks_set;  // MAASO_THREAD_BLOCKS was given: also caps the resident warps per SM in arena mode
     int thread_blocks;   // one-warp blocks of the thread-mapping kernel per SM its pool is sized for
     uint32_t thread_theta;     // waiting lanes of a warp that trigger a distributor round in the thread mapping
-    uint32_t thread_min_cand;  // MAASO_MAP_AUTO takes the thread mapping from this many candidates on
+    uint32_t thread_min_cand;  // MAASO_MAP_AUTO considers the thread mapping from this many candidates on
+    uint32_t walk_all;         // MAASO_MAP_AUTO takes the walking kernel up to this many placements x traces, whatever their load
     uint32_t last_mapping;     // mapping the most recent scoring call resolved to
     int fail_allocs;           // test hook: this many of the next scratch allocations are refused
     bool timing;
@@ -235,12 +240,14 @@ MAASO_API int maaso_create(maaso_ctx** out, int cuda_device) {
         int v = atoi(tt);
         if (v >= 1 && v <= 32) ctx->thread_theta = (uint32_t)v;
     }
-    ctx->thread_min_cand = 16384;  // fewer loaded placements than this do not fill the GPU one per lane
+    ctx->thread_min_cand = 262144;  // loaded sweeps of 300,000 placements: 183 ms on the threads, 194 ms walking; of 100,000: 132 and 122
     const char* tm = getenv("MAASO_THREAD_MIN_CAND");
     if (tm) {
         long v = atol(tm);
         if (v >= 0) ctx->thread_min_cand = (uint32_t)v;
     }
+    ctx->walk_all = 16384;
+    if (const char* v = getenv("MAASO_WALK_ALL")) ctx->walk_all = (uint32_t)atol(v);
     ctx->last_mapping = MAASO_MAP_GROUP;
     ctx->fail_allocs = 0;
     const char* gb = getenv("MAASO_GROUP_BLOCKS");
@@ -331,6 +338,14 @@ MAASO_API int maaso_load_profile(maaso_ctx* ctx, const maaso_profile_desc* d) {
     ctx->h_devices.assign(d->devices, d->devices + S);
     ctx->h_min_devices.assign(d->min_devices, d->min_devices + M);
     ctx->h_rows = rows;
+    ctx->max_step = ctx->max_pre_base = ctx->max_q16 = 0;
+    for (uint32_t r = 0; r < R; r++) {
+        const int32_t* row = rows.data() + (size_t)r * kRowStride;
+        if (row[0] > ctx->max_pre_base) ctx->max_pre_base = row[0];
+        if (row[1] > ctx->max_q16) ctx->max_q16 = row[1];
+        for (uint32_t w = 0; w < MAASO_WMAX; w++)
+            if (row[2 + w] > ctx->max_step) ctx->max_step = row[2 + w];
+    }
     ctx->n_models = M;
     ctx->n_strategies = S;
     ctx->n_rows = R;
@@ -378,6 +393,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     // mapping starts from "everything counted was rejected" and takes the served ones out)
     std::vector<uint64_t> class_tot((size_t)n_classes * 2, 0);
     uint64_t tok_sum = 0;
+    uint32_t max_in = 0;
     for (uint64_t r = 0; r < n; r++) {
         const maaso_request& q = host[r];
         if (q.arrival_us < prev || q.arrival_us > kArrMax)
@@ -388,6 +404,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         if (q.model >= ctx->n_models) return fail(ctx, MAASO_EINVAL, "trace: unknown model");
         if (q.model > max_model) max_model = q.model;
         tok_sum += q.out_tokens;
+        if (q.in_tokens > max_in) max_in = q.in_tokens;
         class_tot[(size_t)q.cls * 2] += 1;
         class_tot[(size_t)q.cls * 2 + 1] += host_rejected_hash((uint32_t)r);
     }
@@ -403,6 +420,9 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     t->n = n;
     t->n_classes = n_classes;
     t->max_model = max_model;
+    t->max_in = max_in;
+    t->small_limits = true;
+    for (int64_t v : cls) t->small_limits = t->small_limits && v < kWalkLimMax;
     {
         const double span_s = n > 1 ? (double)(host[n - 1].arrival_us - host[0].arrival_us) * 1e-6 : 0.0;
         t->tok_rate = span_s > 0.0 ? (double)tok_sum / span_s : 0.0;
@@ -505,6 +525,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         P.trace_scan[t] = traces[t]->d_scan;
         P.trace_class_tot[t] = traces[t]->d_class_tot;
         P.trace_n[t] = (uint32_t)traces[t]->n;
+        P.trace_reqs[t] = traces[t]->d_reqs;
     }
     P.rows = ctx->d_rows;
     P.devices = ctx->d_devices;
@@ -535,8 +556,19 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     // wave is bound by its longest dependent chains, which run faster with fewer warps sharing a
     // scheduler; a larger batch is bound by instruction issue and wants all four.  Lanes needed
     // ~ instances x 1.3 (group widths are powers of two).
-    const bool threads = o.mapping == MAASO_MAP_THREAD || o.mapping == MAASO_MAP_AUTO;
-    const bool groups = o.mapping == MAASO_MAP_GROUP || o.mapping == MAASO_MAP_AUTO;
+    // the default engine runs on the walking kernel, the other readings on the lane-group kernel
+    // and whatever the walking kernel's 32-bit times cannot hold
+    bool walk = !variant && o.mapping == MAASO_MAP_AUTO && C < ctx->thread_min_cand && ctx->max_step < kWalkStepMax;
+    for (uint32_t t = 0; t < n_traces && walk; t++)
+        walk = traces[t]->small_limits &&
+               (double)ctx->max_pre_base + (double)ctx->max_q16 * traces[t]->max_in / 65536.0 + 1.0 < (double)kWalkPreMax;
+    const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
+    P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;
+    P.walk_all = walk && (uint64_t)C * n_traces <= ctx->walk_all ? 1u : 0u;
+    const bool groups = !P.walk_all && (o.mapping == MAASO_MAP_GROUP || o.mapping == MAASO_MAP_AUTO);
+    if (walk) {
+        P.walk_bytes = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes).pool) / kWalkWarps) & ~15u;
+    }
     int group_blocks = ctx->group_blocks;
     if (group_blocks == 0) {
         const uint64_t est_warps = ((cands->n_inst * 13 / 10 + 31) / 32 + 6) * n_traces;
@@ -607,7 +639,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     // unless the batch goes to the threads; whatever the thread kernel's pools cannot hold): one warp per
     // placement with the lane-group code
     int grid_w = 0;
-    if (o.mapping != MAASO_MAP_BLOCK && cands->n_inst > 32) {
+    if (o.mapping != MAASO_MAP_BLOCK && (cands->n_inst > 32 || walk)) {
         // As many warps per SM as the registers allow (8) where the batch is made of large placements (more
         // than 16 instances per placement on average): the kernel waits on dependent chains, and four more
         // warps per SM are worth a third of its time.  Elsewhere 4 per SM, which needs no more scratch than
@@ -619,6 +651,10 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         // a placement that needs this kernel has more than 32 instances (or, thread mapping forced, more state
         // than a warp's pools): the batch cannot hold more of them than instances / 33
         uint64_t max_items_w = (o.mapping == MAASO_MAP_THREAD ? (uint64_t)C : cands->n_inst / 33u) * n_traces;
+        if (walk) {  // and placements that the walking kernel hands over
+            const uint64_t over = ((uint64_t)C * n_traces + 3) / 4;
+            if (over > max_items_w) max_items_w = over;
+        }
         if (max_items_w < 1) max_items_w = 1;
         if ((uint64_t)grid_w > max_items_w) grid_w = (int)max_items_w;
         const size_t need = ((size_t)grid_w * wide_scratch_per_warp() + sizeof(Payload) - 1) / sizeof(Payload);
@@ -641,6 +677,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     P.work_ctr = P.bucket_count + 32;
     P.hist = P.bucket_count + 64;
     P.sm_ctr = P.hist + kHistRows * kCostBins;
+    P.walk_ctr = P.work_ctr + 16;
     P.n_sm = (uint32_t)(ctx->sm_count < 1024 ? ctx->sm_count : 1024);
     P.code = reinterpret_cast<uint32_t*>(sb + off_code);
     P.code2 = reinterpret_cast<uint32_t*>(sb + off_code2);
@@ -651,7 +688,6 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     static_assert(64 + kHistRows * kCostBins + 1024 <= kCounterWords, "counter region");
     P.group_warps = (uint32_t)grid_g * (kGroupThreads / 32);
     P.mapping = o.mapping;  // block, lane groups, threads, or auto (routed by the validation kernels)
-    P.thread_min_cand = ctx->thread_min_cand;
     {   // output tokens per second the trace(s) ask for (mean over the traces of the call)
         double d = 0.0;
         for (uint32_t t = 0; t < n_traces; t++) d += traces[t]->tok_rate;
@@ -672,6 +708,11 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         e = launch_eval_group(P, grid_g, tile, group_blocks, ctx->smem_per_sm, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel launch");
+    }
+    if (walk) {
+        e = launch_eval_walk(P, ctx->sm_count, stream);
+        launches++;
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[2], stream);
     if (threads) {

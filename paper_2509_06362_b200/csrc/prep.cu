@@ -1,6 +1,6 @@
 // Candidate decode + validation (constraints (c) and (d) of Sec. IV-C, table ranges) and
 // sorting of valid candidates into launch buckets; helpers for the per-request dump buffers.
-#include "common.cuh"
+#include "walk.cuh"
 
 namespace maaso {
 
@@ -8,15 +8,17 @@ namespace maaso {
 // (0..9) and its cost bin, `code2` = its bucket among the thread-mapping buckets (10..18) and the
 // bin; 0xFFFFFFFF = it has no such place.  A candidate with both is placed by the batch-wide choice
 // plan_kernel makes (MAASO_MAP_AUTO).
+__device__ __forceinline__ int t_row(int b) { return b < kWalkBucket0 ? b - kThreadBucket0 : kThreadBuckets + b - kWalkBucket0; }
 __global__ void prep_kernel(const EvalParams P) {
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= P.n_cand) return;
     const uint32_t lo = P.offsets[c], hi = P.offsets[c + 1];
     uint32_t status = 0, n = 0, sum_b = 0;
     uint32_t units = 0;  // thread mapping: 16-byte units of cold instance state (per instance 2 + key blocks + minima)
+    uint32_t slot_bytes = 0;  // walking kernel: shared memory of its instances' slots
     uint64_t supply = 0; // decode tokens per second the placement can produce with every slot busy
     const bool variant = (P.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_TBT_MAXGAP | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
-    const bool threads_ok = !variant && (P.mapping == MAASO_MAP_THREAD || P.mapping == MAASO_MAP_AUTO);
+    const bool threads_ok = !variant && (P.mapping == MAASO_MAP_THREAD || (P.mapping == MAASO_MAP_AUTO && !P.walk_bytes));
     const bool groups_ok = P.mapping != MAASO_MAP_THREAD;
     if (hi < lo || hi > P.n_inst) {
         status = MAASO_CAND_EBADINST;  // malformed CSR row
@@ -34,6 +36,7 @@ __global__ void prep_kernel(const EvalParams P) {
                     continue;
                 }
                 sum_b += b;
+                slot_bytes += walk_slot_bytes((b + 7u) >> 3);
                 units += 2u + 2u * ((b + 7u) >> 3) + 2u;
                 supply += (uint64_t)b * 1000000ull / (uint64_t)P.rows[(m * P.n_strategies + s) * kRowStride + 1 + b];
                 devsum += (uint64_t)P.devices[s];
@@ -51,6 +54,12 @@ __global__ void prep_kernel(const EvalParams P) {
             const uint32_t lanes[9] = {32, 24, 16, 12, 8, 6, 4, 2, 1};
             for (int i = 0; i < 9; i++)
                 if (fit >= lanes[i]) { bt = kThreadBucket0 + i; break; }
+        }
+        if (P.walk_bytes) {
+            // one warp's part of the walking kernel's pool, or 2, 4, 8, 16 of them
+            const uint32_t need = walk_region_bytes(P.n_models, n, slot_bytes);
+            for (uint32_t k = 0; n <= 32u && k < (uint32_t)kWalkModes && bt < 0; k++)
+                if (need <= (P.walk_bytes << k)) bt = kWalkBucket0 + (int)k;
         }
         if (P.mapping == MAASO_MAP_BLOCK) bg = n <= 2 ? 6 : (n <= 4 ? 7 : (n <= 8 ? 8 : kGenericBlockBucket));
         else if (groups_ok && n <= 32) bg = n <= 1 ? 0 : 32 - __clz((int)(n - 1));
@@ -84,7 +93,7 @@ __global__ void prep_kernel(const EvalParams P) {
     P.code2[c] = bt >= 0 ? (((uint32_t)bt << 8) | bin) : 0xFFFFFFFFu;
     if (bg >= 0 && bt >= 0) {
         atomicAdd(&P.hist[(bg == kWideBucket ? kHistBothW : kHistBothG + bg) * kCostBins + bin], 1u);
-        atomicAdd(&P.hist[(kHistBothT + bt - kThreadBucket0) * kCostBins + bin], 1u);
+        atomicAdd(&P.hist[(kHistBothT + t_row(bt)) * kCostBins + bin], 1u);
         // loaded beyond what it can decode: most of its requests will be turned away, which the
         // thread mapping does for next to nothing
         atomicAdd(&P.bucket_count[kCtrBoth], 1u);
@@ -94,7 +103,7 @@ __global__ void prep_kernel(const EvalParams P) {
     } else if (bg >= 0) {
         atomicAdd(&P.hist[(kHistOnlyG + bg) * kCostBins + bin], 1u);
     } else {
-        atomicAdd(&P.hist[(kHistOnlyT + bt - kThreadBucket0) * kCostBins + bin], 1u);
+        atomicAdd(&P.hist[(kHistOnlyT + t_row(bt)) * kCostBins + bin], 1u);
     }
 }
 
@@ -125,14 +134,14 @@ __global__ void __launch_bounds__(kCostBins) plan_kernel(const EvalParams P) {
     __shared__ uint32_t tot[6];
     const int bin = threadIdx.x;
     const uint32_t n_both = P.bucket_count[kCtrBoth], n_loaded = P.bucket_count[kCtrLoaded];
-    const bool use_threads = n_loaded >= P.thread_min_cand && 2u * n_loaded >= n_both;
+    const bool use_threads = P.walk_all || (n_loaded >= P.thread_min_cand && 2u * n_loaded >= n_both);
     // final counts of this bin per bucket
     uint32_t cnt[kNumBuckets];
     for (int b = 0; b < kThreadBucket0; b++)
         cnt[b] = P.hist[(kHistOnlyG + b) * kCostBins + bin] + (use_threads ? 0u : P.hist[(kHistBothG + b) * kCostBins + bin]);
-    for (int b = kThreadBucket0; b < kThreadBucket0 + kThreadBuckets; b++)
-        cnt[b] = P.hist[(kHistOnlyT + b - kThreadBucket0) * kCostBins + bin] +
-                 (use_threads ? P.hist[(kHistBothT + b - kThreadBucket0) * kCostBins + bin] : 0u);
+    for (int b = kThreadBucket0; b < kNumBuckets; b++)
+        if (b != kWideBucket)
+            cnt[b] = P.hist[(kHistOnlyT + t_row(b)) * kCostBins + bin] + (use_threads ? P.hist[(kHistBothT + t_row(b)) * kCostBins + bin] : 0u);
     cnt[kWideBucket] = P.hist[kHistWide * kCostBins + bin] + (use_threads ? 0u : P.hist[kHistBothW * kCostBins + bin]);
     uint32_t cut = 0;  // bins below `cut` are promoted
     uint32_t narrow = 0;
