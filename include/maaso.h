@@ -353,7 +353,7 @@ MAASO_API int maaso_partition(maaso_ctx *ctx, const maaso_trace *trace, uint32_t
  * a latency-critical serving loop where an allocation would synchronise the device, or a
  * process that is already close to its memory limit.  Same inputs, outputs and ordering
  * as maaso_topk, no context needed; the partial lists of the selection passes live in a
- * fixed array of about 0.8 MB inside the library image (every GPU that loads the library
+ * fixed array of about 0.4 MB inside the library image (every GPU that loads the library
  * holds it until the process exits) instead of context scratch memory.
  * Limits: n_cand <= MAASO_NOALLOC_MAX_CAND and k <= MAASO_NOALLOC_MAX_K; anything larger
  * returns MAASO_ETOOBIG and does nothing.  The call uses the current CUDA device and calls
