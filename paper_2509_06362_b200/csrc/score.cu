@@ -53,25 +53,64 @@ struct PermilleList {
     uint32_t v[16];
 };
 
-// One thread per candidate: cumulative counts over the 64 bins, one pass per requested rank.
-__global__ void ttft_percentile_kernel(const uint32_t* hist, uint64_t n, PermilleList pm, uint32_t n_p, int64_t* out) {
-    const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const uint32_t* h = hist + c * MAASO_TTFT_BINS;
-    uint64_t total = 0;
-    for (int b = 0; b < MAASO_TTFT_BINS; b++) total += h[b];
-    for (uint32_t j = 0; j < n_p; j++) {
-        int64_t r = -1;
-        if (total > 0) {
-            uint64_t target = ((uint64_t)pm.v[j] * total + 999u) / 1000u;
-            if (target < 1) target = 1;
-            uint64_t cum = 0;
-            for (int b = 0; b < MAASO_TTFT_BINS; b++) {
-                cum += h[b];
-                if (cum >= target) { r = ttft_bin_upper((uint32_t)b); break; }
-            }
+// Eight lanes per candidate: lane l holds bins 8l .. 8l+7 (two 16-byte loads; a warp reads four histograms), a scan
+// over the lanes gives the cumulative counts, lane j works out the target of rank j and keeps the bin it falls
+// into.  Bound by the read of the histograms; with 16 lanes and every lane working out every target it was bound
+// by instructions (10^6 histograms: 74 us, 218 that way, 496 with one thread per candidate).
+template <class U>
+__device__ __forceinline__ void percentiles_of(const U (&c)[8], U incl, uint32_t l, const PermilleList& pm, uint32_t n_p, int64_t* o, bool write) {
+    const U below = incl - c[7], total = __shfl_sync(0xFFFFFFFFu, incl, 7, 8);
+    for (uint32_t j0 = 0; j0 < n_p; j0 += 8u) {
+        const uint32_t p = j0 + l < n_p ? pm.v[j0 + l] : 1u;
+        U target = (U)(((uint64_t)p * total + 999u) / 1000u);
+        if (target < 1) target = 1;
+        uint32_t bin = 0;
+        for (uint32_t j = 0; j < 8u && j0 + j < n_p; j++) {
+            const U t = __shfl_sync(0xFFFFFFFFu, target, (int)j, 8);
+            uint32_t k = 8u * l;
+#pragma unroll
+            for (int i = 0; i < 7; i++) k += below + c[i] < t ? 1u : 0u;
+            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, below < t && t <= incl) >> (threadIdx.x & 24u);
+            const uint32_t found = __shfl_sync(0xFFFFFFFFu, k, __ffs((int)(votes & 0xFFu)) - 1, 8);
+            if (j == l) bin = found;
         }
-        out[c * n_p + j] = r;
+        if (write && j0 + l < n_p) o[j0 + l] = total ? ttft_bin_upper(bin) : -1;
+    }
+}
+
+__global__ void __launch_bounds__(256) ttft_percentile_kernel(const uint32_t* hist, uint64_t n, const __grid_constant__ PermilleList pm, uint32_t n_p, int64_t* out) {
+    const uint64_t c = ((uint64_t)blockIdx.x * 256u + threadIdx.x) >> 3;
+    const uint32_t l = threadIdx.x & 7u;
+    uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+    if (c < n) {
+        const uint4* h = reinterpret_cast<const uint4*>(hist + c * MAASO_TTFT_BINS) + 2u * l;
+        a = __ldg(h);
+        b = __ldg(h + 1);
+    }
+    const bool small = (a.x | a.y | a.z | a.w | b.x | b.y | b.z | b.w) < (1u << 25);  // 64 of them stay below 2^31
+    int64_t* const o = out + c * n_p;
+    if (__all_sync(0xFFFFFFFFu, small)) {
+        uint32_t s[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 1; i < 8; i++) s[i] += s[i - 1];
+        uint32_t incl = s[7];
+#pragma unroll
+        for (int k = 1; k < 8; k <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, k, 8);
+            if (l >= (uint32_t)k) incl += v;
+        }
+        percentiles_of(s, incl, l, pm, n_p, o, c < n);
+    } else {
+        unsigned long long s[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 1; i < 8; i++) s[i] += s[i - 1];
+        unsigned long long incl = s[7];
+#pragma unroll
+        for (int k = 1; k < 8; k <<= 1) {
+            const unsigned long long v = __shfl_up_sync(0xFFFFFFFFu, incl, k, 8);
+            if (l >= (uint32_t)k) incl += v;
+        }
+        percentiles_of(s, incl, l, pm, n_p, o, c < n);
     }
 }
 
@@ -79,7 +118,7 @@ cudaError_t launch_ttft_percentiles(const uint32_t* hist, uint64_t n, const uint
                                     int64_t* out, cudaStream_t stream) {
     PermilleList pm;
     for (uint32_t j = 0; j < 16; j++) pm.v[j] = j < n_p ? permille[j] : 0;
-    if (n) ttft_percentile_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(hist, n, pm, n_p, out);
+    if (n) ttft_percentile_kernel<<<(unsigned)((n + 31) / 32), 256, 0, stream>>>(hist, n, pm, n_p, out);
     return cudaGetLastError();
 }
 
