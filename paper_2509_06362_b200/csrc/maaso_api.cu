@@ -57,6 +57,7 @@ struct maaso_trace {
     uint64_t n;
     uint32_t n_classes;
     uint32_t max_model;
+    std::vector<uint32_t> h_count;  // [n_classes][MAASO_MAX_MODELS] requests
     uint32_t max_in;  // most input tokens of a request
     bool small_limits;  // every finite SLO limit fits the walking kernel's 32-bit times
     double tok_rate;  // output tokens per second the trace asks for (routing hint of MAASO_MAP_AUTO)
@@ -394,6 +395,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     std::vector<uint64_t> class_tot((size_t)n_classes * 2, 0);
     uint64_t tok_sum = 0;
     uint32_t max_in = 0;
+    std::vector<uint32_t> count((size_t)n_classes * MAASO_MAX_MODELS, 0);
     for (uint64_t r = 0; r < n; r++) {
         const maaso_request& q = host[r];
         if (q.arrival_us < prev || q.arrival_us > kArrMax)
@@ -405,6 +407,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         if (q.model > max_model) max_model = q.model;
         tok_sum += q.out_tokens;
         if (q.in_tokens > max_in) max_in = q.in_tokens;
+        count[(size_t)q.cls * MAASO_MAX_MODELS + q.model]++;
         class_tot[(size_t)q.cls * 2] += 1;
         class_tot[(size_t)q.cls * 2 + 1] += host_rejected_hash((uint32_t)r);
     }
@@ -420,6 +423,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     t->n = n;
     t->n_classes = n_classes;
     t->max_model = max_model;
+    t->h_count = std::move(count);
     t->max_in = max_in;
     t->small_limits = true;
     for (int64_t v : cls) t->small_limits = t->small_limits && v < kWalkLimMax;
@@ -879,6 +883,8 @@ struct DeployProblem {
     uint32_t* istar_inst;
 };
 
+constexpr uint32_t kAhead = 8;  // instances a chain can be ahead of its accepted placement in one round
+
 static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const DeployProblem* prob, uint32_t n_prob,
                             const maaso_config* configs, uint32_t n_configs, const maaso_score_params* score,
                             uint32_t flags) {
@@ -898,10 +904,11 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
 
     // device staging: offsets | inst | mask | results | scores | rejected-by-model
     const size_t C = (size_t)n_configs * n_prob;
-    const size_t cap_spec = 1u << 16;  // speculative follow-ups only while the batch stays this small
-    const size_t per_chain = C * (2 + (size_t)ctx->n_models) <= cap_spec ? 2 + (size_t)ctx->n_models : 1;
-    const size_t cap_cand = C * per_chain > n_prob ? C * per_chain : n_prob;
-    const size_t cap_inst = cap_cand * (MAASO_MAX_INSTANCES + 2);
+    // Placements scored per round.  A round takes as long as its longest replay, and up to about two warps per
+    // scheduler share one without slowing it down much: that is the room for what the chains may need next.
+    const size_t room = (size_t)ctx->sm_count * 8;
+    const size_t cap_cand = C > room ? C : room;
+    const size_t cap_inst = cap_cand * (MAASO_MAX_INSTANCES + kAhead);
     size_t off = 0;
     const size_t o_off = off;  off = align_up(off + (cap_cand + 1) * 4, 256);
     const size_t o_inst = off; off = align_up(off + cap_inst * 4, 256);
@@ -951,13 +958,6 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
     // a problem without a mask counts every class (masks are ignored anyway beyond 32 classes)
     auto mask_of = [&](uint32_t p) { return prob[p].use_mask ? prob[p].class_mask : 0xFFFFFFFFu; };
 
-    // R_res = R_x before anything is deployed: the empty placement rejects every request of R_x
-    for (uint32_t p = 0; p <= n_prob; p++) h_off[p] = 0;
-    for (uint32_t p = 0; p < n_prob; p++) h_mask[p] = mask_of(p);
-    h_inst.clear();
-    rc = run_batch(n_prob);
-    if (rc != MAASO_OK) return rc;
-
     struct Step {
         uint32_t k;    // device count of the placement the step leaves (the one stored under Phi*[k], I*[k])
         uint32_t len;  // instances of the accepted placement after the step
@@ -972,48 +972,139 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
         uint32_t dev;
         uint32_t gpus;  // device count of the chain's problem
         uint32_t mask;
-        int tentative;  // model of the tentative instance, -1 = chain finished
+        uint32_t gain[MAASO_MAX_MODELS];  // requests of the model that the last accepted instance of it took on
+        bool done;
     };
     std::vector<Chain> chains(C);  // chain p * n_configs + c
-    for (uint32_t p = 0; p < n_prob; p++)
+    for (uint32_t p = 0; p < n_prob; p++) {
+        std::vector<uint32_t> unserved0(MAASO_MAX_MODELS, 0);
+        for (uint32_t k = 0; k < trace->n_classes; k++)
+            if (!prob[p].use_mask || trace->n_classes > 32 || ((prob[p].class_mask >> k) & 1u))
+                for (uint32_t m = 0; m < MAASO_MAX_MODELS; m++) unserved0[m] += trace->h_count[(size_t)k * MAASO_MAX_MODELS + m];
         for (uint32_t c = 0; c < n_configs; c++) {
             Chain& ch = chains[(size_t)p * n_configs + c];
             memset(ch.sat, 0, sizeof(ch.sat));
-            memcpy(ch.unserved, h_rbm.data() + (size_t)p * MAASO_MAX_MODELS, sizeof(ch.unserved));
+            memset(ch.gain, 0, sizeof(ch.gain));
+            // R_res = R_x before anything is deployed: nothing is served yet
+            memcpy(ch.unserved, unserved0.data(), sizeof(ch.unserved));
             ch.phi = 0.0;
             ch.dev = (uint32_t)ctx->h_devices[configs[c].strategy];
             ch.gpus = prob[p].gpus;
             ch.mask = mask_of(p);
-            ch.tentative = 0;
+            ch.done = false;
         }
-    // Two greedy steps per batch.  Besides its tentative placement A = I + m' every chain also
-    // proposes what its NEXT step would score, for both outcomes of this one: if A is rejected the
-    // next tentative model is already known (m' becomes saturated, nothing else changes): B; if A is
-    // accepted the unserved counts change, so the next model is not known: I + m' + m for every model
-    // m still open.  After the batch the first step is taken with A's result and the second with the
-    // speculative result that matches the actual state.  The batches are a few times larger, the
-    // number of trace replays halves; the steps taken are those of the sequential algorithm.
+    }
+    // Several greedy steps per batch.  A chain's next tentative placement is known; what it will propose after that
+    // depends on whether this one is accepted and on what it leaves unserved.  So every chain also submits the
+    // placements it is most likely to need next (plan_ahead), the batch is scored, and steps are taken for as long as
+    // the placement the chain really proposes is among the scored ones: exactly the steps of the sequential algorithm,
+    // with fewer trace replays one after the other.
     const uint32_t n_models = ctx->n_models;
-    const bool speculate = C * (2 + (size_t)n_models) <= cap_spec;
-    auto next_model = [&](const Chain& ch, const bool* sat, size_t len) -> int {
+    auto next_model = [&](const Chain& ch, const bool* sat, const uint32_t* unserved, size_t len) -> int {
         int mp = -1;  // model with the most unserved requests among the non-saturated ones
         if ((uint64_t)len * ch.dev < ch.gpus && len <= MAASO_MAX_INSTANCES)
             for (uint32_t m = 0; m < n_models; m++)
-                if (!sat[m] && (mp < 0 || ch.unserved[m] > ch.unserved[mp])) mp = (int)m;
+                if (!sat[m] && (mp < 0 || unserved[m] > unserved[mp])) mp = (int)m;
         return mp;
     };
+    // A scored placement of the round: the chain's accepted instances plus `seq` (models, in order).
+    struct Node {
+        uint32_t len;
+        uint8_t seq[kAhead];
+        int index;  // in the batch
+    };
+    // A point the chain may reach in this round, with a guess how likely.
+    struct State {
+        uint32_t len;
+        uint8_t seq[kAhead];
+        bool sat[MAASO_MAX_MODELS];
+        uint32_t unserved[MAASO_MAX_MODELS];
+        bool guessed;  // `unserved` is an estimate
+        double p;
+    };
+    std::vector<std::vector<Node>> ahead(C);
+    std::vector<State> frontier;
     uint32_t n_batch = 0;
     std::vector<char> batch_over;  // the placement needs more devices than its problem has
-    auto propose = [&](const Chain& ch, const maaso_config& cf, int m1, int m2) -> int {
-        // candidate I + m1 (+ m2); returns its index in the batch
+    auto find_node = [&](const std::vector<Node>& v, const uint8_t* seq, uint32_t len) -> int {
+        for (const Node& nd : v)
+            if (nd.len == len && memcmp(nd.seq, seq, len) == 0) return nd.index;
+        return -1;
+    };
+    auto propose = [&](const Chain& ch, const maaso_config& cf, const uint8_t* seq, uint32_t len) -> int {
         h_off[n_batch] = (uint32_t)h_inst.size();
         h_mask[n_batch] = ch.mask;
         h_inst.insert(h_inst.end(), ch.inst.begin(), ch.inst.end());
-        const uint32_t w = ((cf.strategy & 0xFFu) << 4) | ((cf.batch & 0xFFu) << 12);
-        h_inst.push_back(((uint32_t)m1 & 0xFu) | w);
-        if (m2 >= 0) h_inst.push_back(((uint32_t)m2 & 0xFu) | w);
-        batch_over.push_back(((uint64_t)ch.inst.size() + (m2 >= 0 ? 2 : 1)) * ch.dev > ch.gpus ? 1 : 0);
+        for (uint32_t i = 0; i < len; i++)
+            h_inst.push_back(((uint32_t)seq[i] & 0xFu) | ((cf.strategy & 0xFFu) << 4) | ((cf.batch & 0xFFu) << 12));
+        batch_over.push_back(((uint64_t)ch.inst.size() + len) * ch.dev > ch.gpus ? 1 : 0);
         return (int)n_batch++;
+    };
+    // Adds up to `most` placements for one chain: the states it may reach, likeliest first.  Accepted three times in
+    // four; the next model after an acceptance is the one with the most unserved requests by estimate (an instance of
+    // a model serves about what the last one accepted did) three times in five.  The guesses decide only what is
+    // scored beforehand.
+    auto plan_ahead = [&](const Chain& ch, const maaso_config& cf, std::vector<Node>& out, size_t most) {
+        frontier.clear();
+        State root;
+        memset(&root, 0, sizeof(root));
+        memcpy(root.sat, ch.sat, sizeof(root.sat));
+        memcpy(root.unserved, ch.unserved, sizeof(root.unserved));
+        root.p = 1.0;
+        frontier.push_back(root);
+        auto push = [&](const State& x) {
+            if (x.p >= 0.002) frontier.push_back(x);
+        };
+        while (out.size() < most && !frontier.empty()) {
+            size_t at = 0;
+            for (size_t i = 1; i < frontier.size(); i++)
+                if (frontier[i].p > frontier[at].p) at = i;
+            const State st = frontier[at];
+            frontier[at] = frontier.back();
+            frontier.pop_back();
+            bool tried[MAASO_MAX_MODELS] = {false};
+            double p_left = st.p;
+            for (uint32_t r = 0; r < (st.guessed ? n_models : 1u) && out.size() < most; r++) {
+                bool skip[MAASO_MAX_MODELS];
+                for (uint32_t m = 0; m < n_models; m++) skip[m] = st.sat[m] || tried[m];
+                const int m = next_model(ch, skip, st.unserved, ch.inst.size() + st.len);
+                if (m < 0) break;
+                // the r-th likeliest model: a state of its own in the queue when it is not the first
+                if (r > 0) {
+                    State later = st;
+                    for (uint32_t k = 0; k < n_models; k++)
+                        if (tried[k]) later.unserved[k] = 0;  // looked at after the models not yet tried
+                    later.p = p_left;
+                    later.guessed = true;
+                    push(later);
+                    break;
+                }
+                tried[m] = true;
+                const double p_m = st.guessed ? 0.6 * st.p : st.p;
+                p_left = st.p - p_m;
+                State nx = st;
+                nx.seq[nx.len++] = (uint8_t)m;
+                if (find_node(out, nx.seq, nx.len) < 0) {
+                    Node nd;
+                    memset(&nd, 0, sizeof(nd));
+                    nd.len = nx.len;
+                    memcpy(nd.seq, nx.seq, sizeof(nd.seq));
+                    nd.index = propose(ch, cf, nx.seq, nx.len);
+                    out.push_back(nd);
+                }
+                State rejected = st;  // the model is saturated, nothing else changes
+                rejected.sat[m] = true;
+                rejected.p = 0.25 * p_m;
+                push(rejected);
+                if (nx.len < kAhead) {
+                    const uint32_t gain = ch.gain[m] ? ch.gain[m] : nx.unserved[m] / 2;
+                    nx.unserved[m] -= gain < nx.unserved[m] ? gain : nx.unserved[m];
+                    nx.guessed = true;
+                    nx.p = 0.75 * p_m;
+                    push(nx);
+                }
+            }
+        }
     };
     auto take_step = [&](Chain& ch, int model, uint32_t word, int j) {
         Step sp;
@@ -1024,7 +1115,9 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
         if (sc > ch.phi) {  // accept the new instance
             ch.phi = sc;
             ch.inst.push_back(word);
-            memcpy(ch.unserved, h_rbm.data() + (size_t)j * MAASO_MAX_MODELS, sizeof(ch.unserved));
+            const uint32_t* left = h_rbm.data() + (size_t)j * MAASO_MAX_MODELS;
+            ch.gain[model] = ch.unserved[model] > left[model] ? ch.unserved[model] - left[model] : 0;
+            memcpy(ch.unserved, left, sizeof(ch.unserved));
             accepted = true;
         } else {
             ch.sat[model] = true;  // stop deploying this model
@@ -1035,60 +1128,38 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
         ch.steps.push_back(sp);
         return accepted;
     };
-    struct Plan {
-        uint32_t chain;
-        int m1, a;           // tentative model, batch index of A
-        int mb, b;           // model and batch index of the "A rejected" follow-up (-1: none)
-        int c[MAASO_MAX_MODELS];  // batch index of the "A accepted, then model m" follow-up (-1: none)
-    };
-    std::vector<Plan> plans;
     for (;;) {
-        // every unfinished chain proposes its next tentative placement I' = I + (m', P, B)
-        plans.clear();
         batch_over.clear();
         h_inst.clear();
         n_batch = 0;
-        for (size_t x = 0; x < C; x++) {
-            Chain& ch = chains[x];
-            const maaso_config& cf = configs[x % n_configs];
-            if (ch.tentative < 0) continue;
-            const int mp = next_model(ch, ch.sat, ch.inst.size());
-            ch.tentative = mp;
-            if (mp < 0) continue;
-            Plan pl;
-            pl.chain = (uint32_t)x;
-            pl.m1 = mp;
-            pl.a = propose(ch, cf, mp, -1);
-            pl.mb = -1;
-            pl.b = -1;
-            for (uint32_t m = 0; m < MAASO_MAX_MODELS; m++) pl.c[m] = -1;
-            if (speculate) {
-                bool sat2[MAASO_MAX_MODELS];
-                memcpy(sat2, ch.sat, sizeof(sat2));
-                sat2[mp] = true;
-                pl.mb = next_model(ch, sat2, ch.inst.size());
-                if (pl.mb >= 0) pl.b = propose(ch, cf, pl.mb, -1);
-                const size_t len2 = ch.inst.size() + 1;
-                if ((uint64_t)len2 * ch.dev < ch.gpus && len2 <= MAASO_MAX_INSTANCES)
-                    for (uint32_t m = 0; m < n_models; m++)
-                        if (!ch.sat[m]) pl.c[m] = propose(ch, cf, mp, (int)m);
-            }
-            plans.push_back(pl);
+        size_t active = 0;
+        for (Chain& ch : chains) {
+            if (!ch.done && next_model(ch, ch.sat, ch.unserved, ch.inst.size()) < 0) ch.done = true;
+            active += ch.done ? 0 : 1;
         }
-        if (plans.empty()) break;
+        if (active == 0) break;
+        const size_t most = room / active > 1 ? room / active : 1;
+        for (size_t x = 0; x < C; x++) {
+            ahead[x].clear();
+            if (!chains[x].done) plan_ahead(chains[x], configs[x % n_configs], ahead[x], most);
+        }
         h_off[n_batch] = (uint32_t)h_inst.size();
         rc = run_batch(n_batch);
         if (rc != MAASO_OK) return rc;
-        for (const Plan& pl : plans) {
-            Chain& ch = chains[pl.chain];
-            const maaso_config& cf = configs[pl.chain % n_configs];
-            const uint32_t w = ((cf.strategy & 0xFFu) << 4) | ((cf.batch & 0xFFu) << 12);
-            const bool accepted = take_step(ch, pl.m1, ((uint32_t)pl.m1 & 0xFu) | w, pl.a);
-            if (!speculate) continue;
-            const int m2 = next_model(ch, ch.sat, ch.inst.size());  // from the state the first step left
-            if (m2 < 0) continue;  // the chain ends; the next round marks it finished
-            const int j = accepted ? pl.c[m2] : (m2 == pl.mb ? pl.b : -1);
-            if (j >= 0) take_step(ch, m2, ((uint32_t)m2 & 0xFu) | w, j);
+        for (size_t x = 0; x < C; x++) {
+            Chain& ch = chains[x];
+            if (ch.done) continue;
+            const maaso_config& cf = configs[x % n_configs];
+            uint8_t seq[kAhead + 1];
+            uint32_t len = 0;
+            for (;;) {
+                const int m = next_model(ch, ch.sat, ch.unserved, ch.inst.size());
+                if (m < 0 || len >= kAhead) break;
+                seq[len] = (uint8_t)m;
+                const int j = find_node(ahead[x], seq, len + 1);
+                if (j < 0) break;
+                if (take_step(ch, m, ((uint32_t)m & 0xFu) | ((cf.strategy & 0xFFu) << 4) | ((cf.batch & 0xFFu) << 12), j)) len++;
+            }
         }
     }
     // Phi*[k] / I*[k]: replay the steps configuration by configuration, as the sequential algorithm
@@ -1245,30 +1316,14 @@ MAASO_API int maaso_partition(maaso_ctx* ctx, const maaso_trace* trace, uint32_t
     if (!ctx || !trace || !out_g || !out_phi || !len_t || !inst_t || !len_l || !inst_l || gpus > 4096)
         return MAASO_EINVAL;
     if (trace->owner != ctx) return fail(ctx, MAASO_ESTATE, "partition: trace belongs to another context");
-    // |R_t|, |R_l|: what the empty placement counts under each mask
-    DeviceGuard g(ctx->device);
-    int rc = grow(ctx, &ctx->deploy, &ctx->deploy_bytes, 4096);
-    if (rc != MAASO_OK) return rc;
-    unsigned char* sb = static_cast<unsigned char*>(ctx->deploy);
-    const uint32_t h_off[3] = {0, 0, 0}, h_mask[2] = {mask_t, mask_l};
-    maaso_result h_res[2];
-    cudaStream_t st = ctx->own_stream;
-    cudaError_t e = cudaMemcpyAsync(sb, h_off, sizeof(h_off), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sb + 256, h_mask, sizeof(h_mask), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "partition: upload");
-    maaso_cand_batch b;
-    memset(&b, 0, sizeof(b));
-    b.offsets = reinterpret_cast<const uint32_t*>(sb);
-    b.inst = reinterpret_cast<const uint32_t*>(sb + 512);
-    b.class_mask = reinterpret_cast<const uint32_t*>(sb + 256);
-    b.n_cand = 2;
-    b.budget = gpus;
-    rc = maaso_eval_placements(ctx, trace, &b, nullptr, reinterpret_cast<maaso_result*>(sb + 1024), st);
-    if (rc != MAASO_OK) return rc;
-    e = cudaMemcpyAsync(h_res, sb + 1024, sizeof(h_res), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "partition: download");
-    const uint64_t n_t = h_res[0].n_counted, n_l = h_res[1].n_counted;
+    // |R_t|, |R_l|: the requests of each mask's classes (masks are ignored beyond 32 classes)
+    uint64_t n_t = 0, n_l = 0;
+    for (uint32_t k = 0; k < trace->n_classes; k++)
+        for (uint32_t m = 0; m < MAASO_MAX_MODELS; m++) {
+            const uint64_t n = trace->h_count[(size_t)k * MAASO_MAX_MODELS + m];
+            if (trace->n_classes > 32 || ((mask_t >> k) & 1u)) n_t += n;
+            if (trace->n_classes > 32 || ((mask_l >> k) & 1u)) n_l += n;
+        }
     const uint32_t gl_max = (n_t + n_l) ? (uint32_t)((n_l * (uint64_t)gpus) / (n_t + n_l)) : 0;
 
     const size_t cells = (size_t)gpus + 1;
@@ -1284,7 +1339,7 @@ MAASO_API int maaso_partition(maaso_ctx* ctx, const maaso_trace* trace, uint32_t
         {gpus, 1, mask_t, phi_t.data(), ln_t.data(), in_t.data()},
         {gpus, 1, mask_t | mask_l, phi_h.data(), ln_h.data(), in_h.data()},
     };
-    rc = ins_deploy_multi(ctx, trace, probs, baseline ? 3u : 2u, configs, n_configs, score, flags);
+    const int rc = ins_deploy_multi(ctx, trace, probs, baseline ? 3u : 2u, configs, n_configs, score, flags);
     double phi_opt = 0.0;
     if (rc == MAASO_OK && baseline)  // homogeneous deployment as the fallback
         for (uint32_t k = 0; k <= gpus; k++)
