@@ -11,8 +11,7 @@
 
 namespace maaso {
 cudaError_t launch_prep(const EvalParams& P, const uint32_t* dump_idx, cudaStream_t stream, int* launches);
-cudaError_t launch_rej_hash(uint64_t* out, uint32_t n);
-cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint32_t n);
+cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n);
 cudaError_t launch_scan_trace(const uint4* reqs, const int64_t* classes, uint4* scan, uint32_t n);
 size_t scan_trace_units(uint32_t n);
 cudaError_t launch_eval_group(const EvalParams& P, int grid, int tile_recs, int blocks_per_sm, int smem_per_sm,
@@ -47,6 +46,8 @@ using namespace maaso;
 
 struct maaso_trace {
     maaso_ctx* owner;
+    void* mem;         // one allocation, everything below is a part of it
+    size_t mem_bytes;
     uint4* d_reqs;
     int64_t* d_classes;
     uint64_t* d_rej_hash;
@@ -76,6 +77,8 @@ struct maaso_ctx {
     std::vector<int32_t> h_min_devices;
     std::vector<int32_t> h_rows;
     std::vector<maaso_trace*> traces;
+    void* spare;          // memory of the trace freed last (at most kSpareMax bytes), for the next one to load
+    size_t spare_bytes;
     void* scratch;
     size_t scratch_bytes;
     void* topk_scratch;
@@ -149,6 +152,8 @@ int grow(maaso_ctx* ctx, void** buf, size_t* have, size_t need) {
     return MAASO_OK;
 }
 
+constexpr size_t kSpareMax = (size_t)256 << 20;
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Checksum term of "request r was rejected": the SplitMix64 output mixer (public domain) of
@@ -177,6 +182,8 @@ MAASO_API int maaso_create(maaso_ctx** out, int cuda_device) {
     ctx->device = cuda_device;
     ctx->has_profile = false;
     ctx->d_rows = ctx->d_devices = ctx->d_min_devices = nullptr;
+    ctx->spare = nullptr;
+    ctx->spare_bytes = 0;
     ctx->scratch = ctx->topk_scratch = ctx->stage = ctx->deploy = nullptr;
     ctx->scratch_bytes = ctx->topk_scratch_bytes = ctx->stage_bytes = ctx->deploy_bytes = 0;
     ctx->launches = 0;
@@ -269,12 +276,14 @@ MAASO_API void maaso_free_trace(maaso_ctx* ctx, maaso_trace* trace) {
             ctx->traces.erase(ctx->traces.begin() + i);
             break;
         }
-    if (trace->d_reqs) cudaFree(trace->d_reqs);
-    if (trace->d_classes) cudaFree(trace->d_classes);
-    if (trace->d_rej_hash) cudaFree(trace->d_rej_hash);
-    if (trace->d_cooked) cudaFree(trace->d_cooked);
-    if (trace->d_scan) cudaFree(trace->d_scan);
-    if (trace->d_class_tot) cudaFree(trace->d_class_tot);
+    // a placer loads a trace per request window: its memory is kept for the next one
+    if (trace->mem_bytes <= kSpareMax) {
+        if (ctx->spare) cudaFree(ctx->spare);
+        ctx->spare = trace->mem;
+        ctx->spare_bytes = trace->mem_bytes;
+    } else {
+        cudaFree(trace->mem);
+    }
     delete trace;
 }
 
@@ -283,6 +292,7 @@ MAASO_API void maaso_destroy(maaso_ctx* ctx) {
     DeviceGuard g(ctx->device);
     cudaDeviceSynchronize();
     while (!ctx->traces.empty()) maaso_free_trace(ctx, ctx->traces.back());
+    if (ctx->spare) cudaFree(ctx->spare);
     if (ctx->d_rows) cudaFree(ctx->d_rows);
     if (ctx->d_devices) cudaFree(ctx->d_devices);
     if (ctx->d_min_devices) cudaFree(ctx->d_min_devices);
@@ -414,12 +424,6 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     maaso_trace* t = new (std::nothrow) maaso_trace();
     if (!t) return MAASO_ENOMEM;
     t->owner = ctx;
-    t->d_reqs = nullptr;
-    t->d_classes = nullptr;
-    t->d_rej_hash = nullptr;
-    t->d_cooked = nullptr;
-    t->d_scan = nullptr;
-    t->d_class_tot = nullptr;
     t->n = n;
     t->n_classes = n_classes;
     t->max_model = max_model;
@@ -432,29 +436,50 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         t->tok_rate = span_s > 0.0 ? (double)tok_sum / span_s : 0.0;
     }
     t->h_classes = cls;
-    cudaError_t e = cudaMalloc(&t->d_reqs, (n ? n : 1) * sizeof(maaso_request));
-    if (e == cudaSuccess) e = cudaMalloc(&t->d_classes, cls.size() * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&t->d_rej_hash, (n ? n : 1) * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&t->d_cooked, (n ? n : 1) * 16 * kCookedWords);
-    if (e == cudaSuccess) e = cudaMalloc(&t->d_scan, scan_trace_units((uint32_t)n) * 16);
-    if (e == cudaSuccess) e = cudaMalloc(&t->d_class_tot, (size_t)n_classes * 16);
-    if (e == cudaSuccess) e = cudaMemcpy(t->d_class_tot, class_tot.data(), (size_t)n_classes * 16, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = launch_rej_hash(t->d_rej_hash, (uint32_t)n);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e == cudaSuccess && n)
-        e = cudaMemcpy(t->d_reqs, reqs, n * sizeof(maaso_request),
-                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(t->d_classes, cls.data(), cls.size() * 8, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = launch_cook_trace(t->d_reqs, t->d_classes, t->d_cooked, (uint32_t)n);
+    // requests | prepared records | scan tiles | rejection hashes | per-class totals, SLO classes
+    size_t off = 0;
+    const size_t n1 = n ? n : 1;
+    const size_t o_reqs = off;   off = align_up(off + n1 * sizeof(maaso_request), 256);
+    const size_t o_cooked = off; off = align_up(off + n1 * 16 * kCookedWords, 256);
+    const size_t o_scan = off;   off = align_up(off + scan_trace_units((uint32_t)n) * 16, 256);
+    const size_t o_hash = off;   off = align_up(off + n1 * 8, 256);
+    const size_t o_small = off;  off = align_up(off + (class_tot.size() + cls.size()) * 8, 256);
+    cudaError_t e = cudaSuccess;
+    if (ctx->spare && ctx->spare_bytes >= off && ctx->spare_bytes / 4 <= off) {
+        t->mem = ctx->spare;
+        t->mem_bytes = ctx->spare_bytes;
+        ctx->spare = nullptr;
+    } else {
+        t->mem_bytes = align_up(off, (size_t)1 << 16);
+        e = cudaMalloc(&t->mem, t->mem_bytes);
+        if (e == cudaErrorMemoryAllocation && ctx->spare) {
+            cudaGetLastError();
+            cudaFree(ctx->spare);
+            ctx->spare = nullptr;
+            e = cudaMalloc(&t->mem, t->mem_bytes);
+        }
+        if (e != cudaSuccess) {
+            delete t;
+            return cuda_fail(ctx, e, "trace alloc");
+        }
+    }
+    unsigned char* const mem = static_cast<unsigned char*>(t->mem);
+    t->d_reqs = reinterpret_cast<uint4*>(mem + o_reqs);
+    t->d_cooked = reinterpret_cast<uint4*>(mem + o_cooked);
+    t->d_scan = reinterpret_cast<uint4*>(mem + o_scan);
+    t->d_rej_hash = reinterpret_cast<uint64_t*>(mem + o_hash);
+    t->d_class_tot = reinterpret_cast<uint64_t*>(mem + o_small);
+    t->d_classes = reinterpret_cast<int64_t*>(mem + o_small) + class_tot.size();
+    std::vector<int64_t> small(class_tot.begin(), class_tot.end());
+    small.insert(small.end(), cls.begin(), cls.end());
+    if (n) e = cudaMemcpyAsync(t->d_reqs, reqs, n * sizeof(maaso_request),
+                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(mem + o_small, small.data(), small.size() * 8, cudaMemcpyHostToDevice, cudaStreamLegacy);
+    if (e == cudaSuccess) e = launch_cook_trace(t->d_reqs, t->d_classes, t->d_cooked, t->d_rej_hash, (uint32_t)n);
     if (e == cudaSuccess) e = launch_scan_trace(t->d_reqs, t->d_classes, t->d_scan, (uint32_t)n);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
-        if (t->d_cooked) cudaFree(t->d_cooked);
-        if (t->d_scan) cudaFree(t->d_scan);
-        if (t->d_class_tot) cudaFree(t->d_class_tot);
-        if (t->d_reqs) cudaFree(t->d_reqs);
-        if (t->d_classes) cudaFree(t->d_classes);
-        if (t->d_rej_hash) cudaFree(t->d_rej_hash);
+        cudaFree(t->mem);
         delete t;
         return cuda_fail(ctx, e, "trace upload");
     }

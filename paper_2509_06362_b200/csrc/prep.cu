@@ -207,13 +207,10 @@ __global__ void dump_fill_kernel(int64_t* finish, int64_t* first, int32_t* inst,
     }
 }
 
-// The checksum term of a rejected request depends on the request alone: computed once per trace.
-__global__ void rej_hash_kernel(uint64_t* out, uint32_t n) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) out[r] = rejected_hash(r);
-}
+// The checksum term of a rejected request depends on the request alone: computed once per trace, with the
+// prepared record.
 // Prepared trace records for the lane-group kernel (layout: common.cuh).
-__global__ void cook_trace_kernel(const uint4* reqs, const int64_t* classes, uint4* out, uint32_t n) {
+__global__ void cook_trace_kernel(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n) {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const Request q = decode_request(reqs[r]);
@@ -222,6 +219,7 @@ __global__ void cook_trace_kernel(const uint4* reqs, const int64_t* classes, uin
     const int64_t dl_e2e = l_e2e < 0 ? INT64_MAX : q.arrival + l_e2e;
     const uint32_t tbt32 = (l_tbt < 0 || l_tbt > 0xFFFFFFFFll) ? 0xFFFFFFFFu : (uint32_t)l_tbt;
     const uint64_t h = rejected_hash(r);
+    rej_hash[r] = h;
     auto lo = [](uint64_t v) { return (uint32_t)v; };
     auto hi = [](uint64_t v) { return (uint32_t)(v >> 32); };
     uint4* o = out + (size_t)r * kCookedWords;
@@ -290,13 +288,8 @@ cudaError_t launch_scan_trace(const uint4* reqs, const int64_t* classes, uint4* 
     if (n) scan_trace_kernel<<<(n + kScanTile - 1) / kScanTile, kScanTile>>>(reqs, classes, scan, n);
     return cudaGetLastError();
 }
-cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint32_t n) {
-    if (n) cook_trace_kernel<<<(n + 255) / 256, 256>>>(reqs, classes, out, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_rej_hash(uint64_t* out, uint32_t n) {
-    if (n) rej_hash_kernel<<<(n + 255) / 256, 256>>>(out, n);
+cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n) {
+    if (n) cook_trace_kernel<<<(n + 255) / 256, 256>>>(reqs, classes, out, rej_hash, n);
     return cudaGetLastError();
 }
 
