@@ -18,23 +18,25 @@ constexpr long long kWaitCycles = 4000000000ll;  // bound on any device-side wai
 // 9:    block layout with 16 warps striding over up to 128 instances, state in shared memory
 // 10..18: thread mapping, by how many lanes of a warp work at a time (32, 24, 16, 12, 8, 6, 4, 2, 1:
 //        the larger the placements, the fewer fit the warp's pools)
-// 20..24: walking kernel, by the room a placement needs: one, 2, 4, 8, 16 times a warp's part (walk.cuh)
-constexpr int kNumBuckets = 25;
-constexpr int kWalkBucket0 = 20;
-constexpr int kWalkBuckets = 5;
-constexpr int kWalkModes = kWalkBuckets;
+// 20..30: walking kernel (walk.cuh): up to 32 instances by the room a placement needs (one, 2, 4, 8, 16 times a
+//        warp's part), more than 32, 64-bit times by the room
+constexpr int kNumBuckets = 31;
+constexpr int kWalkModes = 5;
+constexpr int kWalkBucket0 = 20, kWalkBig0 = kWalkBucket0 + kWalkModes, kWalkLong0 = kWalkBig0 + 1;
+constexpr int kWalkBuckets = 2 * kWalkModes + 1;
 constexpr int kGenericBlockBucket = 9;
 constexpr int kThreadBucket0 = 10;  // buckets 10..18: the thread mapping, by lanes per warp
 constexpr int kThreadBuckets = 9;
 constexpr int kWideBucket = 19;     // 33..128 instances under the engines of the lane-group code: one warp per placement
+constexpr int kPrepOne = 1024;   // candidates one block of the validation kernel takes
 constexpr int kCostBins = 256;   // bin 0 = most expensive (largest total batch cap)
-constexpr int kCounterWords = 20480;  // counters | work counters | histograms + cursors, cleared per call
+constexpr int kCounterWords = 28160;  // counters | work counters | histograms + cursors, cleared per call
 // histogram sets (rows of kCostBins words in EvalParams::hist): candidates that can only go to a lane-group
 // or block bucket, only to a walking or thread bucket, or either way (counted once per side); then the write cursors
-constexpr int kHistOnlyG = 0, kHistBothG = 10, kHistOnlyT = 20, kHistBothT = 34, kHistWide = 48, kHistBothW = 49, kHistCursor = 50;
+constexpr int kHistOnlyG = 0, kHistBothG = 10, kHistOnlyT = 20, kHistBothT = 40, kHistWide = 60, kHistBothW = 61, kHistCursor = 62;
 constexpr int kHistRows = kHistCursor + kNumBuckets;
-// counters beside the bucket counts (EvalParams::bucket_count[0..31])
-constexpr int kCtrBoth = 28, kCtrLoaded = 29, kCtrCut = 30, kCtrUseThreads = 31;
+// counters beside the bucket counts (EvalParams::bucket_count[0..63])
+constexpr int kCtrBoth = 40, kCtrLoaded = 41, kCtrCut = 42, kCtrUseThreads = 43;
 constexpr int kGroupThreads = 128;
 constexpr int kScanTile = 256;       // requests per scan tile of the thread mapping
 constexpr int kScanHdrUnits = 40;    // 16-byte units of a scan tile's header (see scan_trace_kernel)
@@ -269,7 +271,7 @@ struct EvalParams {
     uint32_t flags;
     uint32_t mapping;
     maaso_result* out;
-    uint32_t* bucket_count;  // [32]: candidates per bucket after planning, and the kCtr* counters
+    uint32_t* bucket_count;  // [64]: candidates per bucket after planning, and the kCtr* counters
     uint32_t* bucket_list;   // [kNumBuckets][n_cand], each bucket sorted by decreasing cost estimate
     uint32_t* work_ctr;      // [16]: next work item of the block kernels [1..4], of the thread buckets [5..13], of the wide kernel [14]
     uint32_t* hist;          // [kHistRows][kCostBins]: candidates per cost bin by set, then write cursors
@@ -285,7 +287,10 @@ struct EvalParams {
     uint32_t thread_pool_units;  // thread mapping: 16-byte units one warp has for the cold part of its placements' state
     uint32_t thread_hot_units;   // and for the hot part (3 units per instance, shared memory)
     uint32_t* walk_ctr;      // [kWalkBuckets]: next placement of each walking bucket
-    uint32_t walk_bytes;     // walking kernel: bytes of shared memory one warp has for a placement, 0 = not used
+    uint32_t walk_bytes;     // walking kernel: bytes of shared memory one of 16 warps has for a placement, 0 = not used
+    uint32_t walk_usual;     // the same for placements of up to 32 instances, with walk_warps warps
+    uint32_t walk_warps;
+    uint32_t walk_long;      // the whole batch with 64-bit times
     long long wait_cycles;   // bound of every device-side wait
     uint32_t stall_test;     // test hook: never issue the trace copies
     int32_t* dump_row;       // [n_cand] or null

@@ -1,0 +1,13 @@
+// Walking kernel, 64-bit times: one instance per engine and estimate.
+#include "walk_kernel.cuh"
+
+namespace maaso {
+
+cudaError_t launch_eval_walk_long(const EvalParams& P, int grid, cudaStream_t stream) {
+    const bool opt = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) != 0;
+    if (P.flags & MAASO_FLAG_ENGINE_FROZEN)
+        return opt ? launch_walk<true, 1, true, true>(P, grid, stream) : launch_walk<false, 1, true, true>(P, grid, stream);
+    return opt ? launch_walk<true, 0, true, true>(P, grid, stream) : launch_walk<false, 0, true, true>(P, grid, stream);
+}
+
+}  // namespace maaso

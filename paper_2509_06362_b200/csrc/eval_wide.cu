@@ -103,13 +103,6 @@ __global__ void __launch_bounds__(32) eval_wide_kernel(const __grid_constant__ E
         const uint32_t n_req = P.trace_n[tr];
         const uint32_t oc = tr * P.n_cand + cand;
         const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
-        // a placement handed over by the walking kernel may have left counts in its side outputs
-        if (P.rej_by_model && lane < (uint32_t)MAASO_MAX_MODELS) P.rej_by_model[(size_t)oc * MAASO_MAX_MODELS + lane] = 0;
-        if (P.ttft_hist)
-            for (uint32_t i = lane; i < (uint32_t)MAASO_TTFT_BINS; i += 32u) P.ttft_hist[(size_t)oc * MAASO_TTFT_BINS + i] = 0;
-        __threadfence();
-        __syncwarp();
-
         Inst ins[kWideStrides];
         LaneEnv envs[kWideStrides];
         bool has[kWideStrides];

@@ -23,7 +23,9 @@ cudaError_t launch_eval_thread(const EvalParams& P, int grid, uint32_t pool_byte
 int occupancy_eval_thread(const EvalParams& P, uint32_t pool_bytes, uint32_t hot_bytes, bool in_smem);
 size_t thread_scratch_per_warp(uint32_t pool_bytes);
 uint32_t thread_fixed_smem(uint32_t n_models, uint32_t n_rows);
-cudaError_t launch_eval_walk(const EvalParams& P, int sm_count, cudaStream_t stream);
+cudaError_t launch_eval_walk(const EvalParams& P, int grid, cudaStream_t stream);
+cudaError_t launch_eval_walk_big(const EvalParams& P, int grid, cudaStream_t stream);
+cudaError_t launch_eval_walk_long(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_wide(const EvalParams& P, int grid, cudaStream_t stream);
 int occupancy_eval_wide(const EvalParams& P);
 size_t wide_scratch_per_warp();
@@ -59,7 +61,7 @@ struct maaso_trace {
     uint32_t n_classes;
     uint32_t max_model;
     std::vector<uint32_t> h_count;  // [n_classes][MAASO_MAX_MODELS] requests
-    uint32_t max_in;  // most input tokens of a request
+    uint32_t max_in, max_out;  // most input and output tokens of a request
     bool small_limits;  // every finite SLO limit fits the walking kernel's 32-bit times
     double tok_rate;  // output tokens per second the trace asks for (routing hint of MAASO_MAP_AUTO)
 };
@@ -100,7 +102,6 @@ struct maaso_ctx {
     int thread_blocks;   // one-warp blocks of the thread-mapping kernel per SM its pool is sized for
     uint32_t thread_theta;     // waiting lanes of a warp that trigger a distributor round in the thread mapping
     uint32_t thread_min_cand;  // MAASO_MAP_AUTO considers the thread mapping from this many candidates on
-    uint32_t walk_all;         // MAASO_MAP_AUTO takes the walking kernel up to this many placements x traces, whatever their load
     uint32_t last_mapping;     // mapping the most recent scoring call resolved to
     int fail_allocs;           // test hook: this many of the next scratch allocations are refused
     bool timing;
@@ -254,8 +255,6 @@ MAASO_API int maaso_create(maaso_ctx** out, int cuda_device) {
         long v = atol(tm);
         if (v >= 0) ctx->thread_min_cand = (uint32_t)v;
     }
-    ctx->walk_all = 16384;
-    if (const char* v = getenv("MAASO_WALK_ALL")) ctx->walk_all = (uint32_t)atol(v);
     ctx->last_mapping = MAASO_MAP_GROUP;
     ctx->fail_allocs = 0;
     const char* gb = getenv("MAASO_GROUP_BLOCKS");
@@ -404,7 +403,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     // mapping starts from "everything counted was rejected" and takes the served ones out)
     std::vector<uint64_t> class_tot((size_t)n_classes * 2, 0);
     uint64_t tok_sum = 0;
-    uint32_t max_in = 0;
+    uint32_t max_in = 0, max_out = 0;
     std::vector<uint32_t> count((size_t)n_classes * MAASO_MAX_MODELS, 0);
     for (uint64_t r = 0; r < n; r++) {
         const maaso_request& q = host[r];
@@ -417,6 +416,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         if (q.model > max_model) max_model = q.model;
         tok_sum += q.out_tokens;
         if (q.in_tokens > max_in) max_in = q.in_tokens;
+        if (q.out_tokens > max_out) max_out = q.out_tokens;
         count[(size_t)q.cls * MAASO_MAX_MODELS + q.model]++;
         class_tot[(size_t)q.cls * 2] += 1;
         class_tot[(size_t)q.cls * 2 + 1] += host_rejected_hash((uint32_t)r);
@@ -429,6 +429,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     t->max_model = max_model;
     t->h_count = std::move(count);
     t->max_in = max_in;
+    t->max_out = max_out;
     t->small_limits = true;
     for (int64_t v : cls) t->small_limits = t->small_limits && v < kWalkLimMax;
     {
@@ -530,9 +531,9 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     if (variant && o.mapping == MAASO_MAP_THREAD)
         return fail(ctx, MAASO_EINVAL,
                     "eval: the fixed-speed engine, per-instance queues and the largest-gap test have no thread mapping");
-    // MAASO_MAP_AUTO: the other engines exist in the lane-group kernel only; for the default engine both the
-    // lane-group and the thread kernel are launched and the validation kernels route the batch
-    if (o.mapping == MAASO_MAP_AUTO && variant) o.mapping = MAASO_MAP_GROUP;
+    // MAASO_MAP_AUTO: the largest-gap test exists in the lane-group code only; otherwise the validation kernels route the
+    // batch
+    if (o.mapping == MAASO_MAP_AUTO && (o.flags & MAASO_FLAG_TBT_MAXGAP)) o.mapping = MAASO_MAP_GROUP;
     ctx->last_mapping = o.mapping;
 
     DeviceGuard g(ctx->device);
@@ -585,24 +586,49 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     // wave is bound by its longest dependent chains, which run faster with fewer warps sharing a
     // scheduler; a larger batch is bound by instruction issue and wants all four.  Lanes needed
     // ~ instances x 1.3 (group widths are powers of two).
-    // the default engine runs on the walking kernel, the other readings on the lane-group kernel
-    // and whatever the walking kernel's 32-bit times cannot hold
-    bool walk = !variant && o.mapping == MAASO_MAP_AUTO && C < ctx->thread_min_cand && ctx->max_step < kWalkStepMax;
-    for (uint32_t t = 0; t < n_traces && walk; t++)
-        walk = traces[t]->small_limits &&
-               (double)ctx->max_pre_base + (double)ctx->max_q16 * traces[t]->max_in / 65536.0 + 1.0 < (double)kWalkPreMax;
+    // the walking kernel runs everything but the largest-gap test of the default engine; with 64-bit times where
+    // 32-bit ones cannot hold the batch's tables or limits
+    const bool walk = o.mapping == MAASO_MAP_AUTO && !(o.flags & MAASO_FLAG_TBT_MAXGAP) && (variant || C < ctx->thread_min_cand);
+    bool may_leave = false;  // a placement may leave the 32-bit horizon in mid-trace
+    if (walk) {
+        bool fits = ctx->max_step < kWalkStepMax;
+        for (uint32_t t = 0; t < n_traces; t++) {
+            const double pre = (double)ctx->max_pre_base + (double)ctx->max_q16 * traces[t]->max_in / 65536.0 + 1.0;
+            fits = fits && traces[t]->small_limits && pre < (double)kWalkPreMax;
+            // one request's time from its admission, everything that can be admitted before it, and a wait for it
+            const double ahead = pre * (double)traces[t]->n + (double)ctx->max_step * traces[t]->max_out;
+            may_leave = may_leave || o.flags != 0 || (double)kWalkNowMax + 2.0 * ahead >= (double)kWalkHorizon;
+        }
+        const bool queues = (o.flags & MAASO_FLAG_INSTANCE_QUEUES) != 0;  // always with 64-bit times
+        P.walk_long = fits || queues ? 0u : 1u;
+        may_leave = may_leave && !queues;
+        P.walk_bytes = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, true, kWalkWarps).pool) / kWalkWarps) & ~15u;
+        P.walk_warps = (uint64_t)C * n_traces <= 3ull * ctx->sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
+        P.walk_usual = P.walk_warps == kWalkWarps ? P.walk_bytes
+                                                  : ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, true, kWalkWarpsFew).pool) / kWalkWarpsFew) & ~15u;
+    }
     const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;
-    P.walk_all = walk && (uint64_t)C * n_traces <= ctx->walk_all ? 1u : 0u;
+    // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,
+    // which several placements of one warp share in the lane-group kernel; with one model all their lanes are at work,
+    // so the line lies lower (10,864 x 5,000, one model, few rejections: 13.7 ms against 19.3 walking; under load 4.1
+    // against 3.2; 6,000 x 8,000 of three models: 16.3 against 11.1).  Queues reject least.
+    const uint64_t walk_most = (o.flags & MAASO_FLAG_INSTANCE_QUEUES) ? 4096u : 6144u * (uint64_t)ctx->n_models;
+    P.walk_all = walk && (uint64_t)C * n_traces <= walk_most ? 1u : 0u;
+    if (walk && (o.flags & MAASO_FLAG_INSTANCE_QUEUES)) P.thread_min_cand = 0xFFFFFFFFu;
     const bool groups = !P.walk_all && (o.mapping == MAASO_MAP_GROUP || o.mapping == MAASO_MAP_AUTO);
-    if (walk) {
-        P.walk_bytes = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes).pool) / kWalkWarps) & ~15u;
-    }
     int group_blocks = ctx->group_blocks;
     if (group_blocks == 0) {
         const uint64_t est_warps = ((cands->n_inst * 13 / 10 + 31) / 32 + 6) * n_traces;
         group_blocks = est_warps <= (uint64_t)ctx->sm_count * 3 * (kGroupThreads / 32) ? 3 : 4;
     }
+    // blocks of the walking kernel for more than 32 instances: a block per placement at most
+    int grid_big = 0;
+    if (walk && !P.walk_long && cands->n_inst > kWalkBig) {
+        const uint64_t most = cands->n_inst / (kWalkBig + 1) * n_traces;
+        grid_big = most < (uint64_t)ctx->sm_count ? (int)most : ctx->sm_count;
+    }
+    const bool away = grid_big > 0 && !variant;  // its running requests are in global memory
     int grid_g = 0, grid_t = 0;
     uint32_t thread_pool = 0, thread_hot = 0;
     size_t pay_entries = 0, pay_thread = 0;  // scratch entries of the lane-group / block kernels, of the thread kernel
@@ -668,7 +694,8 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     // unless the batch goes to the threads; whatever the thread kernel's pools cannot hold): one warp per
     // placement with the lane-group code
     int grid_w = 0;
-    if (o.mapping != MAASO_MAP_BLOCK && (cands->n_inst > 32 || walk)) {
+    // (the walking kernel takes all of them, unless tables of more than a hundred rows leave its pool no room)
+    if (o.mapping != MAASO_MAP_BLOCK && cands->n_inst > 32 && !(walk && (P.walk_bytes << (kWalkModes - 1)) >= kWalkMost)) {
         // As many warps per SM as the registers allow (8) where the batch is made of large placements (more
         // than 16 instances per placement on average): the kernel waits on dependent chains, and four more
         // warps per SM are worth a third of its time.  Elsewhere 4 per SM, which needs no more scratch than
@@ -680,10 +707,6 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         // a placement that needs this kernel has more than 32 instances (or, thread mapping forced, more state
         // than a warp's pools): the batch cannot hold more of them than instances / 33
         uint64_t max_items_w = (o.mapping == MAASO_MAP_THREAD ? (uint64_t)C : cands->n_inst / 33u) * n_traces;
-        if (walk) {  // and placements that the walking kernel hands over
-            const uint64_t over = ((uint64_t)C * n_traces + 3) / 4;
-            if (over > max_items_w) max_items_w = over;
-        }
         if (max_items_w < 1) max_items_w = 1;
         if ((uint64_t)grid_w > max_items_w) grid_w = (int)max_items_w;
         const size_t need = ((size_t)grid_w * wide_scratch_per_warp() + sizeof(Payload) - 1) / sizeof(Payload);
@@ -698,13 +721,14 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     const size_t off_lists = off;    off = align_up(off + (size_t)kNumBuckets * C * 4, 256);
     const size_t off_dump = off;     off = align_up(off + (o.dump_n ? (size_t)C * 4 : 0), 256);
     const size_t off_pay = off;      off = align_up(off + pay_entries * sizeof(Payload), 256);
+    const size_t off_pay_b = off;    off = align_up(off + (away ? (size_t)grid_big * walk_big_scratch(P.walk_bytes * kWalkWarps) : 0), 256);
     const size_t off_pay_t = off;    off = align_up(off + pay_thread * sizeof(Payload), 256);
     int rc = grow(ctx, &ctx->scratch, &ctx->scratch_bytes, off);
     if (rc != MAASO_OK) return rc;
     unsigned char* sb = static_cast<unsigned char*>(ctx->scratch);
     P.bucket_count = reinterpret_cast<uint32_t*>(sb + off_counters);
-    P.work_ctr = P.bucket_count + 32;
-    P.hist = P.bucket_count + 64;
+    P.work_ctr = P.bucket_count + 64;
+    P.hist = P.bucket_count + 128;
     P.sm_ctr = P.hist + kHistRows * kCostBins;
     P.walk_ctr = P.work_ctr + 16;
     P.n_sm = (uint32_t)(ctx->sm_count < 1024 ? ctx->sm_count : 1024);
@@ -714,17 +738,19 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     P.dump_row = o.dump_n ? reinterpret_cast<int32_t*>(sb + off_dump) : nullptr;
     P.payload = reinterpret_cast<Payload*>(sb + off_pay);
 
-    static_assert(64 + kHistRows * kCostBins + 1024 <= kCounterWords, "counter region");
+    static_assert(128 + kHistRows * kCostBins + 1024 <= kCounterWords, "counter region");
     P.group_warps = (uint32_t)grid_g * (kGroupThreads / 32);
     P.mapping = o.mapping;  // block, lane groups, threads, or auto (routed by the validation kernels)
-    {   // output tokens per second the trace(s) ask for (mean over the traces of the call)
-        double d = 0.0;
-        for (uint32_t t = 0; t < n_traces; t++) d += traces[t]->tok_rate;
-        d /= n_traces;
+    {   // output tokens per second the trace(s) ask for (harmonic mean over the traces of the call: what share of the
+        // requests can be served is decided by the inverse, and it is the light traces that take the time)
+        double inv = 0.0;
+        for (uint32_t t = 0; t < n_traces; t++) inv += traces[t]->tok_rate > 0.0 ? 1.0 / traces[t]->tok_rate : 1.0;
+        const double d = n_traces / inv;
         P.demand_tok_s = d >= 4.0e9 ? 4000000000u : (uint32_t)d;
     }
     P.promote_pct = (uint32_t)ctx->promote_pct;
-    cudaError_t e = cudaMemsetAsync(sb + off_counters, 0, kCounterWords * 4, stream);
+    cudaError_t e = cudaSuccess;
+    if (!(C <= (uint32_t)kPrepOne && P.walk_all)) e = cudaMemsetAsync(sb + off_counters, 0, kCounterWords * 4, stream);
     if (e == cudaSuccess && o.ttft_hist)
         e = cudaMemsetAsync(o.ttft_hist, 0, (size_t)C * n_traces * MAASO_TTFT_BINS * 4, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "memset");
@@ -738,7 +764,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel launch");
     }
-    if (walk) {
+    if (walk && !P.walk_long) {
         e = launch_eval_walk(P, ctx->sm_count, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
@@ -756,6 +782,18 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         if (e != cudaSuccess) return cuda_fail(ctx, e, "thread kernel launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[6], stream);
+    if (grid_big > 0) {
+        EvalParams PB = P;
+        PB.payload = reinterpret_cast<Payload*>(sb + off_pay_b);
+        e = launch_eval_walk_big(PB, grid_big, stream);
+        launches++;
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
+    }
+    if (walk && (P.walk_long || may_leave)) {
+        e = launch_eval_walk_long(P, ctx->sm_count, stream);
+        launches++;
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
+    }
     if (grid_w > 0) {
         e = launch_eval_wide(P, grid_w, stream);
         launches++;

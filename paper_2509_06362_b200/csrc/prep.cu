@@ -4,20 +4,30 @@
 
 namespace maaso {
 
-// Where a valid candidate can be scored.  `code` = its bucket among the lane-group / block buckets
-// (0..9) and its cost bin, `code2` = its bucket among the thread-mapping buckets (10..18) and the
-// bin; 0xFFFFFFFF = it has no such place.  A candidate with both is placed by the batch-wide choice
-// plan_kernel makes (MAASO_MAP_AUTO).
+// Where a valid candidate can be scored.  `code` = its bucket among the lane-group / block buckets (0..9, or the
+// one-warp bucket) and its cost bin, `code2` = its bucket among the thread-mapping and walking buckets and the bin;
+// 0xFFFFFFFF = it has no such place.  A candidate with both is placed by the batch-wide choice plan_kernel makes
+// (MAASO_MAP_AUTO).
+constexpr uint32_t kNowhere = 0xFFFFFFFFu;
 __device__ __forceinline__ int t_row(int b) { return b < kWalkBucket0 ? b - kThreadBucket0 : kThreadBuckets + b - kWalkBucket0; }
-__global__ void prep_kernel(const EvalParams P) {
-    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= P.n_cand) return;
+
+struct Place {
+    uint32_t status, code, code2;
+    bool loaded;  // the trace asks for more than the placement can decode
+};
+
+// Validation (constraints (c) and (d) of Sec. IV-C, table ranges) and routing of candidate c; writes the record of an
+// invalid one and marks a valid one "not scored" (ETIMEOUT): the scoring kernel overwrites the record when it
+// finishes the candidate, so a kernel that gave up leaves no record undefined.
+__device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c) {
     const uint32_t lo = P.offsets[c], hi = P.offsets[c + 1];
     uint32_t status = 0, n = 0, sum_b = 0;
     uint32_t units = 0;  // thread mapping: 16-byte units of cold instance state (per instance 2 + key blocks + minima)
-    uint32_t slot_bytes = 0;  // walking kernel: shared memory of its instances' slots
+    uint32_t slot_bytes = 0, slot_bytes64 = 0;  // walking kernel: shared memory of its instances' slots, with 64-bit times too
     uint64_t supply = 0; // decode tokens per second the placement can produce with every slot busy
     const bool variant = (P.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_TBT_MAXGAP | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
+    const bool fixed_speed = (P.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
+    const bool queues = (P.flags & MAASO_FLAG_INSTANCE_QUEUES) != 0;  // always with 64-bit times
     const bool threads_ok = !variant && (P.mapping == MAASO_MAP_THREAD || (P.mapping == MAASO_MAP_AUTO && !P.walk_bytes));
     const bool groups_ok = P.mapping != MAASO_MAP_THREAD;
     if (hi < lo || hi > P.n_inst) {
@@ -27,6 +37,7 @@ __global__ void prep_kernel(const EvalParams P) {
         if (n > MAASO_MAX_INSTANCES) {
             status = MAASO_CAND_ETOOMANY;
         } else {
+            const uint32_t key_bytes = fixed_speed && (P.walk_long || queues) ? 8u : 4u;
             uint64_t devsum = 0;
             for (uint32_t i = 0; i < n; i++) {
                 const uint32_t word = P.inst[lo + i];
@@ -36,9 +47,10 @@ __global__ void prep_kernel(const EvalParams P) {
                     continue;
                 }
                 sum_b += b;
-                slot_bytes += walk_slot_bytes((b + 7u) >> 3);
+                slot_bytes += walk_slot_bytes((b + 7u) >> 3, key_bytes, fixed_speed || (n > kWalkBig && !P.walk_long));
+                slot_bytes64 += walk_slot_bytes((b + 7u) >> 3, fixed_speed ? 8u : 4u, fixed_speed);
                 units += 2u + 2u * ((b + 7u) >> 3) + 2u;
-                supply += (uint64_t)b * 1000000ull / (uint64_t)P.rows[(m * P.n_strategies + s) * kRowStride + 1 + b];
+                supply += b * 1000000u / (uint32_t)P.rows[(m * P.n_strategies + s) * kRowStride + 1 + b];
                 devsum += (uint64_t)P.devices[s];
                 if (P.devices[s] < P.min_devices[m]) status |= MAASO_CAND_EMEMFIT;
             }
@@ -47,6 +59,7 @@ __global__ void prep_kernel(const EvalParams P) {
     }
     // where it can go
     int bg = -1, bt = -1;
+    uint32_t need = 0;  // room in the walking kernel
     if (!status) {
         if (threads_ok) {
             // as many lanes per item as placements of this size fit the warp's pools
@@ -56,17 +69,24 @@ __global__ void prep_kernel(const EvalParams P) {
                 if (fit >= lanes[i]) { bt = kThreadBucket0 + i; break; }
         }
         if (P.walk_bytes) {
-            // one warp's part of the walking kernel's pool, or 2, 4, 8, 16 of them
-            const uint32_t need = walk_region_bytes(P.n_models, n, slot_bytes);
-            for (uint32_t k = 0; n <= 32u && k < (uint32_t)kWalkModes && bt < 0; k++)
-                if (need <= (P.walk_bytes << k)) bt = kWalkBucket0 + (int)k;
+            const bool big = n > kWalkBig && !P.walk_long;
+            need = walk_region_bytes(P.n_models, n, slot_bytes, P.walk_long || queues ? kWalkLongKind : (big ? kWalkBigKind : kWalkUsual));
+            if (big) {
+                // (and all of the pool has to hold it if it is handed over)
+                if (max(need, walk_region_bytes(P.n_models, n, slot_bytes64, kWalkLongKind)) <= P.walk_bytes * (uint32_t)kWalkWarps) bt = kWalkBig0;
+            } else {
+                // one warp's part of the walking kernel's pool, or 2, 4, 8 of them (16 with 64-bit times)
+                const uint32_t part = P.walk_long ? P.walk_bytes : P.walk_usual;
+                for (uint32_t k = 0; k < (uint32_t)kWalkModes - 1u && bt < 0; k++)
+                    if (need <= (part << k)) bt = (P.walk_long ? kWalkLong0 : kWalkBucket0) + (int)k;
+                if (bt < 0 && P.walk_long && need <= part * 16u) bt = kWalkLong0 + 4;
+            }
         }
         if (P.mapping == MAASO_MAP_BLOCK) bg = n <= 2 ? 6 : (n <= 4 ? 7 : (n <= 8 ? 8 : kGenericBlockBucket));
         else if (groups_ok && n <= 32) bg = n <= 1 ? 0 : 32 - __clz((int)(n - 1));
-        // More than 32 instances: one warp per placement with the lane-group code (every engine), or the thread
-        // mapping where that exists and can hold the placement; the batch-wide choice of plan_kernel decides
-        // between the two.  (One block per placement only when the block mapping is asked for.)
-        if (bg < 0 && (groups_ok || bt < 0)) bg = kWideBucket;
+        // More than 32 instances outside the walking and the thread kernel: one warp per placement with the lane-group
+        // code.  (One block per placement only when the block mapping is asked for.)
+        else if (bt < 0 || (groups_ok && !P.walk_bytes)) bg = kWideBucket;
     }
     if (P.dump_row) P.dump_row[c] = -1;
     const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
@@ -74,105 +94,133 @@ __global__ void prep_kernel(const EvalParams P) {
         const size_t oc = (size_t)t * P.n_cand + c;  // the candidate's record in trace t's block
         if (P.rej_by_model)
             for (int m = 0; m < MAASO_MAX_MODELS; m++) P.rej_by_model[oc * MAASO_MAX_MODELS + m] = 0;
-        // Invalid candidates get their final record here.  Valid ones are pre-marked "not scored"
-        // (ETIMEOUT); the scoring kernel overwrites the record when it finishes the candidate, so a
-        // kernel that gave up on a bounded wait leaves no record undefined.
         uint4* o = reinterpret_cast<uint4*>(P.out + oc);
         o[0] = make_uint4(status ? status : MAASO_CAND_ETIMEOUT, 0, 0, 0);
         for (int i = 1; i < 8; i++) o[i] = make_uint4(0, 0, 0, 0);
     }
-    if (status) {
-        P.code[c] = 0xFFFFFFFFu;
-        P.code2[c] = 0xFFFFFFFFu;
-        return;
-    }
     // Cost estimate: the total batch cap (how many requests the placement can have in flight;
     // it tracks the number of served requests and so the number of simulation events).
     const uint32_t bin = (kCostBins - 1) - min((uint32_t)(kCostBins - 1), sum_b / 8u);
-    P.code[c] = bg >= 0 ? (((uint32_t)bg << 8) | bin) : 0xFFFFFFFFu;
-    P.code2[c] = bt >= 0 ? (((uint32_t)bt << 8) | bin) : 0xFFFFFFFFu;
-    if (bg >= 0 && bt >= 0) {
+    Place r;
+    r.status = status;
+    r.code = bg >= 0 ? (((uint32_t)bg << 8) | bin) : kNowhere;
+    r.code2 = bt >= 0 ? (((uint32_t)bt << 8) | (bt == kWalkBig0 ? walk_big_bin(need) : bin)) : kNowhere;
+    r.loaded = (uint64_t)P.demand_tok_s >= 2ull * supply;
+    return r;
+}
+
+__global__ void prep_kernel(const EvalParams P) {
+    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= P.n_cand) return;
+    const Place r = place_candidate(P, c);
+    P.code[c] = r.code;
+    P.code2[c] = r.code2;
+    const uint32_t bin = (r.code != kNowhere ? r.code : r.code2) & 0xFFu;
+    const int bg = (int)(r.code >> 8), bt = (int)(r.code2 >> 8);
+    if (r.code != kNowhere && r.code2 != kNowhere) {
         atomicAdd(&P.hist[(bg == kWideBucket ? kHistBothW : kHistBothG + bg) * kCostBins + bin], 1u);
         atomicAdd(&P.hist[(kHistBothT + t_row(bt)) * kCostBins + bin], 1u);
         // loaded beyond what it can decode: most of its requests will be turned away, which the
-        // thread mapping does for next to nothing
+        // walking and the thread kernel do for next to nothing
         atomicAdd(&P.bucket_count[kCtrBoth], 1u);
-        if ((uint64_t)P.demand_tok_s >= 2ull * supply) atomicAdd(&P.bucket_count[kCtrLoaded], 1u);
-    } else if (bg == kWideBucket) {
-        atomicAdd(&P.hist[kHistWide * kCostBins + bin], 1u);
-    } else if (bg >= 0) {
-        atomicAdd(&P.hist[(kHistOnlyG + bg) * kCostBins + bin], 1u);
-    } else {
+        if (r.loaded) atomicAdd(&P.bucket_count[kCtrLoaded], 1u);
+    } else if (r.code != kNowhere) {
+        atomicAdd(&P.hist[(bg == kWideBucket ? kHistWide : kHistOnlyG + bg) * kCostBins + bin], 1u);
+    } else if (r.code2 != kNowhere) {
         atomicAdd(&P.hist[(kHistOnlyT + t_row(bt)) * kCostBins + bin], 1u);
     }
 }
 
-// One block, one thread per cost bin: (0) the batch-wide choice between lane groups and threads for
-// the candidates that can go either way (MAASO_MAP_AUTO): threads if most of them are loaded beyond
-// their decode capacity and there are enough of them to fill the GPU one placement per lane; (1) if the
-// resident lane-group grid has warps to spare, promote the most expensive candidates of the narrower
-// lane-group buckets to a warp of their own (bucket 5) so that their event handling is not
-// serialised with other candidates' in the same warp; (2) turn the per-bin histograms into write
-// cursors (bins in decreasing cost order).
-__device__ __forceinline__ uint32_t block_inclusive_scan(uint32_t v, uint32_t* buf) {
-    const int t = threadIdx.x;
-    buf[t] = v;
-    __syncthreads();
-    for (int off = 1; off < kCostBins; off <<= 1) {
-        const uint32_t add = t >= off ? buf[t - off] : 0u;
-        __syncthreads();
-        buf[t] += add;
-        __syncthreads();
+// Exclusive prefix sums of 256 counts by one warp (lane l holds counts 8l .. 8l+7); returns the total.
+__device__ __forceinline__ uint32_t warp_scan_256(uint32_t (&v)[8]) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const uint32_t x = v[i];
+        v[i] = sum;
+        sum += x;
     }
-    const uint32_t r = buf[t];
-    __syncthreads();
-    return r;
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += x;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] += incl - sum;
+    return __shfl_sync(0xFFFFFFFFu, incl, 31);
 }
 
-__global__ void __launch_bounds__(kCostBins) plan_kernel(const EvalParams P) {
-    __shared__ uint32_t buf[kCostBins];
-    __shared__ uint32_t tot[6];
-    const int bin = threadIdx.x;
+// One block, one warp per bucket, eight cost bins per lane: (0) the batch-wide choice for the candidates that can go
+// either way (MAASO_MAP_AUTO): the walking (or thread) kernel if the batch is small, or if most of them are loaded
+// beyond their decode capacity, else the lane groups; (1) if the resident lane-group grid has warps to spare, promote
+// the most expensive candidates of the narrower lane-group buckets to a warp of their own (bucket 5) so that their
+// event handling is not serialised with other candidates' in the same warp; (2) turn the per-bin histograms into
+// write cursors (bins in decreasing cost order).
+__global__ void __launch_bounds__(1024) plan_kernel(const EvalParams P) {
+    __shared__ uint32_t tot[6], s_cut;
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     const uint32_t n_both = P.bucket_count[kCtrBoth], n_loaded = P.bucket_count[kCtrLoaded];
     const bool use_threads = P.walk_all || (n_loaded >= P.thread_min_cand && 2u * n_loaded >= n_both);
-    // final counts of this bin per bucket
-    uint32_t cnt[kNumBuckets];
-    for (int b = 0; b < kThreadBucket0; b++)
-        cnt[b] = P.hist[(kHistOnlyG + b) * kCostBins + bin] + (use_threads ? 0u : P.hist[(kHistBothG + b) * kCostBins + bin]);
-    for (int b = kThreadBucket0; b < kNumBuckets; b++)
-        if (b != kWideBucket)
-            cnt[b] = P.hist[(kHistOnlyT + t_row(b)) * kCostBins + bin] + (use_threads ? P.hist[(kHistBothT + t_row(b)) * kCostBins + bin] : 0u);
-    cnt[kWideBucket] = P.hist[kHistWide * kCostBins + bin] + (use_threads ? 0u : P.hist[kHistBothW * kCostBins + bin]);
-    uint32_t cut = 0;  // bins below `cut` are promoted
-    uint32_t narrow = 0;
-    for (int b = 0; b < 5; b++) narrow += cnt[b];
-    if (P.mapping != MAASO_MAP_BLOCK && P.mapping != MAASO_MAP_THREAD) {
-        // warps the lane-group buckets need: bucket totals = sums over the bins
-        uint32_t need = 0;
-        for (int b = 0; b <= 5; b++) {
-            const uint32_t incl = block_inclusive_scan(cnt[b], buf);
-            if (bin == kCostBins - 1) tot[b] = incl;
+    auto counts = [&](int b, uint32_t (&v)[8]) {  // final counts of bucket b in this lane's bins
+        const uint32_t only = b == kWideBucket ? kHistWide : (b < kThreadBucket0 ? kHistOnlyG + b : kHistOnlyT + t_row(b));
+        const uint32_t both = b == kWideBucket ? kHistBothW : (b < kThreadBucket0 ? kHistBothG + b : kHistBothT + t_row(b));
+        const bool take = (b == kWideBucket || b < kThreadBucket0) ? !use_threads : use_threads;
+#pragma unroll
+        for (int i = 0; i < 8; i++) v[i] = P.hist[only * kCostBins + 8u * lane + i] + (take ? P.hist[both * kCostBins + 8u * lane + i] : 0u);
+    };
+    if (threadIdx.x == 0) s_cut = 0;
+    uint32_t v[8];
+    if (P.group_warps) {
+        if (warp <= 5) {
+            counts((int)warp, v);
+            const uint32_t t = warp_scan_256(v);
+            if (lane == 0) tot[warp] = t;
         }
         __syncthreads();
-        for (int b = 0; b <= 5; b++) need += (tot[b] + (32u >> b) - 1) / (32u >> b);
-        // every work item exists once per trace, and a promoted candidate takes a warp in each of them
-        const uint32_t n_tr = P.n_traces > 1 ? P.n_traces : 1u;
-        const uint64_t need_all = (uint64_t)need * n_tr;
-        const uint32_t spare = P.group_warps > need_all
-                                   ? (uint32_t)((P.group_warps - need_all) / n_tr * P.promote_pct / 100) : 0;
-        const uint32_t incl = block_inclusive_scan(narrow, buf);
-        cut = (uint32_t)__syncthreads_count(incl <= spare);  // prefix sums are monotone
+        if (warp == 0) {
+            // warps the lane-group buckets need; every work item exists once per trace, and a promoted candidate takes a
+            // warp in each of them
+            uint32_t need = 0, narrow[8] = {0, 0, 0, 0, 0, 0, 0, 0}, add[8];
+            for (int b = 0; b <= 5; b++) need += (tot[b] + (32u >> b) - 1) / (32u >> b);
+            const uint32_t n_tr = P.n_traces > 1 ? P.n_traces : 1u;
+            const uint64_t need_all = (uint64_t)need * n_tr;
+            const uint32_t spare = P.group_warps > need_all ? (uint32_t)((P.group_warps - need_all) / n_tr * P.promote_pct / 100) : 0;
+            for (int b = 0; b < 5; b++) {
+                counts(b, add);
+#pragma unroll
+                for (int i = 0; i < 8; i++) narrow[i] += add[i];
+            }
+            uint32_t before[8], n = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i++) before[i] = narrow[i];
+            warp_scan_256(before);
+#pragma unroll
+            for (int i = 0; i < 8; i++) n += before[i] + narrow[i] <= spare ? 1u : 0u;  // prefix sums are monotone
+            n = __reduce_add_sync(0xFFFFFFFFu, n);
+            if (lane == 0) s_cut = n;
+        }
     }
     __syncthreads();
-    for (int b = 0; b < kNumBuckets; b++) {
-        uint32_t v = cnt[b];
-        if (b < 5 && (uint32_t)bin < cut) v = 0;
-        if (b == 5 && (uint32_t)bin < cut) v += narrow;
-        const uint32_t incl = block_inclusive_scan(v, buf);
-        P.hist[(kHistCursor + b) * kCostBins + bin] = incl - v;
-        if (bin == kCostBins - 1) P.bucket_count[b] = incl;
+    const uint32_t cut = s_cut;  // bins below `cut` are promoted
+    for (int b = (int)warp; b < kNumBuckets; b += 32) {
+        counts(b, v);
+        if (b <= 5 && cut) {
+            uint32_t add[8];
+            for (int x = 0; x < 5; x++) {
+                if (b == 5) counts(x, add);
+#pragma unroll
+                for (int i = 0; i < 8; i++)
+                    if (8u * lane + i < cut) v[i] = b == 5 ? v[i] + add[i] : 0u;
+            }
+        }
+        const uint32_t total = warp_scan_256(v);
+#pragma unroll
+        for (int i = 0; i < 8; i++) P.hist[(kHistCursor + b) * kCostBins + 8u * lane + i] = v[i];
+        if (lane == 0) P.bucket_count[b] = total;
     }
-    if (bin == 0) {
+    if (threadIdx.x == 0) {
         P.bucket_count[kCtrCut] = cut;
         P.bucket_count[kCtrUseThreads] = use_threads ? 1u : 0u;
     }
@@ -182,14 +230,47 @@ __global__ void scatter_kernel(const EvalParams P) {
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= P.n_cand) return;
     const uint32_t cg = P.code[c], ct = P.code2[c];
-    if (cg == 0xFFFFFFFFu && ct == 0xFFFFFFFFu) return;
-    const uint32_t code = (cg != 0xFFFFFFFFu && ct != 0xFFFFFFFFu) ? (P.bucket_count[kCtrUseThreads] ? ct : cg)
-                                                                    : (cg != 0xFFFFFFFFu ? cg : ct);
+    if (cg == kNowhere && ct == kNowhere) return;
+    const uint32_t code = (cg != kNowhere && ct != kNowhere) ? (P.bucket_count[kCtrUseThreads] ? ct : cg) : (cg != kNowhere ? cg : ct);
     uint32_t b = code >> 8;
     const uint32_t bin = code & 0xFFu;
     if (b < 5 && bin < P.bucket_count[kCtrCut]) b = 5;
     const uint32_t pos = atomicAdd(&P.hist[(kHistCursor + b) * kCostBins + bin], 1u);
     P.bucket_list[(size_t)b * P.n_cand + pos] = c;
+}
+
+// All of the above in one launch, for a batch of at most kPrepOne candidates that the walking kernel takes whatever
+// its load: one block, histograms in shared memory, nothing to be cleared beforehand.  Three launches and a clear
+// are 20 us of a small call's 300.
+__global__ void __launch_bounds__(kPrepOne) prep_one_kernel(const EvalParams P) {
+    extern __shared__ uint32_t one_hist[];  // [kNumBuckets][kCostBins]
+    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
+    for (uint32_t i = tid; i < (uint32_t)(kNumBuckets * kCostBins); i += kPrepOne) one_hist[i] = 0;
+    for (uint32_t i = tid; i < 128u; i += kPrepOne) P.bucket_count[i] = 0;  // bucket counts and work counters
+    __syncthreads();
+    uint32_t code = kNowhere;
+    if (tid < P.n_cand) {
+        const Place r = place_candidate(P, tid);
+        code = r.code2 != kNowhere ? r.code2 : r.code;
+        P.code[tid] = code;
+        P.code2[tid] = code;
+    }
+    if (code != kNowhere) atomicAdd(&one_hist[code], 1u);  // bucket << 8 | bin is its place in the histograms
+    __syncthreads();
+    for (uint32_t b = warp; b < (uint32_t)kNumBuckets; b += kPrepOne / 32) {
+        uint32_t v[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) v[i] = one_hist[b * kCostBins + 8u * lane + i];
+        const uint32_t total = warp_scan_256(v);
+#pragma unroll
+        for (int i = 0; i < 8; i++) one_hist[b * kCostBins + 8u * lane + i] = v[i];
+        if (lane == 0) P.bucket_count[b] = total;
+    }
+    __syncthreads();
+    if (code != kNowhere) {
+        const uint32_t pos = atomicAdd(&one_hist[code], 1u);
+        P.bucket_list[(size_t)(code >> 8) * P.n_cand + pos] = tid;
+    }
 }
 
 __global__ void dump_map_kernel(const EvalParams P, const uint32_t* dump_idx) {
@@ -302,10 +383,15 @@ cudaError_t launch_prep(const EvalParams& P, const uint32_t* dump_idx, cudaStrea
             (*launches)++;
         }
     }
-    prep_kernel<<<(P.n_cand + 255) / 256, 256, 0, stream>>>(P);
-    plan_kernel<<<1, kCostBins, 0, stream>>>(P);
-    scatter_kernel<<<(P.n_cand + 255) / 256, 256, 0, stream>>>(P);
-    (*launches) += 3;
+    if (P.n_cand <= (uint32_t)kPrepOne && P.walk_all) {
+        prep_one_kernel<<<1, kPrepOne, kNumBuckets * kCostBins * 4, stream>>>(P);
+        (*launches)++;
+    } else {
+        prep_kernel<<<(P.n_cand + 255) / 256, 256, 0, stream>>>(P);
+        plan_kernel<<<1, 1024, 0, stream>>>(P);
+        scatter_kernel<<<(P.n_cand + 255) / 256, 256, 0, stream>>>(P);
+        (*launches) += 3;
+    }
     if (P.dump_n) {
         dump_map_kernel<<<(P.dump_n + 255) / 256, 256, 0, stream>>>(P, dump_idx);
         (*launches)++;

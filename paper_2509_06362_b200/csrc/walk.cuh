@@ -1,47 +1,72 @@
-// Layout of the walking kernel's shared memory (eval_walk.cu), used by the validation kernel too, which
+// Layout of the walking kernel's shared memory (walk_kernel.cuh), used by the validation kernel too, which
 // has to know how much of it a placement needs.
 #pragma once
 #include "lane_sim.cuh"
 
 namespace maaso {
 
-constexpr int kWalkWarps = 16;                    // one block per SM
-constexpr int kWalkThreads = 32 * kWalkWarps;
+// Warps per block, one block per SM: 16 with 128 registers each, or 12 with 168 for a batch of at most three
+// placements per warp, which its longest chains bound (2,000 x 17,000 of the paper's shape: 13.7 ms against 15.0;
+// 100,000 x 100,000 under load: 144 against 122).
+constexpr int kWalkWarps = 16, kWalkWarpsFew = 12;
 constexpr int kWalkRing = 64;                     // ring entries per warp
 
-// One block: decode-step tables, SLO limits, the completion rings, the pool.
+// One block: the completion rings, SLO limits, decode-step tables, the pool.
 struct WalkLayout {
-    uint32_t steps;   // [n_rows][64] u32
-    uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
     uint32_t ring;    // [warps][kWalkRing] {finish, first token}
     uint32_t ring_b;  // [warps][kWalkRing] {request, instance}
+    uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
+    uint32_t wide;    // 64-bit times: [n_classes] {TTFT limit (2^62 = none), TBT limit (negative = none)}
+    uint32_t steps;   // [n_rows][64] u32
     uint32_t pool;
 };
-__host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes) {
+__host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes, bool wide, uint32_t warps) {
     WalkLayout l;
     l.ring = 0;
-    l.ring_b = (uint32_t)(kWalkWarps * kWalkRing) * 16u;
-    l.lims = l.ring_b + (uint32_t)(kWalkWarps * kWalkRing) * 8u;
-    l.steps = l.lims + n_classes * 16u;
+    l.ring_b = warps * (uint32_t)kWalkRing * 16u;
+    l.lims = l.ring_b + warps * (uint32_t)kWalkRing * 8u;
+    l.wide = l.lims + n_classes * 16u;
+    l.steps = l.wide + (wide ? n_classes * 16u : 0u);
     l.pool = (l.steps + n_rows * 256u + 127u) & ~127u;
     return l;
 }
 
 // One placement's region: sums (kWalkSums bytes: one set of four 16-byte units per lane, unit-major, then hits by
-// class bin), 16 bytes per model, 16 per instance, then per instance its slots: the eight block minima, the stack
-// of free slots (a byte each), then blocks of 8 slots with the keys (end index << 6 | slot), the request indices
-// and the first-token times.
+// class bin), 16 bytes per model, 16 per instance, with more than 32 instances their resting state (unit-major) and
+// a lower bound per model, then per instance its slots: the eight block minima, the stack of free slots (a byte
+// each), then blocks of 8 slots with the keys (end index << 6 | slot), the request indices and the first-token
+// times.  Keys alone (finish times) in the engines that fix a request's speed at admission, and with more than 32
+// instances, where the rest (16 bytes per slot) is in global memory: shared memory decides how many such placements
+// are resident.
+enum WalkKind : uint32_t { kWalkUsual = 0, kWalkBigKind = 1, kWalkLongKind = 2 };
 constexpr uint32_t kWalkLaneSums = 4u * 32u * 16u;
 constexpr uint32_t kWalkSums = kWalkLaneSums + 48u;
-__host__ __device__ inline uint32_t walk_slot_bytes(uint32_t nblk) { return 32u + ((8u * nblk + 15u) & ~15u) + nblk * 128u; }
-__host__ __device__ inline uint32_t walk_region_bytes(uint32_t n_models, uint32_t n_inst, uint32_t slot_bytes) {
-    return kWalkSums + 16u * (n_models + n_inst) + slot_bytes;
+constexpr uint32_t kWalkBig = 32u;  // more instances than this rest in shared memory
+__host__ __device__ inline uint32_t walk_slots_at(uint32_t nblk, uint32_t key_bytes) { return 8u * key_bytes + ((8u * nblk + 15u) & ~15u); }
+__host__ __device__ inline uint32_t walk_slot_bytes(uint32_t nblk, uint32_t key_bytes, bool keys_alone) {
+    return walk_slots_at(nblk, key_bytes) + nblk * (keys_alone ? 8u * key_bytes : 128u);
 }
+__host__ __device__ inline uint32_t walk_rest_bytes(WalkKind kind) { return kind == kWalkUsual ? 0u : (kind == kWalkBigKind ? 48u : 80u); }
+__host__ __device__ inline uint32_t walk_region_bytes(uint32_t n_models, uint32_t n_inst, uint32_t slot_bytes, WalkKind kind) {
+    return kWalkSums + 16u * (n_models + n_inst) + (kind ? walk_rest_bytes(kind) * n_inst + ((8u * n_models + 15u) & ~15u) : 0u) + slot_bytes;
+}
+// Placements of more than 32 instances are sorted by the room they need, in steps of kWalkStepBytes; a block's first is
+// its largest and decides how many of its warps work side by side.
+constexpr uint32_t kWalkStepBytes = 640u;
+__host__ __device__ inline uint32_t walk_big_bin(uint32_t need) {
+    const uint32_t k = need / kWalkStepBytes;
+    return 255u - (k < 255u ? k : 255u);
+}
+// Global memory for one block's running requests: four bytes of it per byte of pool.
+__host__ __device__ inline size_t walk_big_scratch(uint32_t pool_bytes) { return (size_t)pool_bytes * 4u; }
 
-// Times are 32-bit offsets from an epoch that each placement moves along (eval_walk.cu).  The bounds below
+// The most a placement can need: 128 instances of 64 slots, 16 models, 8-byte keys or requests beside 4-byte keys.
+constexpr uint32_t kWalkMost = 160u * 1024u;
+
+// Times are 32-bit offsets from an epoch that each placement moves along (walk_kernel.cuh).  The bounds below
 // keep every sum of a round inside 31 bits; a batch whose tables or limits exceed them, checked on the host,
-// runs on the lane-group kernel, and a single placement that gets beyond kWalkHorizon is handed to the
-// one-warp-per-placement kernel, both of which compute in 64 bits.
+// runs with 64-bit times, and so does, from its start again, a single placement that gets beyond kWalkHorizon.
+constexpr int32_t kWalkFar = 0x7FFFFFFF;         // no completion in sight; an arrival beyond the epoch's reach
 constexpr int32_t kWalkNowMax = 1 << 27;         // the epoch moves when the dispatcher's clock is this far ahead
 constexpr int32_t kWalkHorizon = 0x60000000;     // largest time
 constexpr int64_t kWalkStepMax = 1 << 24;        // decode step
