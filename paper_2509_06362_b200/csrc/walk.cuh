@@ -35,16 +35,17 @@ __host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_cl
 // class bin), 16 bytes per model, 16 per instance, with more than 32 instances their resting state (unit-major) and
 // a lower bound per model, then per instance its slots: the eight block minima, the stack of free slots (a byte
 // each), then blocks of 8 slots with the keys (end index << 6 | slot), the request indices and the first-token
-// times.  Keys alone (finish times) in the engines that fix a request's speed at admission, and with more than 32
-// instances, where the rest (16 bytes per slot) is in global memory: shared memory decides how many such placements
-// are resident.
+// times.  Keys alone with more than 32 instances, where the rest (16 bytes per slot) is in global memory: shared memory
+// decides how many such placements are resident.  In the engines that fix a request's speed at admission: the finish
+// times in falling order, so that the next to free is popped off the end.
 enum WalkKind : uint32_t { kWalkUsual = 0, kWalkBigKind = 1, kWalkLongKind = 2 };
 constexpr uint32_t kWalkLaneSums = 4u * 32u * 16u;
 constexpr uint32_t kWalkSums = kWalkLaneSums + 48u;
 constexpr uint32_t kWalkBig = 32u;  // more instances than this rest in shared memory
-__host__ __device__ inline uint32_t walk_slots_at(uint32_t nblk, uint32_t key_bytes) { return 8u * key_bytes + ((8u * nblk + 15u) & ~15u); }
-__host__ __device__ inline uint32_t walk_slot_bytes(uint32_t nblk, uint32_t key_bytes, bool keys_alone) {
-    return walk_slots_at(nblk, key_bytes) + nblk * (keys_alone ? 8u * key_bytes : 128u);
+__host__ __device__ inline uint32_t walk_slots_at(uint32_t nblk) { return 32u + ((8u * nblk + 15u) & ~15u); }
+__host__ __device__ inline uint32_t walk_slot_bytes(uint32_t b, bool fixed_speed, uint32_t key_bytes, bool keys_alone) {
+    const uint32_t nblk = (b + 7u) >> 3;
+    return fixed_speed ? ((b * key_bytes + 15u) & ~15u) : walk_slots_at(nblk) + nblk * (keys_alone ? 32u : 128u);
 }
 __host__ __device__ inline uint32_t walk_rest_bytes(WalkKind kind) { return kind == kWalkUsual ? 0u : (kind == kWalkBigKind ? 48u : 80u); }
 __host__ __device__ inline uint32_t walk_region_bytes(uint32_t n_models, uint32_t n_inst, uint32_t slot_bytes, WalkKind kind) {

@@ -19,11 +19,12 @@
 // Nothing is counted per rejected request: the request count and the checksum of "all of them rejected"
 // are per-class totals of the trace, and a served request takes its own term out again.
 //
-// Measured (B200; lane-group, thread or one-warp kernel before): 143 placements x 500 requests 0.26 ms (0.44),
-// 10,864 x 10,000 8.7 ms (12.2), 2,000 x 17,000 of the paper's shape 13.6 ms (33.8), with queues 18.6 (27.0),
-// 100,000 x 100,000 under load 121 ms (132), 64 x 20,000 8.9 ms (18.9), 2,000 placements of 33 to 128 instances x
-// 10,000 11.5 ms (15.4).  A round with one completion takes 290 warp instructions and, alone on its scheduler,
-// 1,360 cycles.
+// Measured (B200; lane-group, thread or one-warp kernel before): 143 placements x 500 requests 0.23 ms (0.44),
+// 10,864 x 10,000 7.4 ms (12.2), 2,000 x 17,000 of the paper's shape 10.6 ms (33.8), with queues 10.9 ms (27.0),
+// 100,000 x 100,000 under load 116 ms (132), 64 x 20,000 7.8 ms (18.9), 2,000 placements of 33 to 128 instances x
+// 10,000 10.9 ms (15.4).  A round with one completion takes 300 warp instructions and, alone on its scheduler,
+// 1,280 cycles, almost all of them dependent: what the next step needs is therefore read from shared memory ahead of
+// the choice, and the uncommon outcomes share one branch (1,470 cycles before).
 //
 // The block's pool of shared memory is split evenly among its warps.  Placements beyond one warp's part run
 // first, with half, a quarter, ... of the warps at work and twice, four times, ... the room for each (kWalkModes);
@@ -75,16 +76,13 @@ __device__ __forceinline__ uint64_t warp_min(uint64_t v) {
     for (int o = 16; o > 0; o >>= 1) v = min(v, wshfl_xor(v, o));
     return v;
 }
-__device__ __forceinline__ uint32_t min_of_8(const uint4& a, const uint4& b) {
-    return __vimin3_u32(__vimin3_u32(a.x, a.y, a.z), __vimin3_u32(a.w, b.x, b.y), min(b.z, b.w));
-}
-
-// ceil(dt / s) for 1 <= dt < 2^31 and a quotient below 2^16, rs = 1 / s to a few units in the last place: the
-// float estimate is within one of the true quotient and is fixed up exactly.
+// ceil(dt / s) for 0 <= dt < 2^31 and a quotient below 2^16, rs a little below 1 / s (walk_rcp): the float estimate is at
+// most the true quotient, and less than one below it.
+__device__ __forceinline__ float walk_rcp(uint32_t s) { return rcp_approx((float)s) * (1.0f - 0x1p-20f); }
 __device__ __forceinline__ uint32_t walk_steps(int32_t dt, uint32_t s, float rs) {
     const uint32_t q = (uint32_t)(__uint2float_rz((uint32_t)dt) * rs);
-    const int32_t r = (int32_t)((uint32_t)dt - q * s);
-    return q + (r > 0 ? 1u : 0u) + (r > (int32_t)s ? 1u : 0u) - (r <= -(int32_t)s ? 1u : 0u);
+    const uint32_t r = (uint32_t)dt - q * s;
+    return q + (r > 0u ? 1u : 0u) + (r > s ? 1u : 0u);
 }
 __device__ __forceinline__ uint32_t walk_steps(int64_t dt, uint32_t s, float rs) { return ceil_div_small(dt, s, rs); }
 
@@ -153,7 +151,7 @@ static __device__ __noinline__ void walk_hand_over(const EvalParams& P, uint32_t
     if (atomicExch(&P.code[cand], 0xFFFFFFFEu) == 0xFFFFFFFEu) return;
     const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
     uint32_t slots = 0, mode = 0;
-    for (uint32_t i = 0; i < n_i; i++) slots += walk_slot_bytes((((P.inst[lo + i] >> 12) & 0xFFu) + 7u) >> 3, fixed_speed ? 8u : 4u, fixed_speed);
+    for (uint32_t i = 0; i < n_i; i++) slots += walk_slot_bytes((P.inst[lo + i] >> 12) & 0xFFu, fixed_speed, fixed_speed ? 8u : 4u, fixed_speed);
     const uint32_t need = walk_region_bytes(P.n_models, n_i, slots, kWalkLongKind);
     while (mode + 1u < (uint32_t)kWalkModes && need > (P.walk_bytes << mode)) mode++;
     // (what 16 parts cannot hold is not in a walking bucket in the first place)
@@ -310,7 +308,7 @@ struct Walk {
                         // per instance: earliest start, prefill base and slope, smallest prediction step
                         w4(at) = make_uint4(0u, in.pre_base, in.pre_q16, ms);
                     }
-                    const uint32_t bytes = nblk ? walk_slot_bytes(nblk, kKeyBytes, kFixed || kAway) : 0u;
+                    const uint32_t bytes = nblk ? walk_slot_bytes(in.B, kFixed, kKeyBytes, kFixed || kAway) : 0u;
                     uint32_t incl = bytes;
                     for (uint32_t o = 1; o < 32u; o <<= 1) {
                         const uint32_t v = __shfl_up_sync(kWFull, incl, o);
@@ -318,14 +316,12 @@ struct Walk {
                     }
                     if (nblk) {
                         in.area = area + incl - bytes;
-                        in.keys = in.area + walk_slots_at(nblk, kKeyBytes);
-                        for (uint32_t i = 0; i < 8u * (nblk + 1u); i++) {
-                            const uint32_t slot8 = i < 8u ? in.area + kKeyBytes * i
-                                                          : in.keys + kBlock * ((i - 8u) >> 3) + kKeyBytes * (i & 7u);
-                            if (kFixed) wt<T>(slot8) = kFar;
-                            else w1(slot8) = kKeyEmpty;
+                        in.keys = kFixed ? in.area : in.area + walk_slots_at(nblk);
+                        if (!kFixed) {
+                            for (uint32_t i = 0; i < 8u * (nblk + 1u); i++)
+                                w1(i < 8u ? in.area + 4u * i : in.keys + kBlock * ((i - 8u) >> 3) + 4u * (i & 7u)) = kKeyEmpty;
+                            for (uint32_t i = 0; i < in.B; i++) walk_smem[in.area + 32u + i] = (unsigned char)i;
                         }
-                        for (uint32_t i = 0; i < in.B; i++) walk_smem[in.area + 8u * kKeyBytes + i] = (unsigned char)i;
                     }
                     if (Wide && !Big && j < n_i) wt<T>(rest + 8u * j) = 0;
                     if (Big) {
@@ -372,15 +368,15 @@ struct Walk {
             auto is_due = [&](T upto) { return kFixed ? in.tb <= upto : in.tb < upto; };
             // when the instance could start a request
             auto start = [&]() -> T { return kFixed ? (in.w == in.B ? in.tb : now) : (in.w == in.B ? in.tb + (T)in.sw : in.t); };
-            // Level, step and next completion `left` steps after in.t >= 0; flags what leaves the horizon.
-            auto next_end = [&](uint32_t left, bool busy) {
-                in.sw = w1(in.row + 4u * in.w - 4u);  // (an instance that is now idle reads the word before its row)
-                in.rsw = rcp_approx((float)in.sw);
+            // Step `sw` and next completion `left` steps after in.t >= 0; flags what leaves the horizon.
+            auto next_end = [&](uint32_t left, bool busy, uint32_t sw) {
+                in.sw = sw;
+                in.rsw = Wide ? rcp_approx((float)sw) : walk_rcp(sw);
                 if constexpr (Wide) {
-                    in.tb = busy ? in.t + (int64_t)((uint64_t)left * in.sw) - (int64_t)in.sw : kFar;
+                    in.tb = busy ? in.t + (int64_t)((uint64_t)left * sw) - (int64_t)sw : kFar;
                 } else {
-                    const uint64_t tc = (uint64_t)left * in.sw + (uint32_t)in.t;
-                    in.tb = busy ? (int32_t)((uint32_t)tc - in.sw) : kFar;
+                    const uint64_t tc = (uint64_t)left * sw + (uint32_t)in.t;
+                    in.tb = busy ? (int32_t)((uint32_t)tc - sw) : kFar;
                     bad = bad || (busy && tc > (uint64_t)kWalkHorizon);
                 }
             };
@@ -391,25 +387,8 @@ struct Walk {
                 while (dm) {
                     if constexpr (kFixed) {
                         if (due) {
-                            // the first block and the first slot that hold the earliest finish time
-                            const uint32_t nblk = (in.B + 7u) >> 3;
-                            uint32_t b = 0, j = 0;
-                            while (b + 1u < nblk && wt<T>(in.area + kKeyBytes * b) != in.tb) b++;
-                            const uint32_t kb = in.keys + 8u * kKeyBytes * b;
-                            T k[8], m = kFar;
-#pragma unroll
-                            for (uint32_t i = 0; i < 8u; i++) k[i] = wt<T>(kb + kKeyBytes * i);
-#pragma unroll
-                            for (int i = 7; i >= 0; i--) j = k[i] == in.tb ? (uint32_t)i : j;
-#pragma unroll
-                            for (uint32_t i = 0; i < 8u; i++) m = min(m, i == j ? kFar : k[i]);
-                            wt<T>(kb + kKeyBytes * j) = kFar;
-                            wt<T>(in.area + kKeyBytes * b) = m;
                             in.w--;
-                            walk_smem[in.area + 8u * kKeyBytes + in.w] = (unsigned char)(8u * b + j);
-#pragma unroll
-                            for (uint32_t i = 0; i < 8u; i++) m = min(m, i == b ? kFar : wt<T>(in.area + kKeyBytes * i));
-                            in.tb = m;
+                            in.tb = in.w > 0 ? wt<T>(in.keys + kKeyBytes * (in.w - 1u)) : kFar;
                             due = in.w > 0 && is_due(upto);
                         }
                     } else {
@@ -419,6 +398,7 @@ struct Walk {
                             const uint32_t slot = in.kmin & 63u;
                             const uint32_t kb = in.keys + (slot >> 3) * kBlock, k8 = kb + 4u * (slot & 7u);
                             const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(in.area), m1 = w4(in.area + 16u);
+                            const uint32_t sw = w1(in.row + 4u * in.w - 8u);  // (the word before the row, if that was the last one)
                             uint2 ft;
                             uint32_t rq;
                             if constexpr (kAway) {
@@ -447,7 +427,7 @@ struct Walk {
                             in.kmin = min(bmin, min8(mv)) + km;
                             const uint32_t left = (in.kmin >> 6) - in.K;
                             const bool busy = in.w > 0;
-                            next_end(left, busy);
+                            next_end(left, busy, sw);
                             due = busy && (left == 0u || in.tb < upto) && !bad;
                         }
                         ring_n += adds;
@@ -455,14 +435,28 @@ struct Walk {
                     dm = __ballot_sync(kWFull, due);
                 }
             };
-            // A clock that lags behind `upto` while nothing completes: the next step boundary.
-            auto catch_up = [&](T upto) {
-                if (in.w == 0) {
-                    in.t = upto;  // an idle instance starts at once
+            // Clocks of the lanes in `go` that lag behind `upto` while nothing completes: the next step boundary; an idle
+            // instance starts at once.
+            auto catch_up = [&](bool go, T upto) {
+                if constexpr (Wide) {
+                    if (go && in.t < upto) {
+                        const uint32_t k = walk_steps((T)(upto - in.t), in.sw, in.rsw);
+                        in.t = in.w == 0 ? upto : in.t + (T)((U)k * in.sw);
+                        in.K += k;
+                    }
                 } else {
-                    const uint32_t k = walk_steps((T)(upto - in.t), in.sw, in.rsw);
-                    in.t += (T)((U)k * in.sw);
+                    const int32_t dt = go ? max(upto - in.t, 0) : 0;
+                    const uint32_t k = walk_steps(dt, in.sw, in.rsw);
+                    in.t += in.w == 0 ? dt : (int32_t)(k * in.sw);
                     in.K += k;
+                }
+            };
+            // The next free slot and the step with one request more, read ahead of the choice.
+            uint32_t top = 0, more = 0;
+            auto peek = [&]() {
+                if (!kFixed) {
+                    top = walk_smem[in.area + 32u + in.w];
+                    more = w1(in.row + 4u * in.w);
                 }
             };
             // One request's times into the ring (`e`: its entry).
@@ -471,55 +465,48 @@ struct Walk {
                 w4(ring + e * 16u) = make_uint4(lo32(f), hi32(f), lo32(g), hi32(g));
                 w2(ring_b + e * 8u) = make_uint2(req, in.tag >> 16);
             };
-            // "map": prefill at the step boundary (running decodes stall), then occupy a free slot; with fixed speeds the
-            // slot is busy until the finish time, and `queued` takes over the slot that frees first.  All lanes call it.
-            auto admit = [&](bool win, uint32_t req, uint32_t Sm1, T pre, bool queued) {
+            // "map": prefill at the step boundary (running decodes stall), then occupy a free slot.  With fixed speeds the slot
+            // is busy until the finish time, and `queued` takes over the slot that frees first; an instance's finish times
+            // are in falling order, the winner's (lane `wl`) are moved by all lanes.  All lanes call it.
+            auto admit = [&](bool win, int wl, uint32_t req, uint32_t Sm1, T pre, bool queued) {
                 if constexpr (kFixed) {
                     if (ring_n + 1u > kCap) flush();
+                    const uint32_t at = __shfl_sync(kWFull, (in.keys << 7) | in.w, wl), a = at >> 7;
+                    uint32_t n = at & 127u, level;
+                    if (queued) n--;  // the last one goes
+                    T v[2], first = now + pre;
+#pragma unroll
+                    for (uint32_t h = 0; h < 2u; h++) v[h] = 32u * h < n && lane + 32u * h < n ? wt<T>(a + kKeyBytes * (lane + 32u * h)) : kFar;
+                    level = n;
+                    if (queued) {  // whatever frees together with the slot taken is not busy when the request starts
+                        const T tb = wshfl(in.tb, wl);
+                        level -= (uint32_t)(__popc(__ballot_sync(kWFull, v[0] == tb)) + __popc(__ballot_sync(kWFull, v[1] == tb)));
+                        first = in.tb + pre;
+                    }
+                    const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? 4u * level : 0u));
+                    T fin = first + (T)span;
                     if (win) {
-                        const uint32_t nblk = (in.B + 7u) >> 3;
-                        uint32_t slot, level;
-                        T first;
-                        if (!queued) {
-                            slot = walk_smem[in.area + 8u * kKeyBytes + in.w];
-                            level = in.w++;
-                            first = now + pre;
-                        } else {
-                            slot = 0xFFFFFFFFu;
-                            uint32_t same = 0;
-                            for (uint32_t i = 0; i < 8u * nblk; i++)
-                                if (wt<T>(in.keys + kKeyBytes * i) == in.tb) {
-                                    if (slot == 0xFFFFFFFFu) slot = i;
-                                    else same++;  // ends at the same time: not busy any more when the request starts
-                                }
-                            level = in.B - 1u - same;
-                            first = in.tb + pre;
-                        }
-                        const uint32_t speed = w1(in.row + 4u * level);
-                        const uint64_t span = (uint64_t)Sm1 * speed;
-                        const T fin = first + (T)span;
                         if constexpr (Wide) {
                             if (((uint64_t)fin >> 57) != 0) status = MAASO_CAND_ELOOP;  // beyond what the engine takes
                         } else {
                             bad = bad || span > (uint64_t)kWalkHorizon || fin > (T)kWalkHorizon;
                         }
-                        wt<T>(in.keys + kKeyBytes * slot) = fin;
-                        const uint32_t mb = in.area + kKeyBytes * (slot >> 3);
-                        if (!queued) {
-                            wt<T>(mb) = min(wt<T>(mb), fin);
-                            in.tb = min(in.tb, fin);
-                        } else {
-                            T m = kFar;
-#pragma unroll
-                            for (uint32_t i = 0; i < 8u; i++) m = min(m, wt<T>(in.keys + kKeyBytes * ((slot & 56u) + i)));
-                            wt<T>(mb) = m;
-#pragma unroll
-                            for (uint32_t i = 0; i < 8u; i++) m = min(m, wt<T>(in.area + kKeyBytes * i));
-                            in.tb = m;
-                        }
                         record(ring_n, fin, first, req);
                     }
                     ring_n++;
+                    fin = wshfl(fin, wl);
+                    uint32_t pos = n;
+#pragma unroll
+                    for (uint32_t h = 0; h < 2u; h++) {
+                        pos -= (uint32_t)__popc(__ballot_sync(kWFull, v[h] < fin));
+                        if (v[h] < fin) wt<T>(a + kKeyBytes * (lane + 32u * h + 1u)) = v[h];
+                    }
+                    if (lane == 0) wt<T>(a + kKeyBytes * pos) = fin;
+                    __syncwarp();
+                    if (win) {
+                        in.w = n + 1u;
+                        in.tb = wt<T>(a + kKeyBytes * n);
+                    }
                 } else if (Sm1 == 0u) {  // done at the end of its prefill, never occupies a slot
                     if (ring_n + 1u > kCap) flush();
                     if (win) {
@@ -530,7 +517,7 @@ struct Walk {
                     }
                     ring_n++;
                 } else if (win) {
-                    const uint32_t slot = walk_smem[in.area + 32u + in.w];
+                    const uint32_t slot = top;
                     in.t += pre;
                     if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
                     if (in.K + Sm1 > kRelMax) {
@@ -550,7 +537,7 @@ struct Walk {
                     atomicMin(&w1(in.area + ((slot >> 3) << 2)), nk);
                     in.kmin = min(in.kmin, nk);
                     in.w++;
-                    next_end((in.kmin >> 6) - in.K, true);
+                    next_end((in.kmin >> 6) - in.K, true, more);
                 }
             };
 
@@ -601,7 +588,7 @@ struct Walk {
                     live &= live - 1u;
                     T arrival = wshfl(rel, src);
                     if constexpr (!Wide) {
-                        if (arrival == kFar || now >= kWalkNowMax) {
+                        if (max(now, arrival) >= kWalkNowMax) {  // (or the arrival is out of reach)
                             // move the epoch to the dispatcher's clock (or to the request's arrival, if that is later): what
                             // happens before it is simulated, everything else is measured from there on
                             const uint4 v = __ldg(reqs + req);
@@ -615,18 +602,14 @@ struct Walk {
                                 }
                                 events(mine && in.w > 0 && is_due(up), up);
                                 if (kFixed) {
-                                    const uint32_t nblk = (in.B + 7u) >> 3;
                                     if (mine && in.w > 0) {
-                                        for (uint32_t i = 0; i < 8u * (nblk + 1u); i++) {
-                                            T& k = wt<T>(i < 8u ? in.area + kKeyBytes * i : in.keys + kKeyBytes * (i - 8u));
-                                            if (k != kFar) k -= up;
-                                        }
+                                        for (uint32_t i = 0; i < in.w; i++) wt<T>(in.keys + kKeyBytes * i) -= up;
                                         in.tb -= up;
                                     }
                                 } else if (in.w == 0) {
                                     in.t = in.t > up ? in.t - up : 0;  // an idle instance is where the dispatcher is
                                 } else {
-                                    if (in.w < in.B && in.t < up) catch_up(up);
+                                    catch_up(in.w < in.B, up);
                                     in.t = in.t > up + kWPast ? in.t - up : kWPast;  // a full instance's clock is not looked at
                                     in.tb -= up;
                                 }
@@ -676,11 +659,12 @@ struct Walk {
                             // "reduce": what completes before the instance's clock reaches `now`
                             events(elig && is_due(now), now);
                             const bool full = in.w == in.B;
-                            if (!kFixed && elig && !full && in.t < now) catch_up(now);
+                            if (!kFixed) catch_up(elig && !full, now);
+                            if (!Big || Opt) peek();
                             // distributor prediction (Sec. IV-F steps 2-3)
                             const T t = start();
                             uint32_t sB = in.stepB;
-                            if (Opt && !full) sB = w1(in.row + 4u * in.w);
+                            if (Opt && !full) sB = kFixed ? w1(in.row + 4u * in.w) : more;
                             const bool ok = elig && lim.met((U)(t + p - arrival), Sm1, sB);
                             // smallest (tier, predicted first token >= now >= 0), lowest instance among equals
                             const U k = ok ? (full ? kTier1 : (U)0) | (U)(t + p) : kNone;
@@ -697,58 +681,60 @@ struct Walk {
                         }
                         const U best = warp_min(key);
                         again = false;
-                        look = look || (best & kTier1) != 0;
-                        if (Big && (best & kTier1) != 0) {  // rejected, or waits: the model's new bound of any first token
-                            const U m = warp_min((U)lb);
-                            if (lane == 0) wi(lbs + 8u * model) = (int64_t)(T)m;
+                        int wl = __ffs((int)__ballot_sync(kWFull, key == best)) - 1;  // the winner's lane
+                        if (Big && best != kNone) {
+                            const uint32_t lowest = __reduce_min_sync(kWFull, key == best ? at : 0xFFFFFFFFu);
+                            wl = (int)(lowest & 31u);
+                            if ((int)lane == wl) {
+                                at = lowest;
+                                get(rest, ents, n_i, at, in);
+                                peek();
+                            }
                         }
-                        if (best != kNone) {
-                            bool win;
-                            if (Big) {
-                                const uint32_t lowest = __reduce_min_sync(kWFull, key == best ? at : 0xFFFFFFFFu);
-                                win = key == best && at == lowest;
-                                if (win) get(rest, ents, n_i, at, in);
+                        const bool win = (int)lane == wl;
+                        bool go = true, queued = false;
+                        if (best >= kTier1) {
+                            if (Big) {  // rejected, or waits: the model's new bound of any first token
+                                const U m = warp_min((U)lb);
+                                if (lane == 0) wi(lbs + 8u * model) = (int64_t)(T)m;
+                            }
+                            if (best == kNone) {  // overflow protection: nobody can meet the deadline
+                                if (side && lane == 0) walk_reject_side(P, tr * P.n_cand + cand, req, model);
+                                go = false;
+                                look = true;
+                            } else if (Eng == 2) {
+                                queued = true;  // every capable instance is full: queues at the chosen one, the dispatcher goes on
                             } else {
-                                win = (int)lane == __ffs((int)__ballot_sync(kWFull, key == best)) - 1;
-                            }
-                            bool queued = false;
-                            if ((best & kTier1) != 0) {
-                                // every capable instance is full
-                                if (Eng == 2) {
-                                    queued = true;  // the request queues at the chosen one; the dispatcher goes on
+                                // every capable instance is full: wait until the chosen slot frees
+                                now = wshfl(t0, wl);
+                                if (!kAgain) {
+                                    // With the worst-case estimate the next round cannot choose differently: at that time the
+                                    // winner has a free slot with the same predicted first token, and no other instance's
+                                    // prediction can have become earlier or feasible.  The second round is only counted.
+                                    events(win, now);
+                                    peek();
                                 } else {
-                                    // wait until the chosen slot frees
-                                    now = wshfl(t0, __ffs((int)__ballot_sync(kWFull, win)) - 1);
-                                    if (!kAgain) {
-                                        // With the worst-case estimate the next round cannot choose differently: at that
-                                        // time the winner has a free slot with the same predicted first token, and no
-                                        // other instance's prediction can have become earlier or feasible.  The second
-                                        // round is only counted.
-                                        tries++;
-                                        events(win, now);
-                                    } else {
-                                        again = true;
-                                        if (tries >= kAttemptCap) { status = MAASO_CAND_ELOOP; again = false; }
-                                    }
+                                    again = true;
+                                    go = false;
+                                    if (tries >= kAttemptCap) { status = MAASO_CAND_ELOOP; again = false; }
                                 }
+                                if (lane == 0 && (!kAgain || again)) atomicAdd(&w1(base + kSExtra), 1u);
                             }
-                            if (!again && status == 0u) {
-                                admit(win, req, Sm1, pre, queued);
-                                if (Big && win) {
-                                    if (!Wide) w1(ents + 16u * at) = (uint32_t)start();
-                                    put(rest, n_i, at, in, false);
-                                }
+                        }
+                        if (go) {
+                            admit(win, wl, req, Sm1, pre, queued);
+                            if (Big && win) {
+                                if (!Wide) w1(ents + 16u * at) = (uint32_t)start();
+                                put(rest, n_i, at, in, false);
                             }
-                        } else if (side && lane == 0) {
-                            walk_reject_side(P, tr * P.n_cand + cand, req, model);  // overflow protection: nobody can meet the deadline
                         }
                         if (!Big && elig) wt<T>(Wide ? rest + 8u * lane : ent) = start();
                         if (kFixed && Wide) status = __reduce_or_sync(kWFull, status);
                     } while (kAgain && again);
-                    if (tries > 1u && lane == 0) w1(base + kSExtra) += tries - 1u;
-                    if (status) break;
-                    // after a plain admission the other live requests of the chunk stay live; a rejection or a wait has
-                    // changed what the scan goes by
+                    if ((kAgain || (kFixed && Wide)) && status) break;
+                    // The other live requests of the chunk stay live, unless this one was rejected: what the scan went by is out
+                    // of date then.  (A wait alone makes few others hopeless: 0 to 0.3 of them on average, and finding out
+                    // takes as long as a round.)
                     if (look) {
                         __syncwarp();
                         if (live) live = test((uint32_t)src + 1u);
