@@ -27,6 +27,7 @@ constexpr int kWalkBuckets = 2 * kWalkModes + 1;
 constexpr int kGenericBlockBucket = 9;
 constexpr int kThreadBucket0 = 10;  // buckets 10..18: the thread mapping, by lanes per warp
 constexpr int kThreadBuckets = 9;
+constexpr int kPack4 = 2, kPack8 = 3;  // in place of the lane groups (EvalParams::pack): up to 4 and up to 8 instances
 constexpr int kWideBucket = 19;     // 33..128 instances under the engines of the lane-group code: one warp per placement
 constexpr int kPrepOne = 1024;   // candidates one block of the validation kernel takes
 constexpr int kCostBins = 256;   // bin 0 = most expensive (largest total batch cap)
@@ -289,6 +290,7 @@ struct EvalParams {
     uint32_t* walk_ctr;      // [kWalkBuckets]: next placement of each walking bucket
     uint32_t walk_bytes;     // walking kernel: bytes of shared memory one of 16 warps has for a placement, 0 = not used
     uint32_t walk_usual;     // the same for placements of up to 32 instances, with walk_warps warps
+    uint32_t pack;           // placements of at most 8 instances that could go to the lane groups share the steps of a warp instead
     uint32_t walk_warps;
     uint32_t walk_long;      // the whole batch with 64-bit times
     long long wait_cycles;   // bound of every device-side wait

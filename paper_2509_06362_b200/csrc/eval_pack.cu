@@ -1,0 +1,391 @@
+// Scoring kernel for many lightly loaded placements of at most 8 instances: the placements of a warp share its steps.
+//
+// What bounds it: instruction issue and the chain of steps together.  Where most requests are served, nearly every request
+// needs a distributor round in every placement, and a round of the walking kernel leaves all but a few lanes idle.  Here a
+// group of 4 or 8 lanes replays one placement, lane = instance, and the groups of a warp take the same request of the same
+// trace at the same time: one step of about 400 warp instructions is 4 or 8 rounds.  The request and its limits are the
+// same in all lanes, the choice is a butterfly inside the group, completions of all groups are worked off together.  Under
+// load the walking kernel is the better one: it skips what is turned away, and a step here waits for every group.
+//
+// The rest is the walking kernel's: 32-bit times from an epoch (here the same for the warp, moved to a request's
+// arrival), keys in shared memory, a ring of completions (one part per group) accounted by the group's lanes.  A running
+// request's first token and index (16 bytes per slot) and the sums, which a step does not wait for, are in global memory:
+// what is left in shared memory is the same for every placement, so that 16 warps always fit.
+//
+// Measured (B200; 64-bit lane groups before): 9,000 placements of one node x 5,000 requests at 2 a second 9.4 ms (13.3),
+// at 8 a second 5.2 (5.9), 10,864 x 10,000 x 16 arrival rates 137 ms (214).  Groups of 2 lanes for placements of one and
+// two instances were slower (12.3 and 142 ms): 16 placements step through more completions one after the other than 8 do.
+#include "walk_kernel.cuh"
+
+namespace maaso {
+
+constexpr uint32_t kPackLane = 32u + 64u + 256u + 16u;  // block minima, free slots, keys; 16 bytes so that lanes start in different banks
+constexpr uint32_t kPackPay = 64u * 16u, kPackScratch = kPackPay + 128u;  // a lane's running requests; then sums (64 bytes), hits by class bin (32)
+
+__host__ __device__ inline WalkLayout pack_layout(uint32_t n_rows, uint32_t n_classes) {
+    return walk_layout(n_rows, n_classes, false, (uint32_t)kWalkWarps);
+}
+size_t pack_scratch(int grid) { return (size_t)grid * 32u * kWalkWarps * kPackScratch; }
+bool pack_fits(uint32_t n_rows, uint32_t n_classes) {
+    return pack_layout(n_rows, n_classes).pool + 32u * kWalkWarps * kPackLane <= 227u * 1024u;
+}
+
+// Accounts a group's ring, one entry per lane and pass (lane `li` of `G`; `mine`: the lane's sums).
+static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumping, uint32_t oc, unsigned char* mine, uint32_t* bins,
+                                                 uint32_t ring, uint32_t ring_b, uint32_t li, uint32_t G, uint32_t cnt, uint32_t lims,
+                                                 const uint4* reqs) {
+    __syncwarp();
+    if (li < cnt) {
+        uint4* const sums = reinterpret_cast<uint4*>(mine);
+        const uint4 u0 = __ldcg(sums), u1 = __ldcg(sums + 1), u2 = __ldcg(sums + 2), u3 = __ldcg(sums + 3);
+        int64_t st = i64_of(u0.x, u0.y), mt = i64_of(u0.z, u0.w), se = i64_of(u1.x, u1.y), me = i64_of(u1.z, u1.w);
+        int64_t mk = i64_of(u2.x, u2.y), tk = i64_of(u3.x, u3.y);
+        uint64_t sum = (uint64_t)i64_of(u2.z, u2.w);
+        uint32_t served = u3.z, hits = u3.w;
+        for (uint32_t e = li; e < cnt; e += G) {
+            const uint2 rb = w2(ring_b + e * 8u);
+            const uint4 rec = __ldg(reqs + rb.x);
+            const uint4 ra = w4(ring + e * 16u);
+            const int64_t fin = i64_of(ra.x, ra.y), first = i64_of(ra.z, ra.w), arrival = i64_of(rec.x, rec.y);
+            const uint32_t S = rec.w & 0xFFFFu, cls = (rec.w >> 16) & 0xFFu;
+            const uint4 lim = w4(lims + cls * 16u);
+            const int64_t ttft = first - arrival, e2e = fin - arrival;
+            const bool hit = e2e <= i64_of(lim.z, lim.w) && (lim.x == 0xFFFFFFFFu || ttft <= (int64_t)lim.x) &&
+                             (lim.y == 0xFFFFFFFFu || (uint64_t)(fin - first) <= (uint64_t)(S - 1u) * lim.y);
+            // the request's term as a served one in, its term as a rejected one out
+            sum += served_hash(rb.x, fin, first, rb.y) - rejected_hash(rb.x);
+            st += ttft;
+            mt = max(mt, ttft);
+            se += e2e;
+            me = max(me, e2e);
+            mk = max(mk, fin);
+            tk += S;
+            served++;
+            hits += hit ? 1u : 0u;
+            if (hit) atomicAdd(bins + (cls < 7u ? cls : 7u), 1u);
+            if (dumping) {
+                const Dump d = dump_for(P, oc);
+                if (d.finish) d.finish[rb.x] = fin;
+                if (d.first) d.first[rb.x] = first;
+                if (d.inst) d.inst[rb.x] = (int32_t)rb.y;
+                if (d.hist) atomicAdd(d.hist + ttft_bin(ttft), 1u);
+            }
+        }
+        __stcg(sums, make_uint4(lo32(st), hi32(st), lo32(mt), hi32(mt)));
+        __stcg(sums + 1, make_uint4(lo32(se), hi32(se), lo32(me), hi32(me)));
+        __stcg(sums + 2, make_uint4(lo32(mk), hi32(mk), (uint32_t)sum, (uint32_t)(sum >> 32)));
+        __stcg(sums + 3, make_uint4(lo32(tk), hi32(tk), served, hits));
+    }
+    __syncwarp();
+}
+
+// One warp takes work items, one after the other: 32 / G placements of the bucket whose groups have G lanes, the largest
+// placements first.  (One numbering for both buckets: starting on each from the same warps would have some replay an item
+// of each in a row where there is one item for each warp.)
+template <bool Opt>
+static __device__ __forceinline__ void pack_items(const EvalParams& P, const WalkLayout& L, uint32_t idx, uint32_t static_total) {
+    using W = Walk<Opt, 0, false, false>;
+    using Limits = typename W::Limits;
+    constexpr int32_t kFar = kWalkFar;
+    constexpr uint32_t kTier1 = 1u << 31, kNone = ~0u;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, below = (1u << lane) - 1u;
+    const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
+    const uint32_t n8 = (P.bucket_count[kPack8] + 3u) / 4u, n4 = (P.bucket_count[kPack4] + 7u) / 8u;
+    const uint32_t total = (n8 + n4) * n_traces;
+    const uint32_t area = L.pool + threadIdx.x * kPackLane, keys = area + 96u;
+    unsigned char* const pay = reinterpret_cast<unsigned char*>(P.payload) + ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * kPackScratch;
+    const bool use_mask = P.class_mask != nullptr && P.n_classes <= 32;
+
+    while (idx < total) {
+        // ---- the next placements ------------------------------------------------------------------------------
+        const uint32_t tr = idx % n_traces, item = idx / n_traces;
+        const bool eight = item < n8;
+        const uint32_t G = eight ? 8u : 4u, g = lane / G, li = lane & (G - 1u), gmask = ((1u << G) - 1u) << (lane - li);
+        const uint32_t bucket = eight ? kPack8 : kPack4, count = P.bucket_count[bucket];
+        const uint32_t at = (eight ? item : item - n8) * (32u / G) + g;
+        const bool valid = at < count;
+        const uint32_t cap = 2u * G;  // a group's part of the ring
+        const uint32_t ring = L.ring + (warp * kWalkRing + g * cap) * 16u;  // (the second part of an entry is half as far in)
+        const uint32_t cand = P.bucket_list[(size_t)bucket * P.n_cand + (valid ? at : count - 1u)], oc = tr * P.n_cand + cand;
+        const uint4* const reqs = P.trace_reqs[tr];
+        const uint32_t n_req = P.trace_n[tr];
+        uint4 nxt = make_uint4(0u, 0u, 0u, 0u);
+        if (n_req) nxt = __ldg(reqs + min(lane, n_req - 1u));
+        WInst<int32_t> in;
+        in.t = 0; in.tb = kFar; in.K = 0; in.kmin = kKeyEmpty; in.w = 0; in.B = 1; in.sw = 1; in.rsw = 1.0f;
+        in.pre_base = in.pre_q16 = 0; in.stepB = 1; in.tag = 0; in.row = L.steps;
+        {
+            const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
+            if (valid && li < n_i) {
+                const uint32_t word = P.inst[lo + li], md = word & 0xFu, r = md * P.n_strategies + ((word >> 4) & 0xFFu);
+                in.tag = 1u << md;
+                in.B = (word >> 12) & 0xFFu;
+                in.row = L.steps + r * 256u;
+                in.pre_base = (uint32_t)P.rows[r * kRowStride];
+                in.pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
+                in.stepB = w1(in.row + 4u * in.B - 4u);
+            }
+        }
+        for (uint32_t i = 0; i < 8u + ((in.B + 7u) & ~7u); i++) w1(i < 8u ? area + 4u * i : keys + 4u * (i - 8u)) = kKeyEmpty;
+        for (uint32_t i = 0; i < in.B; i++) walk_smem[area + 32u + i] = (unsigned char)i;
+#pragma unroll
+        for (uint32_t i = 0; i < 6u; i++) __stcg(reinterpret_cast<uint4*>(pay + kPackPay) + i, make_uint4(0u, 0u, 0u, 0u));
+        __threadfence();
+        __syncwarp();
+        const uint32_t cmask = use_mask ? P.class_mask[cand] : 0xFFFFFFFFu;
+        const bool side = valid && (P.rej_by_model != nullptr || (P.dump_row && P.dump_row[cand] >= 0));
+        uint32_t ring_n = 0, status = 0, extra = 0;
+        int64_t epoch = 0;
+        int32_t now = 0, rel = 0;
+        uint32_t c_in = 0, c_meta = 0;
+        bool bad = false;  // a time of this lane has left the horizon
+
+        auto bins = [&]() { return reinterpret_cast<uint32_t*>(pay - li * kPackScratch + kPackPay + 64u); };
+        auto flush = [&]() {
+            pack_account(P, P.dump_row || P.ttft_hist, oc, pay + kPackPay, bins(), ring, L.ring_b + ((ring - L.ring) >> 1), li, G, ring_n, L.lims, reqs);
+            ring_n = 0;
+        };
+        auto take_chunk = [&](const uint4& v) {
+            const int64_t d = i64_of(v.x, v.y) - epoch;
+            rel = d >= (int64_t)kWalkNowMax ? kFar : (d < (int64_t)kWPast ? kWPast : (int32_t)d);
+            c_in = v.z;
+            c_meta = v.w;
+        };
+        auto next_end = [&](uint32_t left, bool busy, uint32_t sw) {
+            in.sw = sw;
+            in.rsw = walk_rcp(sw);
+            const uint64_t tc = (uint64_t)left * sw + (uint32_t)in.t;
+            in.tb = busy ? (int32_t)((uint32_t)tc - sw) : kFar;
+            bad = bad || (busy && tc > (uint64_t)kWalkHorizon);
+        };
+        // Completions of the lanes in `due` before `upto`, one per lane and iteration.
+        auto events = [&](bool due, int32_t upto) {
+            uint32_t dm = __ballot_sync(kWFull, due);
+            while (dm) {
+                const uint32_t adds = (uint32_t)__popc(dm & gmask);
+                if (__any_sync(kWFull, ring_n + adds > cap)) flush();
+                if (due) {
+                    const uint32_t slot = in.kmin & 63u, kb = keys + ((slot >> 3) << 5);
+                    const uint4 ft = __ldcg(reinterpret_cast<const uint4*>(pay) + slot);
+                    const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(area), m1 = w4(area + 16u);
+                    const uint32_t sw = w1(in.row + 4u * in.w - 8u);  // (the word before the row, if that was the last one)
+                    in.t = in.tb + (int32_t)in.sw;
+                    in.K = in.kmin >> 6;
+                    in.w--;
+                    walk_smem[area + 32u + in.w] = (unsigned char)slot;
+                    // the smallest of the other keys: keys are unique, so the retired one wraps to all ones
+                    const uint32_t km = in.kmin + 1u;
+                    const uint32_t kv[8] = {k0.x - km, k0.y - km, k0.z - km, k0.w - km, k1.x - km, k1.y - km, k1.z - km, k1.w - km};
+                    const uint32_t mv[8] = {m0.x - km, m0.y - km, m0.z - km, m0.w - km, m1.x - km, m1.y - km, m1.z - km, m1.w - km};
+                    const uint32_t bmin = min8(kv);
+                    w1(keys + (slot << 2)) = kKeyEmpty;
+                    w1(area + ((slot >> 3) << 2)) = bmin + km;
+                    in.kmin = min(bmin, min8(mv)) + km;
+                    const uint32_t left = (in.kmin >> 6) - in.K;
+                    const bool busy = in.w > 0;
+                    next_end(left, busy, sw);
+                    due = busy && (left == 0u || in.tb < upto) && !bad;
+                    const uint32_t e = ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below));
+                    const int64_t fin = epoch + in.t;
+                    w2(L.ring_b + ((e - L.ring) >> 1)) = make_uint2(ft.z, li);
+                    w4(e) = make_uint4(lo32(fin), hi32(fin), ft.x, ft.y);
+                }
+                ring_n += adds;
+                dm = __ballot_sync(kWFull, due);
+            }
+        };
+        // A clock that lags behind `upto` while nothing completes: the next step boundary; an idle instance starts at once.
+        auto catch_up = [&](bool go, int32_t upto) {
+            const int32_t dt = go ? max(upto - in.t, 0) : 0;
+            const uint32_t k = walk_steps(dt, in.sw, in.rsw);
+            in.t += in.w == 0 ? dt : (int32_t)(k * in.sw);
+            in.K += k;
+        };
+
+        for (uint32_t cb = 0; cb < n_req; cb += 32u) {
+            take_chunk(nxt);
+            nxt = __ldg(reqs + min(cb + 32u + lane, n_req - 1u));
+            const uint32_t n_chunk = min(32u, n_req - cb);
+            for (uint32_t i = 0; i < n_chunk; i++) {
+                int32_t arrival = __shfl_sync(kWFull, rel, (int)i);
+                const uint32_t in_tok = __shfl_sync(kWFull, c_in, (int)i), meta = __shfl_sync(kWFull, c_meta, (int)i);
+                if (arrival == kFar) {
+                    // move the epoch to this arrival: what happens before it is simulated, the rest is measured from there on
+                    const uint4 v = __ldg(reqs + cb + i);
+                    const int64_t to = i64_of(v.x, v.y);
+                    const int32_t up = to - epoch >= (int64_t)kFar ? kFar : (int32_t)(to - epoch);
+                    events(in.w > 0 && in.tb < up && !bad, up);
+                    if (in.w == 0) {
+                        in.t = in.t > up ? in.t - up : 0;
+                    } else {
+                        catch_up(in.w < in.B, up);
+                        in.t = in.t > up + kWPast ? in.t - up : kWPast;  // a full instance's clock is not looked at
+                        in.tb -= up;
+                    }
+                    now = max(now - up, 0);
+                    epoch = to;
+                    take_chunk(__ldg(reqs + min(cb + lane, n_req - 1u)));
+                    arrival = 0;
+                }
+                const uint32_t Sm1 = (meta & 0xFFFFu) - 1u, model = meta >> 24;
+                const bool counted = (cmask >> ((meta >> 16) & 31u)) & 1u;
+                Limits lim;
+                lim.load(L, (meta >> 12) & 0xFF0u);
+                now = max(now, arrival);  // pending time: the dispatcher never goes back
+                const int32_t pre = W::prefill(in.pre_base, in.pre_q16, in_tok);
+                bool act = counted;  // this group still has to place the request
+                for (uint32_t tries = 1;; tries++) {
+                    const bool elig = act && ((in.tag >> model) & 1u);
+                    events(elig && in.tb < now, now);
+                    const bool full = in.w == in.B;
+                    catch_up(elig && !full, now);
+                    uint32_t top = walk_smem[area + 32u + in.w], more = w1(in.row + 4u * in.w);
+                    // distributor prediction (Sec. IV-F steps 2-3)
+                    const int32_t t = full ? in.tb + (int32_t)in.sw : in.t;
+                    const bool ok = elig && lim.met((uint32_t)(t + pre - arrival), Sm1, Opt && !full ? more : in.stepB);
+                    // smallest (tier, predicted first token), lowest instance among equals
+                    const uint32_t key = ok ? (full ? kTier1 : 0u) | (uint32_t)(t + pre) : kNone;
+                    uint32_t best = min(key, __shfl_xor_sync(kWFull, key, 1));
+                    best = min(best, __shfl_xor_sync(kWFull, best, 2));
+                    if (G > 4u) best = min(best, __shfl_xor_sync(kWFull, best, 4));
+                    const int wl = __ffs((int)(__ballot_sync(kWFull, key == best) & gmask)) - 1;
+                    bool win = (int)lane == wl && best < kTier1;
+                    const bool slow = act && best >= kTier1;
+                    bool again = false;
+                    if (__any_sync(kWFull, slow)) {
+                        const bool waits = slow && best != kNone;
+                        // overflow protection: nobody can meet the deadline
+                        if (side && slow && !waits && li == 0u && status == 0u) walk_reject_side(P, oc, cb + i, model);
+                        // every capable instance is full: wait until the chosen slot frees
+                        const int32_t frees = __shfl_sync(kWFull, t, wl);
+                        if (waits) now = frees;
+                        if (!Opt) {
+                            // the second round cannot choose differently (see the walking kernel): it is only counted
+                            const bool mine = waits && (int)lane == wl;
+                            events(mine, now);
+                            win = win || mine;
+                            top = walk_smem[area + 32u + in.w];
+                            more = w1(in.row + 4u * in.w);
+                        } else {
+                            again = waits;
+                            if (waits && tries >= kAttemptCap) { status = MAASO_CAND_ELOOP; again = false; }
+                        }
+                        if (waits && (!Opt || again)) extra++;
+                    }
+                    // prefill at the step boundary (running decodes stall), then occupy a free slot
+                    if (Sm1 == 0u) {  // done at the end of its prefill, never occupies a slot
+                        const uint32_t adds = __ballot_sync(kWFull, win) & gmask ? 1u : 0u;
+                        if (__any_sync(kWFull, ring_n + adds > cap)) flush();
+                        if (win) {
+                            in.t += pre;
+                            if (in.w > 0) in.tb += pre;
+                            bad = bad || in.t > kWalkHorizon || (in.w > 0 && in.tb > kWalkHorizon);
+                            const int64_t fin = epoch + in.t;
+                            w4(ring + ring_n * 16u) = make_uint4(lo32(fin), hi32(fin), lo32(fin), hi32(fin));
+                            w2(L.ring_b + ((ring - L.ring) >> 1) + ring_n * 8u) = make_uint2(cb + i, li);
+                        }
+                        ring_n += adds;
+                    } else if (win) {
+                        in.t += pre;
+                        if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
+                        if (in.K + Sm1 > kRelMax) {
+                            in.kmin = walk_rebase(area, keys, 32u, (in.B + 7u) >> 3, in.K, in.kmin);
+                            in.K = 0;
+                        }
+                        const uint32_t nk = ((in.K + Sm1) << 6) | top;
+                        const int64_t first = epoch + in.t;
+                        w1(keys + 4u * top) = nk;
+                        __stcg(reinterpret_cast<uint4*>(pay) + top, make_uint4(lo32(first), hi32(first), cb + i, 0u));
+                        atomicMin(&w1(area + ((top >> 3) << 2)), nk);
+                        in.kmin = min(in.kmin, nk);
+                        in.w++;
+                        next_end((in.kmin >> 6) - in.K, true, more);
+                    }
+                    if (!Opt) break;
+                    act = again;
+                    if (!__any_sync(kWFull, again)) break;
+                }
+            }
+            // a group that has left the horizon, or ran out of rounds, is out
+            const uint32_t out = __ballot_sync(kWFull, bad || status);
+            if (out & gmask) {
+                in.tag = 0; in.w = 0; in.tb = kFar; in.kmin = kKeyEmpty; in.t = 0; in.sw = 1; now = 0;
+            }
+        }
+
+        // ---- through the trace: drain, account, write the records -----------------------------------------------------
+        events(in.w > 0 && !bad, kFar);
+        flush();
+        if (lane == 0) idx = static_total + atomicAdd(&P.work_ctr[0], 1u);
+        idx = __shfl_sync(kWFull, idx, 0);
+        const bool away = (__ballot_sync(kWFull, bad) & gmask) != 0u;
+        __threadfence();
+        __syncwarp();
+        const uint4* const sums = reinterpret_cast<const uint4*>(pay + kPackPay);
+        const uint4 u0 = __ldcg(sums), u1 = __ldcg(sums + 1), u2 = __ldcg(sums + 2), u3 = __ldcg(sums + 3);
+        Stats st;
+        st.sum_ttft = i64_of(u0.x, u0.y); st.max_ttft = i64_of(u0.z, u0.w);
+        st.sum_e2e = i64_of(u1.x, u1.y);  st.max_e2e = i64_of(u1.z, u1.w);
+        st.makespan = i64_of(u2.x, u2.y); st.checksum = (uint64_t)i64_of(u2.z, u2.w);
+        st.tokens = (uint64_t)i64_of(u3.x, u3.y);
+        st.served = u3.z;
+        st.hit = u3.w;
+        // the request count and the checksum of "everything rejected", from the per-class totals
+        uint32_t counted_all = 0;
+        for (uint32_t c = li; c < P.n_classes; c += G)
+            if (!use_mask || ((cmask >> c) & 1u)) {
+                counted_all += (uint32_t)P.trace_class_tot[tr][2u * c];
+                st.checksum += P.trace_class_tot[tr][2u * c + 1u];
+            }
+        for (uint32_t o = 1; o < G; o <<= 1) {
+            st.sum_ttft += (int64_t)wshfl_xor((uint64_t)st.sum_ttft, (int)o);
+            st.sum_e2e += (int64_t)wshfl_xor((uint64_t)st.sum_e2e, (int)o);
+            st.tokens += wshfl_xor(st.tokens, (int)o);
+            st.checksum += wshfl_xor(st.checksum, (int)o);
+            st.max_ttft = max(st.max_ttft, (int64_t)wshfl_xor((uint64_t)st.max_ttft, (int)o));
+            st.max_e2e = max(st.max_e2e, (int64_t)wshfl_xor((uint64_t)st.max_e2e, (int)o));
+            st.makespan = max(st.makespan, (int64_t)wshfl_xor((uint64_t)st.makespan, (int)o));
+            st.served += __shfl_xor_sync(kWFull, st.served, (int)o);
+            st.hit += __shfl_xor_sync(kWFull, st.hit, (int)o);
+            counted_all += __shfl_xor_sync(kWFull, counted_all, (int)o);
+        }
+        if (valid && li == 0u) {
+            if (away) {
+                walk_hand_over(P, cand, false);
+            } else {
+                uint32_t h[8];
+#pragma unroll
+                for (int i = 0; i < 8; i++) h[i] = __ldcg(bins() + i);
+                write_result(P.out + oc, status, counted_all, counted_all - st.served, (uint64_t)counted_all + extra, st, h);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <bool Opt>
+__global__ void __launch_bounds__(32 * kWalkWarps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
+    if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
+    if (P.bucket_count[kPack4] + P.bucket_count[kPack8] == 0) return;
+    const WalkLayout L = pack_layout(P.n_rows, P.n_classes);
+    const uint32_t tid = threadIdx.x, warp = tid >> 5;
+    for (uint32_t i = tid; i < P.n_rows * 64u; i += 32u * kWalkWarps)
+        w1(L.steps + 4u * i) = (uint32_t)P.rows[(i >> 6) * kRowStride + 2 + (i & 63u)];
+    for (uint32_t c = tid; c < P.n_classes; c += 32u * kWalkWarps) {
+        const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u], le = e < 0 ? (int64_t)1 << 62 : e;
+        w4(L.lims + 16u * c) = make_uint4(a < 0 ? 0xFFFFFFFFu : (uint32_t)a, b < 0 ? 0xFFFFFFFFu : (uint32_t)b, lo32(le), hi32(le));
+    }
+    __syncthreads();
+    pack_items<Opt>(P, L, warp * gridDim.x + blockIdx.x, gridDim.x * kWalkWarps);
+}
+
+cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
+    const size_t smem = pack_layout(P.n_rows, P.n_classes).pool + 32u * kWalkWarps * kPackLane;
+    auto kernel = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) ? eval_pack_kernel<true> : eval_pack_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, 32 * kWalkWarps, smem, stream>>>(P);
+    return cudaGetLastError();
+}
+
+}  // namespace maaso

@@ -24,6 +24,9 @@ int occupancy_eval_thread(const EvalParams& P, uint32_t pool_bytes, uint32_t hot
 size_t thread_scratch_per_warp(uint32_t pool_bytes);
 uint32_t thread_fixed_smem(uint32_t n_models, uint32_t n_rows);
 cudaError_t launch_eval_walk(const EvalParams& P, int grid, cudaStream_t stream);
+cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream);
+size_t pack_scratch(int grid);
+bool pack_fits(uint32_t n_rows, uint32_t n_classes);
 cudaError_t launch_eval_walk_big(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_walk_long(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_wide(const EvalParams& P, int grid, cudaStream_t stream);
@@ -610,13 +613,16 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;
     // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,
-    // which several placements of one warp share in the lane-group kernel; with one model all their lanes are at work,
-    // so the line lies lower (10,864 x 5,000, one model, few rejections: 13.7 ms against 19.3 walking; under load 4.1
-    // against 3.2; 6,000 x 8,000 of three models: 16.3 against 11.1).  Queues reject least.
-    const uint64_t walk_most = (o.flags & MAASO_FLAG_INSTANCE_QUEUES) ? 4096u : 6144u * (uint64_t)ctx->n_models;
+    // which several placements of one warp share in the packed kernel; its steps take the same time however few placements
+    // there are, so that the line lies where the walking kernel needs as long (4,000 requests, walking and packed: one model,
+    // 4,000 placements 6.3 and 6.8 ms, 6,000 9.0 and 7.0; three models, where a third of the lanes of a step work, 12,000
+    // placements 8.0 and 13.2, 20,000 about 13 each).  With fixed speeds or queues the alternative is the lane-group kernel,
+    // and the line much the same (queues, one model, 6,000 placements: 9.6 and 8.4 ms).
+    const uint64_t walk_most = ctx->n_models == 1 ? 4096u : 6144u * (uint64_t)ctx->n_models;
     P.walk_all = walk && (uint64_t)C * n_traces <= walk_most ? 1u : 0u;
-    if (walk && (o.flags & MAASO_FLAG_INSTANCE_QUEUES)) P.thread_min_cand = 0xFFFFFFFFu;
-    const bool groups = !P.walk_all && (o.mapping == MAASO_MAP_GROUP || o.mapping == MAASO_MAP_AUTO);
+    const bool packs = walk && !P.walk_all && !P.walk_long && !variant && pack_fits(P.n_rows, P.n_classes);
+    P.pack = packs ? 1u : 0u;
+    const bool groups = !packs && !P.walk_all && (o.mapping == MAASO_MAP_GROUP || o.mapping == MAASO_MAP_AUTO);
     int group_blocks = ctx->group_blocks;
     if (group_blocks == 0) {
         const uint64_t est_warps = ((cands->n_inst * 13 / 10 + 31) / 32 + 6) * n_traces;
@@ -676,6 +682,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         if ((uint64_t)grid_g > max_items_g) grid_g = (int)max_items_g;
         pay_entries = (size_t)grid_g * kGroupThreads * (group_scratch_per_lane() / sizeof(Payload));
     }
+    if (packs) pay_entries = pack_scratch(ctx->sm_count) / sizeof(Payload);
     int grid_b[4];
     for (int b = 6; b <= kGenericBlockBucket; b++) {
         // the block kernels run only when the block mapping is asked for
@@ -764,6 +771,11 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel launch");
     }
+    if (packs) {
+        e = launch_eval_pack(P, ctx->sm_count, stream);
+        launches++;
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "packed kernel launch");
+    }
     if (walk && !P.walk_long) {
         e = launch_eval_walk(P, ctx->sm_count, stream);
         launches++;
@@ -789,7 +801,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     }
-    if (walk && (P.walk_long || may_leave)) {
+    if (walk && (P.walk_long || may_leave || packs)) {
         e = launch_eval_walk_long(P, ctx->sm_count, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");

@@ -83,6 +83,7 @@ __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c
             }
         }
         if (P.mapping == MAASO_MAP_BLOCK) bg = n <= 2 ? 6 : (n <= 4 ? 7 : (n <= 8 ? 8 : kGenericBlockBucket));
+        else if (P.pack) bg = n <= 4 ? kPack4 : (n <= 8 ? kPack8 : -1);  // (what the pack kernel needs room for leaves the walking kernel room for all)
         else if (groups_ok && n <= 32) bg = n <= 1 ? 0 : 32 - __clz((int)(n - 1));
         // More than 32 instances outside the walking and the thread kernel: one warp per placement with the lane-group
         // code.  (One block per placement only when the block mapping is asked for.)
