@@ -198,18 +198,19 @@ MAASO_API int maaso_create(maaso_ctx** out, int cuda_device) {
     ctx->ev_eval = ctx->ev_topk = false;
     for (int i = 0; i < 7; i++) ctx->ev[i] = nullptr;
     DeviceGuard g(cuda_device);
-    cudaDeviceProp prop;
-    e = cudaGetDeviceProperties(&prop, cuda_device);
+    // (single attributes: the whole property record takes 2 ms, most of this call)
+    int major = 0;
+    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cuda_device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, cuda_device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, cuda_device);
     if (e != cudaSuccess || !g.ok) {
         delete ctx;
-        return cuda_fail(nullptr, e, "cudaGetDeviceProperties");
+        return cuda_fail(nullptr, e, "cudaDeviceGetAttribute");
     }
-    if (prop.major < 10) {  // the kernels are built for sm_100a only
+    if (major < 10) {  // the kernels are built for sm_100a only
         delete ctx;
         return MAASO_ESTATE;
     }
-    ctx->sm_count = prop.multiProcessorCount;
-    ctx->smem_per_sm = (int)prop.sharedMemPerMultiprocessor;
     e = cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         delete ctx;
