@@ -400,9 +400,11 @@ def main():
     peak, peak_kind = measured_peak()
     mean_ms = {k: statistics.mean(x[k] for x in kernel_ms) for k in kernel_ms[0]}
     dom = max(("thread_ms", "group_ms", "block_ms"), key=lambda k: mean_ms[k])
-    # block_ms covers the block kernels (block mapping) and the one-warp-per-placement kernel (other mappings)
-    dom_kernel = {"thread_ms": "eval_thread_kernel", "group_ms": "eval_group_kernel",
-                  "block_ms": "eval_block_kernel" if args.mapping == 1 else "eval_wide_kernel"}[dom]
+    # group_ms and block_ms cover the walking kernel (up to 32 instances with the packed kernel, and beyond) unless a mapping
+    # is forced or the largest-gap test (flag 4) is on: then the lane groups, and the block or one-warp-per-placement kernel
+    walks = args.mapping == 0 and not args.flags & 4
+    dom_kernel = {"thread_ms": "eval_thread_kernel", "group_ms": "eval_walk_kernel" if walks else "eval_group_kernel",
+                  "block_ms": "eval_walk_kernel" if walks else ("eval_block_kernel" if args.mapping == 1 else "eval_wide_kernel")}[dom]
     dom_ms = mean_ms[dom]
     # the dominant kernel's launch on rank 0 processes rank 0's shard
     abytes = algorithmic_bytes({"offsets": off_np, "inst": inst_np, "profile": cfg["profile"]}, evals_rank)

@@ -100,8 +100,8 @@ extern "C" {
                                              and the call must return normally */
 
 /* maaso_eval_opts.mapping */
-#define MAASO_MAP_AUTO 0u   /* the library routes the batch: threads for large batches of placements the trace
-                               overloads (default engine), else lane groups; see maaso_eval_placements */
+#define MAASO_MAP_AUTO 0u   /* the library routes the batch: one warp per candidate, or several candidates per warp
+                               for large, lightly loaded batches; see maaso_eval_placements */
 #define MAASO_MAP_BLOCK 1u  /* one thread block per candidate, one warp per instance, lanes = slots */
 #define MAASO_MAP_GROUP 2u  /* one lane per instance, groups of lanes per candidate (<= 32 instances; beyond
                                that one warp per candidate with four instances per lane) */
@@ -223,9 +223,10 @@ MAASO_API void maaso_free_trace(maaso_ctx *ctx, maaso_trace *trace);
  * through the distributor (Sec. IV-F) and per-instance continuous batching with virtual
  * slots (Sec. V-A), and write one record per candidate to out_results (device,
  * [n_cand]).  Work is enqueued on `cuda_stream` (a cudaStream_t, NULL = default stream).
- * opts->mapping chooses the kernel: MAASO_MAP_AUTO (default) lets the library route the batch (large
- * batches of placements that the trace overloads go to the thread kernel, the rest to the lane groups,
- * where a placement of more than 32 instances gets a warp of its own); the records do not depend on it.
+ * opts->mapping chooses the kernel: MAASO_MAP_AUTO (default) lets the library route the batch (a
+ * warp walks the trace for one placement; in large batches that the trace does not overload, placements of at
+ * most 8 instances share a warp, which walks it for four or eight of them at once); the records do not depend
+ * on it.
  * The context's scratch memory grows on demand (this may allocate and synchronise on the
  * first call or when a batch is larger than any before). */
 MAASO_API int maaso_eval_placements(maaso_ctx *ctx, const maaso_trace *trace, const maaso_cand_batch *cands,
@@ -237,10 +238,8 @@ MAASO_API int maaso_eval_placements(maaso_ctx *ctx, const maaso_trace *trace, co
  * out_results (device): n_traces blocks of n_cand records, record c of trace t at
  * out_results[t * n_cand + c]; opts->rejected_by_model and opts->ttft_hist, if given, are laid out
  * the same way ([n_traces * n_cand][...]).  Each record equals what maaso_eval_placements returns
- * for that trace alone; scoring them together lets small candidate sets fill the GPU.  Lane-group
- * and thread mappings only: dump buffers and MAASO_MAP_BLOCK are refused.  A placement of more than 32
- * instances is scored by the thread kernel where the batch goes there, else one warp replays it with the
- * lane-group code (four instances per lane).  No engine and no mapping refuses a placement of
+ * for that trace alone; scoring them together lets small candidate sets fill the GPU.
+ * Dump buffers and MAASO_MAP_BLOCK are refused.  No engine and no mapping refuses a placement of
  * MAASO_MAX_INSTANCES instances or fewer.  Enqueued on cuda_stream. */
 MAASO_API int maaso_eval_placements_multi(maaso_ctx *ctx, const maaso_trace *const *traces, uint32_t n_traces,
                                           const maaso_cand_batch *cands, const maaso_eval_opts *opts,
@@ -375,8 +374,8 @@ MAASO_API int maaso_topk_noalloc(const maaso_result *results, uint64_t n_cand, u
  * run).  Off by default; costs a few event records per call when on. */
 typedef struct {
     float prep_ms;  /* validation, routing + bucket sort (+ dump buffer fill) */
-    float group_ms; /* lane-group scoring kernel */
-    float block_ms; /* block-layout scoring kernels and the one-warp-per-placement kernel for more than 32 instances */
+    float group_ms; /* walking, packed and lane-group scoring kernels (up to 32 instances) */
+    float block_ms; /* scoring kernels for more than 32 instances; block-layout scoring kernels */
     float topk_ms;  /* all passes of the last maaso_topk */
     float thread_ms; /* thread-mapping scoring kernel */
 } maaso_timing;

@@ -5,6 +5,8 @@
 // The trace (and the per-request checksum term of a rejection) is staged once per thread
 // block in shared-memory tiles by 1-D bulk copies (TMA) and shared by every candidate of
 // the block.  No global memory access sits on the per-request path.
+// Used for the largest-gap test, for large lightly loaded batches under the engines that fix a request's speed at admission,
+// for tables beyond the packed kernel's shared memory, and when this mapping is asked for.
 #include "lane_frozen.cuh"
 
 namespace maaso {

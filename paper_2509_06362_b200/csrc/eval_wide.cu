@@ -1,6 +1,5 @@
-// Scoring kernel for placements of 33 to 128 instances under the engines that exist in the
-// lane-group code only (the fixed-speed engine, per-instance queues, the largest-gap test; also the
-// default engine when the lane-group mapping is forced with several traces in one pass): one warp
+// Scoring kernel for placements of 33 to 128 instances with the lane-group code (the largest-gap test, the lane-group
+// mapping when it is forced, tables so large that the walking kernel has no room left beside them): one warp
 // replays one placement, lane l owns instances l, l + 32, l + 64, l + 96.  It reuses the
 // per-instance code of the lane-group kernel (lane_sim.cuh, lane_frozen.cuh) unchanged: every
 // (lane, stride) pair is a "virtual lane" with its own instance state, slot keys (in global
@@ -10,8 +9,7 @@
 //
 // This is the slow, plain member of the family: it reads the prepared trace records straight from
 // global memory (one look-ahead record in registers) and keeps nothing but the queues and the
-// tables in shared memory.  Placements of this size are rare in the sweeps; the default engine
-// scores them in the thread kernel.
+// tables in shared memory.
 #include "lane_frozen.cuh"
 
 namespace maaso {

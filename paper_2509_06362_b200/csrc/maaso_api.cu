@@ -253,7 +253,9 @@ MAASO_API int maaso_create(maaso_ctx** out, int cuda_device) {
         int v = atoi(tt);
         if (v >= 1 && v <= 32) ctx->thread_theta = (uint32_t)v;
     }
-    ctx->thread_min_cand = 262144;  // loaded sweeps of 300,000 placements: 183 ms on the threads, 194 ms walking; of 100,000: 132 and 122
+    // Batches from this size on may go to the thread kernel; none does by itself any more (loaded sweeps of 300,000 placements
+    // x 40,000: 150 ms on the threads, 148 walking; 10^6 x 20,000: 301 and 279; 10^6 x 30,000 of the scale sweep: 453 and 321).
+    ctx->thread_min_cand = 0xFFFFFFFFu;
     const char* tm = getenv("MAASO_THREAD_MIN_CAND");
     if (tm) {
         long v = atol(tm);
