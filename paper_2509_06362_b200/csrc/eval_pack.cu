@@ -50,8 +50,8 @@ static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumpi
             const uint32_t S = rec.w & 0xFFFFu, cls = (rec.w >> 16) & 0xFFu;
             const uint4 lim = w4(lims + cls * 16u);
             const int64_t ttft = first - arrival, e2e = fin - arrival;
-            const bool hit = e2e <= i64_of(lim.z, lim.w) && (lim.x == 0xFFFFFFFFu || ttft <= (int64_t)lim.x) &&
-                             (lim.y == 0xFFFFFFFFu || (uint64_t)(fin - first) <= (uint64_t)(S - 1u) * lim.y);
+            const bool hit = (e2e <= i64_of(lim.z, lim.w)) & ((lim.x == 0xFFFFFFFFu) | (ttft <= (int64_t)lim.x)) &
+                             ((lim.y == 0xFFFFFFFFu) | ((uint64_t)(fin - first) <= (uint64_t)(S - 1u) * lim.y));
             // the request's term as a served one in, its term as a rejected one out
             sum += served_hash(rb.x, fin, first, rb.y) - rejected_hash(rb.x);
             st += ttft;
@@ -156,7 +156,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
             in.rsw = walk_rcp(sw);
             const uint64_t tc = (uint64_t)left * sw + (uint32_t)in.t;
             in.tb = busy ? (int32_t)((uint32_t)tc - sw) : kFar;
-            bad = bad || (busy && tc > (uint64_t)kWalkHorizon);
+            bad = bad | (busy & (tc > (uint64_t)kWalkHorizon));
         };
         // Completions of the lanes in `due` before `upto`, one per lane and iteration.
         auto events = [&](bool due, int32_t upto) {
@@ -184,7 +184,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                     const uint32_t left = (in.kmin >> 6) - in.K;
                     const bool busy = in.w > 0;
                     next_end(left, busy, sw);
-                    due = busy && (left == 0u || in.tb < upto) && !bad;
+                    due = busy & ((left == 0u) | (in.tb < upto)) & !bad;
                     const uint32_t e = ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below));
                     const int64_t fin = epoch + in.t;
                     w2(L.ring_b + ((e - L.ring) >> 1)) = make_uint2(ft.z, li);

@@ -19,12 +19,13 @@
 // Nothing is counted per rejected request: the request count and the checksum of "all of them rejected"
 // are per-class totals of the trace, and a served request takes its own term out again.
 //
-// Measured (B200; lane-group, thread or one-warp kernel before): 143 placements x 500 requests 0.23 ms (0.44),
-// 10,864 x 10,000 7.4 ms (12.2), 2,000 x 17,000 of the paper's shape 10.6 ms (33.8), with queues 10.9 ms (27.0),
-// 100,000 x 100,000 under load 116 ms (132), 64 x 20,000 7.8 ms (18.9), 2,000 placements of 33 to 128 instances x
-// 10,000 10.9 ms (15.4).  A round with one completion takes 300 warp instructions and, alone on its scheduler,
-// 1,280 cycles, almost all of them dependent: what the next step needs is therefore read from shared memory ahead of
-// the choice, and the uncommon outcomes share one branch (1,470 cycles before).
+// Measured (B200; lane-group, thread or one-warp kernel before): 143 placements x 500 requests 0.20 ms (0.44),
+// 10,864 x 10,000 6.7 ms (12.2), 2,000 x 17,000 of the paper's shape 9.6 ms (33.8), with queues 10.5 ms (27.0),
+// 100,000 x 100,000 under load 100 ms (132), 64 x 20,000 7.0 ms (18.9), 2,000 placements of 33 to 128 instances x
+// 10,000 10.1 ms (15.4).  A round with one completion takes 300 warp instructions and, alone on its scheduler,
+// 1,130 cycles, almost all of them dependent: what the next step needs is therefore read from shared memory ahead of
+// the choice, the uncommon outcomes share one branch, and tests of several conditions are written without branches
+// (& and | for && and ||: 652 -> 576 ns a round, 100,000 x 100,000 under load 115 -> 100 ms).
 //
 // The block's pool of shared memory is split evenly among its warps.  Placements beyond one warp's part run
 // first, with half, a quarter, ... of the warps at work and twice, four times, ... the room for each (kWalkModes);
@@ -103,13 +104,13 @@ static __device__ __noinline__ void walk_account(const EvalParams& P, bool dumpi
         const uint32_t S = rec.w & 0xFFFFu, cls = (rec.w >> 16) & 0xFFu;
         const uint4 lim = w4(lims + cls * 16u);
         const int64_t ttft = first - arrival, e2e = fin - arrival;
-        bool hit = e2e <= i64_of(lim.z, lim.w);
+        bool hit = e2e <= i64_of(lim.z, lim.w);  // (no branches)
         if (Wide) {
             const int64_t l_ttft = wi(wide + cls * 16u), l_tbt = wi(wide + cls * 16u + 8u);
-            hit = hit && ttft <= l_ttft && (l_tbt < 0 || fin - first <= (int64_t)(S - 1u) * l_tbt);
+            hit = hit & (ttft <= l_ttft) & ((l_tbt < 0) | (fin - first <= (int64_t)(S - 1u) * l_tbt));
         } else {
-            hit = hit && (lim.x == 0xFFFFFFFFu || ttft <= (int64_t)lim.x) &&
-                  (lim.y == 0xFFFFFFFFu || (uint64_t)(fin - first) <= (uint64_t)(S - 1u) * lim.y);
+            hit = hit & ((lim.x == 0xFFFFFFFFu) | (ttft <= (int64_t)lim.x)) &
+                  ((lim.y == 0xFFFFFFFFu) | ((uint64_t)(fin - first) <= (uint64_t)(S - 1u) * lim.y));
         }
         // the request's term as a served one in, its term as a rejected one out
         const uint64_t sum = i64_of(u2.z, u2.w) + served_hash(rb.x, fin, first, rb.y) - rejected_hash(rb.x);
@@ -120,7 +121,7 @@ static __device__ __noinline__ void walk_account(const EvalParams& P, bool dumpi
         w4(sums + 512u) = make_uint4(lo32(se), hi32(se), lo32(me), hi32(me));
         w4(sums + 1024u) = make_uint4(lo32(mk), hi32(mk), (uint32_t)sum, (uint32_t)(sum >> 32));
         w4(sums + 1536u) = make_uint4(lo32(tk), hi32(tk), u3.z + 1u, u3.w + (hit ? 1u : 0u));
-        if (hit) atomicAdd(&w1(base + kSByClass + 4u * (cls < 7u ? cls : 7u)), 1u);
+        if (hit) atomicAdd(&w1(base + kSByClass + 4u * min(cls, 7u)), 1u);
         if (dumping) {
             const Dump d = dump_for(P, oc);
             if (d.finish) d.finish[rb.x] = fin;
@@ -204,9 +205,9 @@ struct Walk {
             }
         }
         __device__ __forceinline__ bool met(U since, uint32_t Sm1, uint32_t step) const {
-            const bool end = (int64_t)((uint64_t)Sm1 * step + since) <= i64_of(a.z, a.w);
+            const bool end = (int64_t)((uint64_t)Sm1 * step + since) <= i64_of(a.z, a.w);  // (no branches)
             if constexpr (Wide) return (int64_t)since <= ttft && (Sm1 == 0u || tbt < 0 || (int64_t)step <= tbt) && end;
-            else return since <= a.x && (Sm1 == 0u || step <= a.y) && end;
+            else return (since <= a.x) & ((Sm1 == 0u) | (step <= a.y)) & end;
         }
     };
     static __device__ __forceinline__ T prefill(uint32_t base, uint32_t q16, uint32_t in_tok) {
@@ -377,7 +378,7 @@ struct Walk {
                 } else {
                     const uint64_t tc = (uint64_t)left * sw + (uint32_t)in.t;
                     in.tb = busy ? (int32_t)((uint32_t)tc - sw) : kFar;
-                    bad = bad || (busy && tc > (uint64_t)kWalkHorizon);
+                    bad = bad | (busy & (tc > (uint64_t)kWalkHorizon));
                 }
             };
             // Completions (fixed speeds: slots that free) of the lanes in `due`, one per lane and iteration, until every
@@ -428,7 +429,7 @@ struct Walk {
                             const uint32_t left = (in.kmin >> 6) - in.K;
                             const bool busy = in.w > 0;
                             next_end(left, busy, sw);
-                            due = busy && (left == 0u || in.tb < upto) && !bad;
+                            due = busy & ((left == 0u) | (in.tb < upto)) & !bad;
                         }
                         ring_n += adds;
                     }
@@ -550,15 +551,13 @@ struct Walk {
                     const uint32_t Sm1 = (c_meta & 0xFFFFu) - 1u, model = c_meta >> 24;
                     const T at = max(now, rel);
                     bool live = lane >= from && counted() && ((hasmodel >> model) & 1u);
-                    uint4 me = make_uint4(0u, 0u, 0u, 0u);
+                    // (without a branch: every lane has a request, behind the last one the last one once more)
+                    const uint4 me = w4(models + 16u * model);
                     Limits lim;
-                    if (live) {
-                        me = w4(models + 16u * model);
-                        lim.load(L, (c_meta >> 12) & 0xFF0u);
-                        U since = (U)(at - rel) + me.x;  // earliest first token, since the arrival
-                        if (Big && rel != kFar) since = max((T)since, (T)wi(lbs + 8u * model) - rel);
-                        live = lim.met(since, Sm1, me.y);
-                    }
+                    lim.load(L, (c_meta >> 12) & 0xFF0u);
+                    U since = (U)(at - rel) + me.x;  // earliest first token, since the arrival
+                    if (Big && rel != kFar) since = max((T)since, (T)wi(lbs + 8u * model) - rel);
+                    live = live & lim.met(since, Sm1, me.y);
                     const uint32_t first = __ballot_sync(kWFull, live);
                     if ((Wide && Big) || first == 0u) return first;
                     // each instance of the model by itself: its start time at the latest look at it, its prefill of this
@@ -568,13 +567,12 @@ struct Walk {
                     const uint32_t j_end = live ? me.w : 0u;
                     if (Big) ok = ok || j_end - j > 8u * 16u;
                     while (__any_sync(kWFull, j < j_end && !ok)) {
-                        if (j < j_end && !ok) {
-                            const uint4 e = w4(j);
-                            const T t = Wide ? wt<T>(rest + ((j - ents) >> 1)) : (T)(int32_t)e.x;
-                            const U since = (U)(max(at, t) - rel) + (U)prefill(e.y, e.z, c_in);
-                            ok = lim.met(since, Sm1, e.w);
-                            j += 16u;
-                        }
+                        const uint32_t jj = j < j_end ? j : ents;  // (no branch)
+                        const uint4 e = w4(jj);
+                        const T t = Wide ? wt<T>(rest + ((jj - ents) >> 1)) : (T)(int32_t)e.x;
+                        const U since = (U)(max(at, t) - rel) + (U)prefill(e.y, e.z, c_in);
+                        ok = ok | ((j < j_end) & lim.met(since, Sm1, e.w));
+                        j += 16u;
                     }
                     return __ballot_sync(kWFull, live && ok);
                 };
