@@ -12,8 +12,8 @@
 // request's first token and index (16 bytes per slot) and the sums, which a step does not wait for, are in global memory:
 // what is left in shared memory is the same for every placement, so that 16 warps always fit.
 //
-// Measured (B200; 64-bit lane groups before): 9,000 placements of one node x 5,000 requests at 2 a second 9.4 ms (13.3),
-// at 8 a second 5.2 (5.9), 10,864 x 10,000 x 16 arrival rates 137 ms (214).  Groups of 2 lanes for placements of one and
+// Measured (B200; 64-bit lane groups before): 9,000 placements of one node x 5,000 requests at 2 a second 8.0 ms (13.3),
+// at 8 a second 5.2 (5.9), 10,864 x 10,000 x 16 arrival rates 131 ms (214).  Groups of 2 lanes for placements of one and
 // two instances were slower (12.3 and 142 ms): 16 placements step through more completions one after the other than 8 do.
 #include "walk_kernel.cuh"
 
@@ -235,22 +235,22 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 const int32_t pre = W::prefill(in.pre_base, in.pre_q16, in_tok);
                 bool act = counted;  // this group still has to place the request
                 for (uint32_t tries = 1;; tries++) {
-                    const bool elig = act && ((in.tag >> model) & 1u);
-                    events(elig && in.tb < now, now);
+                    const bool elig = act & (((in.tag >> model) & 1u) != 0u);
+                    events(elig & (in.tb < now), now);
                     const bool full = in.w == in.B;
-                    catch_up(elig && !full, now);
+                    catch_up(elig & !full, now);
                     uint32_t top = walk_smem[area + 32u + in.w], more = w1(in.row + 4u * in.w);
                     // distributor prediction (Sec. IV-F steps 2-3)
                     const int32_t t = full ? in.tb + (int32_t)in.sw : in.t;
-                    const bool ok = elig && lim.met((uint32_t)(t + pre - arrival), Sm1, Opt && !full ? more : in.stepB);
+                    const bool ok = elig & lim.met((uint32_t)(t + pre - arrival), Sm1, Opt && !full ? more : in.stepB);
                     // smallest (tier, predicted first token), lowest instance among equals
                     const uint32_t key = ok ? (full ? kTier1 : 0u) | (uint32_t)(t + pre) : kNone;
                     uint32_t best = min(key, __shfl_xor_sync(kWFull, key, 1));
                     best = min(best, __shfl_xor_sync(kWFull, best, 2));
                     if (G > 4u) best = min(best, __shfl_xor_sync(kWFull, best, 4));
                     const int wl = __ffs((int)(__ballot_sync(kWFull, key == best) & gmask)) - 1;
-                    bool win = (int)lane == wl && best < kTier1;
-                    const bool slow = act && best >= kTier1;
+                    bool win = ((int)lane == wl) & (best < kTier1);
+                    const bool slow = act & (best >= kTier1);
                     bool again = false;
                     if (__any_sync(kWFull, slow)) {
                         const bool waits = slow && best != kNone;
@@ -363,29 +363,37 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     }
 }
 
-template <bool Opt>
-__global__ void __launch_bounds__(32 * kWalkWarps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
+// `Warps`: 16, or 12 with 168 registers each (launch_eval_pack).
+template <bool Opt, int Warps>
+__global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
     if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
     if (P.bucket_count[kPack4] + P.bucket_count[kPack8] == 0) return;
     const WalkLayout L = pack_layout(P.n_rows, P.n_classes);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
-    for (uint32_t i = tid; i < P.n_rows * 64u; i += 32u * kWalkWarps)
+    for (uint32_t i = tid; i < P.n_rows * 64u; i += 32u * Warps)
         w1(L.steps + 4u * i) = (uint32_t)P.rows[(i >> 6) * kRowStride + 2 + (i & 63u)];
-    for (uint32_t c = tid; c < P.n_classes; c += 32u * kWalkWarps) {
+    for (uint32_t c = tid; c < P.n_classes; c += 32u * Warps) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u], le = e < 0 ? (int64_t)1 << 62 : e;
         w4(L.lims + 16u * c) = make_uint4(a < 0 ? 0xFFFFFFFFu : (uint32_t)a, b < 0 ? 0xFFFFFFFFu : (uint32_t)b, lo32(le), hi32(le));
     }
     __syncthreads();
-    pack_items<Opt>(P, L, warp * gridDim.x + blockIdx.x, gridDim.x * kWalkWarps);
+    pack_items<Opt>(P, L, warp * gridDim.x + blockIdx.x, gridDim.x * Warps);
 }
 
-cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
-    const size_t smem = pack_layout(P.n_rows, P.n_classes).pool + 32u * kWalkWarps * kPackLane;
-    auto kernel = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) ? eval_pack_kernel<true> : eval_pack_kernel<false>;
+template <int Warps>
+static cudaError_t launch_pack(const EvalParams& P, int grid, cudaStream_t stream) {
+    const size_t smem = pack_layout(P.n_rows, P.n_classes).pool + 32u * Warps * kPackLane;
+    auto kernel = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) ? eval_pack_kernel<true, Warps> : eval_pack_kernel<false, Warps>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, 32 * kWalkWarps, smem, stream>>>(P);
+    kernel<<<grid, 32 * Warps, smem, stream>>>(P);
     return cudaGetLastError();
+}
+// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which spill
+// nothing there: 9,000 x 5,000 8.0 ms against 8.6; the load sweep of many waves 145 against 131.
+cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
+    const uint64_t placements = (uint64_t)P.n_cand * (P.n_traces > 1 ? P.n_traces : 1u);
+    return placements <= 6ull * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kWalkWarps>(P, grid, stream);
 }
 
 }  // namespace maaso
