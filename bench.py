@@ -30,11 +30,11 @@ TOPK = 64
 # ncu counters of the dominant kernel on the default workload (see profiles/).  They describe the
 # kernels whose source hashes to `csrc_sha256`; with any other source they are not printed.
 PROFILED = {
-    "workload": "multimodel", "mapping": 0, "kernel": "eval_thread_kernel",
-    # profiles/eval_thread_kernel_multimodel_sweep_counters.md: one launch of the default workload
-    "warp_inst_per_launch": 46573414946,                 # smsp__inst_executed.sum
-    "dram_bytes_per_launch": 8540173312 + 6593907712,    # dram__bytes_read.sum + dram__bytes_write.sum
-    "csrc_sha256": "38d6462581e8b3e93e08ae6faacbcde5536639edd825c4f14a4a1d54dd9372cb",
+    "workload": "multimodel", "mapping": 0, "kernel": "eval_walk_kernel",
+    # profiles/eval_thread_kernel_multimodel_sweep_counters.md, first table: one launch of the default workload
+    "warp_inst_per_launch": 75909936388,                 # smsp__inst_executed.sum
+    "dram_bytes_per_launch": 4910080 + 0,                # dram__bytes_read.sum + dram__bytes_write.sum
+    "csrc_sha256": "f764ac3c3b3880a428e3dff087399b6894c16baa65e31dd3d55dfcfb8b6e89ca",
 }
 SM_COUNT, ISSUE_PER_SM = 148, 4   # B200: 148 SMs x 4 warp schedulers, one warp instruction per cycle each
 
