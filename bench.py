@@ -34,7 +34,7 @@ PROFILED = {
     # profiles/eval_thread_kernel_multimodel_sweep_counters.md, first table: one launch of the default workload
     "warp_inst_per_launch": 75909936388,                 # smsp__inst_executed.sum
     "dram_bytes_per_launch": 4910080 + 0,                # dram__bytes_read.sum + dram__bytes_write.sum
-    "csrc_sha256": "f764ac3c3b3880a428e3dff087399b6894c16baa65e31dd3d55dfcfb8b6e89ca",
+    "csrc_sha256": "ddecd5ed7be2da69a0029d7d9c8a41085c9aaccfe83baf9549894b3df75eee42",
 }
 SM_COUNT, ISSUE_PER_SM = 148, 4   # B200: 148 SMs x 4 warp schedulers, one warp instruction per cycle each
 

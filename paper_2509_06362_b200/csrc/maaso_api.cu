@@ -1091,7 +1091,7 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
         uint8_t seq[kAhead];
         int index;  // in the batch
     };
-    // A point the chain may reach in this round, with a guess how likely.
+    // A point the chain may reach with this batch, with a guess how likely.
     struct State {
         uint32_t len;
         uint8_t seq[kAhead];
