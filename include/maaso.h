@@ -275,8 +275,8 @@ typedef struct {
     double alpha, beta, gamma_t, gamma_l;
 } maaso_score_params;
 
-/* Latency percentiles from the histograms maaso_eval_placements filled (opts.ttft_hist): for
- * every candidate c and every requested rank permille[j] (1..1000, host array, n_p <= 16),
+/* Latency percentiles from the histograms maaso_eval_placements filled (opts.ttft_hist, which may start at
+ * any 4-byte boundary): for every candidate c and every requested rank permille[j] (1..1000, host array, n_p <= 16),
  * out[c * n_p + j] (device, int64) = the upper edge in microseconds of the first bin at which the
  * cumulative count reaches ceil(permille[j] * served / 1000), i.e. an upper bound of that
  * percentile that is tight to a factor 1.5; INT64_MAX if it falls in the open last bin, -1 if

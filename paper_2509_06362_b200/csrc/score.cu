@@ -56,7 +56,8 @@ struct PermilleList {
 // Eight lanes per candidate: lane l holds bins 8l .. 8l+7 (two 16-byte loads; a warp reads four histograms), a scan
 // over the lanes gives the cumulative counts, lane j works out the target of rank j and keeps the bin it falls
 // into.  Bound by the read of the histograms; with 16 lanes and every lane working out every target it was bound
-// by instructions (10^6 histograms: 74 us, 218 that way, 496 with one thread per candidate).
+// by instructions (10^6 histograms: 74 us, 218 that way, 496 with one thread per candidate).  Histograms are words, so
+// they may start at any word: beside a 16-byte boundary they are read word by word (`Words`).
 template <class U>
 __device__ __forceinline__ void percentiles_of(const U (&c)[8], U incl, uint32_t l, const PermilleList& pm, uint32_t n_p, int64_t* o, bool write) {
     const U below = incl - c[7], total = __shfl_sync(0xFFFFFFFFu, incl, 7, 8);
@@ -78,14 +79,20 @@ __device__ __forceinline__ void percentiles_of(const U (&c)[8], U incl, uint32_t
     }
 }
 
+template <bool Words>
 __global__ void __launch_bounds__(256) ttft_percentile_kernel(const uint32_t* hist, uint64_t n, const __grid_constant__ PermilleList pm, uint32_t n_p, int64_t* out) {
     const uint64_t c = ((uint64_t)blockIdx.x * 256u + threadIdx.x) >> 3;
     const uint32_t l = threadIdx.x & 7u;
     uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
     if (c < n) {
-        const uint4* h = reinterpret_cast<const uint4*>(hist + c * MAASO_TTFT_BINS) + 2u * l;
-        a = __ldg(h);
-        b = __ldg(h + 1);
+        const uint32_t* h = hist + c * MAASO_TTFT_BINS + 8u * l;
+        if (Words) {
+            a = make_uint4(__ldg(h), __ldg(h + 1), __ldg(h + 2), __ldg(h + 3));
+            b = make_uint4(__ldg(h + 4), __ldg(h + 5), __ldg(h + 6), __ldg(h + 7));
+        } else {
+            a = __ldg(reinterpret_cast<const uint4*>(h));
+            b = __ldg(reinterpret_cast<const uint4*>(h) + 1);
+        }
     }
     const bool small = (a.x | a.y | a.z | a.w | b.x | b.y | b.z | b.w) < (1u << 25);  // 64 of them stay below 2^31
     int64_t* const o = out + c * n_p;
@@ -118,7 +125,10 @@ cudaError_t launch_ttft_percentiles(const uint32_t* hist, uint64_t n, const uint
                                     int64_t* out, cudaStream_t stream) {
     PermilleList pm;
     for (uint32_t j = 0; j < 16; j++) pm.v[j] = j < n_p ? permille[j] : 0;
-    if (n) ttft_percentile_kernel<<<(unsigned)((n + 31) / 32), 256, 0, stream>>>(hist, n, pm, n_p, out);
+    if (n) {
+        auto kernel = reinterpret_cast<uintptr_t>(hist) % 16u ? ttft_percentile_kernel<true> : ttft_percentile_kernel<false>;
+        kernel<<<(unsigned)((n + 31) / 32), 256, 0, stream>>>(hist, n, pm, n_p, out);
+    }
     return cudaGetLastError();
 }
 

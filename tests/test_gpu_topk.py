@@ -71,3 +71,19 @@ def test_percentiles_of_partial_warps_and_large_counts(ctx, oracle_mod, n, most)
     permille = rng.integers(1, 1001, {3: 1, 5_000: 3}.get(most, 16)).astype(np.uint32)
     got = ctx.ttft_percentiles(torch.from_numpy(hist.view(np.int32)).cuda(), permille).cpu().numpy()
     assert (got == oracle_mod.ttft_percentiles(hist, permille)).all()
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3, 4])
+def test_percentiles_of_histograms_at_any_word(ctx, oracle_mod, offset):
+    """The histograms are an array of words and may start at any of them (a slice of a larger buffer)."""
+    import torch
+    n = 37
+    rng = np.random.default_rng(offset)
+    hist = rng.integers(0, 5_000, (n, 64)).astype(np.uint32)
+    hist[::5] = 0
+    buffer = torch.full((n * 64 + 8,), -1, dtype=torch.int32, device="cuda")
+    view = buffer[offset:offset + n * 64].view(n, 64)
+    view.copy_(torch.from_numpy(hist.view(np.int32)))
+    permille = np.array((1, 500, 900, 990, 1000), dtype=np.uint32)
+    assert view.is_contiguous() and (view.data_ptr() % 16 != 0) == (offset != 4)
+    assert (ctx.ttft_percentiles(view, permille).cpu().numpy() == oracle_mod.ttft_percentiles(hist, permille)).all()
