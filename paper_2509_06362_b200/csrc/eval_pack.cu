@@ -138,7 +138,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         int64_t epoch = 0;
         int32_t now = 0, rel = 0;
         uint32_t c_in = 0, c_meta = 0;
-        bool bad = false;  // a time of this lane has left the horizon
+        bool bad = false;  // a time of this lane has left the horizon: nothing is asked of it any more (see the walking kernel)
 
         auto bins = [&]() { return reinterpret_cast<uint32_t*>(pay - li * kPackScratch + kPackPay + 64u); };
         auto flush = [&]() {
@@ -235,7 +235,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 const int32_t pre = W::prefill(in.pre_base, in.pre_q16, in_tok);
                 bool act = counted;  // this group still has to place the request
                 for (uint32_t tries = 1;; tries++) {
-                    const bool elig = act & (((in.tag >> model) & 1u) != 0u);
+                    const bool elig = act & (((in.tag >> model) & 1u) != 0u) & !bad;
                     events(elig & (in.tb < now), now);
                     const bool full = in.w == in.B;
                     catch_up(elig & !full, now);

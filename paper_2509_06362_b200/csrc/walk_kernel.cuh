@@ -351,7 +351,11 @@ struct Walk {
             uint32_t ring_n = 0, status = 0;
             int64_t epoch = 0;
             T now = 0;
-            bool bad = false;              // a time of this lane has left the horizon
+            // A time of this lane has left the horizon.  Its next completion may have wrapped then, so from the next round on nothing
+            // is asked of the lane, up to the end of the chunk, when the placement is given up: no completion is taken from it (it
+            // might have none running), no clock runs past a completion, and no prediction of it is compared (bit 31 of a key
+            // says "full").  In the round in which it happens the lane has a free slot and a clock that is right.
+            bool bad = false;
             T rel = 0;                     // this lane's request of the chunk: arrival,
             uint32_t c_in = 0, c_meta = 0; // input tokens, output tokens | class | model
 
@@ -598,7 +602,7 @@ struct Walk {
                                     if (mine) get(rest, ents, n_i, s + lane, in);
                                     else in.tag = 0;
                                 }
-                                events(mine && in.w > 0 && is_due(up), up);
+                                events(mine && in.w > 0 && is_due(up) && !bad, up);
                                 if (kFixed) {
                                     if (mine && in.w > 0) {
                                         for (uint32_t i = 0; i < in.w; i++) wt<T>(in.keys + kKeyBytes * i) -= up;
@@ -652,7 +656,7 @@ struct Walk {
                                 if (s + lane < n_i) get(rest, ents, n_i, s + lane, in);
                                 else in.tag = 0;
                             }
-                            elig = (in.tag >> model) & 1u;
+                            elig = (((in.tag >> model) & 1u) != 0u) & !bad;
                             const T p = prefill(in.pre_base, in.pre_q16, in_tok);
                             // "reduce": what completes before the instance's clock reaches `now`
                             events(elig && is_due(now), now);

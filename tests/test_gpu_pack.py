@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import gen
-from test_gpu_walk import _check, _lists
+from test_gpu_walk import _check, _lists, _past_the_horizon
 
 pytestmark = pytest.mark.gpu
 
@@ -17,8 +17,27 @@ def _trace(n, rate, seed, models, far):
     if far:  # pauses beyond the reach of an epoch, and decodes beyond the horizon
         tr["arrival_us"][n // 3:] += 200_000_000
         tr["arrival_us"][n // 2:] += 7_000_000_000
-        tr["out_tokens"][rng.random(n) < 0.02] = 65535
+        tr["out_tokens"][rng.random(n) < 0.2] = 65535
     return tr
+
+
+def _leave(want):
+    """Do some placements leave the 32-bit horizon, and most not?  (Times count from an epoch that is no later than a request's
+    arrival, and less than 2^27 us earlier.)"""
+    e2e = want["max_e2e_us"]
+    return (e2e > 0x60000000).any() and (e2e < 0x60000000 - (1 << 27)).mean() > 0.5
+
+
+def _mostly_not_loaded(prof, lists, traces):
+    """Do the traces together (harmonic mean of their output tokens a second) leave most placements unloaded?  That and the
+    size of the batch decide that it is packed."""
+    rates = []
+    for t in traces:
+        span = (t["arrival_us"][-1] - t["arrival_us"][0]) * 1e-6 if len(t) > 1 else 0.0
+        rates.append(t["out_tokens"].astype(np.int64).sum() / span if span else 1.0)
+    demand = len(traces) / sum(1.0 / r for r in rates)
+    supply = [sum(b * 1_000_000 // int(prof["step_us"][m, s, b - 1]) for m, s, b in lst) for lst in lists if 0 < len(lst) <= 8]
+    return 2 * sum(demand >= 2 * x for x in supply) < len(supply)
 
 
 @pytest.mark.parametrize("flags", [0, 1])
@@ -33,6 +52,18 @@ def test_one_model(oracle_mod, flags, far):
     mask = None if far else rng.integers(0, 8, size=len(lists)).astype(np.uint32)
     want = _check(oracle_mod, m, prof, _trace(150, 3.0, 7, (1.0,), far), classes, off, inst, flags, mask)
     assert (want["attempts"] > want["n_counted"]).any() and (want["n_served"] > 0).mean() > 0.5
+    assert not far or _leave(want)
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+def test_steps_behind_one_that_left_the_horizon(oracle_mod, flags):
+    import paper_2509_06362_b200 as m
+    prof, tr, lists = _past_the_horizon(3, 4300, heavy=0.1)
+    off, inst = gen.candidates_from_lists(lists)
+    assert _mostly_not_loaded(prof, lists, [tr])
+    want = _check(oracle_mod, m, prof, tr, gen.make_classes([(None, None, None)]), off, inst, flags)
+    gone = want["max_e2e_us"] > 0x60000000
+    assert gone.mean() > 0.3 and (~gone).mean() > 0.05
 
 
 @pytest.mark.parametrize("flags", [0, 1])

@@ -1,4 +1,4 @@
-"""The walking kernel (csrc/eval_walk.cu) at its edges: placements of 0 to 128 instances, whose state is at and
+"""The walking kernel (csrc/walk_kernel.cuh) at its edges: placements of 0 to 128 instances, whose state is at and
 beyond one and several warps' parts of the pool, and the 32-bit times: arrivals far beyond the
 epoch, long waits, and placements that leave the horizon and are handed over in mid-trace."""
 import numpy as np
@@ -112,3 +112,36 @@ def test_overloaded_without_limits(oracle_mod):
     mask = np.array([7, 7, 1], dtype=np.uint32)
     want = _check(oracle_mod, m, prof, tr, classes, off, inst, 0, mask)
     assert (want["max_ttft_us"] > 1 << 31).any()
+
+
+def _past_the_horizon(seed, n_lists, n=96, heavy=0.2):
+    """Placements of one model that get beyond the horizon in the middle of a chunk of 32 requests, with more requests behind:
+    decodes of hours, prefills of minutes in a row, one-token requests, nothing has a limit."""
+    rng = np.random.default_rng(seed)
+    W = gen.WMAX
+    step = np.empty((1, 6, W), dtype=np.int32)
+    step[0, :4] = np.array([[1], [40], [33_500], [(1 << 24) - 1]])
+    step[0, 4:] = rng.choice([1, 7, 1000, 33_500, 1 << 20, (1 << 24) - 1], size=(2, W))
+    prof = {"n_models": 1, "n_strategies": 6, "wmax": W, "devices": np.ones(6, dtype=np.int32),
+            "min_devices": np.ones(1, dtype=np.int32), "prefill_base_us": np.array([[0, 1, 2000, 0, 0, 5]], dtype=np.int32),
+            "prefill_q16": np.full((1, 6), 65536, dtype=np.int32), "step_us": step}
+    tr = np.zeros(n, dtype=gen.REQUEST_DTYPE)
+    gaps = rng.choice([0, 1000, 10 ** 6, 10 ** 7], size=n)
+    gaps[n - 1] = 2 * 10 ** 11  # and a long pause, so that little is asked of a placement on average
+    tr["arrival_us"] = np.cumsum(gaps)
+    tr["in_tokens"] = rng.choice([0, 1, 1000, 1 << 24, (1 << 28) - 4096], size=n, p=[0.2, 0.2, 0.4 - heavy, 0.2, heavy])
+    tr["out_tokens"] = rng.choice([1, 2, 301, 65535], size=n, p=[0.4, 0.2, 0.4 - heavy, heavy])
+    lists = [[(0, int(rng.choice(6, p=[0.3, 0.2, 0.2, 0.1, 0.1, 0.1])), int(rng.choice([1, 1, 2, 3, 8, 9, 64])))
+              for _ in range(int(rng.choice([1, 1, 2, 3, 5, 8])))] for _ in range(n_lists)]
+    lists[:2] = [[(0, 2, 1)], [(0, 0, 2)] * 40]
+    return prof, tr, lists
+
+
+@pytest.mark.parametrize("flags", [0, 1, 2, 3])
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_rounds_behind_one_that_left_the_horizon(oracle_mod, seed, flags):
+    import paper_2509_06362_b200 as m
+    prof, tr, lists = _past_the_horizon(seed, 300)
+    off, inst = gen.candidates_from_lists(lists)
+    want = _check(oracle_mod, m, prof, tr, gen.make_classes([(None, None, None)]), off, inst, flags)
+    assert (want["max_e2e_us"] > 0x60000000).mean() > 0.3
