@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import gen
+from gpu_common import assert_records_equal
 from test_gpu_walk import _check, _lists, _past_the_horizon
 
 pytestmark = pytest.mark.gpu
@@ -74,3 +75,44 @@ def test_three_models(oracle_mod, flags):
     classes = gen.make_classes([(500_000, 50_000, None), (2_000_000, 150_000, None), (None, None, 180_000_000)])
     off, inst = gen.candidates_from_lists(lists)
     _check(oracle_mod, m, prof, _trace(60, 2.0, 8, (0.6, 0.3, 0.1), False), classes, off, inst, flags)
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+@pytest.mark.parametrize("far", [False, True])
+@pytest.mark.parametrize("copies", [1, 3])  # 4,464 items: 12 warps per SM hold them at once; 13,392: 16 take several each
+def test_several_traces(oracle_mod, copies, far, flags):
+    """Every item of the packed kernel exists once per trace: records, unserved requests and histograms go to the trace's own
+    block, traces of other lengths (an empty one among them) end at other times, and a placement that leaves the horizon under
+    one trace is replayed under all of them."""
+    import torch
+    import paper_2509_06362_b200 as m
+    prof, rng = gen.profile_node(1), np.random.default_rng(15)
+    lists = _lists(prof, rng, (1, 2, 3, 4, 5, 8), (2, 16, 32, 64), 183) + _lists(prof, rng, (1, 3, 7, 9, 17, 33), (1, 2), 3)
+    classes = gen.make_classes([(None, None, None)] * 3 if far else [(500_000, 50_000, None), (2_000_000, 150_000, None), (None, None, 180_000_000)])
+    off, inst = gen.candidates_from_lists(lists)
+    traces = [_trace(150, 3.0, 7, (1.0,), False), _trace(97, 2.0, 8, (1.0,), far), _trace(1, 2.0, 9, (1.0,), False)[:0],
+              _trace(131, 1.0, 10, (1.0,), False)] * copies
+    mask = None if far else rng.integers(0, 8, size=len(lists)).astype(np.uint32)
+    n, n_tr = len(lists), len(traces)
+    assert n * n_tr > 4096 and _mostly_not_loaded(prof, lists, traces)
+    c = m.Context(0)
+    c.load_profile(prof)
+    handles = [c.load_trace(t, classes) for t in traces]
+    rej = torch.full((n_tr * n, 16), 77, dtype=torch.int32, device="cuda")
+    hist = torch.full((n_tr * n, 64), 77, dtype=torch.int32, device="cuda")
+    out = c.eval_placements_multi(handles, c.to_device(off), c.to_device(inst), 10 ** 6, None if mask is None else c.to_device(mask),
+                                  flags, rejected_by_model=rej, ttft_hist=hist)
+    torch.cuda.synchronize()
+    got = c.results_to_numpy(out).reshape(n_tr, n)
+    rej, hist = (x.cpu().numpy().view(np.uint32).reshape(n_tr, n, -1) for x in (rej, hist))
+    c.close()
+    wanted = []
+    for k, t in enumerate(traces[:4]):
+        want = oracle_mod.eval_placements(prof, t, classes, off, inst, 10 ** 6, mask, flags)
+        want_rej = oracle_mod.rejected_by_model(prof, t, classes, off, inst, 10 ** 6, mask, flags)
+        want_hist = oracle_mod.ttft_hist(prof, t, classes, off, inst, 10 ** 6, mask, flags)
+        for j in range(k, n_tr, 4):
+            assert_records_equal(got[j], want, f"trace {j}, flags {flags}")
+            assert (rej[j] == want_rej).all() and (hist[j] == want_hist).all(), j
+        wanted.append(want)
+    assert [_leave(w) for w in wanted] == [False, far, False, False]
