@@ -214,7 +214,9 @@ MAASO_API int maaso_load_profile(maaso_ctx *ctx, const maaso_profile_desc *desc)
  * or a device pointer, `classes` is a host pointer.  Checks: n >= 0, n < 2^32, arrivals
  * non-negative and non-decreasing, out_tokens >= 1, cls < n_classes, model < n_models of
  * the loaded profile (MAASO_ESTATE if none).  Synchronous.  *out must be released with
- * maaso_free_trace (or by maaso_destroy). */
+ * maaso_free_trace (or by maaso_destroy).  The context keeps the memory of the trace freed last (at most
+ * 256 MB) for the next one to load; it gives it back when it is out of device memory otherwise, and in
+ * maaso_destroy. */
 MAASO_API int maaso_load_trace(maaso_ctx *ctx, const maaso_request *reqs, uint64_t n,
                      const maaso_slo_class *classes, uint32_t n_classes, maaso_trace **out);
 MAASO_API void maaso_free_trace(maaso_ctx *ctx, maaso_trace *trace);
@@ -387,7 +389,8 @@ MAASO_API uint64_t maaso_launch_count(const maaso_ctx *ctx);
 
 /* Test hook for the out-of-memory paths (no counterpart in the paper): the next `count` times the
  * context would grow one of its scratch buffers, the growth is refused as if the device had no
- * memory left.  The call that needed it returns MAASO_ENOMEM and enqueues nothing; the context
+ * memory left.  If the context holds the memory of a freed trace, that is given back and the growth
+ * tried again.  Otherwise the call that needed it returns MAASO_ENOMEM and enqueues nothing; the context
  * keeps the buffers it had, stays usable, and the next call allocates normally.  count = 0
  * switches the hook off. */
 MAASO_API int maaso_test_fail_allocs(maaso_ctx *ctx, int count);

@@ -138,11 +138,20 @@ int fail(maaso_ctx* ctx, int code, const char* what) {
     return code;
 }
 
+// Gives back the memory of a freed trace, if the context holds some.
+bool drop_spare(maaso_ctx* ctx) {
+    if (!ctx->spare) return false;
+    cudaFree(ctx->spare);
+    ctx->spare = nullptr;
+    ctx->spare_bytes = 0;
+    return true;
+}
+
 int grow(maaso_ctx* ctx, void** buf, size_t* have, size_t need) {
     if (need <= *have) return MAASO_OK;
-    if (ctx && ctx->fail_allocs > 0) {  // test hook: behave as if the allocation had been refused
+    while (ctx->fail_allocs > 0) {  // test hook: behave as if the allocation had been refused
         ctx->fail_allocs--;
-        return fail(ctx, MAASO_ENOMEM, "scratch allocation refused (test hook)");
+        if (!drop_spare(ctx)) return fail(ctx, MAASO_ENOMEM, "scratch allocation refused (test hook)");
     }
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "synchronize before growing scratch");
@@ -151,6 +160,10 @@ int grow(maaso_ctx* ctx, void** buf, size_t* have, size_t need) {
     *have = 0;
     need = (need + (size_t)(1 << 20) - 1) & ~((size_t)(1 << 20) - 1);
     e = cudaMalloc(buf, need);
+    if (e == cudaErrorMemoryAllocation && drop_spare(ctx)) {
+        cudaGetLastError();
+        e = cudaMalloc(buf, need);
+    }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation");
     *have = need;
     return MAASO_OK;
@@ -283,7 +296,7 @@ MAASO_API void maaso_free_trace(maaso_ctx* ctx, maaso_trace* trace) {
         }
     // a placer loads a trace per request window: its memory is kept for the next one
     if (trace->mem_bytes <= kSpareMax) {
-        if (ctx->spare) cudaFree(ctx->spare);
+        drop_spare(ctx);
         ctx->spare = trace->mem;
         ctx->spare_bytes = trace->mem_bytes;
     } else {
@@ -297,7 +310,7 @@ MAASO_API void maaso_destroy(maaso_ctx* ctx) {
     DeviceGuard g(ctx->device);
     cudaDeviceSynchronize();
     while (!ctx->traces.empty()) maaso_free_trace(ctx, ctx->traces.back());
-    if (ctx->spare) cudaFree(ctx->spare);
+    drop_spare(ctx);
     if (ctx->d_rows) cudaFree(ctx->d_rows);
     if (ctx->d_devices) cudaFree(ctx->d_devices);
     if (ctx->d_min_devices) cudaFree(ctx->d_min_devices);
@@ -456,13 +469,12 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         t->mem = ctx->spare;
         t->mem_bytes = ctx->spare_bytes;
         ctx->spare = nullptr;
+        ctx->spare_bytes = 0;
     } else {
         t->mem_bytes = align_up(off, (size_t)1 << 16);
         e = cudaMalloc(&t->mem, t->mem_bytes);
-        if (e == cudaErrorMemoryAllocation && ctx->spare) {
+        if (e == cudaErrorMemoryAllocation && drop_spare(ctx)) {
             cudaGetLastError();
-            cudaFree(ctx->spare);
-            ctx->spare = nullptr;
             e = cudaMalloc(&t->mem, t->mem_bytes);
         }
         if (e != cudaSuccess) {

@@ -1124,3 +1124,33 @@ def test_refused_scratch_allocation_is_reported_and_survived(oracle_mod):
 
     clean = used_by(False)
     assert used_by(True) <= clean
+
+
+def test_memory_of_a_freed_trace_is_given_back_when_there_is_no_other(oracle_mod):
+    """The context keeps the memory of the trace freed last for the next one to load.  A scratch growth that the device
+    refuses (test hook) takes place after that memory has gone back; refused once more, the call fails as it does without."""
+    import torch
+    import paper_2509_06362_b200 as m
+    cfg = gen.make_config("tiny", n_req=300)
+    off, inst = cfg["offsets"][:9], cfg["inst"][:int(cfg["offsets"][8])]
+    want = oracle_mod.eval_placements(cfg["profile"], cfg["traces"][0], cfg["classes"], off, inst, 4)
+    long = gen.make_trace(200_000, 8.0, 3)
+    for refused in (1, 2):
+        c = m.Context(0)
+        c.load_profile(cfg["profile"])
+        t = c.load_trace(cfg["traces"][0], cfg["classes"])
+        c.free_trace(c.load_trace(long, cfg["classes"]))
+        d_off, d_inst = c.to_device(off), c.to_device(inst)
+        out = torch.empty((8, 128), dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        c.test_fail_allocs(refused)
+        if refused == 2:
+            with pytest.raises(m.MaasoError) as err:
+                c.eval_placements(t, d_off, d_inst, 4, out=out)
+            assert err.value.code == -3
+        c.eval_placements(t, d_off, d_inst, 4, out=out)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] > free + 8_000_000   # 16 MB back, a small scratch taken
+        assert c.results_to_numpy(out).tobytes() == want.tobytes()
+        c.close()
