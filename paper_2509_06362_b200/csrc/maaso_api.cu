@@ -169,6 +169,25 @@ int grow(maaso_ctx* ctx, void** buf, size_t* have, size_t need) {
     return MAASO_OK;
 }
 
+// What every call that scores on a trace refuses.
+int check_trace(maaso_ctx* ctx, const maaso_trace* t) {
+    if (t->owner != ctx) return fail(ctx, MAASO_ESTATE, "eval: trace belongs to another context");
+    if (t->n && t->max_model >= ctx->n_models)
+        return fail(ctx, MAASO_ESTATE, "eval: trace refers to a model the current profile lacks");
+    return MAASO_OK;
+}
+
+int check_flags(maaso_ctx* ctx, uint32_t flags) {
+    if (flags & ~(MAASO_FLAG_PRED_OPTIMISTIC | MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_TBT_MAXGAP | MAASO_FLAG_INSTANCE_QUEUES |
+                  MAASO_FLAG_TEST_STALL))
+        return fail(ctx, MAASO_EINVAL, "eval: unknown flag");
+    return MAASO_OK;
+}
+
+bool score_params_ok(const maaso_score_params* p) {
+    return p->gamma_t > 0.0 && p->gamma_l > 0.0 && p->gamma_t <= 1e300 && p->gamma_l <= 1e300;
+}
+
 constexpr size_t kSpareMax = (size_t)256 << 20;
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -518,9 +537,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     for (uint32_t t = 0; t < n_traces; t++) {
         const maaso_trace* x = traces[t];
         if (!x) return MAASO_EINVAL;
-        if (x->owner != ctx) return fail(ctx, MAASO_ESTATE, "eval: trace belongs to another context");
-        if (x->n && x->max_model >= ctx->n_models)
-            return fail(ctx, MAASO_ESTATE, "eval: trace refers to a model the current profile lacks");
+        if (const int rc = check_trace(ctx, x)) return rc;
         if (x->h_classes != trace->h_classes)
             return fail(ctx, MAASO_EINVAL, "eval: traces scored in one call must have the same SLO classes");
         if (x->n > n_max) n_max = x->n;
@@ -538,9 +555,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     if (o.dump_n && !o.dump_cand_idx) return fail(ctx, MAASO_EINVAL, "eval: dump_n without dump_cand_idx");
     if (n_traces > 1 && (o.dump_n || o.mapping == MAASO_MAP_BLOCK))
         return fail(ctx, MAASO_EINVAL, "eval: several traces in one call allow no dump buffers and no block mapping");
-    if (o.flags & ~(MAASO_FLAG_PRED_OPTIMISTIC | MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_TBT_MAXGAP | MAASO_FLAG_INSTANCE_QUEUES |
-                    MAASO_FLAG_TEST_STALL))
-        return fail(ctx, MAASO_EINVAL, "eval: unknown flag");
+    if (const int rc = check_flags(ctx, o.flags)) return rc;
     if ((o.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_TBT_MAXGAP | MAASO_FLAG_INSTANCE_QUEUES)) &&
         o.mapping == MAASO_MAP_BLOCK)
         return fail(ctx, MAASO_EINVAL,
@@ -916,8 +931,7 @@ MAASO_API int maaso_score(maaso_ctx* ctx, const maaso_result* results, uint64_t 
                           const maaso_score_params* params, double* out_scores, void* cuda_stream) {
     if (!ctx || !params) return MAASO_EINVAL;
     if (n_cand == 0) return MAASO_OK;
-    if (!results || !out_scores || !(params->gamma_t > 0.0) || !(params->gamma_l > 0.0) ||
-        params->gamma_t > 1e300 || params->gamma_l > 1e300)
+    if (!results || !out_scores || !score_params_ok(params))
         return fail(ctx, MAASO_EINVAL, "score: null pointer or non-positive threshold");
     DeviceGuard g(ctx->device);
     cudaError_t e = launch_score(results, n_cand, *params, out_scores, (cudaStream_t)cuda_stream);
@@ -990,6 +1004,10 @@ static int ins_deploy_multi(maaso_ctx* ctx, const maaso_trace* trace, const Depl
         any_mask = any_mask || prob[p].use_mask;
     }
     if (n_configs == 0 || n_prob == 0) return MAASO_OK;
+    // (also where there is nothing to deploy on, so that no placement is ever scored)
+    if (const int rc = check_trace(ctx, trace)) return rc;
+    if (const int rc = check_flags(ctx, flags)) return rc;
+    if (!score_params_ok(score)) return fail(ctx, MAASO_EINVAL, "score: null pointer or non-positive threshold");
     DeviceGuard g(ctx->device);
 
     // device staging: offsets | inst | mask | results | scores | rejected-by-model

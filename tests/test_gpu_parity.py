@@ -1154,3 +1154,23 @@ def test_memory_of_a_freed_trace_is_given_back_when_there_is_no_other(oracle_mod
         assert torch.cuda.mem_get_info()[0] > free + 8_000_000   # 16 MB back, a small scratch taken
         assert c.results_to_numpy(out).tobytes() == want.tobytes()
         c.close()
+
+
+@pytest.mark.parametrize("gpus", [0, 4])
+def test_ins_deploy_refuses_what_scoring_refuses(ctx, gpus):
+    """A foreign trace, an unknown flag and a threshold of zero are refused on any number of devices, none among them."""
+    import paper_2509_06362_b200 as m
+    cfg = gen.make_config("tiny", n_req=60)
+    ctx.load_profile(cfg["profile"])
+    t = ctx.load_trace(cfg["traces"][0], cfg["classes"])
+    other = m.Context(0)
+    other.load_profile(cfg["profile"])
+    foreign = other.load_trace(cfg["traces"][0], cfg["classes"])
+    for trace, gamma, flags, code in ((foreign, 1.0, 0, -2), (t, 0.0, 0, -1), (t, 1.0, 1 << 20, -1)):
+        with pytest.raises(m.MaasoError) as err:
+            ctx.ins_deploy(trace, gpus, [(0, 1)], 4.0, 0.3, gamma, 1.0, flags=flags)
+        assert err.value.code == code
+    phi, placements = ctx.ins_deploy(t, gpus, [(0, 1)], 4.0, 0.3, 1.0, 1.0)
+    assert len(phi) == gpus + 1 and phi[0] == 0.0
+    ctx.free_trace(t)
+    other.close()
