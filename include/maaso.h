@@ -72,18 +72,15 @@ extern "C" {
                                       admission to the request's finish time, first token = admission +
                                       prefill, one token every step[running + 1] afterwards; later
                                       admissions slow nobody down and prefills stall nobody.  Same
-                                      distributor.  Lane-group code only: MAASO_MAP_BLOCK and
-                                      MAASO_MAP_THREAD are refused; a placement with more than 32 instances
-                                      (up to MAASO_MAX_INSTANCES) is replayed by one warp, four instances
-                                      per lane; finish times must stay below 2^57 us (else
-                                      MAASO_CAND_ELOOP). */
+                                      distributor.  MAASO_MAP_BLOCK and MAASO_MAP_THREAD are refused;
+                                      finish times must stay below 2^57 us (else MAASO_CAND_ELOOP). */
 
 #define MAASO_FLAG_TBT_MAXGAP 4u /* the TBT term of the hit test (Phi_S indicator) looks at the largest gap
                                     between two consecutive tokens of a request, prefill stalls included,
                                     instead of the mean gap; a request of one token has no gap.  The
                                     distributor's prediction is unchanged.  Same limits as
-                                    MAASO_FLAG_ENGINE_FROZEN (lane-group code; one warp per placement
-                                    beyond 32 instances). */
+                                    MAASO_FLAG_ENGINE_FROZEN; lane-group code (one warp per placement
+                                    beyond 32 instances), whatever the mapping. */
 
 #define MAASO_FLAG_INSTANCE_QUEUES 8u /* a request whose chosen instance is full queues THERE (Sec. II-A: requests
                                         beyond the batch cap wait in the instance's queue) instead of at the

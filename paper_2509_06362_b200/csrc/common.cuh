@@ -44,7 +44,7 @@ constexpr int kScanHdrUnits = 40;    // 16-byte units of a scan tile's header (s
 constexpr int kScanHdrBase = 4;      // unit of the tile's base arrival time
 constexpr int kScanHdrClassBits = 5; // first unit of the 8 per-class bitmaps (2 units = 256 bits each)
 constexpr int kScanHdrModelBits = 21; // first unit of the 8 per-model bitmaps
-constexpr int kMaxTraces = 16;  // traces one call of the lane-group kernel can replay side by side
+constexpr int kMaxTraces = 16;  // traces one call can replay side by side
 
 struct Request {
     int64_t arrival;

@@ -12,8 +12,9 @@
 // request's first token and index (16 bytes per slot) and the sums, which a step does not wait for, are in global memory:
 // what is left in shared memory is the same for every placement, so that 16 warps always fit.
 //
-// Measured (B200; 64-bit lane groups before): 9,000 placements of one node x 5,000 requests at 2 a second 8.0 ms (13.3),
-// at 8 a second 5.2 (5.9), 10,864 x 10,000 x 16 arrival rates 131 ms (214).  Groups of 2 lanes for placements of one and
+// Measured (B200; 64-bit lane groups before, walking kernel in place of this one): 9,000 placements of one node x 5,000
+// requests at 2 a second 8.0 ms (13.3, 14.2), 10,864 x 10,000 x 16 arrival rates, optimistic estimate, 132 ms (214, 307); at 8 a
+// second half of the 9,000 are loaded and they walk (5.3 ms).  Groups of 2 lanes for placements of one and
 // two instances were slower (12.3 and 142 ms): 16 placements step through more completions one after the other than 8 do.
 #include "walk_kernel.cuh"
 
@@ -363,7 +364,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     }
 }
 
-// `Warps`: 16, or 12 with 168 registers each (launch_eval_pack).
+// `Warps`: 16 with 128 registers each, or 12 with room for 168 (launch_eval_pack).
 template <bool Opt, int Warps>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
     if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
@@ -389,8 +390,12 @@ static cudaError_t launch_pack(const EvalParams& P, int grid, cudaStream_t strea
     kernel<<<grid, 32 * Warps, smem, stream>>>(P);
     return cudaGetLastError();
 }
-// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which spill
-// nothing there: 9,000 x 5,000 8.0 ms against 8.6; the load sweep of many waves 145 against 131.
+// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which take
+// 150 to 154 registers there and spill nothing (16 warps: 68 to 76 bytes).  Measured, 12 and 16 warps: one node at 2 requests
+// a second, 9,000 x 5,000 8.0 and 9.2 ms; its 10,864 placements x 10,000 under 1, 2, 4 and 16 traces 13.7 and 16.0, 25.2 and
+// 28.8, 46.7 and 48.5, 134 and 127 (optimistic estimate 15.2 and 16.8, 27.4 and 29.7, 49.9 and 49.4, 144 and 131); three
+// models at 1 a second, 20,000 x 4,000 9.9 and 10.0, 40,000 17.7 and 16.4.  So the line is where it must lie for several
+// models and early for one, which 12 warps serve better up to about 40,000 placements.
 cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
     const uint64_t placements = (uint64_t)P.n_cand * (P.n_traces > 1 ? P.n_traces : 1u);
     return placements <= 6ull * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kWalkWarps>(P, grid, stream);

@@ -285,8 +285,9 @@ MAASO_API int maaso_create(maaso_ctx** out, int cuda_device) {
         int v = atoi(tt);
         if (v >= 1 && v <= 32) ctx->thread_theta = (uint32_t)v;
     }
-    // Batches from this size on may go to the thread kernel; none does by itself any more (loaded sweeps of 300,000 placements
-    // x 40,000: 150 ms on the threads, 148 walking; 10^6 x 20,000: 301 and 279; 10^6 x 30,000 of the scale sweep: 453 and 321).
+    // Batches from this size on may go to the thread kernel; none does by itself any more (loaded sweeps of three models,
+    // threads and walking: 300,000 placements x 40,000 150 and 129 ms, 10^6 x 20,000 295 and 241; of the scale sweep, 10^6 x
+    // 30,000 456 and 279).
     ctx->thread_min_cand = 0xFFFFFFFFu;
     const char* tm = getenv("MAASO_THREAD_MIN_CAND");
     if (tm) {
@@ -644,10 +645,20 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;
     // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,
     // which several placements of one warp share in the packed kernel; its steps take the same time however few placements
-    // there are, so that the line lies where the walking kernel needs as long (4,000 requests, walking and packed: one model,
-    // 4,000 placements 6.3 and 6.8 ms, 6,000 9.0 and 7.0; three models, where a third of the lanes of a step work, 12,000
-    // placements 8.0 and 13.2, 20,000 about 13 each).  With fixed speeds or queues the alternative is the lane-group kernel,
-    // and the line much the same (queues, one model, 6,000 placements: 9.6 and 8.4 ms).
+    // there are, so that the line lies where the walking kernel needs as long.  Measured on 4,000 requests, walking and packed:
+    //   one model     at 1 a second 3,000 placements 5.5 and 5.7 ms, 4,096 7.9 and 5.7; at 2 a second 4,096 6.1 and 6.0, 5,000
+    //                 8.0 and 6.1; at 4 a second 6,144 6.1 and 6.4, 8,192 7.9 and 6.6
+    //   two models    at 1 a second 8,192 7.7 and 8.3, 10,240 9.4 and 8.5; at 2 a second 12,288 8.5 and 9.3, 16,384 10.7 and 10.4;
+    //                 at 4 a second 32,768 12.7 and 14.0
+    //   three models  (a third of the lanes of a step at work) at 1 a second 10,240 7.9 and 7.9; at 2 a second 16,384 9.2 and 9.5,
+    //                 24,576 13.0 and 12.9; at 4 a second 32,768 11.5 and 12.9
+    //   16 models     (which the placements serve few of) at 2 a second 16,384 3.3 and 4.5, 98,304 18.2 and 22.3, 163,840 30.1 and
+    //                 35.9: walking is the better one at every size
+    // that is between 3,100 and 6,500 placements for one model and between 9,000 and more than 32,768 for several.  With fixed
+    // speeds or queues the alternative is the lane-group kernel.  Fixed speeds: 4,500 to 9,800, 9,000 to more than 24,576.
+    // Queues cost the walking kernel more, and for several models the line is late there: one model at 2 a second 4,096 7.3 and
+    // 8.1, 5,000 9.6 and 8.3; two models 6,144 7.2 and 7.8, 8,192 9.0 and 7.9; three 8,192 7.4 and 7.7, 10,240 8.9 and 7.7, 16,384
+    // 13.0 and 10.0.
     const uint64_t walk_most = ctx->n_models == 1 ? 4096u : 6144u * (uint64_t)ctx->n_models;
     P.walk_all = walk && (uint64_t)C * n_traces <= walk_most ? 1u : 0u;
     const bool packs = walk && !P.walk_all && !P.walk_long && !variant && pack_fits(P.n_rows, P.n_classes);

@@ -154,8 +154,9 @@ __device__ __forceinline__ uint32_t warp_scan_256(uint32_t (&v)[8]) {
 }
 
 // One block, one warp per bucket, eight cost bins per lane: (0) the batch-wide choice for the candidates that can go
-// either way (MAASO_MAP_AUTO): the walking (or thread) kernel if the batch is small, or if most of them are loaded
-// beyond their decode capacity, else the lane groups; (1) if the resident lane-group grid has warps to spare, promote
+// either way (MAASO_MAP_AUTO): the walking kernel if the batch is small, or if most of them are loaded beyond their decode
+// capacity, else the packed kernel or the lane groups (the thread kernel in the walking kernel's place, and from
+// P.thread_min_cand loaded ones on, only where MAASO_THREAD_MIN_CAND allows it: 0 otherwise); (1) if the resident lane-group grid has warps to spare, promote
 // the most expensive candidates of the narrower lane-group buckets to a warp of their own (bucket 5) so that their
 // event handling is not serialised with other candidates' in the same warp; (2) turn the per-bin histograms into
 // write cursors (bins in decreasing cost order).

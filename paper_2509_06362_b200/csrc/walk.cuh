@@ -5,9 +5,11 @@
 
 namespace maaso {
 
-// Warps per block, one block per SM: 16 with 128 registers each, or 12 with 168 for a batch of at most three
-// placements per warp, which its longest chains bound (2,000 x 17,000 of the paper's shape: 13.7 ms against 15.0;
-// 100,000 x 100,000 under load: 144 against 122).
+// Warps per block, one block per SM: 16 with 128 registers each, or 12 with room for 168 (142 to 156 are used) for a batch of
+// at most three placements per warp, which its longest chains bound.  Measured, 12 and 16 warps: 2,000 x 17,000 of the
+// paper's shape 9.7 and 10.2 ms; three models under load, 1,000 to 4,440 x 10,000, 1.15 to 1.28 and 1.19 to 1.34; 100,000 x
+// 100,000 117 and 100.  The line is a compromise: a lightly loaded batch, whose placements all take as long, has it at one
+// placement per warp (one node at 2 requests a second, 1,776 x 5,000 3.5 and 3.6 ms, 2,368 6.3 and 4.0, 5,328 10.0 and 8.3).
 constexpr int kWalkWarps = 16, kWalkWarpsFew = 12;
 constexpr int kWalkRing = 64;                     // ring entries per warp
 

@@ -19,10 +19,10 @@
 // Nothing is counted per rejected request: the request count and the checksum of "all of them rejected"
 // are per-class totals of the trace, and a served request takes its own term out again.
 //
-// Measured (B200; lane-group, thread or one-warp kernel before): 143 placements x 500 requests 0.20 ms (0.44),
-// 10,864 x 10,000 6.7 ms (12.2), 2,000 x 17,000 of the paper's shape 9.6 ms (33.8), with queues 10.5 ms (27.0),
-// 100,000 x 100,000 under load 100 ms (132), 64 x 20,000 7.0 ms (18.9), 2,000 placements of 33 to 128 instances x
-// 10,000 10.1 ms (15.4).  A round with one completion takes 300 warp instructions and, alone on its scheduler,
+// Measured (B200, whole calls with routing and top-k; lane-group, thread or one-warp kernel before): 143 placements x 500
+// requests 0.23 ms (0.56), one node's 10,864 x 10,000 6.8 ms (12.0), 2,000 x 17,000 of the paper's shape 9.5 ms (33.9), with
+// queues 11.0 ms (27.8), three models, 100,000 x 100,000 under load 99.7 ms (135), 64 of their placements x 20,000 with all side
+// outputs 2.0 to 3.1 ms (13.8 to 14.1), 2,000 placements of 33 to 128 instances x 10,000 7.9 to 8.3 ms (13.8).  A round with one completion takes 300 warp instructions and, alone on its scheduler,
 // 1,130 cycles, almost all of them dependent: what the next step needs is therefore read from shared memory ahead of
 // the choice, the uncommon outcomes share one branch, and tests of several conditions are written without branches
 // (& and | for && and ||: 652 -> 576 ns a round, 100,000 x 100,000 under load 115 -> 100 ms).

@@ -1017,11 +1017,11 @@ def test_several_traces_in_one_pass(ctx, oracle_mod, flags):
 
 @pytest.mark.parametrize("flags", [0, 1])
 def test_several_traces_in_one_pass_on_the_thread_kernel(oracle_mod, monkeypatch, flags):
-    """Several traces in one pass under both routings of the default mapping: with the routing threshold
-    at zero the loaded batch goes to the thread kernel, placements of more than 32 instances included;
-    with a threshold out of reach the lane groups take it and one warp per placement replays the large
-    ones (no ETOOMANY below 129 instances either way); records, per-model rejection counts and histograms
-    must equal the oracle's for every trace."""
+    """Several traces in one pass under both routings of the default mapping: with MAASO_THREAD_MIN_CAND at
+    zero the loaded batch goes to the thread kernel, placements of more than 32 instances included; with it
+    out of reach the batch walks, the large placements in the walking kernel's variant for them (no
+    ETOOMANY below 129 instances either way); records, per-model rejection counts and histograms must equal
+    the oracle's for every trace."""
     import torch
     import paper_2509_06362_b200 as m
     prof = gen.profile_multimodel(0)
@@ -1036,7 +1036,7 @@ def test_several_traces_in_one_pass_on_the_thread_kernel(oracle_mod, monkeypatch
     classes = cfg["classes"]
     traces_np = [gen.make_trace(900 - 150 * i, 40.0 * (i + 1), 30 + i, model_mix=(0.6, 0.3, 0.1)) for i in range(3)]
     n_cand, n_tr = len(off) - 1, len(traces_np)
-    for min_cand in ("0", "1000000"):        # the whole batch on the thread kernel / only the large placements
+    for min_cand in ("0", "1000000"):        # the whole batch on the thread kernel / all of it walks
         monkeypatch.setenv("MAASO_THREAD_MIN_CAND", min_cand)
         c = m.Context(0)
         c.load_profile(prof)
@@ -1061,7 +1061,7 @@ def test_several_traces_in_one_pass_on_the_thread_kernel(oracle_mod, monkeypatch
         if min_cand == "0":
             assert tm["thread_ms"] > 0.5 and tm["block_ms"] < 0.5      # everything on the thread kernel
         else:
-            assert tm["thread_ms"] < 0.5 and tm["block_ms"] > 0.5      # lane groups + one warp per large placement
+            assert tm["thread_ms"] < 0.5 and tm["block_ms"] > 0.5      # walking kernels: up to 32 instances, and beyond
         c.close()
 
 

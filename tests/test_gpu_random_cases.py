@@ -80,7 +80,7 @@ def test_random_case_every_engine_and_mapping(ctx, oracle_mod, seed):
 @pytest.mark.parametrize("seed", range(6))
 def test_random_case_several_traces_in_one_pass(oracle_mod, seed, monkeypatch):
     """The same kind of workload against three traces in one call, under both routings of the default
-    mapping (the thread kernel takes the loaded part of the batch / only what the lane groups cannot)."""
+    mapping (MAASO_THREAD_MIN_CAND brings the thread kernel back / the batch walks)."""
     import torch
     import paper_2509_06362_b200 as m
     prof, off, inst, classes, tr, mask = _case(100 + seed)

@@ -145,3 +145,32 @@ def test_rounds_behind_one_that_left_the_horizon(oracle_mod, seed, flags):
     off, inst = gen.candidates_from_lists(lists)
     want = _check(oracle_mod, m, prof, tr, gen.make_classes([(None, None, None)]), off, inst, flags)
     assert (want["max_e2e_us"] > 0x60000000).mean() > 0.3
+
+
+@pytest.mark.parametrize("flags", [0, 1, 2, 3, 8, 9])
+def test_tables_and_limits_beyond_32_bit_times(oracle_mod, flags):
+    """A batch that 32-bit times cannot hold runs with 64-bit ones from its start: decode steps and prefill bases of 2^30 us,
+    inputs of four billion tokens, limits of 2^40 us, arrivals up to 2^50; placements of 1 to 128 instances."""
+    import paper_2509_06362_b200 as m
+    W = gen.WMAX
+    rng = np.random.default_rng(23)
+    step = np.zeros((2, 3, W), dtype=np.int32)
+    step[:, 0] = 1 + np.arange(W)
+    step[:, 1] = (1 << 30) - np.arange(W)
+    step[:, 2] = rng.integers(1, 1 << 20, size=(2, W))
+    prof = {"n_models": 2, "n_strategies": 3, "wmax": W, "devices": np.ones(3, dtype=np.int32), "min_devices": np.ones(2, dtype=np.int32),
+            "prefill_base_us": np.array([[0, 1 << 30, 7], [3, 0, 1 << 20]], dtype=np.int32),
+            "prefill_q16": np.array([[0, (1 << 31) - 1, 65536], [1, 0, 123456]], dtype=np.int32), "step_us": step}
+    n = 500
+    tr = np.zeros(n, dtype=gen.REQUEST_DTYPE)
+    gaps = rng.choice([0, 1, 1000, 10 ** 7, 5 * 10 ** 9, 3 * 10 ** 12], size=n, p=[0.2, 0.2, 0.3, 0.2, 0.07, 0.03])
+    tr["arrival_us"] = np.minimum(np.cumsum(gaps) * 20, (1 << 50) - 1)
+    tr["in_tokens"] = rng.choice([0, 1, 4096, 2 ** 32 - 1], size=n, p=[0.4, 0.3, 0.25, 0.05])
+    tr["out_tokens"] = rng.choice([1, 2, 300, 40000, 65535], size=n)
+    tr["cls"] = rng.integers(0, 3, size=n)
+    tr["model"] = rng.integers(0, 2, size=n)
+    classes = gen.make_classes([(None, None, None), (1 << 40, 1 << 40, 1 << 40), (10 ** 9, 10 ** 6, None)])
+    lists = _lists(prof, rng, (1, 2, 5, 8, 17, 32), (1, 2, 7, 64), 6) + _lists(prof, rng, (33, 64, 128), (1, 9, 64), 3)
+    off, inst = gen.candidates_from_lists(lists)
+    want = _check(oracle_mod, m, prof, tr, classes, off, inst, flags)
+    assert (want["makespan_us"] > 1 << 40).all() and (want["status"] == 0).mean() > 0.5
