@@ -31,10 +31,10 @@ TOPK = 64
 # kernels whose source hashes to `csrc_sha256`; with any other source they are not printed.
 PROFILED = {
     "workload": "multimodel", "mapping": 0, "kernel": "eval_walk_kernel",
-    # profiles/eval_thread_kernel_multimodel_sweep_counters.md, first table: one launch of the default workload
-    "warp_inst_per_launch": 75909936388,                 # smsp__inst_executed.sum
-    "dram_bytes_per_launch": 4910080 + 0,                # dram__bytes_read.sum + dram__bytes_write.sum
-    "csrc_sha256": "ddecd5ed7be2da69a0029d7d9c8a41085c9aaccfe83baf9549894b3df75eee42",
+    # profiles/eval_walk_kernel_multimodel_sweep_counters.md: one launch of the default workload
+    "warp_inst_per_launch": 76319382253,                 # smsp__inst_executed.sum
+    "dram_bytes_per_launch": 4908032 + 512,               # dram__bytes_read.sum + dram__bytes_write.sum
+    "csrc_sha256": "fdd8cdd12aef03086dd4e52fb4e6df6325b21526eab3f213ee3ede400cd3bc54",
 }
 SM_COUNT, ISSUE_PER_SM = 148, 4   # B200: 148 SMs x 4 warp schedulers, one warp instruction per cycle each
 

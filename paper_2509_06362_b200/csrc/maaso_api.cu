@@ -654,8 +654,8 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     //                 24,576 13.0 and 12.9; at 4 a second 32,768 11.5 and 12.9
     //   16 models     (which the placements serve few of) at 2 a second 16,384 3.3 and 4.5, 98,304 18.2 and 22.3, 163,840 30.1 and
     //                 35.9: walking is the better one at every size
-    // that is between 3,100 and 6,500 placements for one model and between 9,000 and more than 32,768 for several.  With fixed
-    // speeds or queues the alternative is the lane-group kernel.  Fixed speeds: 4,500 to 9,800, 9,000 to more than 24,576.
+    // that is between 3,100 and 6,600 placements for one model and between 9,000 and more than 32,768 for several.  With fixed
+    // speeds or queues the alternative is the lane-group kernel.  Fixed speeds: 6,200 and more, 9,100 and more.
     // Queues cost the walking kernel more, and for several models the line is late there: one model at 2 a second 4,096 7.3 and
     // 8.1, 5,000 9.6 and 8.3; two models 6,144 7.2 and 7.8, 8,192 9.0 and 7.9; three 8,192 7.4 and 7.7, 10,240 8.9 and 7.7, 16,384
     // 13.0 and 10.0.

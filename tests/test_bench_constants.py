@@ -15,7 +15,7 @@ def test_profiled_constants_match_the_committed_summary():
         return
     assert set(p) >= {"workload", "mapping", "kernel", "warp_inst_per_launch", "dram_bytes_per_launch", "csrc_sha256"}
     assert re.fullmatch(r"[0-9a-f]{64}", p["csrc_sha256"])
-    text = open(os.path.join(ROOT, "profiles", "eval_thread_kernel_multimodel_sweep_counters.md")).read()
+    text = open(os.path.join(ROOT, "profiles", "eval_walk_kernel_multimodel_sweep_counters.md")).read()
     num = lambda key: int(re.search(re.escape(key) + r" \| ([0-9,]+)", text).group(1).replace(",", ""))
     assert num("smsp__inst_executed.sum") == p["warp_inst_per_launch"]
     assert num("dram__bytes_read.sum") + num("dram__bytes_write.sum") == p["dram_bytes_per_launch"]
