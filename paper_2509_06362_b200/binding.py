@@ -398,6 +398,8 @@ class Context:
         kw = {}
         if dump_idx is not None:
             d = self.to_device(np.asarray(dump_idx, dtype=np.uint32))
+            if isinstance(stream, torch.cuda.Stream):
+                d.record_stream(stream)  # it is let go on return, and the call reads it on its own stream
             dumps = {"finish_us": torch.empty((len(dump_idx), trace.n), dtype=torch.int64, device=self.device),
                      "first_us": torch.empty((len(dump_idx), trace.n), dtype=torch.int64, device=self.device),
                      "inst": torch.empty((len(dump_idx), trace.n), dtype=torch.int32, device=self.device)}

@@ -1174,3 +1174,29 @@ def test_ins_deploy_refuses_what_scoring_refuses(ctx, gpus):
     assert len(phi) == gpus + 1 and phi[0] == 0.0
     ctx.free_trace(t)
     other.close()
+
+
+def test_dumps_on_a_stream_that_is_busy(ctx, oracle_mod):
+    """The list of placements to dump lives until the stream of the call has read it, whatever is allocated meanwhile."""
+    import torch
+    cfg = gen.make_config("tiny", n_req=120)
+    idx = np.arange(0, 143, 2, dtype=np.uint32)
+    want, wd = oracle_mod.eval_placements(cfg["profile"], cfg["traces"][0], cfg["classes"], cfg["offsets"], cfg["inst"], 4, dump_idx=idx)
+    ctx.load_profile(cfg["profile"])
+    t = ctx.load_trace(cfg["traces"][0], cfg["classes"])
+    d_off, d_inst = ctx.to_device(cfg["offsets"]), ctx.to_device(cfg["inst"])
+    ctx.eval_placements(t, d_off, d_inst, 4, dump_idx=idx)  # the scratch has its size, the kernels are loaded
+    over = [torch.zeros(len(idx), dtype=torch.int32, device="cuda")]
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(100_000_000)  # about 50 ms
+    out, dumps = ctx.eval_placements(t, d_off, d_inst, 4, dump_idx=idx, stream=side)
+    over += [torch.zeros(len(idx), dtype=torch.int32, device="cuda") for _ in range(500)]
+    assert not side.query()  # it was still asleep
+    torch.cuda.synchronize()
+    del over
+    assert_records_equal(ctx.results_to_numpy(out), want, "busy stream")
+    for k in wd:
+        assert (dumps[k].cpu().numpy() == wd[k]).all(), k
+    ctx.free_trace(t)
