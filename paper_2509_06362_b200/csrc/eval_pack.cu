@@ -32,9 +32,10 @@ bool pack_fits(uint32_t n_rows, uint32_t n_classes) {
     return pack_layout(n_rows, n_classes).pool + 32u * kWalkWarps * kPackLane <= 227u * 1024u;
 }
 
-// Accounts a group's ring, one entry per lane and pass (lane `li` of `G`; `mine`: the lane's sums).
+// Accounts a group's ring, one entry per lane and pass (lane `li` of `G`; `mine`: the lane's sums).  An entry: finish time from
+// the epoch, first-token time (61 bits), the instance in the group (3 bits), the request.
 static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumping, uint32_t oc, unsigned char* mine, uint32_t* bins,
-                                                 uint32_t ring, uint32_t ring_b, uint32_t li, uint32_t G, uint32_t cnt, uint32_t lims,
+                                                 uint32_t ring, int64_t epoch, uint32_t li, uint32_t G, uint32_t cnt, uint32_t lims,
                                                  const uint4* reqs) {
     __syncwarp();
     if (li < cnt) {
@@ -45,10 +46,10 @@ static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumpi
         uint64_t sum = (uint64_t)i64_of(u2.z, u2.w);
         uint32_t served = u3.z, hits = u3.w;
         for (uint32_t e = li; e < cnt; e += G) {
-            const uint2 rb = w2(ring_b + e * 8u);
-            const uint4 rec = __ldg(reqs + rb.x);
             const uint4 ra = w4(ring + e * 16u);
-            const int64_t fin = i64_of(ra.x, ra.y), first = i64_of(ra.z, ra.w), arrival = i64_of(rec.x, rec.y);
+            const uint2 rb = make_uint2(ra.w, ra.z >> 29);
+            const uint4 rec = __ldg(reqs + rb.x);
+            const int64_t fin = epoch + (int32_t)ra.x, first = i64_of(ra.y, ra.z & 0x1FFFFFFFu), arrival = i64_of(rec.x, rec.y);
             const uint32_t S = rec.w & 0xFFFFu, cls = (rec.w >> 16) & 0xFFu;
             const uint4 lim = w4(lims + cls * 16u);
             const int64_t ttft = first - arrival, e2e = fin - arrival;
@@ -107,7 +108,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         const uint32_t at = (eight ? item : item - n8) * (32u / G) + g;
         const bool valid = at < count;
         const uint32_t cap = 2u * G;  // a group's part of the ring
-        const uint32_t ring = L.ring + (warp * kWalkRing + g * cap) * 16u;  // (the second part of an entry is half as far in)
+        const uint32_t ring = L.ring + (warp * kWalkRing + g * cap) * 16u;
         const uint32_t cand = P.bucket_list[(size_t)bucket * P.n_cand + (valid ? at : count - 1u)], oc = tr * P.n_cand + cand;
         const uint4* const reqs = P.trace_reqs[tr];
         const uint32_t n_req = P.trace_n[tr];
@@ -144,7 +145,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
 
         auto bins = [&]() { return reinterpret_cast<uint32_t*>(pay - li * kPackScratch + kPackPay + 64u); };
         auto flush = [&]() {
-            pack_account(P, P.dump_row || P.ttft_hist, oc, pay + kPackPay, bins(), ring, L.ring_b + ((ring - L.ring) >> 1), li, G, ring_n, L.lims, reqs);
+            pack_account(P, P.dump_row || P.ttft_hist, oc, pay + kPackPay, bins(), ring, epoch, li, G, ring_n, L.lims, reqs);
             ring_n = 0;
         };
         auto take_chunk = [&](const uint4& v) {
@@ -187,10 +188,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                     const bool busy = in.w > 0;
                     next_end(left, busy, sw);
                     due = busy & ((left == 0u) | (in.tb < upto)) & !bad;
-                    const uint32_t e = ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below));
-                    const int64_t fin = epoch + in.t;
-                    w2(L.ring_b + ((e - L.ring) >> 1)) = make_uint2(ft.z, li);
-                    w4(e) = make_uint4(lo32(fin), hi32(fin), ft.x, ft.y);
+                    w4(ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below))) = make_uint4((uint32_t)in.t, ft.x, ft.y, ft.z);
                 }
                 ring_n += adds;
                 dm = __ballot_sync(kWFull, due);
@@ -225,6 +223,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                         in.tb -= up;
                     }
                     now = max(now - up, 0);
+                    flush();
                     epoch = to;
                     take_chunk(__ldg(reqs + min(cb + lane, n_req - 1u)));
                     arrival = 0;
@@ -283,21 +282,20 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                             if (in.w > 0) in.tb += pre;
                             bad = bad || in.t > kWalkHorizon || (in.w > 0 && in.tb > kWalkHorizon);
                             const int64_t fin = epoch + in.t;
-                            w4(ring + ring_n * 16u) = make_uint4(lo32(fin), hi32(fin), lo32(fin), hi32(fin));
-                            w2(L.ring_b + ((ring - L.ring) >> 1) + ring_n * 8u) = make_uint2(cb + i, li);
+                            w4(ring + ring_n * 16u) = make_uint4((uint32_t)in.t, lo32(fin), hi32(fin) | (li << 29), cb + i);
                         }
                         ring_n += adds;
                     } else if (win) {
                         in.t += pre;
                         if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
                         if (in.K + Sm1 > kRelMax) {
-                            in.kmin = walk_rebase(area, keys, 32u, (in.B + 7u) >> 3, in.K, in.kmin);
+                            in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K, in.kmin);
                             in.K = 0;
                         }
                         const uint32_t nk = ((in.K + Sm1) << 6) | top;
                         const int64_t first = epoch + in.t;
                         w1(keys + 4u * top) = nk;
-                        __stcg(reinterpret_cast<uint4*>(pay) + top, make_uint4(lo32(first), hi32(first), cb + i, 0u));
+                        __stcg(reinterpret_cast<uint4*>(pay) + top, make_uint4(lo32(first), hi32(first) | (li << 29), cb + i, 0u));
                         atomicMin(&w1(area + ((top >> 3) << 2)), nk);
                         in.kmin = min(in.kmin, nk);
                         in.w++;

@@ -47,8 +47,8 @@ __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c
                     continue;
                 }
                 sum_b += b;
-                slot_bytes += walk_slot_bytes(b, fixed_speed, key_bytes, fixed_speed || (n > kWalkBig && !P.walk_long));
-                slot_bytes64 += walk_slot_bytes(b, fixed_speed, fixed_speed ? 8u : 4u, fixed_speed);
+                slot_bytes += walk_slot_bytes(b, fixed_speed, key_bytes, P.walk_long ? kWalkBlockLong : (n > kWalkBig ? kWalkBlockKeys : kWalkBlock));
+                slot_bytes64 += walk_slot_bytes(b, fixed_speed, fixed_speed ? 8u : 4u, kWalkBlockLong);
                 units += 2u + 2u * ((b + 7u) >> 3) + 2u;
                 supply += b * 1000000u / (uint32_t)P.rows[(m * P.n_strategies + s) * kRowStride + 1 + b];
                 devsum += (uint64_t)P.devices[s];

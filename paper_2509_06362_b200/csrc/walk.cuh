@@ -15,8 +15,8 @@ constexpr int kWalkRing = 64;                     // ring entries per warp
 
 // One block: the completion rings, SLO limits, decode-step tables, the pool.
 struct WalkLayout {
-    uint32_t ring;    // [warps][kWalkRing] {finish, first token}
-    uint32_t ring_b;  // [warps][kWalkRing] {request, instance}
+    uint32_t ring;    // [warps][kWalkRing] {finish, first token, request, instance}; 64-bit times: {finish, first token}
+    uint32_t ring_b;  // 64-bit times: [warps][kWalkRing] {request, instance}
     uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
     uint32_t wide;    // 64-bit times: [n_classes] {TTFT limit (2^62 = none), TBT limit (negative = none)}
     uint32_t steps;   // [n_rows][64] u32
@@ -26,7 +26,7 @@ __host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_cl
     WalkLayout l;
     l.ring = 0;
     l.ring_b = warps * (uint32_t)kWalkRing * 16u;
-    l.lims = l.ring_b + warps * (uint32_t)kWalkRing * 8u;
+    l.lims = l.ring_b + (wide ? warps * (uint32_t)kWalkRing * 8u : 0u);
     l.wide = l.lims + n_classes * 16u;
     l.steps = l.wide + (wide ? n_classes * 16u : 0u);
     l.pool = (l.steps + n_rows * 256u + 127u) & ~127u;
@@ -36,18 +36,20 @@ __host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_cl
 // One placement's region: sums (kWalkSums bytes: one set of four 16-byte units per lane, unit-major, then hits by
 // class bin), 16 bytes per model, 16 per instance, with more than 32 instances their resting state (unit-major) and
 // a lower bound per model, then per instance its slots: the eight block minima, the stack of free slots (a byte
-// each), then blocks of 8 slots with the keys (end index << 6 | slot), the request indices and the first-token
-// times.  Keys alone with more than 32 instances, where the rest (16 bytes per slot) is in global memory: shared memory
-// decides how many such placements are resident.  In the engines that fix a request's speed at admission: the finish
+// each), the keys (end index << 6 | slot, in blocks of 8), then what a running request must remember: {first-token time,
+// request index}, 8 bytes (64-bit times: the request indices, then the first-token times).  Keys alone with more than 32
+// instances, where the rest is in global memory: shared memory decides how many such placements are resident.  In the engines that fix a request's speed at admission: the finish
 // times in falling order, so that the next to free is popped off the end.
 enum WalkKind : uint32_t { kWalkUsual = 0, kWalkBigKind = 1, kWalkLongKind = 2 };
 constexpr uint32_t kWalkLaneSums = 4u * 32u * 16u;
 constexpr uint32_t kWalkSums = kWalkLaneSums + 48u;
 constexpr uint32_t kWalkBig = 32u;  // more instances than this rest in shared memory
 __host__ __device__ inline uint32_t walk_slots_at(uint32_t nblk) { return 32u + ((8u * nblk + 15u) & ~15u); }
-__host__ __device__ inline uint32_t walk_slot_bytes(uint32_t b, bool fixed_speed, uint32_t key_bytes, bool keys_alone) {
+// `block`: bytes of 8 slots
+constexpr uint32_t kWalkBlock = 96u, kWalkBlockLong = 128u, kWalkBlockKeys = 32u;
+__host__ __device__ inline uint32_t walk_slot_bytes(uint32_t b, bool fixed_speed, uint32_t key_bytes, uint32_t block) {
     const uint32_t nblk = (b + 7u) >> 3;
-    return fixed_speed ? ((b * key_bytes + 15u) & ~15u) : walk_slots_at(nblk) + nblk * (keys_alone ? 32u : 128u);
+    return fixed_speed ? ((b * key_bytes + 15u) & ~15u) : walk_slots_at(nblk) + nblk * block;
 }
 __host__ __device__ inline uint32_t walk_rest_bytes(WalkKind kind) { return kind == kWalkUsual ? 0u : (kind == kWalkBigKind ? 48u : 80u); }
 __host__ __device__ inline uint32_t walk_region_bytes(uint32_t n_models, uint32_t n_inst, uint32_t slot_bytes, WalkKind kind) {
@@ -60,8 +62,8 @@ __host__ __device__ inline uint32_t walk_big_bin(uint32_t need) {
     const uint32_t k = need / kWalkStepBytes;
     return 255u - (k < 255u ? k : 255u);
 }
-// Global memory for one block's running requests: four bytes of it per byte of pool.
-__host__ __device__ inline size_t walk_big_scratch(uint32_t pool_bytes) { return (size_t)pool_bytes * 4u; }
+// Global memory for one block's running requests: two bytes of it per byte of pool.
+__host__ __device__ inline size_t walk_big_scratch(uint32_t pool_bytes) { return (size_t)pool_bytes * 2u; }
 
 // The most a placement can need: 128 instances of 64 slots, 16 models, 8-byte keys or requests beside 4-byte keys.
 constexpr uint32_t kWalkMost = 160u * 1024u;

@@ -92,15 +92,17 @@ __device__ __forceinline__ uint32_t walk_steps(int64_t dt, uint32_t s, float rs)
 //   3: output tokens, requests served, hits
 template <bool Wide>
 static __device__ __noinline__ void walk_account(const EvalParams& P, bool dumping, uint32_t oc, uint32_t base, uint32_t ring,
-                                                 uint32_t ring_b, uint32_t cnt, uint32_t lims, uint32_t wide, const uint4* reqs) {
+                                                 uint32_t ring_b, uint32_t cnt, int64_t epoch, uint32_t lims, uint32_t wide,
+                                                 const uint4* reqs) {
     const uint32_t lane = threadIdx.x & 31u, sums = base + 16u * lane;
     __syncwarp();
     for (uint32_t e = lane; e < cnt; e += 32u) {
-        const uint2 rb = w2(ring_b + e * 8u);
-        const uint4 rec = __ldg(reqs + rb.x);
         const uint4 ra = w4(ring + e * 16u);
+        const uint2 rb = Wide ? w2(ring_b + e * 8u) : make_uint2(ra.z, ra.w);
+        const uint4 rec = __ldg(reqs + rb.x);
         const uint4 u0 = w4(sums), u1 = w4(sums + 512u), u2 = w4(sums + 1024u), u3 = w4(sums + 1536u);
-        const int64_t fin = i64_of(ra.x, ra.y), first = i64_of(ra.z, ra.w), arrival = i64_of(rec.x, rec.y);
+        const int64_t fin = Wide ? i64_of(ra.x, ra.y) : epoch + (int32_t)ra.x, first = Wide ? i64_of(ra.z, ra.w) : epoch + (int32_t)ra.y;
+        const int64_t arrival = i64_of(rec.x, rec.y);
         const uint32_t S = rec.w & 0xFFFFu, cls = (rec.w >> 16) & 0xFFu;
         const uint4 lim = w4(lims + cls * 16u);
         const int64_t ttft = first - arrival, e2e = fin - arrival;
@@ -134,10 +136,10 @@ static __device__ __noinline__ void walk_account(const EvalParams& P, bool dumpi
 }
 
 // All live end indices of one instance move down by the counter value K (which restarts at 0).  Rare.
-static __device__ __noinline__ uint32_t walk_rebase(uint32_t area, uint32_t keys, uint32_t block, uint32_t nblk, uint32_t K, uint32_t kmin) {
+static __device__ __noinline__ uint32_t walk_rebase(uint32_t area, uint32_t keys, uint32_t nblk, uint32_t K, uint32_t kmin) {
     const uint32_t d = K << 6;
     for (uint32_t b = 0; b <= nblk; b++) {
-        const uint32_t p = b ? keys + block * (b - 1u) : area;  // the minima, then the keys of each block
+        const uint32_t p = b ? keys + 32u * (b - 1u) : area;  // the minima, then the keys of each block
         for (uint32_t i = 0; i < 8u; i++) {
             const uint32_t k = w1(p + 4u * i);
             if (k != kKeyEmpty) w1(p + 4u * i) = k - d;
@@ -152,7 +154,7 @@ static __device__ __noinline__ void walk_hand_over(const EvalParams& P, uint32_t
     if (atomicExch(&P.code[cand], 0xFFFFFFFEu) == 0xFFFFFFFEu) return;
     const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
     uint32_t slots = 0, mode = 0;
-    for (uint32_t i = 0; i < n_i; i++) slots += walk_slot_bytes((P.inst[lo + i] >> 12) & 0xFFu, fixed_speed, fixed_speed ? 8u : 4u, fixed_speed);
+    for (uint32_t i = 0; i < n_i; i++) slots += walk_slot_bytes((P.inst[lo + i] >> 12) & 0xFFu, fixed_speed, fixed_speed ? 8u : 4u, kWalkBlockLong);
     const uint32_t need = walk_region_bytes(P.n_models, n_i, slots, kWalkLongKind);
     while (mode + 1u < (uint32_t)kWalkModes && need > (P.walk_bytes << mode)) mode++;
     // (what 16 parts cannot hold is not in a walking bucket in the first place)
@@ -174,7 +176,7 @@ struct WInst {
     uint32_t tag;  // 1 << model (0 for a lane without an instance) | place in the placement as given << 16
     uint32_t area, keys, row;  // byte offsets of its slots, of its first block of keys and of its decode-step row
     uint32_t pre_base, pre_q16, stepB;
-    uint32_t pad;
+    uint32_t pay;  // of what its running requests must remember
 };
 
 template <bool Opt, int Eng, bool Wide, bool Big>
@@ -189,7 +191,7 @@ struct Walk {
     static constexpr U kNone = ~(U)0;
     static constexpr uint32_t kKeyBytes = kFixed ? (uint32_t)sizeof(T) : 4u;
     static constexpr bool kAway = Big && !Wide && !kFixed;  // running requests' data in global memory
-    static constexpr uint32_t kBlock = kFixed || kAway ? 8u * kKeyBytes : 128u;  // bytes of a block of 8 slots
+    static constexpr uint32_t kBlock = Wide ? kWalkBlockLong : (Big ? kWalkBlockKeys : kWalkBlock);
     static constexpr WalkKind kKind = Wide ? kWalkLongKind : (Big ? kWalkBigKind : kWalkUsual);
     static constexpr uint32_t kRest = Wide ? 80u : 48u;
 
@@ -236,7 +238,7 @@ struct Walk {
     }
 
     // One warp takes the placements of a bucket, one after the other.  `base`: its part of shared memory;
-    // `away`: the block's global memory for running requests, four bytes per byte of pool (kAway).
+    // `away`: the block's global memory for running requests, two bytes per byte of pool (kAway).
     static __device__ __forceinline__ void bucket(const EvalParams& P, const WalkLayout& L, int bucket, uint32_t base,
                                                   uint32_t static_idx, uint32_t static_total, unsigned char* away) {
         constexpr uint32_t kCap = (uint32_t)kWalkRing;
@@ -287,7 +289,7 @@ struct Walk {
                 for (uint32_t s = 0; s < (Big ? n_i : 1u); s += 32u) {
                     const uint32_t j = s + lane, at = ents + 16u * j;
                     in.t = 0; in.tb = kFar; in.K = 0; in.kmin = kKeyEmpty; in.w = 0; in.B = 1; in.sw = 1; in.rsw = 1.0f;
-                    in.pre_base = in.pre_q16 = 0; in.stepB = 1; in.tag = 0; in.area = in.keys = in.row = L.steps; in.pad = 0;
+                    in.pre_base = in.pre_q16 = 0; in.stepB = 1; in.tag = 0; in.area = in.keys = in.pay = in.row = L.steps;
                     uint32_t nblk = 0;
                     if (j < n_i) {
                         const uint2 e = w2(at);
@@ -309,7 +311,7 @@ struct Walk {
                         // per instance: earliest start, prefill base and slope, smallest prediction step
                         w4(at) = make_uint4(0u, in.pre_base, in.pre_q16, ms);
                     }
-                    const uint32_t bytes = nblk ? walk_slot_bytes(in.B, kFixed, kKeyBytes, kFixed || kAway) : 0u;
+                    const uint32_t bytes = nblk ? walk_slot_bytes(in.B, kFixed, kKeyBytes, kBlock) : 0u;
                     uint32_t incl = bytes;
                     for (uint32_t o = 1; o < 32u; o <<= 1) {
                         const uint32_t v = __shfl_up_sync(kWFull, incl, o);
@@ -318,9 +320,9 @@ struct Walk {
                     if (nblk) {
                         in.area = area + incl - bytes;
                         in.keys = kFixed ? in.area : in.area + walk_slots_at(nblk);
+                        in.pay = in.keys + 32u * nblk;
                         if (!kFixed) {
-                            for (uint32_t i = 0; i < 8u * (nblk + 1u); i++)
-                                w1(i < 8u ? in.area + 4u * i : in.keys + kBlock * ((i - 8u) >> 3) + 4u * (i & 7u)) = kKeyEmpty;
+                            for (uint32_t i = 0; i < 8u * (nblk + 1u); i++) w1(i < 8u ? in.area + 4u * i : in.keys + 4u * (i - 8u)) = kKeyEmpty;
                             for (uint32_t i = 0; i < in.B; i++) walk_smem[in.area + 32u + i] = (unsigned char)i;
                         }
                     }
@@ -360,7 +362,7 @@ struct Walk {
             uint32_t c_in = 0, c_meta = 0; // input tokens, output tokens | class | model
 
             auto flush = [&]() {
-                walk_account<Wide>(P, P.dump_row || P.ttft_hist, tr * P.n_cand + cand, base, ring, ring_b, ring_n, L.lims, L.wide, reqs);
+                walk_account<Wide>(P, P.dump_row || P.ttft_hist, tr * P.n_cand + cand, base, ring, ring_b, ring_n, epoch, L.lims, L.wide, reqs);
                 ring_n = 0;
             };
             auto take_chunk = [&](const uint4& v) {
@@ -385,6 +387,21 @@ struct Walk {
                     bad = bad | (busy & (tc > (uint64_t)kWalkHorizon));
                 }
             };
+            auto firsts = [&]() { return in.pay + 32u * ((in.B + 7u) >> 3); };  // 64-bit times: first tokens of the running requests
+            // Running requests' first tokens, when the epoch moves by `up`.  (Further back than 32 bits reach: the lane has left
+            // the horizon.)
+            auto rebase_firsts = [&](T up) {
+                if constexpr (!kFixed && !Wide) {
+                    for (uint32_t i = 0; i < in.B && in.w > 0; i++) {
+                        if (w1(in.keys + 4u * i) == kKeyEmpty) continue;
+                        int32_t* const f = kAway ? reinterpret_cast<int32_t*>(away + 2u * (in.keys + 4u * i - L.pool)) : &wt<int32_t>(in.pay + 8u * i);
+                        const int64_t v = (int64_t)(kAway ? __ldcg(f) : *f) - up;
+                        bad = bad || v < -(int64_t)kWalkFar;
+                        if (kAway) __stcg(f, (int32_t)v);
+                        else *f = (int32_t)v;
+                    }
+                }
+            };
             // Completions (fixed speeds: slots that free) of the lanes in `due`, one per lane and iteration, until every
             // clock has reached `upto`.
             auto events = [&](bool due, T upto) {
@@ -401,19 +418,14 @@ struct Walk {
                         if (ring_n + adds > kCap) flush();
                         if (due) {
                             const uint32_t slot = in.kmin & 63u;
-                            const uint32_t kb = in.keys + (slot >> 3) * kBlock, k8 = kb + 4u * (slot & 7u);
+                            const uint32_t k8 = in.keys + 4u * slot, kb = in.keys + 4u * (slot & 56u);
                             const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(in.area), m1 = w4(in.area + 16u);
                             const uint32_t sw = w1(in.row + 4u * in.w - 8u);  // (the word before the row, if that was the last one)
-                            uint2 ft;
-                            uint32_t rq;
-                            if constexpr (kAway) {
-                                const uint4 v = __ldcg(reinterpret_cast<const uint4*>(away + 4u * (k8 - L.pool)));
-                                ft = make_uint2(v.x, v.y);
-                                rq = v.z;
-                            } else {
-                                ft = w2(k8 + 64u + 4u * (slot & 7u));
-                                rq = w1(k8 + 32u);
-                            }
+                            uint2 run;  // first token, request; 64-bit times: first token
+                            uint32_t rq = 0;
+                            if constexpr (kAway) run = __ldcg(reinterpret_cast<const uint2*>(away + 2u * (k8 - L.pool)));
+                            else if constexpr (!Wide) run = w2(in.pay + 8u * slot);
+                            else run = w2(firsts() + 8u * slot), rq = w1(in.pay + 4u * slot);
                             in.t = in.tb + (T)in.sw;
                             in.K = in.kmin >> 6;
                             in.w--;
@@ -424,9 +436,12 @@ struct Walk {
                             const uint32_t mv[8] = {m0.x - km, m0.y - km, m0.z - km, m0.w - km, m1.x - km, m1.y - km, m1.z - km, m1.w - km};
                             const uint32_t bmin = min8(kv);
                             const uint32_t e = ring_n + (uint32_t)__popc(dm & below);
-                            const int64_t fin = epoch + in.t;
-                            w4(ring + 16u * e) = make_uint4(lo32(fin), hi32(fin), ft.x, ft.y);
-                            w2(ring_b + 8u * e) = make_uint2(rq, in.tag >> 16);
+                            if constexpr (Wide) {
+                                w4(ring + 16u * e) = make_uint4(lo32(in.t), hi32(in.t), run.x, run.y);
+                                w2(ring_b + 8u * e) = make_uint2(rq, in.tag >> 16);
+                            } else {
+                                w4(ring + 16u * e) = make_uint4((uint32_t)in.t, run.x, run.y, in.tag >> 16);
+                            }
                             w1(k8) = kKeyEmpty;
                             w1(in.area + ((slot >> 3) << 2)) = bmin + km;
                             in.kmin = min(bmin, min8(mv)) + km;
@@ -466,9 +481,12 @@ struct Walk {
             };
             // One request's times into the ring (`e`: its entry).
             auto record = [&](uint32_t e, T fin, T first, uint32_t req) {
-                const int64_t f = epoch + fin, g = epoch + first;
-                w4(ring + e * 16u) = make_uint4(lo32(f), hi32(f), lo32(g), hi32(g));
-                w2(ring_b + e * 8u) = make_uint2(req, in.tag >> 16);
+                if constexpr (Wide) {
+                    w4(ring + e * 16u) = make_uint4(lo32(fin), hi32(fin), lo32(first), hi32(first));
+                    w2(ring_b + e * 8u) = make_uint2(req, in.tag >> 16);
+                } else {
+                    w4(ring + e * 16u) = make_uint4((uint32_t)fin, (uint32_t)first, req, in.tag >> 16);
+                }
             };
             // "map": prefill at the step boundary (running decodes stall), then occupy a free slot.  With fixed speeds the slot
             // is busy until the finish time, and `queued` takes over the slot that frees first; an instance's finish times
@@ -526,18 +544,19 @@ struct Walk {
                     in.t += pre;
                     if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
                     if (in.K + Sm1 > kRelMax) {
-                        in.kmin = walk_rebase(in.area, in.keys, kBlock, (in.B + 7u) >> 3, in.K, in.kmin);
+                        in.kmin = walk_rebase(in.area, in.keys, (in.B + 7u) >> 3, in.K, in.kmin);
                         in.K = 0;
                     }
                     const uint32_t nk = ((in.K + Sm1) << 6) | slot;
-                    const uint32_t k8 = in.keys + (slot >> 3) * kBlock + 4u * (slot & 7u);
-                    const int64_t first = epoch + in.t;
+                    const uint32_t k8 = in.keys + 4u * slot;
                     w1(k8) = nk;
                     if constexpr (kAway) {
-                        __stcg(reinterpret_cast<uint4*>(away + 4u * (k8 - L.pool)), make_uint4(lo32(first), hi32(first), req, 0u));
+                        __stcg(reinterpret_cast<uint2*>(away + 2u * (k8 - L.pool)), make_uint2((uint32_t)in.t, req));
+                    } else if constexpr (!Wide) {
+                        w2(in.pay + 8u * slot) = make_uint2((uint32_t)in.t, req);
                     } else {
-                        w1(k8 + 32u) = req;
-                        w2(k8 + 64u + 4u * (slot & 7u)) = make_uint2(lo32(first), hi32(first));
+                        w1(in.pay + 4u * slot) = req;
+                        w2(firsts() + 8u * slot) = make_uint2(lo32(in.t), hi32(in.t));
                     }
                     atomicMin(&w1(in.area + ((slot >> 3) << 2)), nk);
                     in.kmin = min(in.kmin, nk);
@@ -596,6 +615,7 @@ struct Walk {
                             const uint4 v = __ldg(reqs + req);
                             const int64_t to = max(epoch + now, i64_of(v.x, v.y));
                             const T up = to - epoch >= (int64_t)kFar ? kFar : (T)(to - epoch);
+                            // (`up` is cut off only if everything is idle by then)
                             for (uint32_t s = 0; s < (Big ? n_i : 1u); s += 32u) {
                                 const bool mine = !Big || s + lane < n_i;
                                 if (Big) {
@@ -614,6 +634,7 @@ struct Walk {
                                     catch_up(in.w < in.B, up);
                                     in.t = in.t > up + kWPast ? in.t - up : kWPast;  // a full instance's clock is not looked at
                                     in.tb -= up;
+                                    if (mine) rebase_firsts(up);
                                 }
                                 if (mine && s + lane < n_i) {
                                     const T t = kFixed && in.w < in.B ? 0 : start();
@@ -625,6 +646,7 @@ struct Walk {
                                 const int64_t lb = wi(lbs + 8u * lane) - up;
                                 wi(lbs + 8u * lane) = lb < kWPast ? (int64_t)kWPast : lb;
                             }
+                            flush();
                             epoch = to;
                             now = 0;
                             take_chunk(__ldg(reqs + min(cb + lane, n_req - 1u)));
