@@ -115,7 +115,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         uint4 nxt = make_uint4(0u, 0u, 0u, 0u);
         if (n_req) nxt = __ldg(reqs + min(lane, n_req - 1u));
         WInst<int32_t> in;
-        in.t = 0; in.tb = kFar; in.K = 0; in.kmin = kKeyEmpty; in.w = 0; in.B = 1; in.sw = 1; in.rsw = 1.0f;
+        in.t = 0; in.tb = kFar; in.K = 0; in.kmin = kKeyEmpty; in.w = 0; in.B = 1; in.sw = 1; in.rsw = ~0u;
         in.pre_base = in.pre_q16 = 0; in.stepB = 1; in.tag = 0; in.row = L.steps;
         {
             const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
@@ -123,10 +123,10 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 const uint32_t word = P.inst[lo + li], md = word & 0xFu, r = md * P.n_strategies + ((word >> 4) & 0xFFu);
                 in.tag = 1u << md;
                 in.B = (word >> 12) & 0xFFu;
-                in.row = L.steps + r * 256u;
+                in.row = L.steps + r * kWalkRow;
                 in.pre_base = (uint32_t)P.rows[r * kRowStride];
                 in.pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
-                in.stepB = w1(in.row + 4u * in.B - 4u);
+                in.stepB = w1(in.row + 8u * in.B);
             }
         }
         for (uint32_t i = 0; i < 8u + ((in.B + 7u) & ~7u); i++) w1(i < 8u ? area + 4u * i : keys + 4u * (i - 8u)) = kKeyEmpty;
@@ -154,9 +154,10 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
             c_in = v.z;
             c_meta = v.w;
         };
-        auto next_end = [&](uint32_t left, bool busy, uint32_t sw) {
+        auto next_end = [&](uint32_t left, bool busy, uint2 step) {
+            const uint32_t sw = step.x;
             in.sw = sw;
-            in.rsw = walk_rcp(sw);
+            in.rsw = step.y;
             const uint64_t tc = (uint64_t)left * sw + (uint32_t)in.t;
             in.tb = busy ? (int32_t)((uint32_t)tc - sw) : kFar;
             bad = bad | (busy & (tc > (uint64_t)kWalkHorizon));
@@ -170,23 +171,22 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 if (due) {
                     const uint32_t slot = in.kmin & 63u, kb = keys + ((slot >> 3) << 5);
                     const uint4 ft = __ldcg(reinterpret_cast<const uint4*>(pay) + slot);
+                    w1(keys + (slot << 2)) = kKeyEmpty;
+                    w1(area + ((slot >> 3) << 2)) = kKeyEmpty;
                     const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(area), m1 = w4(area + 16u);
-                    const uint32_t sw = w1(in.row + 4u * in.w - 8u);  // (the word before the row, if that was the last one)
+                    const uint2 step = w2(in.row + 8u * in.w - 8u);
                     in.t = in.tb + (int32_t)in.sw;
                     in.K = in.kmin >> 6;
                     in.w--;
                     walk_smem[area + 32u + in.w] = (unsigned char)slot;
-                    // the smallest of the other keys: keys are unique, so the retired one wraps to all ones
-                    const uint32_t km = in.kmin + 1u;
-                    const uint32_t kv[8] = {k0.x - km, k0.y - km, k0.z - km, k0.w - km, k1.x - km, k1.y - km, k1.z - km, k1.w - km};
-                    const uint32_t mv[8] = {m0.x - km, m0.y - km, m0.z - km, m0.w - km, m1.x - km, m1.y - km, m1.z - km, m1.w - km};
+                    const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                    const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
                     const uint32_t bmin = min8(kv);
-                    w1(keys + (slot << 2)) = kKeyEmpty;
-                    w1(area + ((slot >> 3) << 2)) = bmin + km;
-                    in.kmin = min(bmin, min8(mv)) + km;
+                    w1(area + ((slot >> 3) << 2)) = bmin;
+                    in.kmin = min(bmin, min8(mv));
                     const uint32_t left = (in.kmin >> 6) - in.K;
                     const bool busy = in.w > 0;
-                    next_end(left, busy, sw);
+                    next_end(left, busy, step);
                     due = busy & ((left == 0u) | (in.tb < upto)) & !bad;
                     w4(ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below))) = make_uint4((uint32_t)in.t, ft.x, ft.y, ft.z);
                 }
@@ -198,7 +198,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         auto catch_up = [&](bool go, int32_t upto) {
             const int32_t dt = go ? max(upto - in.t, 0) : 0;
             const uint32_t k = walk_steps(dt, in.sw, in.rsw);
-            in.t += in.w == 0 ? dt : (int32_t)(k * in.sw);
+            in.t += (int32_t)(k * in.sw);
             in.K += k;
         };
 
@@ -240,10 +240,11 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                     events(elig & (in.tb < now), now);
                     const bool full = in.w == in.B;
                     catch_up(elig & !full, now);
-                    uint32_t top = walk_smem[area + 32u + in.w], more = w1(in.row + 4u * in.w);
+                    uint32_t top = walk_smem[area + 32u + in.w];
+                    uint2 more = w2(in.row + 8u * in.w + 8u);
                     // distributor prediction (Sec. IV-F steps 2-3)
                     const int32_t t = full ? in.tb + (int32_t)in.sw : in.t;
-                    const bool ok = elig & lim.met((uint32_t)(t + pre - arrival), Sm1, Opt && !full ? more : in.stepB);
+                    const bool ok = elig & lim.met((uint32_t)(t + pre - arrival), Sm1, Opt && !full ? more.x : in.stepB);
                     // smallest (tier, predicted first token), lowest instance among equals
                     const uint32_t key = ok ? (full ? kTier1 : 0u) | (uint32_t)(t + pre) : kNone;
                     uint32_t best = min(key, __shfl_xor_sync(kWFull, key, 1));
@@ -266,7 +267,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                             events(mine, now);
                             win = win || mine;
                             top = walk_smem[area + 32u + in.w];
-                            more = w1(in.row + 4u * in.w);
+                            more = w2(in.row + 8u * in.w + 8u);
                         } else {
                             again = waits;
                             if (waits && tries >= kAttemptCap) { status = MAASO_CAND_ELOOP; again = false; }
@@ -309,7 +310,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
             // a group that has left the horizon, or ran out of rounds, is out
             const uint32_t out = __ballot_sync(kWFull, bad || status);
             if (out & gmask) {
-                in.tag = 0; in.w = 0; in.tb = kFar; in.kmin = kKeyEmpty; in.t = 0; in.sw = 1; now = 0;
+                in.tag = 0; in.w = 0; in.tb = kFar; in.kmin = kKeyEmpty; in.t = 0; in.sw = 1; in.rsw = ~0u; now = 0;
             }
         }
 
@@ -370,8 +371,7 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_c
     if (P.bucket_count[kPack4] + P.bucket_count[kPack8] == 0) return;
     const WalkLayout L = pack_layout(P.n_rows, P.n_classes);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
-    for (uint32_t i = tid; i < P.n_rows * 64u; i += 32u * Warps)
-        w1(L.steps + 4u * i) = (uint32_t)P.rows[(i >> 6) * kRowStride + 2 + (i & 63u)];
+    for (uint32_t i = tid; i < P.n_rows * 65u; i += 32u * Warps) w2(L.steps + 8u * i) = walk_step_entry(P, i);
     for (uint32_t c = tid; c < P.n_classes; c += 32u * Warps) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u], le = e < 0 ? (int64_t)1 << 62 : e;
         w4(L.lims + 16u * c) = make_uint4(a < 0 ? 0xFFFFFFFFu : (uint32_t)a, b < 0 ? 0xFFFFFFFFu : (uint32_t)b, lo32(le), hi32(le));

@@ -13,13 +13,15 @@ namespace maaso {
 constexpr int kWalkWarps = 16, kWalkWarpsFew = 12;
 constexpr int kWalkRing = 64;                     // ring entries per warp
 
+constexpr uint32_t kWalkRow = 65u * 8u;           // bytes of a decode-step row
+
 // One block: the completion rings, SLO limits, decode-step tables, the pool.
 struct WalkLayout {
     uint32_t ring;    // [warps][kWalkRing] {finish, first token, request, instance}; 64-bit times: {finish, first token}
     uint32_t ring_b;  // 64-bit times: [warps][kWalkRing] {request, instance}
     uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
     uint32_t wide;    // 64-bit times: [n_classes] {TTFT limit (2^62 = none), TBT limit (negative = none)}
-    uint32_t steps;   // [n_rows][64] u32
+    uint32_t steps;   // [n_rows][65] {decode step, 2^32 / step} by running count; a count of 0: {1, 2^32}, an idle clock
     uint32_t pool;
 };
 __host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes, bool wide, uint32_t warps) {
@@ -29,7 +31,7 @@ __host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_cl
     l.lims = l.ring_b + (wide ? warps * (uint32_t)kWalkRing * 8u : 0u);
     l.wide = l.lims + n_classes * 16u;
     l.steps = l.wide + (wide ? n_classes * 16u : 0u);
-    l.pool = (l.steps + n_rows * 256u + 127u) & ~127u;
+    l.pool = (l.steps + n_rows * kWalkRow + 127u) & ~127u;
     return l;
 }
 

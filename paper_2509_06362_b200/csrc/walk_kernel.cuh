@@ -77,15 +77,23 @@ __device__ __forceinline__ uint64_t warp_min(uint64_t v) {
     for (int o = 16; o > 0; o >>= 1) v = min(v, wshfl_xor(v, o));
     return v;
 }
-// ceil(dt / s) for 0 <= dt < 2^31 and a quotient below 2^16, rs a little below 1 / s (walk_rcp): the float estimate is at
-// most the true quotient, and less than one below it.
-__device__ __forceinline__ float walk_rcp(uint32_t s) { return rcp_approx((float)s) * (1.0f - 0x1p-20f); }
-__device__ __forceinline__ uint32_t walk_steps(int32_t dt, uint32_t s, float rs) {
-    const uint32_t q = (uint32_t)(__uint2float_rz((uint32_t)dt) * rs);
-    const uint32_t r = (uint32_t)dt - q * s;
-    return q + (r > 0u ? 1u : 0u) + (r > s ? 1u : 0u);
+// ceil(dt / s) for 0 <= dt < 2^31, s < 2^31, rs = (2^32 - 1) / s rounded down: the estimate is at most the quotient and less
+// than two below it, since rs > 2^32 / s - 1.
+__device__ __forceinline__ uint32_t walk_rcp(uint32_t s) { return 0xFFFFFFFFu / s; }
+__device__ __forceinline__ uint32_t walk_steps(int32_t dt, uint32_t s, uint32_t rs) {
+    const uint32_t d = (uint32_t)dt + s - 1u, q = __umulhi(d, rs);
+    return q + (d - q * s >= s ? 1u : 0u);
 }
-__device__ __forceinline__ uint32_t walk_steps(int64_t dt, uint32_t s, float rs) { return ceil_div_small(dt, s, rs); }
+__device__ __forceinline__ uint32_t walk_steps(int64_t dt, uint32_t s, uint32_t rs) {
+    const uint64_t d = (uint64_t)dt + (s - 1u);
+    return (d >> 32) == 0 ? walk_steps((int32_t)dt, s, rs) : (uint32_t)(d / s);
+}
+// Entry i of the decode-step rows in shared memory (WalkLayout::steps).
+__device__ __forceinline__ uint2 walk_step_entry(const EvalParams& P, uint32_t i) {
+    const uint32_t r = i / 65u, w = i - 65u * r;
+    const uint32_t s = w ? max((uint32_t)P.rows[r * kRowStride + 1u + w], 1u) : 1u;
+    return make_uint2(s, walk_rcp(s));
+}
 
 // Accounts the completion ring, one entry per lane and pass, into the lane's own sums in the region `base`:
 //   unit 0: sum and maximum of the time to first token; 1: of the end-to-end time; 2: last completion, checksum;
@@ -171,8 +179,8 @@ struct WInst {
     uint32_t K;    // decode steps done at t since the counter last restarted
     uint32_t kmin; // smallest slot key
     uint32_t w, B;
-    uint32_t sw;   // one decode step at the current level (valid while w > 0)
-    float rsw;     // 1 / sw
+    uint32_t sw;   // one decode step at the current level (1 while idle)
+    uint32_t rsw;  // 2^32 / sw
     uint32_t tag;  // 1 << model (0 for a lane without an instance) | place in the placement as given << 16
     uint32_t area, keys, row;  // byte offsets of its slots, of its first block of keys and of its decode-step row
     uint32_t pre_base, pre_q16, stepB;
@@ -234,7 +242,7 @@ struct Walk {
             u[3] = make_uint4(e.y, e.z, e.w, 0u);
         }
         memcpy(&in, u, sizeof(Inst));
-        if (!Wide && Opt) in.stepB = w1(in.row + 4u * in.B - 4u);
+        if (!Wide && Opt) in.stepB = w1(in.row + 8u * in.B);
     }
 
     // One warp takes the placements of a bucket, one after the other.  `base`: its part of shared memory;
@@ -288,7 +296,7 @@ struct Walk {
                 __syncwarp();
                 for (uint32_t s = 0; s < (Big ? n_i : 1u); s += 32u) {
                     const uint32_t j = s + lane, at = ents + 16u * j;
-                    in.t = 0; in.tb = kFar; in.K = 0; in.kmin = kKeyEmpty; in.w = 0; in.B = 1; in.sw = 1; in.rsw = 1.0f;
+                    in.t = 0; in.tb = kFar; in.K = 0; in.kmin = kKeyEmpty; in.w = 0; in.B = 1; in.sw = 1; in.rsw = ~0u;
                     in.pre_base = in.pre_q16 = 0; in.stepB = 1; in.tag = 0; in.area = in.keys = in.pay = in.row = L.steps;
                     uint32_t nblk = 0;
                     if (j < n_i) {
@@ -297,15 +305,15 @@ struct Walk {
                         in.tag = (1u << md) | (e.y << 16);
                         in.B = (e.x >> 12) & 0xFFu;
                         nblk = (in.B + 7u) >> 3;
-                        in.row = L.steps + r * 256u;
+                        in.row = L.steps + r * kWalkRow;
                         in.pre_base = (uint32_t)P.rows[r * kRowStride];
                         in.pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
-                        in.stepB = w1(in.row + 4u * in.B - 4u);
+                        in.stepB = w1(in.row + 8u * in.B);
                         // the smallest step a prediction can use: the step at the batch cap, or (optimistic estimate) at any
                         // level up to it
                         uint32_t ms = in.stepB;
                         if (Opt)
-                            for (uint32_t w = 0; w + 1u < in.B; w++) ms = min(ms, w1(in.row + 4u * w));
+                            for (uint32_t w = 1; w < in.B; w++) ms = min(ms, w1(in.row + 8u * w));
                         atomicMin(&w1(models + 16u * md), in.pre_base);
                         atomicMin(&w1(models + 16u * md + 4u), ms);
                         // per instance: earliest start, prefill base and slope, smallest prediction step
@@ -376,9 +384,10 @@ struct Walk {
             // when the instance could start a request
             auto start = [&]() -> T { return kFixed ? (in.w == in.B ? in.tb : now) : (in.w == in.B ? in.tb + (T)in.sw : in.t); };
             // Step `sw` and next completion `left` steps after in.t >= 0; flags what leaves the horizon.
-            auto next_end = [&](uint32_t left, bool busy, uint32_t sw) {
+            auto next_end = [&](uint32_t left, bool busy, uint2 step) {
+                const uint32_t sw = step.x;
                 in.sw = sw;
-                in.rsw = Wide ? rcp_approx((float)sw) : walk_rcp(sw);
+                in.rsw = step.y;
                 if constexpr (Wide) {
                     in.tb = busy ? in.t + (int64_t)((uint64_t)left * sw) - (int64_t)sw : kFar;
                 } else {
@@ -418,9 +427,12 @@ struct Walk {
                         if (ring_n + adds > kCap) flush();
                         if (due) {
                             const uint32_t slot = in.kmin & 63u;
-                            const uint32_t k8 = in.keys + 4u * slot, kb = in.keys + 4u * (slot & 56u);
+                            const uint32_t k8 = in.keys + 4u * slot, kb = in.keys + 4u * (slot & 56u), mb = in.area + ((slot >> 3) << 2);
+                            // (the key and its block's minimum go first: what is left is read without them)
+                            w1(k8) = kKeyEmpty;
+                            w1(mb) = kKeyEmpty;
                             const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(in.area), m1 = w4(in.area + 16u);
-                            const uint32_t sw = w1(in.row + 4u * in.w - 8u);  // (the word before the row, if that was the last one)
+                            const uint2 step = w2(in.row + 8u * in.w - 8u);
                             uint2 run;  // first token, request; 64-bit times: first token
                             uint32_t rq = 0;
                             if constexpr (kAway) run = __ldcg(reinterpret_cast<const uint2*>(away + 2u * (k8 - L.pool)));
@@ -430,10 +442,8 @@ struct Walk {
                             in.K = in.kmin >> 6;
                             in.w--;
                             walk_smem[in.area + 32u + in.w] = (unsigned char)slot;
-                            // the smallest of the other keys: keys are unique, so the retired one wraps to all ones
-                            const uint32_t km = in.kmin + 1u;
-                            const uint32_t kv[8] = {k0.x - km, k0.y - km, k0.z - km, k0.w - km, k1.x - km, k1.y - km, k1.z - km, k1.w - km};
-                            const uint32_t mv[8] = {m0.x - km, m0.y - km, m0.z - km, m0.w - km, m1.x - km, m1.y - km, m1.z - km, m1.w - km};
+                            const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                            const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
                             const uint32_t bmin = min8(kv);
                             const uint32_t e = ring_n + (uint32_t)__popc(dm & below);
                             if constexpr (Wide) {
@@ -442,12 +452,11 @@ struct Walk {
                             } else {
                                 w4(ring + 16u * e) = make_uint4((uint32_t)in.t, run.x, run.y, in.tag >> 16);
                             }
-                            w1(k8) = kKeyEmpty;
-                            w1(in.area + ((slot >> 3) << 2)) = bmin + km;
-                            in.kmin = min(bmin, min8(mv)) + km;
+                            w1(mb) = bmin;
+                            in.kmin = min(bmin, min8(mv));
                             const uint32_t left = (in.kmin >> 6) - in.K;
                             const bool busy = in.w > 0;
-                            next_end(left, busy, sw);
+                            next_end(left, busy, step);
                             due = busy & ((left == 0u) | (in.tb < upto)) & !bad;
                         }
                         ring_n += adds;
@@ -467,16 +476,17 @@ struct Walk {
                 } else {
                     const int32_t dt = go ? max(upto - in.t, 0) : 0;
                     const uint32_t k = walk_steps(dt, in.sw, in.rsw);
-                    in.t += in.w == 0 ? dt : (int32_t)(k * in.sw);
+                    in.t += (int32_t)(k * in.sw);
                     in.K += k;
                 }
             };
             // The next free slot and the step with one request more, read ahead of the choice.
-            uint32_t top = 0, more = 0;
+            uint32_t top = 0;
+            uint2 more = make_uint2(0u, 0u);
             auto peek = [&]() {
                 if (!kFixed) {
                     top = walk_smem[in.area + 32u + in.w];
-                    more = w1(in.row + 4u * in.w);
+                    more = w2(in.row + 8u * in.w + 8u);
                 }
             };
             // One request's times into the ring (`e`: its entry).
@@ -506,7 +516,7 @@ struct Walk {
                         level -= (uint32_t)(__popc(__ballot_sync(kWFull, v[0] == tb)) + __popc(__ballot_sync(kWFull, v[1] == tb)));
                         first = in.tb + pre;
                     }
-                    const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? 4u * level : 0u));
+                    const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? 8u * level : 0u) + 8u);
                     T fin = first + (T)span;
                     if (win) {
                         if constexpr (Wide) {
@@ -688,7 +698,7 @@ struct Walk {
                             // distributor prediction (Sec. IV-F steps 2-3)
                             const T t = start();
                             uint32_t sB = in.stepB;
-                            if (Opt && !full) sB = kFixed ? w1(in.row + 4u * in.w) : more;
+                            if (Opt && !full) sB = kFixed ? w1(in.row + 8u * in.w + 8u) : more.x;
                             const bool ok = elig && lim.met((U)(t + p - arrival), Sm1, sB);
                             // smallest (tier, predicted first token >= now >= 0), lowest instance among equals
                             const U k = ok ? (full ? kTier1 : (U)0) | (U)(t + p) : kNone;
@@ -835,8 +845,7 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
     if (any == 0) return;
     const WalkLayout L = walk_layout(P.n_rows, P.n_classes, Wide, Warps);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
-    for (uint32_t i = tid; i < P.n_rows * 64u; i += (32 * Warps))
-        w1(L.steps + 4u * i) = (uint32_t)P.rows[(i >> 6) * kRowStride + 2 + (i & 63u)];
+    for (uint32_t i = tid; i < P.n_rows * 65u; i += (32 * Warps)) w2(L.steps + 8u * i) = walk_step_entry(P, i);
     for (uint32_t c = tid; c < P.n_classes; c += (32 * Warps)) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u];
         const int64_t none = (int64_t)1 << 62, le = e < 0 ? none : e;
