@@ -638,7 +638,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         may_leave = may_leave && !queues;
         P.walk_bytes = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, true, kWalkWarps).pool) / kWalkWarps) & ~15u;
         P.walk_warps = (uint64_t)C * n_traces <= 3ull * ctx->sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
-        P.walk_usual = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, queues, P.walk_warps).pool) / P.walk_warps) & ~15u;
+        P.walk_usual = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, queues, P.walk_warps, !(o.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES))).pool) / P.walk_warps) & ~15u;
     }
     const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;

@@ -14,6 +14,7 @@ constexpr int kWalkWarps = 16, kWalkWarpsFew = 12;
 constexpr int kWalkRing = 64;                     // ring entries per warp
 
 constexpr uint32_t kWalkRow = 65u * 8u;           // bytes of a decode-step row
+constexpr uint32_t kWalkList = 33u * 32u + 128u;  // list of 32 requests and one behind it, what lanes without an instance read
 
 // One block: the completion rings, SLO limits, decode-step tables, the pool.
 struct WalkLayout {
@@ -22,16 +23,18 @@ struct WalkLayout {
     uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
     uint32_t wide;    // 64-bit times: [n_classes] {TTFT limit (2^62 = none), TBT limit (negative = none)}
     uint32_t steps;   // [n_rows][65] {decode step, 2^32 / step} by running count; a count of 0: {1, 2^32}, an idle clock
+    uint32_t list;    // `list`: [warps][kWalkList], requests that need a round, and the dummy region (walk_dynamic.cuh)
     uint32_t pool;
 };
-__host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes, bool wide, uint32_t warps) {
+__host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes, bool wide, uint32_t warps, bool list = false) {
     WalkLayout l;
     l.ring = 0;
     l.ring_b = warps * (uint32_t)kWalkRing * 16u;
     l.lims = l.ring_b + (wide ? warps * (uint32_t)kWalkRing * 8u : 0u);
     l.wide = l.lims + n_classes * 16u;
     l.steps = l.wide + (wide ? n_classes * 16u : 0u);
-    l.pool = (l.steps + n_rows * kWalkRow + 127u) & ~127u;
+    l.list = (l.steps + n_rows * kWalkRow + 15u) & ~15u;
+    l.pool = (l.list + (list ? warps * kWalkList : 0u) + 127u) & ~127u;
     return l;
 }
 
@@ -47,11 +50,12 @@ constexpr uint32_t kWalkLaneSums = 4u * 32u * 16u;
 constexpr uint32_t kWalkSums = kWalkLaneSums + 48u;
 constexpr uint32_t kWalkBig = 32u;  // more instances than this rest in shared memory
 __host__ __device__ inline uint32_t walk_slots_at(uint32_t nblk) { return 32u + ((8u * nblk + 15u) & ~15u); }
-// `block`: bytes of 8 slots
+// `block`: bytes of 8 slots; kWalkBlock: {keys, what the running requests must remember} by block, from a fixed offset on
+constexpr uint32_t kWalkKeys = 96u;
 constexpr uint32_t kWalkBlock = 96u, kWalkBlockLong = 128u, kWalkBlockKeys = 32u;
 __host__ __device__ inline uint32_t walk_slot_bytes(uint32_t b, bool fixed_speed, uint32_t key_bytes, uint32_t block) {
     const uint32_t nblk = (b + 7u) >> 3;
-    return fixed_speed ? ((b * key_bytes + 15u) & ~15u) : walk_slots_at(nblk) + nblk * block;
+    return fixed_speed ? ((b * key_bytes + 15u) & ~15u) : (block == kWalkBlock ? kWalkKeys : walk_slots_at(nblk)) + nblk * block;
 }
 __host__ __device__ inline uint32_t walk_rest_bytes(WalkKind kind) { return kind == kWalkUsual ? 0u : (kind == kWalkBigKind ? 48u : 80u); }
 __host__ __device__ inline uint32_t walk_region_bytes(uint32_t n_models, uint32_t n_inst, uint32_t slot_bytes, WalkKind kind) {

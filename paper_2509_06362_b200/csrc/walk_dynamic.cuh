@@ -1,0 +1,530 @@
+// Walking kernel's body for the engine whose decode speed follows the running count, placements of at most 32 instances,
+// 32-bit times: what nearly every call runs.  Same scan and same round as Walk (walk_kernel.cuh), written for the shortest chain.
+//
+// What bounds it: the chain of rounds of the longest placements, each instruction waited for in turn (5 to 6 cycles for an
+// addition, 13 more where a comparison is waited for, 18 for a warp-wide minimum, 30 for shared memory or a shuffle, 36 for
+// finding a lowest bit, 20 to 40 for a vote and its branch: clock() around chains of each), and over a large batch the ALU
+// pipe, which takes a warp instruction every second cycle.  So
+//   - the scan leaves a list of the requests that need a round, with what a round needs of them, in shared memory, and a round
+//     reads the next entry ahead: no bit search, no shuffles, no limits to look up;
+//   - everything an admission needs is there before the choice: next free slot, its block's minimum, the step with one
+//     request more;
+//   - the choice's key names the lane: one minimum and one comparison;
+//   - the usual path shares no value with the uncommon ones (what merged with them cost 30 instructions a round);
+//   - a wait is one operation on the winner's slots: the request takes over the slot that frees;
+//   - a step count is a high product and a shift (exact reciprocals), without a correction;
+//   - chunks that need no round are skipped in a loop of their own;
+//   - shared memory is addressed directly (5 % against references into the block's array).
+// Measured against the body that it replaced here (that of Walk): warp instructions of a round that admits 189 -> 160, with a
+// completion before 286 -> 246, with a wait 304 -> 190; 2,000 x 17,000 of the paper's shape 8.9 -> 6.8 ms, one node's 10,864 x
+// 10,000 6.4 -> 4.9, three models under load 12,000 x 30,000 4.51 -> 4.35, masked sub-clusters 9,000 x 12,000 18.3 -> 16.3.
+// Dropped: completions and admissions without a branch, lanes that have none writing to a dummy region (a lone warp as fast,
+// +5 % instructions); the accounting of completions inlined (+7 %).
+#pragma once
+
+namespace maaso {
+
+// ceil(dt / s) = (2 (dt + s - 1) m >> 32) >> L with L = ceil(log2 s), m = ceil(2^(31 + L) / s) < 2^32: exact for dt + s - 1 <
+// 2^31 (m s - 2^(31 + L) < s <= 2^L; Granlund and Montgomery's division by an invariant).  A row's entry: {s << 5 | L, m}.
+__device__ __forceinline__ uint2 walk_exact_entry(const EvalParams& P, uint32_t i) {
+    const uint32_t r = i / 65u, w = i - 65u * r;
+    const uint32_t s = w ? max((uint32_t)P.rows[r * kRowStride + 1u + w], 1u) : 1u;
+    const uint32_t sh = s > 1u ? 32u - (uint32_t)__clz((int)(s - 1u)) : 0u;
+    return make_uint2((s << 5) | sh, (uint32_t)((((uint64_t)1 << (31u + sh)) + (s - 1u)) / s));
+}
+
+// A load that stays where it is written, ahead of what it is for (the compiler moves a plain one down to its use).
+__device__ __forceinline__ uint4 load_ahead(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
+// Shared memory by its own 32-bit addresses (the layout's offsets with the base of the block's part added).
+__device__ __forceinline__ uint4 ld4(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint2 ld2(uint32_t a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld1(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t ldb(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void st4(uint32_t a, const uint4& v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void st2(uint32_t a, const uint2& v) {
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void st1(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void stb(uint32_t a, uint32_t v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void min_shared(uint32_t a, uint32_t v) { asm volatile("red.shared.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+
+template <bool Opt>
+struct WalkDynamic {
+    using Limits = typename Walk<Opt, 0, false, false>::Limits;
+    static constexpr int32_t kFar = kWalkFar;
+    // A key: tier << 31 | (predicted first token - now, at most kOffMax) << 5 | lane.  From kOffMax on (a minute ahead) the
+    // offsets are compared in full.
+    static constexpr uint32_t kTier1 = 1u << 31, kNone = ~0u, kOffMax = (1u << 26) - 2u, kFast = kOffMax << 5;
+    static constexpr uint32_t kRoom = 32u;         // the ring is accounted when it has as many entries: one iteration adds up to 32
+
+    static __device__ __forceinline__ void bucket(const EvalParams& P, const WalkLayout& L0, int bucket, uint32_t base0,
+                                                  uint32_t static_idx, uint32_t static_total, unsigned char*) {
+        const uint32_t smem = smem_addr(walk_smem), base = base0 + smem;
+        WalkLayout L = L0;
+        L.ring += smem; L.lims += smem; L.steps += smem; L.list += smem;
+        const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, below = (1u << lane) - 1u;
+        const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
+        const uint32_t total = P.bucket_count[bucket] * n_traces;
+        const uint32_t ring = L.ring + warp * kWalkRing * 16u, list = L.list + warp * kWalkList, dummy = list + 33u * 32u;
+        const bool use_mask = P.class_mask != nullptr && P.n_classes <= 32;
+        const uint32_t models = base + kWalkSums, ents = models + 16u * P.n_models;
+
+        uint32_t idx = static_idx;
+        while (idx < total) {
+            // ---- the next placement ------------------------------------------------------------------------
+            const uint32_t tr = idx % n_traces;
+            const uint32_t cand = P.bucket_list[(size_t)bucket * P.n_cand + idx / n_traces];
+            const uint4* const reqs = P.trace_reqs[tr];
+            const uint32_t n_req = P.trace_n[tr];
+            uint4 nxt = make_uint4(0u, 0u, 0u, 0u);  // the lane's request of the next chunk, as loaded
+            if (n_req) nxt = __ldg(reqs + min(lane, n_req - 1u));
+            const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
+            // this lane's instance (see WInst)
+            int32_t t = 0, tb = kFar;
+            uint32_t K = 0, kmin = kKeyEmpty, w = 0, B = 1, tag = 0, area = dummy, row = L.steps, pre_base = 0, pre_q16 = 0, stepB = 1;
+            uint32_t ent = dummy + 96u;
+            {
+                for (uint32_t i = lane; i < kWalkSums / 16u; i += 32u) st4(base + 16u * i, make_uint4(0u, 0u, 0u, 0u));
+                // instances sorted by model, in their given order within a model (the order in which ties are broken)
+                const uint32_t word = lane < n_i ? P.inst[lo + lane] : 0xFu, m = lane < n_i ? word & 0xFu : 0xFFFFFFFFu;
+                uint32_t before = 0;
+                for (uint32_t k = 0; k < P.n_models; k++) {
+                    const uint32_t b = __ballot_sync(kWFull, m == k), n = (uint32_t)__popc(b);
+                    if (m == k) st2(ents + 16u * (before + (uint32_t)__popc(b & below)), make_uint2(word, lane));
+                    // per model: smallest prefill base, smallest prediction step, its instances (byte offsets of their entries)
+                    if (lane == k) st4(models + 16u * k, make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, ents + 16u * before, ents + 16u * (before + n)));
+                    before += n;
+                }
+                __syncwarp();
+                uint32_t bytes = 0;
+                if (lane < n_i) {
+                    ent = ents + 16u * lane;
+                    const uint2 e = ld2(ent);
+                    const uint32_t md = e.x & 0xFu, r = md * P.n_strategies + ((e.x >> 4) & 0xFFu);
+                    tag = (1u << md) | (e.y << 16);
+                    B = (e.x >> 12) & 0xFFu;
+                    row = L.steps + r * kWalkRow;
+                    pre_base = (uint32_t)P.rows[r * kRowStride];
+                    pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
+                    stepB = ld1(row + 8u * B) >> 5;
+                    // the smallest step a prediction can use: the step at the batch cap, or (optimistic estimate) at any
+                    // level up to it
+                    uint32_t ms = stepB;
+                    if (Opt)
+                        for (uint32_t l = 1; l < B; l++) ms = min(ms, ld1(row + 8u * l) >> 5);
+                    min_shared(models + 16u * md, pre_base);
+                    min_shared(models + 16u * md + 4u, ms);
+                    // per instance: earliest start, prefill base and slope, smallest prediction step
+                    st4(ent, make_uint4(0u, pre_base, pre_q16, ms));
+                    bytes = walk_slot_bytes(B, false, 4u, kWalkBlock);
+                }
+                uint32_t incl = bytes;
+                for (uint32_t o = 1; o < 32u; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(kWFull, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                if (bytes) {
+                    area = ents + 16u * n_i + incl - bytes;
+                    for (uint32_t i = 0; i < 8u; i++) st1(area + 4u * i, kKeyEmpty);
+                    for (uint32_t i = 0; i < ((B + 7u) & ~7u); i++) st1(area + kWalkKeys + (i >> 3) * kWalkBlock + 4u * (i & 7u), kKeyEmpty);
+                    for (uint32_t i = 0; i < B; i++) stb(area + 32u + i, i);
+                }
+            }
+            uint32_t hasmodel = 0;
+            for (uint32_t k = 0; k < P.n_models; k++) {
+                const uint2 r = ld2(models + 16u * k + 8u);
+                hasmodel |= r.x < r.y ? 1u << k : 0u;
+            }
+            const uint32_t cmask = use_mask ? P.class_mask[cand] : 0xFFFFFFFFu;
+            const bool side = P.rej_by_model != nullptr || (P.dump_row && P.dump_row[cand] >= 0);
+            __syncwarp();
+
+            uint32_t step = 32u, rcp = 0x80000000u;  // entry of the current level (0: an idle clock)
+            // the next free slot, its block's smallest key, the entry of one request more
+            uint32_t top = 0, top_min = 0;
+            uint2 more = make_uint2(0u, 0u);
+            uint32_t ring_n = 0, status = 0, extra = 0;  // extra: distributor rounds beyond one per request
+            int64_t epoch = 0;
+            int32_t now = 0;
+            bool bad = false;               // a time of this lane has left the horizon: nothing is asked of it any more (see Walk)
+            int32_t rel = 0;                // this lane's request of the chunk: arrival,
+            uint32_t c_in = 0, c_meta = 0;  // input tokens, output tokens | class | model
+
+            auto flush = [&]() {
+                walk_account<false>(P, P.dump_row || P.ttft_hist, tr * P.n_cand + cand, base0, ring - smem, 0u, ring_n, epoch, L0.lims, 0u, reqs);
+                ring_n = 0;
+            };
+            auto take_chunk = [&](const uint4& v) {
+                const int64_t d = i64_of(v.x, v.y) - epoch;
+                rel = d >= (int64_t)kWalkNowMax ? kFar : (d < (int64_t)kWPast ? kWPast : (int32_t)d);
+                c_in = v.z;
+                c_meta = v.w;
+            };
+            auto peek = [&]() {
+                more = ld2(row + 8u * w + 8u);
+                top = ldb(area + 32u + w) & 63u;
+                top_min = ld1(area + ((top >> 1) & 28u));
+            };
+            peek();
+            // The next completion, counted from the clock; flags what leaves the horizon.
+            auto next_end = [&](bool busy) {
+                const uint64_t tc = (uint64_t)((kmin >> 6) - K) * (step >> 5) + (uint32_t)t;
+                tb = busy ? (int32_t)((uint32_t)tc - (step >> 5)) : kFar;
+                bad = bad | (busy & (tc > (uint64_t)kWalkHorizon));
+            };
+            // One completion in each of the lanes in `due` (their set: `dm`); then whether another one is due.
+            // `stay`: at the time `now`, while the clock is already beyond it (see the wait).
+            auto retire = [&](bool due, uint32_t dm, int32_t upto, bool stay) -> bool {
+                if (due) {
+                    const uint32_t s = kmin & 63u, kb = area + kWalkKeys + (s >> 3) * kWalkBlock, k8 = kb + 4u * (s & 7u), mb = area + 4u * (s >> 3);
+                    // (the key and its block's minimum go first: what is left is read without them)
+                    st1(k8, kKeyEmpty);
+                    st1(mb, kKeyEmpty);
+                    const uint4 k0 = ld4(kb), k1 = ld4(kb + 16u), m0 = ld4(area), m1 = ld4(area + 16u);
+                    const uint2 cur = ld2(row + 8u * w - 8u), run = ld2(kb + 32u + 8u * (s & 7u));
+                    const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                    const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                    const int32_t fin = stay ? now : tb + (int32_t)(step >> 5);
+                    if (!stay) {
+                        t = fin;
+                        K = kmin >> 6;
+                    }
+                    w--;
+                    stb(area + 32u + w, s);
+                    st4(ring + 16u * (ring_n + (uint32_t)__popc(dm & below)), make_uint4((uint32_t)fin, run.x, run.y, tag >> 16));
+                    top = s;
+                    more = make_uint2(step, rcp);
+                    step = cur.x;
+                    rcp = cur.y;
+                    top_min = min8(kv);
+                    st1(mb, top_min);
+                    kmin = min(top_min, min8(mv));
+                    const bool busy = w > 0u;
+                    next_end(busy);
+                    due = busy & (((kmin >> 6) == K) | (!stay & (tb < upto))) & !bad;
+                }
+                return due;
+            };
+            // Completions of the lanes in `due` until every clock has reached `upto`.  (`w` of a lane that is due is not 0.)
+            auto events = [&](bool due, int32_t upto) {
+                uint32_t dm = __ballot_sync(kWFull, due);
+                while (dm) {
+                    if (ring_n >= kRoom) flush();
+                    due = retire(due, dm, upto, false);
+                    ring_n += (uint32_t)__popc(dm);
+                    dm = __ballot_sync(kWFull, due);
+                }
+            };
+            // Decode steps until `dt` later; 2 (dt + step - 1) < 2^32.
+            auto steps_of = [&](int32_t dt) -> uint32_t {
+                return __funnelshift_r(__umulhi(2u * ((uint32_t)dt + (step >> 5) - 1u), rcp), 0u, step);
+            };
+            auto start = [&]() -> int32_t { return w == B ? tb + (int32_t)(step >> 5) : t; };
+            // What is rare, out of the rounds' way.  Moves the epoch for request `src` of the chunk at `cb`, to the dispatcher's
+            // clock (or to the request's arrival, if that is later): what happens before it is simulated, everything else is
+            // measured from there on.
+            auto move_epoch = [&](uint32_t cb, uint32_t src) {
+                const uint4 v = __ldg(reqs + cb + src);
+                const int64_t to = max(epoch + now, i64_of(v.x, v.y));
+                const int32_t up = to - epoch >= (int64_t)kFar ? kFar : (int32_t)(to - epoch);  // (cut off only if all is idle by then)
+                events(w > 0 && tb < up && !bad, up);
+                if (w == 0) {
+                    t = t > up ? t - up : 0;  // an idle instance is where the dispatcher is
+                } else {
+                    if (w < B && t < up) {
+                        const uint32_t k = steps_of(up - t);
+                        t += (int32_t)(k * (step >> 5));
+                        K += k;
+                    }
+                    t = t > up + kWPast ? t - up : kWPast;  // a full instance's clock is not looked at
+                    tb -= up;
+                    // running requests' first tokens (further back than 32 bits reach: the lane has left the horizon)
+                    for (uint32_t i = 0; i < B; i++) {
+                        const uint32_t kb = area + kWalkKeys + (i >> 3) * kWalkBlock;
+                        if (ld1(kb + 4u * (i & 7u)) == kKeyEmpty) continue;
+                        const int64_t f = (int64_t)(int32_t)ld1(kb + 32u + 8u * (i & 7u)) - up;
+                        bad = bad || f < -(int64_t)kFar;
+                        st1(kb + 32u + 8u * (i & 7u), (int32_t)f);
+                    }
+                }
+                st1(ent, (uint32_t)start());
+                flush();
+                epoch = to;
+                now = 0;
+                take_chunk(__ldg(reqs + min(cb + lane, n_req - 1u)));
+                __syncwarp();
+            };
+
+            uint32_t cb = 0;  // the chunk
+            auto counted = [&]() { return cb + lane < n_req && ((cmask >> ((c_meta >> 16) & 31u)) & 1u); };
+            // Which of the chunk's requests from lane `from` on may need the distributor.
+            auto test = [&](uint32_t from) -> uint32_t {
+                const uint32_t Sm1 = (c_meta & 0xFFFFu) - 1u, model = c_meta >> 24;
+                const int32_t at = max(now, rel);
+                bool live = (lane >= from) & counted() & ((hasmodel >> model) & 1u);
+                // (without a branch: every lane has a request, behind the last one the last one once more)
+                const uint4 me = ld4(models + 16u * model);
+                Limits lim;
+                lim.a = ld4(L.lims + ((c_meta >> 12) & 0xFF0u));
+                live = live & lim.met((uint32_t)(at - rel) + me.x, Sm1, me.y);  // earliest first token, since the arrival
+                const uint32_t first = __ballot_sync(kWFull, live);
+                if (first == 0u) return 0u;
+                // each instance of the model by itself: its start time at the latest look at it, its prefill of this
+                // request, its step
+                bool ok = rel == kFar;
+                uint32_t j = live ? me.z : 0u;
+                const uint32_t j_end = live ? me.w : 0u;
+                while (__any_sync(kWFull, j < j_end && !ok)) {
+                    const uint4 e = ld4(j < j_end ? j : ents);  // (no branch)
+                    const uint32_t since = (uint32_t)(max(at, (int32_t)e.x) - rel) + (uint32_t)Walk<Opt, 0, false, false>::prefill(e.y, e.z, c_in);
+                    ok = ok | ((j < j_end) & lim.met(since, Sm1, e.w));
+                    j += 16u;
+                }
+                return __ballot_sync(kWFull, live && ok);
+            };
+            auto report = [&](uint32_t served, uint32_t end) {
+                if (lane < end && counted() && !((served >> lane) & 1u)) walk_reject_side(P, tr * P.n_cand + cand, cb + lane, c_meta >> 24);
+            };
+
+            for (;; cb += 32u) {
+                uint32_t live = 0;
+                for (; cb < n_req; cb += 32u) {  // (a loop of its own: under load most chunks need no round)
+                    take_chunk(nxt);
+                    nxt = load_ahead(reqs + min(cb + 32u + lane, n_req - 1u));
+                    live = test(0u);
+                    if (live) break;
+                    if (side) report(0u, 32u);
+                }
+                if (cb >= n_req) break;
+                uint32_t from = 0, served = 0, end = 32u;  // `end`: where a failed placement stops
+                do {
+                    // The list of requests that need a round, up to one that is out of the epoch's reach; what the keys need room
+                    // for (an end index is at most 2^16 beyond one before it).
+                    const uint32_t far = __ballot_sync(kWFull, max(now, rel) >= kWalkNowMax) & live;
+                    if (__any_sync(kWFull, (w > 0) & (K > kRelMax - (40u << 16)))) {
+                        if (w > 0) {
+                            const uint32_t d = K << 6;
+                            for (uint32_t i = 0; i < 8u + ((B + 7u) & ~7u); i++) {
+                                const uint32_t at = i < 8u ? area + 4u * i : area + kWalkKeys + ((i - 8u) >> 3) * kWalkBlock + 4u * (i & 7u);
+                                const uint32_t k = ld1(at);
+                                if (k != kKeyEmpty) st1(at, k - d);
+                            }
+                            if (kmin != kKeyEmpty) kmin -= d;
+                            peek();
+                        }
+                        K = 0;
+                    }
+                    if (far) live &= (far & (0u - far)) - 1u;
+                    uint32_t n = (uint32_t)__popc(live);
+                    if ((live >> lane) & 1u) {
+                        // {arrival, input tokens, output tokens - 1 | model << 16 | lane << 24, keys below this take the usual path}
+                        // {bound of the first token after the arrival, of the step, of the end + 1, output tokens - 1 as far as that bound goes}
+                        const uint32_t out = c_meta & 0xFFFFu, at = list + 32u * (uint32_t)__popc(live & below);
+                        const uint4 l = ld4(L.lims + ((c_meta >> 12) & 0xFF0u));
+                        const bool endless = (l.w >> 30) != 0u;
+                        st4(at, make_uint4((uint32_t)rel, c_in, (out - 1u) | ((c_meta >> 24) << 16) | (lane << 24), out == 1u ? 0u : kFast));
+                        st4(at + 16u, make_uint4(min(l.x, 0xFFFFFFFEu) + 1u, out == 1u ? 0xFFFFFFFFu : l.y, endless ? 0xFFFFFFFFu : l.z + 1u, endless ? 0u : out - 1u));
+                    }
+                    __syncwarp();
+                    bool move = far != 0u;
+                    from = move ? (uint32_t)__ffs((int)far) - 1u : 32u;  // where the next pass over the chunk starts
+                    uint32_t i = 0;
+                    uint4 q = ld4(list), lim = ld4(list + 16u);  // the request of this round, its limits
+                    uint32_t tries = 0;
+                    while (i < n) {
+                        const uint4 qn = ld4(list + 32u * i + 32u), ln = ld4(list + 32u * i + 48u);
+                        const int32_t arrival = (int32_t)q.x;
+                        const uint32_t Sm1 = q.z & 0xFFFFu, req = cb + (q.z >> 24);
+                        now = max(now, arrival);  // pending time: the dispatcher never goes back
+                        const bool elig = (((tag >> ((q.z >> 16) & 15u)) & 1u) != 0u) & !bad;
+                        const int32_t pre = (int32_t)(pre_base + (uint32_t)(((uint64_t)pre_q16 * q.y + 32768u) >> 16));
+                        // "reduce": what completes before the instance's clock reaches `now`
+                        bool due = elig & (tb < now);
+                        uint32_t dm = __ballot_sync(kWFull, due);
+                        while (dm) {
+                            due = retire(due, dm, now, false);
+                            ring_n += (uint32_t)__popc(dm);
+                            dm = __ballot_sync(kWFull, due);
+                            if (ring_n >= kRoom) flush();
+                        }
+                        const bool full = w == B;
+                        {
+                            const uint32_t k = steps_of(elig & !full ? max(now - t, 0) : 0);
+                            t += (int32_t)(k * (step >> 5));
+                            K += k;
+                        }
+                        // distributor prediction (Sec. IV-F steps 2-3): the bound that the class and the step put on the first token
+                        const uint32_t sB = Opt && !full ? more.x >> 5 : stepB;
+                        const int64_t left = (int64_t)lim.z - (int64_t)((uint64_t)lim.w * sB);
+                        const uint32_t bound = min(lim.x, lo32(left) & ~(uint32_t)((int32_t)hi32(left) >> 31));
+                        const int32_t t0 = full ? tb + (int32_t)(step >> 5) : t, first = t0 + pre;
+                        const bool ok = elig & (sB <= lim.y) & ((uint32_t)(first - arrival) < bound);
+                        // smallest (tier, predicted first token >= now), lowest instance among equals
+                        const uint32_t key = ok ? (min((uint32_t)(first - now), kOffMax) << 5) + (full ? lane + kTier1 : lane) : kNone;
+                        const uint32_t best = __reduce_min_sync(kWFull, key);
+                        if (best < q.w) {
+                            // "map": prefill at the step boundary (running decodes stall), then occupy a free slot
+                            if (key == best) {
+                                const uint32_t kb = area + kWalkKeys + (top >> 3) * kWalkBlock, nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
+                                st1(kb + 4u * (top & 7u), nk);
+                                st2(kb + 32u + 8u * (top & 7u), make_uint2((uint32_t)first, req));
+                                st1(area + 4u * (top >> 3), min(top_min, nk));
+                                t = first;
+                                K = nK;
+                                kmin = min(kmin, nk);
+                                w++;
+                                step = more.x;
+                                rcp = more.y;
+                                next_end(true);
+                            }
+                            peek();
+                        } else if (best == kNone) {
+                            // overflow protection: nobody can meet the deadline.  What the scan went by is out of date: once more
+                            from = (q.z >> 24) + 1u;
+                            move = false;
+                            break;
+                        } else {
+                            const bool waits = best >= kTier1;
+                            uint32_t wl = best & 31u;  // the winner's lane
+                            if (((best >> 5) & 0x3FFFFFFu) == kOffMax) {  // more than a minute ahead: compared in full
+                                const uint32_t k = ok & (full == waits) ? (uint32_t)first : kNone, b = __reduce_min_sync(kWFull, k);
+                                wl = (uint32_t)__ffs((int)__ballot_sync(kWFull, k == b)) - 1u;
+                            }
+                            const bool win = lane == wl;
+                            if (waits) {
+                                // every capable instance is full: wait until the chosen slot frees
+                                now = __shfl_sync(kWFull, t0, (int)wl);
+                                extra++;
+                                if (Opt || q.w == 0u) {  // a new choice
+                                    if (Opt && ++tries >= kAttemptCap) {
+                                        status = MAASO_CAND_ELOOP;
+                                        from = end = q.z >> 24;
+                                        break;
+                                    }
+                                    if (now >= kWalkNowMax) {  // (for the same request)
+                                        from = q.z >> 24;
+                                        move = true;
+                                        break;
+                                    }
+                                    continue;
+                                }
+                                // With the worst-case estimate the next round cannot choose differently: at that time the winner has
+                                // a free slot with the same predicted first token, and no other instance's prediction can have become
+                                // earlier or feasible.  So it is only counted, and the request takes the slot over.
+                                bool twin = false;
+                                if (win) {
+                                    const uint32_t s = kmin & 63u, kb = area + kWalkKeys + (s >> 3) * kWalkBlock, k8 = kb + 4u * (s & 7u), mb = area + 4u * (s >> 3);
+                                    st1(k8, kKeyEmpty);
+                                    st1(mb, kKeyEmpty);
+                                    const uint4 k0 = ld4(kb), k1 = ld4(kb + 16u), m0 = ld4(area), m1 = ld4(area + 16u);
+                                    const uint2 run = ld2(kb + 32u + 8u * (s & 7u));
+                                    const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                                    const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                                    const uint32_t bmin = min8(kv), others = min(bmin, min8(mv));
+                                    K = kmin >> 6;
+                                    const uint32_t nk = ((K + Sm1) << 6) | s;
+                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t0, run.x, run.y, tag >> 16));
+                                    st1(k8, nk);
+                                    st2(kb + 32u + 8u * (s & 7u), make_uint2((uint32_t)first, req));
+                                    st1(mb, min(bmin, nk));
+                                    t = first;
+                                    kmin = min(others, nk);
+                                    next_end(true);
+                                    twin = (others >> 6) == K;
+                                }
+                                if (++ring_n >= kRoom) flush();
+                                uint32_t tm = __ballot_sync(kWFull, twin | (now >= kWalkNowMax));
+                                if (tm) {
+                                    // others that complete at the very boundary the request waited for
+                                    while ((tm = __ballot_sync(kWFull, twin)) != 0u) {
+                                        twin = retire(twin, tm, 0, true);
+                                        if (++ring_n >= kRoom) flush();
+                                    }
+                                    peek();
+                                    if (now >= kWalkNowMax && i + 1u < n) {
+                                        n = i + 1u;
+                                        from = qn.z >> 24;
+                                        move = true;
+                                    }
+                                }
+                            } else if (q.w == 0u) {  // one token: done at the end of its prefill, never occupies a slot
+                                if (win) {
+                                    t = first;
+                                    if (w > 0) tb += pre;
+                                    bad = bad || t > (int32_t)kWalkHorizon || (w > 0 && tb > (int32_t)kWalkHorizon);
+                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t, (uint32_t)t, req, tag >> 16));
+                                }
+                                if (++ring_n >= kRoom) flush();
+                            } else {  // (as above)
+                                if (win) {
+                                    const uint32_t kb = area + kWalkKeys + (top >> 3) * kWalkBlock, nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
+                                    st1(kb + 4u * (top & 7u), nk);
+                                    st2(kb + 32u + 8u * (top & 7u), make_uint2((uint32_t)first, req));
+                                    st1(area + 4u * (top >> 3), min(top_min, nk));
+                                    t = first;
+                                    K = nK;
+                                    kmin = min(kmin, nk);
+                                    w++;
+                                    step = more.x;
+                                    rcp = more.y;
+                                    next_end(true);
+                                }
+                                peek();
+                            }
+                        }
+                        st1(ent, (uint32_t)start());
+                        i++;
+                        q = qn;
+                        lim = ln;
+                        tries = 0;
+                    }
+                    // (listed requests are admitted, up to where the list was left)
+                    served |= live & (from < 32u ? (1u << from) - 1u : ~0u) & ~(i < n && !move && !status ? 1u << (from - 1u) : 0u);
+                    __syncwarp();
+                    if (status) break;
+                    if (move) move_epoch(cb, from);
+                    else if (from >= 32u) break;
+                    live = test(from);
+                } while (live);
+                if (side) report(served, end);
+                if (__any_sync(kWFull, bad) || status) break;
+            }
+
+            // ---- through the trace: drain, account, write the record ------------------------------------------------
+            if (status == 0u) events(w > 0 && !bad, kFar);
+            flush();
+            if (lane == 0) idx = static_total + atomicAdd(&P.walk_ctr[bucket - kWalkBucket0], 1u);
+            idx = __shfl_sync(kWFull, idx, 0);
+            if (__any_sync(kWFull, bad)) {
+                if (lane == 0) walk_hand_over(P, cand, false);
+                continue;
+            }
+            walk_finish(P, base0, tr, cand, use_mask, cmask, status, extra);
+        }
+    }
+};
+
+}  // namespace maaso

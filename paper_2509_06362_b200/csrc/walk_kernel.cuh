@@ -170,6 +170,46 @@ static __device__ __noinline__ void walk_hand_over(const EvalParams& P, uint32_t
     P.bucket_list[(size_t)bucket * P.n_cand + at] = cand;
 }
 
+// The record of a placement that is through, from its sums in the region `base`.
+static __device__ __forceinline__ void walk_finish(const EvalParams& P, uint32_t base, uint32_t tr, uint32_t cand, bool use_mask,
+                                                   uint32_t cmask, uint32_t status, uint32_t extra) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint4 u0 = w4(base + 16u * lane), u1 = w4(base + 16u * lane + 512u), u2 = w4(base + 16u * lane + 1024u), u3 = w4(base + 16u * lane + 1536u);
+    Stats st;
+    st.sum_ttft = i64_of(u0.x, u0.y); st.max_ttft = i64_of(u0.z, u0.w);
+    st.sum_e2e = i64_of(u1.x, u1.y);  st.max_e2e = i64_of(u1.z, u1.w);
+    st.makespan = i64_of(u2.x, u2.y); st.checksum = (uint64_t)i64_of(u2.z, u2.w);
+    st.tokens = (uint64_t)i64_of(u3.x, u3.y);
+    st.served = __reduce_add_sync(kWFull, u3.z);
+    st.hit = __reduce_add_sync(kWFull, u3.w);
+    // the request count and the checksum of "everything rejected", from the per-class totals
+    uint32_t counted_all = 0;
+    for (uint32_t c = lane; c < P.n_classes; c += 32u)
+        if (!use_mask || ((cmask >> c) & 1u)) {
+            counted_all += (uint32_t)P.trace_class_tot[tr][2u * c];
+            st.checksum += P.trace_class_tot[tr][2u * c + 1u];
+        }
+    counted_all = __reduce_add_sync(kWFull, counted_all);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        st.sum_ttft += (int64_t)wshfl_xor((uint64_t)st.sum_ttft, o);
+        st.sum_e2e += (int64_t)wshfl_xor((uint64_t)st.sum_e2e, o);
+        st.tokens += wshfl_xor(st.tokens, o);
+        st.checksum += wshfl_xor(st.checksum, o);
+        st.max_ttft = max(st.max_ttft, (int64_t)wshfl_xor((uint64_t)st.max_ttft, o));
+        st.max_e2e = max(st.max_e2e, (int64_t)wshfl_xor((uint64_t)st.max_e2e, o));
+        st.makespan = max(st.makespan, (int64_t)wshfl_xor((uint64_t)st.makespan, o));
+    }
+    if (lane == 0) {
+        uint32_t h[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) h[i] = w1(base + kSByClass + 4u * i);
+        write_result(P.out + tr * P.n_cand + cand, status, counted_all, counted_all - st.served,
+                     (uint64_t)counted_all + extra, st, h);
+    }
+    __syncwarp();
+}
+
 // What one lane knows of its instance.
 template <class T>
 struct WInst {
@@ -218,6 +258,14 @@ struct Walk {
             const bool end = (int64_t)((uint64_t)Sm1 * step + since) <= i64_of(a.z, a.w);  // (no branches)
             if constexpr (Wide) return (int64_t)since <= ttft && (Sm1 == 0u || tbt < 0 || (int64_t)step <= tbt) && end;
             else return (since <= a.x) & ((Sm1 == 0u) | (step <= a.y)) & end;
+        }
+        // The same for 32-bit times as a bound of `since`, so that one comparison is left when the start is known:
+        // met(since) = since < before().
+        __device__ __forceinline__ uint32_t before(uint32_t Sm1, uint32_t step) const {
+            const int64_t left = i64_of(a.z, a.w) - (int64_t)((uint64_t)Sm1 * step);  // up to 2^62, or negative
+            const uint32_t e = (uint32_t)(left >> 32) == 0u ? lo32(left) : 0xFFFFFFFEu;  // (no time is as long)
+            const bool never = (left < 0) | ((Sm1 != 0u) & (step > a.y));
+            return never ? 0u : min(min(a.x, e), 0xFFFFFFFEu) + 1u;
         }
     };
     static __device__ __forceinline__ T prefill(uint32_t base, uint32_t q16, uint32_t in_tok) {
@@ -795,43 +843,14 @@ struct Walk {
                 if (lane == 0) walk_hand_over(P, cand, kFixed);
                 continue;
             }
-            const uint4 u0 = w4(base + 16u * lane), u1 = w4(base + 16u * lane + 512u), u2 = w4(base + 16u * lane + 1024u), u3 = w4(base + 16u * lane + 1536u);
-            Stats st;
-            st.sum_ttft = i64_of(u0.x, u0.y); st.max_ttft = i64_of(u0.z, u0.w);
-            st.sum_e2e = i64_of(u1.x, u1.y);  st.max_e2e = i64_of(u1.z, u1.w);
-            st.makespan = i64_of(u2.x, u2.y); st.checksum = (uint64_t)i64_of(u2.z, u2.w);
-            st.tokens = (uint64_t)i64_of(u3.x, u3.y);
-            st.served = __reduce_add_sync(kWFull, u3.z);
-            st.hit = __reduce_add_sync(kWFull, u3.w);
-            // the request count and the checksum of "everything rejected", from the per-class totals
-            uint32_t counted_all = 0;
-            for (uint32_t c = lane; c < P.n_classes; c += 32u)
-                if (!use_mask || ((cmask >> c) & 1u)) {
-                    counted_all += (uint32_t)P.trace_class_tot[tr][2u * c];
-                    st.checksum += P.trace_class_tot[tr][2u * c + 1u];
-                }
-            counted_all = __reduce_add_sync(kWFull, counted_all);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                st.sum_ttft += (int64_t)wshfl_xor((uint64_t)st.sum_ttft, o);
-                st.sum_e2e += (int64_t)wshfl_xor((uint64_t)st.sum_e2e, o);
-                st.tokens += wshfl_xor(st.tokens, o);
-                st.checksum += wshfl_xor(st.checksum, o);
-                st.max_ttft = max(st.max_ttft, (int64_t)wshfl_xor((uint64_t)st.max_ttft, o));
-                st.max_e2e = max(st.max_e2e, (int64_t)wshfl_xor((uint64_t)st.max_e2e, o));
-                st.makespan = max(st.makespan, (int64_t)wshfl_xor((uint64_t)st.makespan, o));
-            }
-            if (lane == 0) {
-                uint32_t h[8];
-#pragma unroll
-                for (int i = 0; i < 8; i++) h[i] = w1(base + kSByClass + 4u * i);
-                write_result(P.out + tr * P.n_cand + cand, status, counted_all, counted_all - st.served,
-                             (uint64_t)counted_all + w1(base + kSExtra), st, h);
-            }
-            __syncwarp();
+            walk_finish(P, base, tr, cand, use_mask, cmask, status, w1(base + kSExtra));
         }
     }
 };
+
+}  // namespace maaso
+#include "walk_dynamic.cuh"
+namespace maaso {
 
 // `Warps`: 16, or 12 for a batch that 12 per SM can hold.  Mode k: the block's warps >> k at work, each with 2^k times one warp's part of the pool.  The first placements
 // are dealt out in order, over the SMs first; after that whoever is free takes the next.
@@ -843,9 +862,11 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
     uint32_t any = 0;
     for (int mode = 0; mode < (Big && !kLong ? 1 : kWalkModes); mode++) any |= P.bucket_count[kFirst + mode];
     if (any == 0) return;
-    const WalkLayout L = walk_layout(P.n_rows, P.n_classes, Wide, Warps);
+    constexpr bool kDynamic = Eng == 0 && !Wide && !Big;
+    const WalkLayout L = walk_layout(P.n_rows, P.n_classes, Wide, Warps, kDynamic);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
-    for (uint32_t i = tid; i < P.n_rows * 65u; i += (32 * Warps)) w2(L.steps + 8u * i) = walk_step_entry(P, i);
+    for (uint32_t i = tid; i < P.n_rows * 65u; i += (32 * Warps)) 
+        w2(L.steps + 8u * i) = kDynamic ? walk_exact_entry(P, i) : walk_step_entry(P, i);
     for (uint32_t c = tid; c < P.n_classes; c += (32 * Warps)) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u];
         const int64_t none = (int64_t)1 << 62, le = e < 0 ? none : e;
@@ -876,8 +897,9 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
         for (int mode = kWalkModes - 1; mode >= 0; mode--) {
             if (P.bucket_count[kFirst + mode] == 0) continue;  // the same for the whole block
             const uint32_t act = (uint32_t)Warps >> mode, part = (kLong ? P.walk_bytes : P.walk_usual) << mode;
+            using Body = typename std::conditional<kDynamic, WalkDynamic<Opt>, Walk<Opt, Eng, Wide, Big>>::type;
             if (warp < act)
-                Walk<Opt, Eng, Wide, Big>::bucket(P, L, kFirst + mode, L.pool + warp * part, warp * gridDim.x + blockIdx.x,
+                Body::bucket(P, L, kFirst + mode, L.pool + warp * part, warp * gridDim.x + blockIdx.x,
                                                   act * gridDim.x, nullptr);
             if (mode) __syncthreads();
         }
@@ -887,7 +909,7 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
 template <bool Opt, int Eng, bool Wide, bool Big, int Warps = kWalkWarps>
 static cudaError_t launch_walk(const EvalParams& P, int grid, cudaStream_t stream) {
     auto kernel = eval_walk_kernel<Opt, Eng, Wide, Big, Warps>;
-    const size_t smem = walk_layout(P.n_rows, P.n_classes, Wide, Warps).pool + (Big || (Wide && Eng != 2) ? P.walk_bytes * kWalkWarps : P.walk_usual * Warps);
+    const size_t smem = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Eng == 0 && !Wide && !Big).pool + (Big || (Wide && Eng != 2) ? P.walk_bytes * kWalkWarps : P.walk_usual * Warps);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<grid, (32 * Warps), smem, stream>>>(P);
