@@ -14,10 +14,11 @@
 //   - a wait is one operation on the winner's slots: the request takes over the slot that frees;
 //   - a step count is a high product and a shift (exact reciprocals), without a correction;
 //   - chunks that need no round are skipped in a loop of their own;
-//   - shared memory is addressed directly (5 % against references into the block's array).
-// Measured against the body that it replaced here (that of Walk): warp instructions of a round that admits 189 -> 160, with a
-// completion before 286 -> 246, with a wait 304 -> 190; 2,000 x 17,000 of the paper's shape 8.9 -> 6.8 ms, one node's 10,864 x
-// 10,000 6.4 -> 4.9, three models under load 12,000 x 30,000 4.51 -> 4.35, masked sub-clusters 9,000 x 12,000 18.3 -> 16.3.
+//   - shared memory is addressed directly (5 % against references into the block's array);
+//   - lower bounds for the scan are written when a list is through, not on every round.
+// Measured against the body that it replaced here (that of Walk): warp instructions of a round that admits 189 -> 135, with a
+// completion before 286 -> 214, with a wait 304 -> 171; 2,000 x 17,000 of the paper's shape 8.9 -> 6.4 ms, one node's 10,864 x
+// 10,000 6.4 -> 4.63, three models under load 12,000 x 30,000 4.51 -> 4.25, masked sub-clusters 9,000 x 12,000 18.3 -> 15.9.
 // Dropped: completions and admissions without a branch, lanes that have none writing to a dummy region (a lone warp as fast,
 // +5 % instructions); the accounting of completions inlined (+7 %).
 #pragma once
@@ -103,8 +104,8 @@ struct WalkDynamic {
             if (n_req) nxt = __ldg(reqs + min(lane, n_req - 1u));
             const uint32_t lo = P.offsets[cand], n_i = P.offsets[cand + 1] - lo;
             // this lane's instance (see WInst)
-            int32_t t = 0, tb = kFar;
-            uint32_t K = 0, kmin = kKeyEmpty, w = 0, B = 1, tag = 0, area = dummy, row = L.steps, pre_base = 0, pre_q16 = 0, stepB = 1;
+            int32_t t = 0, tc = kFar;  // clock, next completion
+            uint32_t K = 0, kmin = kKeyEmpty, w = 0, B = 1, bit = 0, place = 0, area = dummy, pay = dummy, row = L.steps, pre_base = 0, pre_q16 = 0, stepB = 1;
             uint32_t ent = dummy + 96u;
             {
                 for (uint32_t i = lane; i < kWalkSums / 16u; i += 32u) st4(base + 16u * i, make_uint4(0u, 0u, 0u, 0u));
@@ -124,7 +125,8 @@ struct WalkDynamic {
                     ent = ents + 16u * lane;
                     const uint2 e = ld2(ent);
                     const uint32_t md = e.x & 0xFu, r = md * P.n_strategies + ((e.x >> 4) & 0xFFu);
-                    tag = (1u << md) | (e.y << 16);
+                    bit = 1u << md;  // of its model; 0 from when it has left the horizon on: nothing is asked of it any more (see Walk)
+                    place = e.y;
                     B = (e.x >> 12) & 0xFFu;
                     row = L.steps + r * kWalkRow;
                     pre_base = (uint32_t)P.rows[r * kRowStride];
@@ -148,8 +150,9 @@ struct WalkDynamic {
                 }
                 if (bytes) {
                     area = ents + 16u * n_i + incl - bytes;
+                    pay = area + kWalkKeys + 4u * ((B + 7u) & ~7u);
                     for (uint32_t i = 0; i < 8u; i++) st1(area + 4u * i, kKeyEmpty);
-                    for (uint32_t i = 0; i < ((B + 7u) & ~7u); i++) st1(area + kWalkKeys + (i >> 3) * kWalkBlock + 4u * (i & 7u), kKeyEmpty);
+                    for (uint32_t i = area + kWalkKeys; i < pay; i += 4u) st1(i, kKeyEmpty);
                     for (uint32_t i = 0; i < B; i++) stb(area + 32u + i, i);
                 }
             }
@@ -162,14 +165,13 @@ struct WalkDynamic {
             const bool side = P.rej_by_model != nullptr || (P.dump_row && P.dump_row[cand] >= 0);
             __syncwarp();
 
-            uint32_t step = 32u, rcp = 0x80000000u;  // entry of the current level (0: an idle clock)
+            uint32_t step = 32u, rcp = 0x80000000u, sw = 1u;  // entry of the current level (0: an idle clock), its step
             // the next free slot, its block's smallest key, the entry of one request more
             uint32_t top = 0, top_min = 0;
             uint2 more = make_uint2(0u, 0u);
             uint32_t ring_n = 0, status = 0, extra = 0;  // extra: distributor rounds beyond one per request
             int64_t epoch = 0;
             int32_t now = 0;
-            bool bad = false;               // a time of this lane has left the horizon: nothing is asked of it any more (see Walk)
             int32_t rel = 0;                // this lane's request of the chunk: arrival,
             uint32_t c_in = 0, c_meta = 0;  // input tokens, output tokens | class | model
 
@@ -185,46 +187,48 @@ struct WalkDynamic {
             };
             auto peek = [&]() {
                 more = ld2(row + 8u * w + 8u);
-                top = ldb(area + 32u + w) & 63u;
+                top = ldb(area + 32u + w);  // (a full instance's is not looked at)
                 top_min = ld1(area + ((top >> 1) & 28u));
             };
             peek();
-            // The next completion, counted from the clock; flags what leaves the horizon.
-            auto next_end = [&](bool busy) {
-                const uint64_t tc = (uint64_t)((kmin >> 6) - K) * (step >> 5) + (uint32_t)t;
-                tb = busy ? (int32_t)((uint32_t)tc - (step >> 5)) : kFar;
-                bad = bad | (busy & (tc > (uint64_t)kWalkHorizon));
+            // The next completion, counted from the clock; false: it leaves the horizon.
+            auto next_end = [&](bool busy) -> bool {
+                const uint64_t ahead = (uint64_t)((kmin >> 6) - K) * sw;
+                const uint32_t end = (uint32_t)ahead + (uint32_t)t;
+                tc = busy ? (int32_t)end : kFar;
+                const bool in = !busy | (((uint32_t)(ahead >> 32) == 0u) & (max((uint32_t)ahead, end) <= (uint32_t)kWalkHorizon));
+                if (!in) bit = 0;
+                return in;
             };
-            // One completion in each of the lanes in `due` (their set: `dm`); then whether another one is due.
-            // `stay`: at the time `now`, while the clock is already beyond it (see the wait).
+            // One completion in each of the lanes in `due` (their set: `dm`); then whether another one is due.  `stay`: at the time
+            // `now`, while the clock is already beyond it (see the wait).
             auto retire = [&](bool due, uint32_t dm, int32_t upto, bool stay) -> bool {
                 if (due) {
-                    const uint32_t s = kmin & 63u, kb = area + kWalkKeys + (s >> 3) * kWalkBlock, k8 = kb + 4u * (s & 7u), mb = area + 4u * (s >> 3);
+                    const uint32_t s = kmin & 63u, keys = area + kWalkKeys, kb = keys + 4u * (s & 56u), mb = area + ((s >> 1) & 28u);
                     // (the key and its block's minimum go first: what is left is read without them)
-                    st1(k8, kKeyEmpty);
+                    st1(keys + 4u * s, kKeyEmpty);
                     st1(mb, kKeyEmpty);
                     const uint4 k0 = ld4(kb), k1 = ld4(kb + 16u), m0 = ld4(area), m1 = ld4(area + 16u);
-                    const uint2 cur = ld2(row + 8u * w - 8u), run = ld2(kb + 32u + 8u * (s & 7u));
+                    const uint2 cur = ld2(row + 8u * w - 8u), run = ld2(pay + 8u * s);
                     const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                     const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-                    const int32_t fin = stay ? now : tb + (int32_t)(step >> 5);
                     if (!stay) {
-                        t = fin;
+                        t = tc;
                         K = kmin >> 6;
                     }
                     w--;
                     stb(area + 32u + w, s);
-                    st4(ring + 16u * (ring_n + (uint32_t)__popc(dm & below)), make_uint4((uint32_t)fin, run.x, run.y, tag >> 16));
+                    st4(ring + 16u * (ring_n + (uint32_t)__popc(dm & below)), make_uint4((uint32_t)(stay ? now : tc), run.x, run.y, place));
                     top = s;
                     more = make_uint2(step, rcp);
                     step = cur.x;
                     rcp = cur.y;
+                    sw = step >> 5;
                     top_min = min8(kv);
                     st1(mb, top_min);
                     kmin = min(top_min, min8(mv));
-                    const bool busy = w > 0u;
-                    next_end(busy);
-                    due = busy & (((kmin >> 6) == K) | (!stay & (tb < upto))) & !bad;
+                    const bool busy = w > 0u, in = next_end(busy);
+                    due = busy & in & (((kmin >> 6) == K) | (!stay & (tc < upto + (int32_t)sw)));
                 }
                 return due;
             };
@@ -240,9 +244,9 @@ struct WalkDynamic {
             };
             // Decode steps until `dt` later; 2 (dt + step - 1) < 2^32.
             auto steps_of = [&](int32_t dt) -> uint32_t {
-                return __funnelshift_r(__umulhi(2u * ((uint32_t)dt + (step >> 5) - 1u), rcp), 0u, step);
+                return __funnelshift_r(__umulhi(2u * ((uint32_t)dt + sw - 1u), rcp), 0u, step);
             };
-            auto start = [&]() -> int32_t { return w == B ? tb + (int32_t)(step >> 5) : t; };
+            auto start = [&]() -> int32_t { return w == B ? tc : t; };
             // What is rare, out of the rounds' way.  Moves the epoch for request `src` of the chunk at `cb`, to the dispatcher's
             // clock (or to the request's arrival, if that is later): what happens before it is simulated, everything else is
             // measured from there on.
@@ -250,24 +254,23 @@ struct WalkDynamic {
                 const uint4 v = __ldg(reqs + cb + src);
                 const int64_t to = max(epoch + now, i64_of(v.x, v.y));
                 const int32_t up = to - epoch >= (int64_t)kFar ? kFar : (int32_t)(to - epoch);  // (cut off only if all is idle by then)
-                events(w > 0 && tb < up && !bad, up);
+                events(w > 0 && bit && tc - (int32_t)sw < up, min(up, kFar - (int32_t)kWalkStepMax));
                 if (w == 0) {
                     t = t > up ? t - up : 0;  // an idle instance is where the dispatcher is
                 } else {
                     if (w < B && t < up) {
                         const uint32_t k = steps_of(up - t);
-                        t += (int32_t)(k * (step >> 5));
+                        t += (int32_t)(k * sw);
                         K += k;
                     }
                     t = t > up + kWPast ? t - up : kWPast;  // a full instance's clock is not looked at
-                    tb -= up;
+                    tc -= up;
                     // running requests' first tokens (further back than 32 bits reach: the lane has left the horizon)
                     for (uint32_t i = 0; i < B; i++) {
-                        const uint32_t kb = area + kWalkKeys + (i >> 3) * kWalkBlock;
-                        if (ld1(kb + 4u * (i & 7u)) == kKeyEmpty) continue;
-                        const int64_t f = (int64_t)(int32_t)ld1(kb + 32u + 8u * (i & 7u)) - up;
-                        bad = bad || f < -(int64_t)kFar;
-                        st1(kb + 32u + 8u * (i & 7u), (int32_t)f);
+                        if (ld1(area + kWalkKeys + 4u * i) == kKeyEmpty) continue;
+                        const int64_t f = (int64_t)(int32_t)ld1(pay + 8u * i) - up;
+                        if (f < -(int64_t)kFar) bit = 0;
+                        st1(pay + 8u * i, (uint32_t)(int32_t)f);
                     }
                 }
                 st1(ent, (uint32_t)start());
@@ -327,8 +330,7 @@ struct WalkDynamic {
                     if (__any_sync(kWFull, (w > 0) & (K > kRelMax - (40u << 16)))) {
                         if (w > 0) {
                             const uint32_t d = K << 6;
-                            for (uint32_t i = 0; i < 8u + ((B + 7u) & ~7u); i++) {
-                                const uint32_t at = i < 8u ? area + 4u * i : area + kWalkKeys + ((i - 8u) >> 3) * kWalkBlock + 4u * (i & 7u);
+                            for (uint32_t at = area; at < pay; at += at == area + 28u ? 68u : 4u) {  // block minima, keys
                                 const uint32_t k = ld1(at);
                                 if (k != kKeyEmpty) st1(at, k - d);
                             }
@@ -340,29 +342,30 @@ struct WalkDynamic {
                     if (far) live &= (far & (0u - far)) - 1u;
                     uint32_t n = (uint32_t)__popc(live);
                     if ((live >> lane) & 1u) {
-                        // {arrival, input tokens, output tokens - 1 | model << 16 | lane << 24, keys below this take the usual path}
-                        // {bound of the first token after the arrival, of the step, of the end + 1, output tokens - 1 as far as that bound goes}
+                        // {arrival, input tokens, model bit | lane << 16, keys below this take the usual path}
+                        // {bound of the first token after the arrival, of the step, of the end + 1, output tokens - 1 | the factor of the step in
+                        // the bound of the end << 16 (the same, 0 without a limit)}
                         const uint32_t out = c_meta & 0xFFFFu, at = list + 32u * (uint32_t)__popc(live & below);
                         const uint4 l = ld4(L.lims + ((c_meta >> 12) & 0xFF0u));
                         const bool endless = (l.w >> 30) != 0u;
-                        st4(at, make_uint4((uint32_t)rel, c_in, (out - 1u) | ((c_meta >> 24) << 16) | (lane << 24), out == 1u ? 0u : kFast));
-                        st4(at + 16u, make_uint4(min(l.x, 0xFFFFFFFEu) + 1u, out == 1u ? 0xFFFFFFFFu : l.y, endless ? 0xFFFFFFFFu : l.z + 1u, endless ? 0u : out - 1u));
+                        st4(at, make_uint4((uint32_t)rel, c_in, (1u << (c_meta >> 24)) | (lane << 16), out == 1u ? 0u : kFast));
+                        st4(at + 16u, make_uint4(min(l.x, 0xFFFFFFFEu) + 1u, out == 1u ? 0xFFFFFFFFu : l.y, endless ? 0xFFFFFFFFu : l.z + 1u, (out - 1u) | (endless ? 0u : (out - 1u) << 16)));
                     }
                     __syncwarp();
                     bool move = far != 0u;
                     from = move ? (uint32_t)__ffs((int)far) - 1u : 32u;  // where the next pass over the chunk starts
                     uint32_t i = 0;
-                    uint4 q = ld4(list), lim = ld4(list + 16u);  // the request of this round, its limits
+                    uint4 q = ld4(list);  // the request of this round
                     uint32_t tries = 0;
                     while (i < n) {
-                        const uint4 qn = ld4(list + 32u * i + 32u), ln = ld4(list + 32u * i + 48u);
+                        const uint4 lim = ld4(list + 32u * i + 16u), qn = ld4(list + 32u * i + 32u);
                         const int32_t arrival = (int32_t)q.x;
-                        const uint32_t Sm1 = q.z & 0xFFFFu, req = cb + (q.z >> 24);
+                        const uint32_t req = cb + (q.z >> 16);
                         now = max(now, arrival);  // pending time: the dispatcher never goes back
-                        const bool elig = (((tag >> ((q.z >> 16) & 15u)) & 1u) != 0u) & !bad;
+                        const bool elig = (bit & q.z) != 0u;
                         const int32_t pre = (int32_t)(pre_base + (uint32_t)(((uint64_t)pre_q16 * q.y + 32768u) >> 16));
                         // "reduce": what completes before the instance's clock reaches `now`
-                        bool due = elig & (tb < now);
+                        bool due = elig & (tc < now + (int32_t)sw);
                         uint32_t dm = __ballot_sync(kWFull, due);
                         while (dm) {
                             due = retire(due, dm, now, false);
@@ -373,14 +376,15 @@ struct WalkDynamic {
                         const bool full = w == B;
                         {
                             const uint32_t k = steps_of(elig & !full ? max(now - t, 0) : 0);
-                            t += (int32_t)(k * (step >> 5));
+                            t += (int32_t)(k * sw);
                             K += k;
                         }
                         // distributor prediction (Sec. IV-F steps 2-3): the bound that the class and the step put on the first token
                         const uint32_t sB = Opt && !full ? more.x >> 5 : stepB;
-                        const int64_t left = (int64_t)lim.z - (int64_t)((uint64_t)lim.w * sB);
+                        const uint32_t Sm1 = lim.w & 0xFFFFu;
+                        const int64_t left = (int64_t)lim.z - (int64_t)((uint64_t)(lim.w >> 16) * sB);
                         const uint32_t bound = min(lim.x, lo32(left) & ~(uint32_t)((int32_t)hi32(left) >> 31));
-                        const int32_t t0 = full ? tb + (int32_t)(step >> 5) : t, first = t0 + pre;
+                        const int32_t t0 = full ? tc : t, first = t0 + pre;
                         const bool ok = elig & (sB <= lim.y) & ((uint32_t)(first - arrival) < bound);
                         // smallest (tier, predicted first token >= now), lowest instance among equals
                         const uint32_t key = ok ? (min((uint32_t)(first - now), kOffMax) << 5) + (full ? lane + kTier1 : lane) : kNone;
@@ -388,22 +392,23 @@ struct WalkDynamic {
                         if (best < q.w) {
                             // "map": prefill at the step boundary (running decodes stall), then occupy a free slot
                             if (key == best) {
-                                const uint32_t kb = area + kWalkKeys + (top >> 3) * kWalkBlock, nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
-                                st1(kb + 4u * (top & 7u), nk);
-                                st2(kb + 32u + 8u * (top & 7u), make_uint2((uint32_t)first, req));
-                                st1(area + 4u * (top >> 3), min(top_min, nk));
+                                const uint32_t nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
+                                st1(area + kWalkKeys + 4u * top, nk);
+                                st2(pay + 8u * top, make_uint2((uint32_t)first, req));
+                                st1(area + ((top >> 1) & 28u), min(top_min, nk));
                                 t = first;
                                 K = nK;
                                 kmin = min(kmin, nk);
                                 w++;
                                 step = more.x;
                                 rcp = more.y;
+                                sw = step >> 5;
                                 next_end(true);
                             }
                             peek();
                         } else if (best == kNone) {
                             // overflow protection: nobody can meet the deadline.  What the scan went by is out of date: once more
-                            from = (q.z >> 24) + 1u;
+                            from = (q.z >> 16) + 1u;
                             move = false;
                             break;
                         } else {
@@ -421,11 +426,11 @@ struct WalkDynamic {
                                 if (Opt || q.w == 0u) {  // a new choice
                                     if (Opt && ++tries >= kAttemptCap) {
                                         status = MAASO_CAND_ELOOP;
-                                        from = end = q.z >> 24;
+                                        from = end = q.z >> 16;
                                         break;
                                     }
                                     if (now >= kWalkNowMax) {  // (for the same request)
-                                        from = q.z >> 24;
+                                        from = q.z >> 16;
                                         move = true;
                                         break;
                                     }
@@ -436,19 +441,19 @@ struct WalkDynamic {
                                 // earlier or feasible.  So it is only counted, and the request takes the slot over.
                                 bool twin = false;
                                 if (win) {
-                                    const uint32_t s = kmin & 63u, kb = area + kWalkKeys + (s >> 3) * kWalkBlock, k8 = kb + 4u * (s & 7u), mb = area + 4u * (s >> 3);
-                                    st1(k8, kKeyEmpty);
+                                    const uint32_t s = kmin & 63u, keys = area + kWalkKeys, kb = keys + 4u * (s & 56u), mb = area + ((s >> 1) & 28u);
+                                    st1(keys + 4u * s, kKeyEmpty);
                                     st1(mb, kKeyEmpty);
                                     const uint4 k0 = ld4(kb), k1 = ld4(kb + 16u), m0 = ld4(area), m1 = ld4(area + 16u);
-                                    const uint2 run = ld2(kb + 32u + 8u * (s & 7u));
+                                    const uint2 run = ld2(pay + 8u * s);
                                     const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                                     const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
                                     const uint32_t bmin = min8(kv), others = min(bmin, min8(mv));
                                     K = kmin >> 6;
                                     const uint32_t nk = ((K + Sm1) << 6) | s;
-                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t0, run.x, run.y, tag >> 16));
-                                    st1(k8, nk);
-                                    st2(kb + 32u + 8u * (s & 7u), make_uint2((uint32_t)first, req));
+                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t0, run.x, run.y, place));
+                                    st1(keys + 4u * s, nk);
+                                    st2(pay + 8u * s, make_uint2((uint32_t)first, req));
                                     st1(mb, min(bmin, nk));
                                     t = first;
                                     kmin = min(others, nk);
@@ -466,41 +471,41 @@ struct WalkDynamic {
                                     peek();
                                     if (now >= kWalkNowMax && i + 1u < n) {
                                         n = i + 1u;
-                                        from = qn.z >> 24;
+                                        from = qn.z >> 16;
                                         move = true;
                                     }
                                 }
                             } else if (q.w == 0u) {  // one token: done at the end of its prefill, never occupies a slot
                                 if (win) {
                                     t = first;
-                                    if (w > 0) tb += pre;
-                                    bad = bad || t > (int32_t)kWalkHorizon || (w > 0 && tb > (int32_t)kWalkHorizon);
-                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t, (uint32_t)t, req, tag >> 16));
+                                    if (w > 0) tc += pre;
+                                    if (t > (int32_t)kWalkHorizon || (w > 0 && (uint32_t)tc > (uint32_t)kWalkHorizon)) bit = 0;
+                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t, (uint32_t)t, req, place));
                                 }
                                 if (++ring_n >= kRoom) flush();
                             } else {  // (as above)
                                 if (win) {
-                                    const uint32_t kb = area + kWalkKeys + (top >> 3) * kWalkBlock, nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
-                                    st1(kb + 4u * (top & 7u), nk);
-                                    st2(kb + 32u + 8u * (top & 7u), make_uint2((uint32_t)first, req));
-                                    st1(area + 4u * (top >> 3), min(top_min, nk));
+                                    const uint32_t nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
+                                    st1(area + kWalkKeys + 4u * top, nk);
+                                    st2(pay + 8u * top, make_uint2((uint32_t)first, req));
+                                    st1(area + ((top >> 1) & 28u), min(top_min, nk));
                                     t = first;
                                     K = nK;
                                     kmin = min(kmin, nk);
                                     w++;
                                     step = more.x;
                                     rcp = more.y;
+                                    sw = step >> 5;
                                     next_end(true);
                                 }
                                 peek();
                             }
                         }
-                        st1(ent, (uint32_t)start());
                         i++;
                         q = qn;
-                        lim = ln;
                         tries = 0;
                     }
+                    st1(ent, (uint32_t)start());  // for the scan
                     // (listed requests are admitted, up to where the list was left)
                     served |= live & (from < 32u ? (1u << from) - 1u : ~0u) & ~(i < n && !move && !status ? 1u << (from - 1u) : 0u);
                     __syncwarp();
@@ -510,15 +515,15 @@ struct WalkDynamic {
                     live = test(from);
                 } while (live);
                 if (side) report(served, end);
-                if (__any_sync(kWFull, bad) || status) break;
+                if (status || __any_sync(kWFull, lane < n_i && bit == 0u)) break;
             }
 
             // ---- through the trace: drain, account, write the record ------------------------------------------------
-            if (status == 0u) events(w > 0 && !bad, kFar);
+            if (status == 0u) events(w > 0 && bit, kFar - (int32_t)kWalkStepMax);
             flush();
             if (lane == 0) idx = static_total + atomicAdd(&P.walk_ctr[bucket - kWalkBucket0], 1u);
             idx = __shfl_sync(kWFull, idx, 0);
-            if (__any_sync(kWFull, bad)) {
+            if (__any_sync(kWFull, lane < n_i && bit == 0u)) {
                 if (lane == 0) walk_hand_over(P, cand, false);
                 continue;
             }
