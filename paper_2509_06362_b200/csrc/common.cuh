@@ -292,6 +292,7 @@ struct EvalParams {
     uint32_t walk_usual;     // the same for placements of up to 32 instances, with walk_warps warps
     uint32_t pack;           // placements of at most 8 instances that could go to the lane groups share the steps of a warp instead
     uint32_t walk_warps;
+    uint32_t walk_parts;     // queues: parts a placement is replayed in, 1 or the number of models
     uint32_t walk_long;      // the whole batch with 64-bit times
     long long wait_cycles;   // bound of every device-side wait
     uint32_t stall_test;     // test hook: never issue the trace copies

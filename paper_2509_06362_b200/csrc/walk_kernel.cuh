@@ -72,10 +72,9 @@ __device__ __forceinline__ int64_t wshfl(int64_t v, int src) {
     return i64_of(__shfl_sync(kWFull, lo32(v), src), __shfl_sync(kWFull, hi32(v), src));
 }
 __device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_sync(kWFull, v); }
-__device__ __forceinline__ uint64_t warp_min(uint64_t v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, wshfl_xor(v, o));
-    return v;
+__device__ __forceinline__ uint64_t warp_min(uint64_t v) {  // the smallest high half, the smallest low half that comes with it
+    const uint32_t hi = (uint32_t)(v >> 32), mh = __reduce_min_sync(kWFull, hi);
+    return ((uint64_t)mh << 32) | __reduce_min_sync(kWFull, hi == mh ? (uint32_t)v : 0xFFFFFFFFu);
 }
 // ceil(dt / s) for 0 <= dt < 2^31, s < 2^31, rs = (2^32 - 1) / s rounded down: the estimate is at most the quotient and less
 // than two below it, since rs > 2^32 / s - 1.
@@ -170,9 +169,42 @@ static __device__ __noinline__ void walk_hand_over(const EvalParams& P, uint32_t
     P.bucket_list[(size_t)bucket * P.n_cand + at] = cand;
 }
 
-// The record of a placement that is through, from its sums in the region `base`.
+// One part of a placement's record: adds its sums to what the other parts left there; the last of `parts` completes the record,
+// which counts them in its reserved word until then.
+static __device__ __noinline__ void walk_add_part(maaso_result* out, uint32_t parts, uint32_t status, uint32_t counted, uint64_t rejected_sum,
+                                                  const Stats& st, const uint32_t* h) {
+    uint32_t* const w = reinterpret_cast<uint32_t*>(out);
+    auto wide = [&](uint32_t at) { return reinterpret_cast<unsigned long long*>(w + at); };
+    atomicAdd(w + 2, st.served);
+    atomicAdd(w + 3, st.hit);
+    for (int i = 0; i < 8; i++)
+        if (h[i]) atomicAdd(w + 6 + i, h[i]);
+    atomicAdd(wide(14), (unsigned long long)st.sum_ttft);
+    atomicMax(wide(16), (unsigned long long)st.max_ttft);
+    atomicAdd(wide(18), (unsigned long long)st.sum_e2e);
+    atomicMax(wide(20), (unsigned long long)st.max_e2e);
+    atomicMax(wide(22), (unsigned long long)st.makespan);
+    atomicAdd(wide(24), (unsigned long long)st.tokens);
+    atomicAdd(wide(26), (unsigned long long)st.checksum);
+    if (status) atomicOr(w + 31, status);
+    __threadfence();
+    if (atomicAdd(w + 30, 1u) + 1u < parts) return;
+    __threadfence();
+    auto get = [&](uint32_t at) { return (int64_t)__ldcg(wide(at)); };
+    Stats all;
+    all.served = __ldcg(w + 2); all.hit = __ldcg(w + 3);
+    all.sum_ttft = get(14); all.max_ttft = get(16);
+    all.sum_e2e = get(18);  all.max_e2e = get(20);
+    all.makespan = get(22); all.tokens = (uint64_t)get(24);
+    all.checksum = (uint64_t)get(26) + rejected_sum;
+    uint32_t hits[8];
+    for (int i = 0; i < 8; i++) hits[i] = __ldcg(w + 6 + i);
+    write_result(out, __ldcg(w + 31), counted, counted - all.served, counted, all, hits);
+}
+
+// The record of a placement that is through, from its sums in the region `base`; of several parts, see above.
 static __device__ __forceinline__ void walk_finish(const EvalParams& P, uint32_t base, uint32_t tr, uint32_t cand, bool use_mask,
-                                                   uint32_t cmask, uint32_t status, uint32_t extra) {
+                                                   uint32_t cmask, uint32_t status, uint32_t extra, uint32_t parts = 1) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint4 u0 = w4(base + 16u * lane), u1 = w4(base + 16u * lane + 512u), u2 = w4(base + 16u * lane + 1024u), u3 = w4(base + 16u * lane + 1536u);
     Stats st;
@@ -184,18 +216,21 @@ static __device__ __forceinline__ void walk_finish(const EvalParams& P, uint32_t
     st.hit = __reduce_add_sync(kWFull, u3.w);
     // the request count and the checksum of "everything rejected", from the per-class totals
     uint32_t counted_all = 0;
+    uint64_t rejected_sum = 0;
     for (uint32_t c = lane; c < P.n_classes; c += 32u)
         if (!use_mask || ((cmask >> c) & 1u)) {
             counted_all += (uint32_t)P.trace_class_tot[tr][2u * c];
-            st.checksum += P.trace_class_tot[tr][2u * c + 1u];
+            rejected_sum += P.trace_class_tot[tr][2u * c + 1u];
         }
     counted_all = __reduce_add_sync(kWFull, counted_all);
+    if (parts == 1u) st.checksum += rejected_sum;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         st.sum_ttft += (int64_t)wshfl_xor((uint64_t)st.sum_ttft, o);
         st.sum_e2e += (int64_t)wshfl_xor((uint64_t)st.sum_e2e, o);
         st.tokens += wshfl_xor(st.tokens, o);
         st.checksum += wshfl_xor(st.checksum, o);
+        rejected_sum += wshfl_xor(rejected_sum, o);
         st.max_ttft = max(st.max_ttft, (int64_t)wshfl_xor((uint64_t)st.max_ttft, o));
         st.max_e2e = max(st.max_e2e, (int64_t)wshfl_xor((uint64_t)st.max_e2e, o));
         st.makespan = max(st.makespan, (int64_t)wshfl_xor((uint64_t)st.makespan, o));
@@ -204,8 +239,9 @@ static __device__ __forceinline__ void walk_finish(const EvalParams& P, uint32_t
         uint32_t h[8];
 #pragma unroll
         for (int i = 0; i < 8; i++) h[i] = w1(base + kSByClass + 4u * i);
-        write_result(P.out + tr * P.n_cand + cand, status, counted_all, counted_all - st.served,
-                     (uint64_t)counted_all + extra, st, h);
+        maaso_result* const out = P.out + (size_t)tr * P.n_cand + cand;
+        if (parts == 1u) write_result(out, status, counted_all, counted_all - st.served, (uint64_t)counted_all + extra, st, h);
+        else walk_add_part(out, parts, status, counted_all, rejected_sum, st, h);
     }
     __syncwarp();
 }
@@ -300,7 +336,11 @@ struct Walk {
         constexpr uint32_t kCap = (uint32_t)kWalkRing;
         const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
         const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
-        const uint32_t total = P.bucket_count[bucket] * n_traces;
+        // With a queue in front of every instance the dispatcher never waits, and requests of one model leave no trace on the
+        // others': a placement can be replayed in parts, a model each, side by side (EvalParams::walk_parts).
+        constexpr bool kParts = Eng == 2 && !Big;
+        const uint32_t n_parts = kParts ? P.walk_parts : 1u;
+        const uint32_t total = P.bucket_count[bucket] * n_parts * n_traces;
         const uint32_t ring = L.ring + (threadIdx.x >> 5) * kWalkRing * 16u, ring_b = L.ring_b + (threadIdx.x >> 5) * kWalkRing * 8u;
         const bool use_mask = P.class_mask != nullptr && P.n_classes <= 32;
         const uint32_t models = base + kWalkSums, ents = models + 16u * P.n_models, ent = ents + 16u * lane;
@@ -309,10 +349,14 @@ struct Walk {
         while (idx < total) {
             // ---- the next placement ------------------------------------------------------------------------
             const uint32_t tr = idx % n_traces;
-            const uint32_t cand = P.bucket_list[(size_t)bucket * P.n_cand + idx / n_traces];
+            const uint32_t cand = P.bucket_list[(size_t)bucket * P.n_cand + idx / n_traces / n_parts];
             const uint4* const reqs = P.trace_reqs[tr];
             const uint32_t n_req = P.trace_n[tr];
             uint32_t n_i;
+            auto next = [&]() {
+                if (lane == 0) idx = static_total + atomicAdd(&P.walk_ctr[bucket - kWalkBucket0], 1u);
+                idx = __shfl_sync(kWFull, idx, 0);
+            };
             uint4 nxt = make_uint4(0u, 0u, 0u, 0u);  // the lane's request of the next chunk, as loaded
             if (n_req) nxt = __ldg(reqs + min(lane, n_req - 1u));
             Inst in;
@@ -394,9 +438,23 @@ struct Walk {
                 const uint2 r = w2(models + 16u * k + 8u);
                 hasmodel |= r.x < r.y ? 1u << k : 0u;
             }
+            uint32_t parts = 1, mine = 0xFFFFFFFFu;  // parts of the placement; models whose requests are this one's to report
+            if constexpr (kParts) {
+                if (n_parts > 1u) {
+                    const uint32_t k = idx / n_traces % n_parts;
+                    const bool first = k == (hasmodel ? (uint32_t)__ffs((int)hasmodel) - 1u : 0u);
+                    if (!first && !((hasmodel >> k) & 1u)) {  // (nothing of this model)
+                        next();
+                        continue;
+                    }
+                    parts = max(1u, (uint32_t)__popc(hasmodel));
+                    mine = (1u << k) | (first ? ~hasmodel : 0u);
+                    hasmodel &= 1u << k;
+                }
+            }
             const uint32_t cmask = use_mask ? P.class_mask[cand] : 0xFFFFFFFFu;
             const bool side = P.rej_by_model != nullptr || (P.dump_row && P.dump_row[cand] >= 0);
-            if (Wide) {
+            if (Wide && Eng != 2) {
                 // a placement handed over has left counts in its side outputs
                 const size_t oc = (size_t)tr * P.n_cand + cand;
                 if (P.rej_by_model && lane < (uint32_t)MAASO_MAX_MODELS) P.rej_by_model[oc * MAASO_MAX_MODELS + lane] = 0;
@@ -626,7 +684,7 @@ struct Walk {
             for (uint32_t cb = 0; cb < n_req; cb += 32u) {
                 take_chunk(nxt);
                 nxt = __ldg(reqs + min(cb + 32u + lane, n_req - 1u));
-                auto counted = [&]() { return cb + lane < n_req && ((cmask >> ((c_meta >> 16) & 31u)) & 1u); };
+                auto counted = [&]() { return cb + lane < n_req && ((cmask >> ((c_meta >> 16) & 31u)) & 1u) && (!kParts || ((mine >> (c_meta >> 24)) & 1u)); };
                 // Which of the chunk's requests from lane `from` on may need the distributor.
                 auto test = [&](uint32_t from) -> uint32_t {
                     const uint32_t Sm1 = (c_meta & 0xFFFFu) - 1u, model = c_meta >> 24;
@@ -837,13 +895,12 @@ struct Walk {
                 }
             }
             flush();
-            if (lane == 0) idx = static_total + atomicAdd(&P.walk_ctr[bucket - kWalkBucket0], 1u);
-            idx = __shfl_sync(kWFull, idx, 0);
+            next();
             if (!Wide && __any_sync(kWFull, bad)) {
                 if (lane == 0) walk_hand_over(P, cand, kFixed);
                 continue;
             }
-            walk_finish(P, base, tr, cand, use_mask, cmask, status, w1(base + kSExtra));
+            walk_finish(P, base, tr, cand, use_mask, cmask, status, w1(base + kSExtra), parts);
         }
     }
 };

@@ -59,3 +59,37 @@ def test_rounds(oracle_mod, case, flags):
     for mk in (None, mask):
         want = _check(oracle_mod, m, prof, tr, classes, off, inst, flags, mk)
     assert want["n_served"].max() > 100 and (want["attempts"] > want["n_counted"]).any()
+
+
+@pytest.mark.parametrize("flags", [8, 9])
+@pytest.mark.parametrize("n_models", [1, 2, 5])
+def test_queues_by_model(oracle_mod, n_models, flags):
+    """With queues the models of a placement are replayed side by side: placements of no, some and all models, requests of models
+    that a placement has no instance of (reported by one part only), several traces in one pass."""
+    import torch
+    import paper_2509_06362_b200 as m
+    from gpu_common import assert_records_equal
+    rng = np.random.default_rng(5)
+    W = gen.WMAX
+    prof = {"n_models": n_models, "n_strategies": 2, "wmax": W, "devices": np.ones(2, dtype=np.int32), "min_devices": np.ones(n_models, dtype=np.int32),
+            "prefill_base_us": rng.integers(0, 3000, size=(n_models, 2)).astype(np.int32), "prefill_q16": np.full((n_models, 2), 9000, dtype=np.int32),
+            "step_us": rng.integers(5000, 30_000, size=(n_models, 2, W)).astype(np.int32)}
+    lists = [[]] + [[(int(rng.integers(n_models)), int(rng.integers(2)), int(rng.choice([1, 3, 8, 64]))) for _ in range(int(rng.integers(1, 33)))] for _ in range(60)]
+    lists += [[(n_models - 1, 1, 2)], [(0, 0, 1)] * 33]
+    off, inst = gen.candidates_from_lists(lists)
+    tr = _requests(700, [0, 1000, 60_000], [1, 2, 100, 400], rng)
+    tr["model"] = rng.integers(0, n_models, size=len(tr))
+    classes = gen.make_classes([(None, None, None), (600_000, 20_000, None), (None, None, 9_000_000)])
+    mask = rng.integers(0, 8, size=len(lists)).astype(np.uint32)
+    for mk in (None, mask):
+        want = _check(oracle_mod, m, prof, tr, classes, off, inst, flags, mk)
+    assert want["n_served"].max() > 100 and (want["n_rejected"] > 0).any()
+    c = m.Context(0)
+    c.load_profile(prof)
+    traces = [tr, tr[:333], tr[:0], tr[100:]]
+    out = c.eval_placements_multi([c.load_trace(t, classes) for t in traces], c.to_device(off), c.to_device(inst), 10 ** 6, c.to_device(mask), flags)
+    torch.cuda.synchronize()
+    got = c.results_to_numpy(out).reshape(len(traces), len(lists))
+    for k, t in enumerate(traces):
+        assert_records_equal(got[k], oracle_mod.eval_placements(prof, t, classes, off, inst, 10 ** 6, mask, flags), f"trace {k}")
+    c.close()
