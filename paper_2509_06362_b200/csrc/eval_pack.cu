@@ -9,34 +9,43 @@
 //
 // The rest is the walking kernel's: 32-bit times from an epoch (here the same for the warp, moved to a request's
 // arrival), keys in shared memory, a ring of completions (one part per group) accounted by the group's lanes.  A running
-// request's first token and index (16 bytes per slot) and the sums are in global memory: what is left in shared memory is
-// the same for every placement, so that 16 warps always fit.  Of these a step waits for a completion's one load only (2.6 of
-// the 8 cycles between two instructions of a warp on 4,000 placements x 3,000 requests x 16 traces).
+// request's first token and index (8 bytes per slot) and the sums are in global memory: what is left in shared memory is
+// the same for every placement.  A completion copies them into its ring entry in the background (cp.async): waited for, that
+// load stopped all groups of the warp and took a quarter of the time (1.7 of 7.2 cycles between two instructions of a warp).
+// A slot has two entries in turn, so that a new occupant does not write what is still being copied.
 //
-// Measured (B200; 64-bit lane groups before, walking kernel in place of this one): 9,000 placements of one node x 5,000
-// requests at 2 a second 8.0 ms (13.3, 14.2), 10,864 x 10,000 x 16 arrival rates, optimistic estimate, 132 ms (214, 307); at 8 a
-// second half of the 9,000 are loaded and they walk (5.3 ms).  Groups of 2 lanes for placements of one and
-// two instances were slower (12.3 and 142 ms): 16 placements step through more completions one after the other than 8 do.
+// Measured (B200; with the load waited for, 64-bit lane groups, walking kernel in place of this one): 9,000 placements of one
+// node x 5,000 requests at 2 a second 6.1 ms (8.0, 13.3, 14.2), 10,864 x 2,500 x 16 arrival rates 29.5 (32.9), with the optimistic
+// estimate 31.9 (34.6); at 8 a second half of the 9,000 are loaded and they walk (5.3 ms, and less since).  Groups of 2 lanes for
+// placements of one and two instances were slower (12.3 against 9.4 and 142 against 132 ms): 16 placements step through more
+// completions one after the other than 8 do.  Dropped: what the next completion has to be accounted with kept in registers, loaded
+// when its key becomes the smallest (+30 % and more: the register's next load waits for the last); this kernel in the manner of
+// walk_dynamic.cuh (+4 to +33 %: it spills at 128 registers); the next request read by all lanes at once (-2 %, optimistic +4 %).
 #include "walk_kernel.cuh"
 
 namespace maaso {
 
+constexpr uint32_t kPackWarps = 14u;  // (launch_eval_pack)
 constexpr uint32_t kPackLane = 32u + 64u + 256u + 16u;  // block minima, free slots, keys; 16 bytes so that lanes start in different banks
-constexpr uint32_t kPackPay = 64u * 16u, kPackScratch = kPackPay + 128u;  // a lane's running requests; then sums (64 bytes), hits by class bin (32)
+// A lane's running requests, two entries per slot in turn: {first token from the epoch, request}; then sums (64 bytes), hits by
+// class bin (32).
+constexpr uint32_t kPackPay = 128u * 8u, kPackScratch = kPackPay + 128u;
+constexpr uint32_t kPackRelMax = (1u << 25) - 2u;  // largest end index of a key: end index << 7 | entry in turn << 6 | slot
 
 __host__ __device__ inline WalkLayout pack_layout(uint32_t n_rows, uint32_t n_classes) {
-    return walk_layout(n_rows, n_classes, false, (uint32_t)kWalkWarps);
+    return walk_layout(n_rows, n_classes, false, kPackWarps);
 }
-size_t pack_scratch(int grid) { return (size_t)grid * 32u * kWalkWarps * kPackScratch; }
+size_t pack_scratch(int grid) { return (size_t)grid * 32u * kPackWarps * kPackScratch; }
 bool pack_fits(uint32_t n_rows, uint32_t n_classes) {
-    return pack_layout(n_rows, n_classes).pool + 32u * kWalkWarps * kPackLane <= 227u * 1024u;
+    return pack_layout(n_rows, n_classes).pool + 32u * kPackWarps * kPackLane <= 227u * 1024u;
 }
 
-// Accounts a group's ring, one entry per lane and pass (lane `li` of `G`; `mine`: the lane's sums).  An entry: finish time from
-// the epoch, first-token time (61 bits), the instance in the group (3 bits), the request.
+// Accounts a group's ring, one entry per lane and pass (lane `li` of `G`; `mine`: the lane's sums).  An entry: first token from the
+// epoch, request, finish time from the epoch, instance.
 static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumping, uint32_t oc, unsigned char* mine, uint32_t* bins,
                                                  uint32_t ring, int64_t epoch, uint32_t li, uint32_t G, uint32_t cnt, uint32_t lims,
                                                  const uint4* reqs) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
     if (li < cnt) {
         uint4* const sums = reinterpret_cast<uint4*>(mine);
@@ -47,9 +56,9 @@ static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumpi
         uint32_t served = u3.z, hits = u3.w;
         for (uint32_t e = li; e < cnt; e += G) {
             const uint4 ra = w4(ring + e * 16u);
-            const uint2 rb = make_uint2(ra.w, ra.z >> 29);
+            const uint2 rb = make_uint2(ra.y, ra.w);
             const uint4 rec = __ldg(reqs + rb.x);
-            const int64_t fin = epoch + (int32_t)ra.x, first = i64_of(ra.y, ra.z & 0x1FFFFFFFu), arrival = i64_of(rec.x, rec.y);
+            const int64_t fin = epoch + (int32_t)ra.z, first = epoch + (int32_t)ra.x, arrival = i64_of(rec.x, rec.y);
             const uint32_t S = rec.w & 0xFFFFu, cls = (rec.w >> 16) & 0xFFu;
             const uint4 lim = w4(lims + cls * 16u);
             const int64_t ttft = first - arrival, e2e = fin - arrival;
@@ -82,6 +91,11 @@ static __device__ __noinline__ void pack_account(const EvalParams& P, bool dumpi
     __syncwarp();
 }
 
+// Copies what a running request must remember into its ring entry, in the background.
+__device__ __forceinline__ void copy_run(uint32_t entry, const uint2* run) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(entry + smem_addr(walk_smem)), "l"(run) : "memory");
+}
+
 // One warp takes work items, one after the other: 32 / G placements of the bucket whose groups have G lanes, the largest
 // placements first.  (One numbering for both buckets: starting on each from the same warps would have some replay an item
 // of each in a row where there is one item for each warp.)
@@ -96,7 +110,8 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     const uint32_t n8 = (P.bucket_count[kPack8] + 3u) / 4u, n4 = (P.bucket_count[kPack4] + 7u) / 8u;
     const uint32_t total = (n8 + n4) * n_traces;
     const uint32_t area = L.pool + threadIdx.x * kPackLane, keys = area + 96u;
-    unsigned char* const pay = reinterpret_cast<unsigned char*>(P.payload) + ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * kPackScratch;
+    unsigned char* const scratch = reinterpret_cast<unsigned char*>(P.payload) + ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * kPackScratch;
+    uint2* const pay = reinterpret_cast<uint2*>(scratch);
     const bool use_mask = P.class_mask != nullptr && P.n_classes <= 32;
 
     while (idx < total) {
@@ -132,7 +147,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         for (uint32_t i = 0; i < 8u + ((in.B + 7u) & ~7u); i++) w1(i < 8u ? area + 4u * i : keys + 4u * (i - 8u)) = kKeyEmpty;
         for (uint32_t i = 0; i < in.B; i++) walk_smem[area + 32u + i] = (unsigned char)i;
 #pragma unroll
-        for (uint32_t i = 0; i < 6u; i++) __stcg(reinterpret_cast<uint4*>(pay + kPackPay) + i, make_uint4(0u, 0u, 0u, 0u));
+        for (uint32_t i = 0; i < 6u; i++) __stcg(reinterpret_cast<uint4*>(scratch + kPackPay) + i, make_uint4(0u, 0u, 0u, 0u));
         __threadfence();
         __syncwarp();
         const uint32_t cmask = use_mask ? P.class_mask[cand] : 0xFFFFFFFFu;
@@ -143,9 +158,9 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         uint32_t c_in = 0, c_meta = 0;
         bool bad = false;  // a time of this lane has left the horizon: nothing is asked of it any more (see the walking kernel)
 
-        auto bins = [&]() { return reinterpret_cast<uint32_t*>(pay - li * kPackScratch + kPackPay + 64u); };
+        auto bins = [&]() { return reinterpret_cast<uint32_t*>(scratch - li * kPackScratch + kPackPay + 64u); };
         auto flush = [&]() {
-            pack_account(P, P.dump_row || P.ttft_hist, oc, pay + kPackPay, bins(), ring, epoch, li, G, ring_n, L.lims, reqs);
+            pack_account(P, P.dump_row || P.ttft_hist, oc, scratch + kPackPay, bins(), ring, epoch, li, G, ring_n, L.lims, reqs);
             ring_n = 0;
         };
         auto take_chunk = [&](const uint4& v) {
@@ -169,26 +184,27 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 const uint32_t adds = (uint32_t)__popc(dm & gmask);
                 if (__any_sync(kWFull, ring_n + adds > cap)) flush();
                 if (due) {
-                    const uint32_t slot = in.kmin & 63u, kb = keys + ((slot >> 3) << 5);
-                    const uint4 ft = __ldcg(reinterpret_cast<const uint4*>(pay) + slot);
+                    const uint32_t slot = in.kmin & 63u, run = in.kmin & 127u, kb = keys + ((slot >> 3) << 5);
+                    const uint32_t e = ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below));
+                    copy_run(e, pay + run);
                     w1(keys + (slot << 2)) = kKeyEmpty;
                     w1(area + ((slot >> 3) << 2)) = kKeyEmpty;
                     const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(area), m1 = w4(area + 16u);
                     const uint2 step = w2(in.row + 8u * in.w - 8u);
                     in.t = in.tb + (int32_t)in.sw;
-                    in.K = in.kmin >> 6;
+                    in.K = in.kmin >> 7;
                     in.w--;
-                    walk_smem[area + 32u + in.w] = (unsigned char)slot;
+                    walk_smem[area + 32u + in.w] = (unsigned char)(run ^ 64u);
+                    w2(e + 8u) = make_uint2((uint32_t)in.t, li);
                     const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                     const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
                     const uint32_t bmin = min8(kv);
                     w1(area + ((slot >> 3) << 2)) = bmin;
                     in.kmin = min(bmin, min8(mv));
-                    const uint32_t left = (in.kmin >> 6) - in.K;
+                    const uint32_t left = (in.kmin >> 7) - in.K;
                     const bool busy = in.w > 0;
                     next_end(left, busy, step);
                     due = busy & ((left == 0u) | (in.tb < upto)) & !bad;
-                    w4(ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below))) = make_uint4((uint32_t)in.t, ft.x, ft.y, ft.z);
                 }
                 ring_n += adds;
                 dm = __ballot_sync(kWFull, due);
@@ -221,6 +237,15 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                         catch_up(in.w < in.B, up);
                         in.t = in.t > up + kWPast ? in.t - up : kWPast;  // a full instance's clock is not looked at
                         in.tb -= up;
+                        // running requests' first tokens (further back than 32 bits reach: the lane has left the horizon)
+                        for (uint32_t s = 0; s < in.B; s++) {
+                            const uint32_t k = w1(keys + 4u * s);
+                            if (k == kKeyEmpty) continue;
+                            int32_t* const f = reinterpret_cast<int32_t*>(pay + (k & 127u));
+                            const int64_t v = (int64_t)*f - up;
+                            bad = bad || v < -(int64_t)kFar;
+                            *f = (int32_t)v;
+                        }
                     }
                     now = max(now - up, 0);
                     flush();
@@ -235,6 +260,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 now = max(now, arrival);  // pending time: the dispatcher never goes back
                 const int32_t pre = W::prefill(in.pre_base, in.pre_q16, in_tok);
                 bool act = counted;  // this group still has to place the request
+                asm volatile("cp.async.commit_group;" ::: "memory");  // what earlier steps copy (see the admission)
                 for (uint32_t tries = 1;; tries++) {
                     const bool elig = act & (((in.tag >> model) & 1u) != 0u) & !bad;
                     events(elig & (in.tb < now), now);
@@ -250,8 +276,9 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                     uint32_t best = min(key, __shfl_xor_sync(kWFull, key, 1));
                     best = min(best, __shfl_xor_sync(kWFull, best, 2));
                     if (G > 4u) best = min(best, __shfl_xor_sync(kWFull, best, 4));
-                    const int wl = __ffs((int)(__ballot_sync(kWFull, key == best) & gmask)) - 1;
-                    bool win = ((int)lane == wl) & (best < kTier1);
+                    const uint32_t equal = __ballot_sync(kWFull, key == best) & gmask;
+                    const bool chosen = (key == best) & ((equal & below) == 0u);  // (the winner, without a search for its bit)
+                    bool win = chosen & (best < kTier1);
                     const bool slow = act & (best >= kTier1);
                     bool again = false;
                     if (__any_sync(kWFull, slow)) {
@@ -259,11 +286,11 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                         // overflow protection: nobody can meet the deadline
                         if (side && slow && !waits && li == 0u && status == 0u) walk_reject_side(P, oc, cb + i, model);
                         // every capable instance is full: wait until the chosen slot frees
-                        const int32_t frees = __shfl_sync(kWFull, t, wl);
+                        const int32_t frees = __shfl_sync(kWFull, t, __ffs((int)equal) - 1);
                         if (waits) now = frees;
                         if (!Opt) {
                             // the second round cannot choose differently (see the walking kernel): it is only counted
-                            const bool mine = waits && (int)lane == wl;
+                            const bool mine = waits & chosen;
                             events(mine, now);
                             win = win || mine;
                             top = walk_smem[area + 32u + in.w];
@@ -282,25 +309,28 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                             in.t += pre;
                             if (in.w > 0) in.tb += pre;
                             bad = bad || in.t > kWalkHorizon || (in.w > 0 && in.tb > kWalkHorizon);
-                            const int64_t fin = epoch + in.t;
-                            w4(ring + ring_n * 16u) = make_uint4((uint32_t)in.t, lo32(fin), hi32(fin) | (li << 29), cb + i);
+                            w4(ring + ring_n * 16u) = make_uint4((uint32_t)in.t, cb + i, (uint32_t)in.t, li);
                         }
                         ring_n += adds;
-                    } else if (win) {
-                        in.t += pre;
-                        if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
-                        if (in.K + Sm1 > kRelMax) {
-                            in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K, in.kmin);
-                            in.K = 0;
+                    } else {
+                        // The entry taken now is the slot's last but one: copies of earlier steps have to be through, this step's not.
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        if (win) {
+                            in.t += pre;
+                            if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
+                            if (in.K + Sm1 > kPackRelMax) {
+                                in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K << 7, in.kmin);
+                                in.K = 0;
+                            }
+                            const uint32_t nk = ((in.K + Sm1) << 7) | top;
+                            w1(keys + 4u * (top & 63u)) = nk;
+                            pay[top] = make_uint2((uint32_t)in.t, cb + i);
+                            const uint32_t mb = area + ((top >> 1) & 28u);
+                            w1(mb) = min(w1(mb), nk);
+                            in.kmin = min(in.kmin, nk);
+                            in.w++;
+                            next_end((in.kmin >> 7) - in.K, true, more);
                         }
-                        const uint32_t nk = ((in.K + Sm1) << 6) | top;
-                        const int64_t first = epoch + in.t;
-                        w1(keys + 4u * top) = nk;
-                        __stcg(reinterpret_cast<uint4*>(pay) + top, make_uint4(lo32(first), hi32(first) | (li << 29), cb + i, 0u));
-                        atomicMin(&w1(area + ((top >> 3) << 2)), nk);
-                        in.kmin = min(in.kmin, nk);
-                        in.w++;
-                        next_end((in.kmin >> 6) - in.K, true, more);
                     }
                     if (!Opt) break;
                     act = again;
@@ -322,7 +352,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
         const bool away = (__ballot_sync(kWFull, bad) & gmask) != 0u;
         __threadfence();
         __syncwarp();
-        const uint4* const sums = reinterpret_cast<const uint4*>(pay + kPackPay);
+        const uint4* const sums = reinterpret_cast<const uint4*>(scratch + kPackPay);
         const uint4 u0 = __ldcg(sums), u1 = __ldcg(sums + 1), u2 = __ldcg(sums + 2), u3 = __ldcg(sums + 3);
         Stats st;
         st.sum_ttft = i64_of(u0.x, u0.y); st.max_ttft = i64_of(u0.z, u0.w);
@@ -364,7 +394,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     }
 }
 
-// `Warps`: 16 with 128 registers each, or 12 with room for 168 (launch_eval_pack).
+// `Warps`: 14 with 128 registers each, or 12 with room for 168 (launch_eval_pack).
 template <bool Opt, int Warps>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
     if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
@@ -389,15 +419,15 @@ static cudaError_t launch_pack(const EvalParams& P, int grid, cudaStream_t strea
     kernel<<<grid, 32 * Warps, smem, stream>>>(P);
     return cudaGetLastError();
 }
-// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which take
-// 150 to 154 registers there and spill nothing (16 warps: 68 to 76 bytes).  Measured, 12 and 16 warps: one node at 2 requests
-// a second, 9,000 x 5,000 8.0 and 9.2 ms; its 10,864 placements x 10,000 under 1, 2, 4 and 16 traces 13.7 and 16.0, 25.2 and
-// 28.8, 46.7 and 48.5, 134 and 127 (optimistic estimate 15.2 and 16.8, 27.4 and 29.7, 49.9 and 49.4, 144 and 131); three
-// models at 1 a second, 20,000 x 4,000 9.9 and 10.0, 40,000 17.7 and 16.4.  So the line is where it must lie for several
-// models and early for one, which 12 warps serve better up to about 40,000 placements.
+// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which take 152 to
+// 156 registers there and spill nothing (14 warps: 88 to 100 bytes).  14 and not 16 for the rest: their shared memory fits a
+// partition that leaves 60 KB of L1 instead of 28 (16 rates, 10,864 x 2,500: 29.5 and 31.7 ms, optimistic estimate 32.0 and 33.5).
+// Measured, 12 and 14 warps: one node's 10,864 x 4,000 under 1, 2 and 4 traces 5.0 and 5.2, 7.7 and 8.0, 13.6 and 13.2, 16 traces x
+// 2,500 30.9 and 29.5; three models at 1 a second, 20,000 x 4,000 11.8 and 11.3, 40,000 20.8 and 19.4.  So the line is where it must
+// lie for several models and early for one, which 12 warps serve better up to about 25,000 placements.
 cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
     const uint64_t placements = (uint64_t)P.n_cand * (P.n_traces > 1 ? P.n_traces : 1u);
-    return placements <= 6ull * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kWalkWarps>(P, grid, stream);
+    return placements <= 6ull * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kPackWarps>(P, grid, stream);
 }
 
 }  // namespace maaso

@@ -142,9 +142,8 @@ static __device__ __noinline__ void walk_account(const EvalParams& P, bool dumpi
     __syncwarp();
 }
 
-// All live end indices of one instance move down by the counter value K (which restarts at 0).  Rare.
-static __device__ __noinline__ uint32_t walk_rebase(uint32_t area, uint32_t keys, uint32_t nblk, uint32_t K, uint32_t kmin) {
-    const uint32_t d = K << 6;
+// All live keys of one instance move down by `d`, the counter's value in a key's place (the counter restarts at 0).  Rare.
+static __device__ __noinline__ uint32_t walk_rebase(uint32_t area, uint32_t keys, uint32_t nblk, uint32_t d, uint32_t kmin) {
     for (uint32_t b = 0; b <= nblk; b++) {
         const uint32_t p = b ? keys + 32u * (b - 1u) : area;  // the minima, then the keys of each block
         for (uint32_t i = 0; i < 8u; i++) {
@@ -660,7 +659,7 @@ struct Walk {
                     in.t += pre;
                     if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
                     if (in.K + Sm1 > kRelMax) {
-                        in.kmin = walk_rebase(in.area, in.keys, (in.B + 7u) >> 3, in.K, in.kmin);
+                        in.kmin = walk_rebase(in.area, in.keys, (in.B + 7u) >> 3, in.K << 6, in.kmin);
                         in.K = 0;
                     }
                     const uint32_t nk = ((in.K + Sm1) << 6) | slot;
