@@ -53,29 +53,34 @@ struct PermilleList {
     uint32_t v[16];
 };
 
-// Eight lanes per candidate: lane l holds bins 8l .. 8l+7 (two 16-byte loads; a warp reads four histograms), a scan
-// over the lanes gives the cumulative counts, lane j works out the target of rank j and keeps the bin it falls
-// into.  Bound by the read of the histograms; with 16 lanes and every lane working out every target it was bound
-// by instructions (10^6 histograms: 74 us, 218 that way, 496 with one thread per candidate).  Histograms are words, so
-// they may start at any word: beside a 16-byte boundary they are read word by word (`Words`).
+// Eight lanes per candidate: lane l holds bins 8l .. 8l+7 (two 16-byte loads; a warp reads four histograms), and a scan over
+// the lanes gives the cumulative counts.  They go to shared memory, where lane j searches for the bin that rank j falls into, six
+// steps for all ranks at once.  Bound by the read of the histograms and the instructions around it: 10^6 histograms, three
+// ranks, 67 us (every lane counting its bins below every target 75, every lane working out every target with 16 lanes a
+// histogram 218, one thread per histogram 496).  Histograms are words, so they may start at any word: beside a 16-byte
+// boundary they are read word by word (`Words`).  `U`: 32 bits where all counts of the warp's histograms are small.
 template <class U>
-__device__ __forceinline__ void percentiles_of(const U (&c)[8], U incl, uint32_t l, const PermilleList& pm, uint32_t n_p, int64_t* o, bool write) {
-    const U below = incl - c[7], total = __shfl_sync(0xFFFFFFFFu, incl, 7, 8);
-    for (uint32_t j0 = 0; j0 < n_p; j0 += 8u) {
-        const uint32_t p = j0 + l < n_p ? pm.v[j0 + l] : 1u;
-        U target = (U)(((uint64_t)p * total + 999u) / 1000u);
-        if (target < 1) target = 1;
-        uint32_t bin = 0;
-        for (uint32_t j = 0; j < 8u && j0 + j < n_p; j++) {
-            const U t = __shfl_sync(0xFFFFFFFFu, target, (int)j, 8);
-            uint32_t k = 8u * l;
+__device__ __forceinline__ void percentiles_of(const U (&c)[8], U below, U* all, uint32_t l, const PermilleList& pm, uint32_t n_p, int64_t* o, bool write) {
+    if constexpr (sizeof(U) == 4) {
+        uint4* const v = reinterpret_cast<uint4*>(all + 8u * l);
+        v[0] = make_uint4(below + c[0], below + c[1], below + c[2], below + c[3]);
+        v[1] = make_uint4(below + c[4], below + c[5], below + c[6], below + c[7]);
+    } else {
 #pragma unroll
-            for (int i = 0; i < 7; i++) k += below + c[i] < t ? 1u : 0u;
-            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, below < t && t <= incl) >> (threadIdx.x & 24u);
-            const uint32_t found = __shfl_sync(0xFFFFFFFFu, k, __ffs((int)(votes & 0xFFu)) - 1, 8);
-            if (j == l) bin = found;
-        }
-        if (write && j0 + l < n_p) o[j0 + l] = total ? ttft_bin_upper(bin) : -1;
+        for (int i = 0; i < 8; i++) all[8u * l + i] = below + c[i];
+    }
+    __syncwarp();
+    const U total = all[MAASO_TTFT_BINS - 1];
+    for (uint32_t j = l; j < n_p; j += 8u) {
+        const uint32_t p = pm.v[j];
+        // the rank's target count: ceil(p total / 1000), at least 1
+        U target = sizeof(U) == 4 && total <= 4000000u ? (U)((p * (uint32_t)total + 999u) / 1000u) : (U)(((uint64_t)p * total + 999u) / 1000u);
+        if (target < 1) target = 1;
+        uint32_t bin = 0;  // how many bins end below it
+#pragma unroll
+        for (uint32_t step = MAASO_TTFT_BINS / 2u; step > 0u; step >>= 1)
+            if (all[bin + step - 1u] < target) bin += step;
+        if (write) o[j] = total ? ttft_bin_upper(bin) : -1;
     }
 }
 
@@ -96,6 +101,8 @@ __global__ void __launch_bounds__(256) ttft_percentile_kernel(const uint32_t* hi
     }
     const bool small = (a.x | a.y | a.z | a.w | b.x | b.y | b.z | b.w) < (1u << 25);  // 64 of them stay below 2^31
     int64_t* const o = out + c * n_p;
+    __shared__ __align__(16) unsigned long long s_all[32 * (MAASO_TTFT_BINS + 2)];  // cumulative counts, a histogram per 8 threads
+    unsigned long long* const mine = s_all + (threadIdx.x >> 3) * (MAASO_TTFT_BINS + 2);
     if (__all_sync(0xFFFFFFFFu, small)) {
         uint32_t s[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
@@ -106,7 +113,7 @@ __global__ void __launch_bounds__(256) ttft_percentile_kernel(const uint32_t* hi
             const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, k, 8);
             if (l >= (uint32_t)k) incl += v;
         }
-        percentiles_of(s, incl, l, pm, n_p, o, c < n);
+        percentiles_of(s, incl - s[7], reinterpret_cast<uint32_t*>(mine), l, pm, n_p, o, c < n);
     } else {
         unsigned long long s[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
@@ -117,7 +124,7 @@ __global__ void __launch_bounds__(256) ttft_percentile_kernel(const uint32_t* hi
             const unsigned long long v = __shfl_up_sync(0xFFFFFFFFu, incl, k, 8);
             if (l >= (uint32_t)k) incl += v;
         }
-        percentiles_of(s, incl, l, pm, n_p, o, c < n);
+        percentiles_of(s, incl - s[7], mine, l, pm, n_p, o, c < n);
     }
 }
 
