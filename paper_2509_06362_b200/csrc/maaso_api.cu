@@ -643,8 +643,9 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         // models under load, 500 x 10,000 1.64 and 1.36, 2,000 2.40 and 1.86, 5,000 2.55 and 2.30, 10,000 3.2 and 4.1, 40,000 11.9 and
         // 15.5; at 16 a second 10,000 x 5,000 4.0 and 4.5.  The warps per block go by the parts (6,000 of them 7.2 ms with 12, 5.3 with 16).
         P.walk_parts = queues && (uint64_t)C * n_traces <= 3ull * ctx->sm_count * kWalkWarpsFew ? ctx->n_models : 1u;
-        P.walk_warps = (uint64_t)C * n_traces * P.walk_parts <= 3ull * ctx->sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
-        P.walk_usual = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, queues, P.walk_warps, !(o.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES))).pool) / P.walk_warps) & ~15u;
+        const bool fixed_speed = (o.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
+        P.walk_warps = fixed_speed && (uint64_t)C * n_traces * P.walk_parts <= 3ull * ctx->sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
+        P.walk_usual = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, queues, P.walk_warps, !fixed_speed).pool) / P.walk_warps) & ~15u;
     }
     const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;

@@ -5,11 +5,12 @@
 
 namespace maaso {
 
-// Warps per block, one block per SM: 16 with 128 registers each, or 12 with room for 168 (142 to 156 are used) for a batch of
-// at most three placements per warp, which its longest chains bound.  Measured, 12 and 16 warps: 2,000 x 17,000 of the
-// paper's shape 9.7 and 10.2 ms; three models under load, 1,000 to 4,440 x 10,000, 1.15 to 1.28 and 1.19 to 1.34; 100,000 x
-// 100,000 117 and 100.  The line is a compromise: a lightly loaded batch, whose placements all take as long, has it at one
-// placement per warp (one node at 2 requests a second, 1,776 x 5,000 3.5 and 3.6 ms, 2,368 6.3 and 4.0, 5,328 10.0 and 8.3).
+// Warps per block, one block per SM: 16 with 128 registers each.  12 with room for 168 serve the engines that fix a request's
+// speed better in a batch of at most three placements (or parts of them) per warp, which its longest chains bound (2,000 x
+// 17,000 of the paper's shape 9.5 and 9.75 ms, with queues 1,000 x 8,000 2.14 and 2.20; 12,000 x 30,000 under load 5.5 and 4.7).
+// With the default engine 12 are 0 to 4 % better where they are better at all (one node, 2,368 x 5,000 1.91 and 1.95 ms, three
+// models under load 7,000 x 10,000 1.43 and 1.48) and lose where 16 hold the batch at once or it is lightly loaded (one node
+// at 2 requests a second, 2,368 x 4,000 3.55 and 2.32; the paper's shape, 3,000 x 8,000 4.1 and 3.4): 16 always.
 constexpr int kWalkWarps = 16, kWalkWarpsFew = 12;
 constexpr int kWalkRing = 64;                     // ring entries per warp
 
