@@ -23,7 +23,8 @@ struct WalkLayout {
     uint32_t ring_b;  // 64-bit times: [warps][kWalkRing] {request, instance}
     uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
     uint32_t wide;    // 64-bit times: [n_classes] {TTFT limit (2^62 = none), TBT limit (negative = none)}
-    uint32_t steps;   // [n_rows][65] {decode step, 2^32 / step} by running count; a count of 0: {1, 2^32}, an idle clock
+    uint32_t steps;   // [n_rows][65] {decode step, 2^32 / step} by running count (walk_dynamic.cuh: exact
+                      // reciprocals); a count of 0: a step of 1, an idle clock
     uint32_t list;    // `list`: [warps][kWalkList], requests that need a round, and the dummy region (walk_dynamic.cuh)
     uint32_t pool;
 };
@@ -44,14 +45,15 @@ __host__ __device__ inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_cl
 // a lower bound per model, then per instance its slots: the eight block minima, the stack of free slots (a byte
 // each), the keys (end index << 6 | slot, in blocks of 8), then what a running request must remember: {first-token time,
 // request index}, 8 bytes (64-bit times: the request indices, then the first-token times).  Keys alone with more than 32
-// instances, where the rest is in global memory: shared memory decides how many such placements are resident.  In the engines that fix a request's speed at admission: the finish
-// times in falling order, so that the next to free is popped off the end.
+// instances, where the rest is in global memory: shared memory decides how many such placements are resident.  In the
+// engines that fix a request's speed at admission: the finish times in falling order, so that the next to free is popped
+// off the end.
 enum WalkKind : uint32_t { kWalkUsual = 0, kWalkBigKind = 1, kWalkLongKind = 2 };
 constexpr uint32_t kWalkLaneSums = 4u * 32u * 16u;
 constexpr uint32_t kWalkSums = kWalkLaneSums + 48u;
 constexpr uint32_t kWalkBig = 32u;  // more instances than this rest in shared memory
 __host__ __device__ inline uint32_t walk_slots_at(uint32_t nblk) { return 32u + ((8u * nblk + 15u) & ~15u); }
-// `block`: bytes of 8 slots; kWalkBlock: {keys, what the running requests must remember} by block, from a fixed offset on
+// `block`: bytes of 8 slots; kWalkBlock (walk_dynamic.cuh): keys and the rest behind them from a fixed offset on
 constexpr uint32_t kWalkKeys = 96u;
 constexpr uint32_t kWalkBlock = 96u, kWalkBlockLong = 128u, kWalkBlockKeys = 32u;
 __host__ __device__ inline uint32_t walk_slot_bytes(uint32_t b, bool fixed_speed, uint32_t key_bytes, uint32_t block) {

@@ -19,13 +19,15 @@
 // Nothing is counted per rejected request: the request count and the checksum of "all of them rejected"
 // are per-class totals of the trace, and a served request takes its own term out again.
 //
+// What nearly every call runs, the default engine with up to 32 instances and 32-bit times, has a body of its own, written for
+// the shortest round (walk_dynamic.cuh).  `Walk` here is the body of all the others.
+//
 // Measured (B200, whole calls with routing and top-k; lane-group, thread or one-warp kernel before): 143 placements x 500
-// requests 0.23 ms (0.56), one node's 10,864 x 10,000 6.8 ms (12.0), 2,000 x 17,000 of the paper's shape 9.5 ms (33.9), with
-// queues 11.0 ms (27.8), three models, 100,000 x 100,000 under load 99.7 ms (135), 64 of their placements x 20,000 with all side
-// outputs 2.0 to 3.1 ms (13.8 to 14.1), 2,000 placements of 33 to 128 instances x 10,000 7.9 to 8.3 ms (13.8).  A round with one completion takes 300 warp instructions and, alone on its scheduler,
-// 1,130 cycles, almost all of them dependent: what the next step needs is therefore read from shared memory ahead of
-// the choice, the uncommon outcomes share one branch, and tests of several conditions are written without branches
-// (& and | for && and ||: 652 -> 576 ns a round, 100,000 x 100,000 under load 115 -> 100 ms).
+// requests 0.17 ms (0.56), one node's 10,864 x 10,000 4.6 ms (12.0), 2,000 x 17,000 of the paper's shape 6.4 to 6.6 ms (33.9), with
+// queues 5.3 ms (27.8), with fixed speeds 9.5 ms, three models, 100,000 x 100,000 under load 92.4 ms (135), 2,000 placements of 33
+// to 128 instances x 10,000 8.1 to 8.7 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
+// needs is therefore read from shared memory ahead of the choice, the uncommon outcomes share one branch, and tests of several
+// conditions are written without branches (& and | for && and ||).
 //
 // The block's pool of shared memory is split evenly among its warps.  Placements beyond one warp's part run
 // first, with half, a quarter, ... of the warps at work and twice, four times, ... the room for each (kWalkModes);
@@ -293,14 +295,6 @@ struct Walk {
             const bool end = (int64_t)((uint64_t)Sm1 * step + since) <= i64_of(a.z, a.w);  // (no branches)
             if constexpr (Wide) return (int64_t)since <= ttft && (Sm1 == 0u || tbt < 0 || (int64_t)step <= tbt) && end;
             else return (since <= a.x) & ((Sm1 == 0u) | (step <= a.y)) & end;
-        }
-        // The same for 32-bit times as a bound of `since`, so that one comparison is left when the start is known:
-        // met(since) = since < before().
-        __device__ __forceinline__ uint32_t before(uint32_t Sm1, uint32_t step) const {
-            const int64_t left = i64_of(a.z, a.w) - (int64_t)((uint64_t)Sm1 * step);  // up to 2^62, or negative
-            const uint32_t e = (uint32_t)(left >> 32) == 0u ? lo32(left) : 0xFFFFFFFEu;  // (no time is as long)
-            const bool never = (left < 0) | ((Sm1 != 0u) & (step > a.y));
-            return never ? 0u : min(min(a.x, e), 0xFFFFFFFEu) + 1u;
         }
     };
     static __device__ __forceinline__ T prefill(uint32_t base, uint32_t q16, uint32_t in_tok) {
