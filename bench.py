@@ -32,9 +32,9 @@ TOPK = 64
 PROFILED = {
     "workload": "multimodel", "mapping": 0, "kernel": "eval_walk_kernel",
     # profiles/eval_walk_kernel_multimodel_sweep_counters.md: one launch of the default workload
-    "warp_inst_per_launch": 76319382253,                 # smsp__inst_executed.sum
-    "dram_bytes_per_launch": 4908032 + 512,               # dram__bytes_read.sum + dram__bytes_write.sum
-    "csrc_sha256": "fdd8cdd12aef03086dd4e52fb4e6df6325b21526eab3f213ee3ede400cd3bc54",
+    "warp_inst_per_launch": 66498140425,                 # smsp__inst_executed.sum
+    "dram_bytes_per_launch": 4945408 + 189696,            # dram__bytes_read.sum + dram__bytes_write.sum
+    "csrc_sha256": "9f92edcd031a9cebb784ff3a27038def3adfefd3878ec6b3ebf69a72719d44a6",
 }
 SM_COUNT, ISSUE_PER_SM = 148, 4   # B200: 148 SMs x 4 warp schedulers, one warp instruction per cycle each
 

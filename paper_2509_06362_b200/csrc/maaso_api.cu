@@ -652,19 +652,14 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,
     // which several placements of one warp share in the packed kernel; its steps take the same time however few placements
     // there are, so that the line lies where the walking kernel needs as long.  Measured on 4,000 requests, walking and packed:
-    //   one model     at 1 a second 3,000 placements 5.5 and 5.7 ms, 4,096 7.9 and 5.7; at 2 a second 4,096 6.1 and 6.0, 5,000
-    //                 8.0 and 6.1; at 4 a second 6,144 6.1 and 6.4, 8,192 7.9 and 6.6
-    //   two models    at 1 a second 8,192 7.7 and 8.3, 10,240 9.4 and 8.5; at 2 a second 12,288 8.5 and 9.3, 16,384 10.7 and 10.4;
-    //                 at 4 a second 32,768 12.7 and 14.0
-    //   three models  (a third of the lanes of a step at work) at 1 a second 10,240 7.9 and 7.9; at 2 a second 16,384 9.2 and 9.5,
-    //                 24,576 13.0 and 12.9; at 4 a second 32,768 11.5 and 12.9
-    //   16 models     (which the placements serve few of) at 2 a second 16,384 3.3 and 4.5, 98,304 18.2 and 22.3, 163,840 30.1 and
-    //                 35.9: walking is the better one at every size
-    // that is between 3,100 and 6,600 placements for one model and between 9,000 and more than 32,768 for several.  With fixed
-    // speeds or queues the alternative is the lane-group kernel.  Fixed speeds: 6,200 and more, 9,100 and more.
-    // Queues cost the walking kernel more, and for several models the line is late there: one model at 2 a second 4,096 7.3 and
-    // 8.1, 5,000 9.6 and 8.3; two models 6,144 7.2 and 7.8, 8,192 9.0 and 7.9; three 8,192 7.4 and 7.7, 10,240 8.9 and 7.7, 16,384
-    // 13.0 and 10.0.
+    //   one model     at 1 a second 3,000 placements 4.1 and 4.1 ms, 4,096 4.5 and 4.15, 5,000 5.5 and 4.3; at 2 a second 4,096 4.4
+    //                 and 4.35, 5,000 4.5 and 4.5, 6,500 6.3 and 4.65; at 4 a second 6,500 4.4 and 4.6, 8,192 5.7 and 4.8
+    //   three models  (a third of the lanes of a step at work) at 1 a second 12,288 7.6 and 8.5, 18,432 10.8 and 10.4; at 2 a second
+    //                 18,432 8.4 and 10.0, 40,000 16.9 and 17.2; at 4 a second 40,000 11.6 and 15.1 (and walking by its load, below)
+    // With the optimistic estimate one model at 2 a second 4,096 5.05 and 4.85, three 12,288 7.4 and 8.1, 24,576 13.7 and 12.4.
+    // With fixed speeds or queues the alternative is the lane-group kernel; measured before the walking kernel's bodies parted: fixed
+    // speeds equal at 6,200 and more, 9,100 and more with several models; queues at 3,600 to 7,300, with two models 4,900 to 10,100,
+    // with three 7,200 to 11,400 (so that for several models the line is late there).
     const uint64_t walk_most = ctx->n_models == 1 ? 4096u : 6144u * (uint64_t)ctx->n_models;
     P.walk_all = walk && (uint64_t)C * n_traces <= walk_most ? 1u : 0u;
     const bool packs = walk && !P.walk_all && !P.walk_long && !variant && pack_fits(P.n_rows, P.n_classes);
