@@ -3,7 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
-#include "../../include/maaso.h"
+#include "route.cuh"
 
 namespace maaso {
 
@@ -12,23 +12,6 @@ constexpr int kRowStride = 66;  // int32 per profile row: prefill base, prefill 
 constexpr uint64_t kKeyInf = ~0ull;
 constexpr long long kWaitCycles = 4000000000ll;  // bound on any device-side wait (~2 s)
 
-// Buckets the validation kernel sorts candidates into.
-// 0..5: lane groups of 1,2,4,8,16,32 lanes (one lane per instance)
-// 6..8: block layout with 2, 4, 8 warps, one warp per instance, state in registers
-// 9:    block layout with 16 warps striding over up to 128 instances, state in shared memory
-// 10..18: thread mapping, by how many lanes of a warp work at a time (32, 24, 16, 12, 8, 6, 4, 2, 1:
-//        the larger the placements, the fewer fit the warp's pools)
-// 20..30: walking kernel (walk.cuh): up to 32 instances by the room a placement needs (one, 2, 4, 8, 16 times a
-//        warp's part), more than 32, 64-bit times by the room
-constexpr int kNumBuckets = 31;
-constexpr int kWalkModes = 5;
-constexpr int kWalkBucket0 = 20, kWalkBig0 = kWalkBucket0 + kWalkModes, kWalkLong0 = kWalkBig0 + 1;
-constexpr int kWalkBuckets = 2 * kWalkModes + 1;
-constexpr int kGenericBlockBucket = 9;
-constexpr int kThreadBucket0 = 10;  // buckets 10..18: the thread mapping, by lanes per warp
-constexpr int kThreadBuckets = 9;
-constexpr int kPack4 = 2, kPack8 = 3;  // in place of the lane groups (EvalParams::pack): up to 4 and up to 8 instances
-constexpr int kWideBucket = 19;     // 33..128 instances under the engines of the lane-group code: one warp per placement
 constexpr int kPrepOne = 1024;   // candidates one block of the validation kernel takes
 constexpr int kCostBins = 256;   // bin 0 = most expensive (largest total batch cap)
 constexpr int kCounterWords = 28160;  // counters | work counters | histograms + cursors, cleared per call
@@ -241,10 +224,9 @@ __device__ __forceinline__ void bulk_load(void* dst_smem, const void* src_gmem, 
 }
 
 // Everything a scoring kernel needs, passed by value.
-struct EvalParams {
+struct EvalParams : Route {
     const uint4* reqs;
     uint32_t n_req;
-    uint32_t n_classes;
     const int64_t* classes;  // [n_classes][3]
     const uint4* cooked;     // [n_req][kCookedWords] prepared records (lane-group kernel)
     // several traces in one launch (lane-group kernel only): trace t of n_traces > 1 has
@@ -262,15 +244,13 @@ struct EvalParams {
     const int32_t* rows;     // [n_rows][kRowStride]
     const int32_t* devices;
     const int32_t* min_devices;
-    uint32_t n_rows, n_models, n_strategies;
+    uint32_t n_strategies;
     uint32_t budget;
     const uint32_t* offsets;
     const uint32_t* inst;
     const uint32_t* class_mask;  // null, or ignored when n_classes > 32
     uint32_t n_cand;
     uint32_t n_inst;
-    uint32_t flags;
-    uint32_t mapping;
     maaso_result* out;
     uint32_t* bucket_count;  // [64]: candidates per bucket after planning, and the kCtr* counters
     uint32_t* bucket_list;   // [kNumBuckets][n_cand], each bucket sorted by decreasing cost estimate
@@ -279,21 +259,12 @@ struct EvalParams {
     uint32_t* code;          // [n_cand] lane-group / block bucket << 8 | cost bin, 0xFFFFFFFF if none
     uint32_t* code2;         // [n_cand] walking or thread bucket << 8 | cost bin, 0xFFFFFFFF if none
     uint32_t demand_tok_s;   // output tokens per second the trace(s) ask for
-    uint32_t walk_all;        // MAASO_MAP_AUTO: the batch goes to the walking kernel whatever its load
     uint32_t thread_min_cand; // MAASO_MAP_AUTO: fewest loaded candidates for which the thread mapping is chosen
     uint32_t group_warps;    // warps the lane-group grid keeps resident (capacity for promotions)
     uint32_t* sm_ctr;        // [n_sm] next work item of each SM's share (lane-group kernel)
     uint32_t n_sm;
     uint32_t promote_pct;
-    uint32_t thread_pool_units;  // thread mapping: 16-byte units one warp has for the cold part of its placements' state
-    uint32_t thread_hot_units;   // and for the hot part (3 units per instance, shared memory)
     uint32_t* walk_ctr;      // [kWalkBuckets]: next placement of each walking bucket
-    uint32_t walk_bytes;     // walking kernel: bytes of shared memory one of 16 warps has for a placement, 0 = not used
-    uint32_t walk_usual;     // the same for placements of up to 32 instances, with walk_warps warps
-    uint32_t pack;           // placements of at most 8 instances that could go to the lane groups share the steps of a warp instead
-    uint32_t walk_warps;
-    uint32_t walk_parts;     // queues: parts a placement is replayed in, 1 or the number of models
-    uint32_t walk_long;      // the whole batch with 64-bit times
     long long wait_cycles;   // bound of every device-side wait
     uint32_t stall_test;     // test hook: never issue the trace copies
     int32_t* dump_row;       // [n_cand] or null

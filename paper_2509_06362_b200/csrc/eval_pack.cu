@@ -25,20 +25,12 @@
 
 namespace maaso {
 
-constexpr uint32_t kPackWarps = 14u;  // (launch_eval_pack)
-constexpr uint32_t kPackLane = 32u + 64u + 256u + 16u;  // block minima, free slots, keys; 16 bytes so that lanes start in different banks
 // A lane's running requests, two entries per slot in turn: {first token from the epoch, request}; then sums (64 bytes), hits by
 // class bin (32).
 constexpr uint32_t kPackPay = 128u * 8u, kPackScratch = kPackPay + 128u;
 constexpr uint32_t kPackRelMax = (1u << 25) - 2u;  // largest end index of a key: end index << 7 | entry in turn << 6 | slot
 
-__host__ __device__ inline WalkLayout pack_layout(uint32_t n_rows, uint32_t n_classes) {
-    return walk_layout(n_rows, n_classes, false, kPackWarps);
-}
 size_t pack_scratch(int grid) { return (size_t)grid * 32u * kPackWarps * kPackScratch; }
-bool pack_fits(uint32_t n_rows, uint32_t n_classes) {
-    return pack_layout(n_rows, n_classes).pool + 32u * kPackWarps * kPackLane <= 227u * 1024u;
-}
 
 // Accounts a group's ring, one entry per lane and pass (lane `li` of `G`; `mine`: the lane's sums).  An entry: first token from the
 // epoch, request, finish time from the epoch, instance.

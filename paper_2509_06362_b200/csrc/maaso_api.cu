@@ -26,7 +26,6 @@ uint32_t thread_fixed_smem(uint32_t n_models, uint32_t n_rows);
 cudaError_t launch_eval_walk(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream);
 size_t pack_scratch(int grid);
-bool pack_fits(uint32_t n_rows, uint32_t n_classes);
 cudaError_t launch_eval_walk_big(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_walk_long(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_wide(const EvalParams& P, int grid, cudaStream_t stream);
@@ -616,10 +615,6 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     P.ttft_hist = o.ttft_hist;
 
     // launch shapes: persistent grids bounded by what the batch can use
-    // Blocks per SM of the lane-group kernel.  A batch that three blocks per SM can hold in one
-    // wave is bound by its longest dependent chains, which run faster with fewer warps sharing a
-    // scheduler; a larger batch is bound by instruction issue and wants all four.  Lanes needed
-    // ~ instances x 1.3 (group widths are powers of two).
     // the walking kernel runs everything but the largest-gap test of the default engine; with 64-bit times where
     // 32-bit ones cannot hold the batch's tables or limits
     const bool walk = o.mapping == MAASO_MAP_AUTO && !(o.flags & MAASO_FLAG_TBT_MAXGAP) && (variant || C < ctx->thread_min_cand);
@@ -633,50 +628,11 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
             const double ahead = pre * (double)traces[t]->n + (double)ctx->max_step * traces[t]->max_out;
             may_leave = may_leave || o.flags != 0 || (double)kWalkNowMax + 2.0 * ahead >= (double)kWalkHorizon;
         }
-        const bool queues = (o.flags & MAASO_FLAG_INSTANCE_QUEUES) != 0;  // always with 64-bit times
-        P.walk_long = fits || queues ? 0u : 1u;
-        may_leave = may_leave && !queues;
-        P.walk_bytes = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, true, kWalkWarps).pool) / kWalkWarps) & ~15u;
-        // With queues the models of a placement are independent of one another and can be replayed side by side, while the batch is
-        // bound by its longest chains: every part scans the whole trace.  Whole and in parts: the paper's shape (three models),
-        // 300 x 8,000 3.4 and 2.0 ms, 1,000 4.15 and 2.15, 5,000 7.9 and 5.7, 18,000 18.3 and 17.7, 2,000 x 17,000 9.25 and 5.35; three
-        // models under load, 500 x 10,000 1.64 and 1.36, 2,000 2.40 and 1.86, 5,000 2.55 and 2.30, 10,000 3.2 and 4.1, 40,000 11.9 and
-        // 15.5; at 16 a second 10,000 x 5,000 4.0 and 4.5.  The warps per block go by the parts (6,000 of them 7.2 ms with 12, 5.3 with 16).
-        P.walk_parts = queues && (uint64_t)C * n_traces <= 3ull * ctx->sm_count * kWalkWarpsFew ? ctx->n_models : 1u;
-        const bool fixed_speed = (o.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
-        P.walk_warps = fixed_speed && (uint64_t)C * n_traces * P.walk_parts <= 3ull * ctx->sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
-        P.walk_usual = ((227u * 1024u - walk_layout(P.n_rows, P.n_classes, queues, P.walk_warps, !fixed_speed).pool) / P.walk_warps) & ~15u;
+        may_leave = may_leave && !(o.flags & MAASO_FLAG_INSTANCE_QUEUES);
+        route_walk(P, (uint64_t)C * n_traces, (uint32_t)ctx->sm_count, fits);
     }
     const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;
-    // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,
-    // which several placements of one warp share in the packed kernel; its steps take the same time however few placements
-    // there are, so that the line lies where the walking kernel needs as long.  Measured on 4,000 requests, walking and packed:
-    //   one model     at 1 a second 3,000 placements 4.1 and 4.1 ms, 4,096 4.5 and 4.15, 5,000 5.5 and 4.3; at 2 a second 4,096 4.4
-    //                 and 4.35, 5,000 4.5 and 4.5, 6,500 6.3 and 4.65; at 4 a second 6,500 4.4 and 4.6, 8,192 5.7 and 4.8
-    //   three models  (a third of the lanes of a step at work) at 1 a second 12,288 7.6 and 8.5, 18,432 10.8 and 10.4; at 2 a second
-    //                 18,432 8.4 and 10.0, 40,000 16.9 and 17.2; at 4 a second 40,000 11.6 and 15.1 (and walking by its load, below)
-    // With the optimistic estimate one model at 2 a second 4,096 5.05 and 4.85, three 12,288 7.4 and 8.1, 24,576 13.7 and 12.4.
-    // With fixed speeds or queues the alternative is the lane-group kernel; measured before the walking kernel's bodies parted: fixed
-    // speeds equal at 6,200 and more, 9,100 and more with several models; queues at 3,600 to 7,300, with two models 4,900 to 10,100,
-    // with three 7,200 to 11,400 (so that for several models the line is late there).
-    const uint64_t walk_most = ctx->n_models == 1 ? 4096u : 6144u * (uint64_t)ctx->n_models;
-    P.walk_all = walk && (uint64_t)C * n_traces <= walk_most ? 1u : 0u;
-    const bool packs = walk && !P.walk_all && !P.walk_long && !variant && pack_fits(P.n_rows, P.n_classes);
-    P.pack = packs ? 1u : 0u;
-    const bool groups = !packs && !P.walk_all && (o.mapping == MAASO_MAP_GROUP || o.mapping == MAASO_MAP_AUTO);
-    int group_blocks = ctx->group_blocks;
-    if (group_blocks == 0) {
-        const uint64_t est_warps = ((cands->n_inst * 13 / 10 + 31) / 32 + 6) * n_traces;
-        group_blocks = est_warps <= (uint64_t)ctx->sm_count * 3 * (kGroupThreads / 32) ? 3 : 4;
-    }
-    // blocks of the walking kernel for more than 32 instances: a block per placement at most
-    int grid_big = 0;
-    if (walk && !P.walk_long && cands->n_inst > kWalkBig) {
-        const uint64_t most = cands->n_inst / (kWalkBig + 1) * n_traces;
-        grid_big = most < (uint64_t)ctx->sm_count ? (int)most : ctx->sm_count;
-    }
-    const bool away = grid_big > 0 && !variant;  // its running requests are in global memory
     int grid_g = 0, grid_t = 0;
     uint32_t thread_pool = 0, thread_hot = 0;
     size_t pay_entries = 0, pay_thread = 0;  // scratch entries of the lane-group / block kernels, of the thread kernel
@@ -684,7 +640,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     if (threads) {
         // thread mapping: one-warp blocks; the pool is what is left of an SM's shared memory when
         // `thread_blocks` of them share it (1 KB per block is reserved by the system)
-        // The hot part of the instances (what a prediction reads: 3 units each) is always in shared memory;
+        // The hot part of the instances (what a prediction reads: 2 units each) is always in shared memory;
         // the cold part (slot masks and keys) is in shared memory too, or in a per-warp arena in global memory,
         // which leaves room for more resident warps.
         size_t pool, hot;
@@ -716,7 +672,24 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         pay_thread = ((size_t)grid_t * (thread_scratch_per_warp(thread_pool) + (ctx->thread_arena_kb > 0 ? thread_pool : 0)) +
                       sizeof(Payload) - 1) / sizeof(Payload);
     }
-    if (groups) {
+    const Launches L = route_launches(P, cands->n_inst, may_leave);
+    // Blocks per SM of the lane-group kernel.  A batch that three blocks per SM can hold in one
+    // wave is bound by its longest dependent chains, which run faster with fewer warps sharing a
+    // scheduler; a larger batch is bound by instruction issue and wants all four.  Lanes needed
+    // ~ instances x 1.3 (group widths are powers of two).
+    int group_blocks = ctx->group_blocks;
+    if (group_blocks == 0) {
+        const uint64_t est_warps = ((cands->n_inst * 13 / 10 + 31) / 32 + 6) * n_traces;
+        group_blocks = est_warps <= (uint64_t)ctx->sm_count * 3 * (kGroupThreads / 32) ? 3 : 4;
+    }
+    // blocks of the walking kernel for more than 32 instances: a block per placement at most
+    int grid_big = 0;
+    if (L.big) {
+        const uint64_t most = cands->n_inst / (kWalkBig + 1) * n_traces;
+        grid_big = most < (uint64_t)ctx->sm_count ? (int)most : ctx->sm_count;
+    }
+    const bool away = grid_big > 0 && !variant;  // its running requests are in global memory
+    if (L.groups) {
         const int occ_g = occupancy_eval_group(P, tile, group_blocks, ctx->smem_per_sm);
         grid_g = ctx->sm_count * occ_g;
         // at most one work item per 4 candidates + bucket tails, once per trace
@@ -724,12 +697,12 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         if ((uint64_t)grid_g > max_items_g) grid_g = (int)max_items_g;
         pay_entries = (size_t)grid_g * kGroupThreads * (group_scratch_per_lane() / sizeof(Payload));
     }
-    if (packs) pay_entries = pack_scratch(ctx->sm_count) / sizeof(Payload);
+    if (L.pack) pay_entries = pack_scratch(ctx->sm_count) / sizeof(Payload);
     int grid_b[4];
     for (int b = 6; b <= kGenericBlockBucket; b++) {
         // the block kernels run only when the block mapping is asked for
         grid_b[b - 6] = 0;
-        if (!(n_traces == 1 && o.mapping == MAASO_MAP_BLOCK)) continue;
+        if (!(n_traces == 1 && L.blocks)) continue;
         // placements with at most 8 instances: one warp per instance with register-resident state
         int gb = ctx->sm_count * (b < kGenericBlockBucket ? occupancy_eval_block_reg(P, b, tile)
                                                         : occupancy_eval_block(P, b, tile));
@@ -739,12 +712,10 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         if (need > pay_entries) pay_entries = need;
     }
 
-    // placements of more than 32 instances outside the thread kernel (the other engines; the default engine
-    // unless the batch goes to the threads; whatever the thread kernel's pools cannot hold): one warp per
-    // placement with the lane-group code
+    // one warp per placement with the lane-group code: placements of more than 32 instances outside the walking and the thread
+    // kernel, and whatever those have no room for
     int grid_w = 0;
-    // (the walking kernel takes all of them, unless tables of more than a hundred rows leave its pool no room)
-    if (o.mapping != MAASO_MAP_BLOCK && cands->n_inst > 32 && !(walk && (P.walk_bytes << (kWalkModes - 1)) >= kWalkMost)) {
+    if (L.wide_from) {
         // As many warps per SM as the registers allow (8) where the batch is made of large placements (more
         // than 16 instances per placement on average): the kernel waits on dependent chains, and four more
         // warps per SM are worth a third of its time.  Elsewhere 4 per SM, which needs no more scratch than
@@ -753,10 +724,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         const int occ_cap = cands->n_inst > 16ull * C ? 8 : 4;
         if (occ_w > occ_cap) occ_w = occ_cap;
         grid_w = ctx->sm_count * occ_w;
-        // a placement that needs this kernel has more than 32 instances (or, thread mapping forced, more state
-        // than a warp's pools): the batch cannot hold more of them than instances / 33
-        uint64_t max_items_w = (o.mapping == MAASO_MAP_THREAD ? (uint64_t)C : cands->n_inst / 33u) * n_traces;
-        if (max_items_w < 1) max_items_w = 1;
+        uint64_t max_items_w = cands->n_inst / L.wide_from * n_traces;  // (it has that many instances at least)
         if ((uint64_t)grid_w > max_items_w) grid_w = (int)max_items_w;
         const size_t need = ((size_t)grid_w * wide_scratch_per_warp() + sizeof(Payload) - 1) / sizeof(Payload);
         if (need > pay_entries) pay_entries = need;
@@ -800,7 +768,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         // and packed, between the two lines: one node 5,000 at 6 and 8 a second 2.5 and 4.5, 2.1 and 4.4 ms, 10,864 at 8 3.9 and 5.1,
         // 14,000 at 6 6.1 and 5.5, 20,000 at 6 and 8 8.5 and 6.1, 6.2 and 5.5; three models at 4 a second 24,576 7.4 and 10.0, 40,000
         // 11.5 and 15.0.  Below both: 10,864 at 6 a second 5.0 and 5.2, three models at 2 a second 24,576 10.9 and 11.3.
-        const bool early = packs && (ctx->n_models > 1 || (uint64_t)C * n_traces <= 7ull * kWalkWarpsFew * ctx->sm_count);
+        const bool early = L.pack && (ctx->n_models > 1 || (uint64_t)C * n_traces <= 7ull * kWalkWarpsFew * ctx->sm_count);
         const double d = n_traces / inv * (early ? 2.0 : 1.0);
         P.demand_tok_s = d >= 4.0e9 ? 4000000000u : (uint32_t)d;
     }
@@ -815,23 +783,23 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
     e = launch_prep(P, o.dump_cand_idx, stream, &launches);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "prep launch");
     if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
-    if (groups) {
+    if (L.groups) {
         e = launch_eval_group(P, grid_g, tile, group_blocks, ctx->smem_per_sm, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel launch");
     }
-    if (packs) {
+    if (L.pack) {
         e = launch_eval_pack(P, ctx->sm_count, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "packed kernel launch");
     }
-    if (walk && !P.walk_long) {
+    if (L.walk) {
         e = launch_eval_walk(P, ctx->sm_count, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[2], stream);
-    if (threads) {
+    if (L.threads) {
         // the thread kernel has scratch of its own; its arena (if any) follows the entries of the running requests
         EvalParams PT = P;
         PT.payload = reinterpret_cast<Payload*>(sb + off_pay_t);
@@ -850,7 +818,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     }
-    if (walk && (P.walk_long || may_leave || packs)) {
+    if (L.far) {
         e = launch_eval_walk_long(P, ctx->sm_count, stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");

@@ -22,14 +22,8 @@ struct Place {
 __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c) {
     const uint32_t lo = P.offsets[c], hi = P.offsets[c + 1];
     uint32_t status = 0, n = 0, sum_b = 0;
-    uint32_t units = 0;  // thread mapping: 16-byte units of cold instance state (per instance 2 + key blocks + minima)
-    uint32_t slot_bytes = 0, slot_bytes64 = 0;  // walking kernel: shared memory of its instances' slots, with 64-bit times too
+    PlacementSize size = {0u, 0u, 0u, 0u};
     uint64_t supply = 0; // decode tokens per second the placement can produce with every slot busy
-    const bool variant = (P.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_TBT_MAXGAP | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
-    const bool fixed_speed = (P.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES)) != 0;
-    const bool queues = (P.flags & MAASO_FLAG_INSTANCE_QUEUES) != 0;  // always with 64-bit times
-    const bool threads_ok = !variant && (P.mapping == MAASO_MAP_THREAD || (P.mapping == MAASO_MAP_AUTO && !P.walk_bytes));
-    const bool groups_ok = P.mapping != MAASO_MAP_THREAD;
     if (hi < lo || hi > P.n_inst) {
         status = MAASO_CAND_EBADINST;  // malformed CSR row
     } else {
@@ -37,7 +31,7 @@ __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c
         if (n > MAASO_MAX_INSTANCES) {
             status = MAASO_CAND_ETOOMANY;
         } else {
-            const uint32_t key_bytes = fixed_speed && (P.walk_long || queues) ? 8u : 4u;
+            size.n = n;
             uint64_t devsum = 0;
             for (uint32_t i = 0; i < n; i++) {
                 const uint32_t word = P.inst[lo + i];
@@ -47,9 +41,7 @@ __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c
                     continue;
                 }
                 sum_b += b;
-                slot_bytes += walk_slot_bytes(b, fixed_speed, key_bytes, P.walk_long ? kWalkBlockLong : (n > kWalkBig ? kWalkBlockKeys : kWalkBlock));
-                slot_bytes64 += walk_slot_bytes(b, fixed_speed, fixed_speed ? 8u : 4u, kWalkBlockLong);
-                units += 2u + 2u * ((b + 7u) >> 3) + 2u;
+                size.add(P, b);
                 supply += b * 1000000u / (uint32_t)P.rows[(m * P.n_strategies + s) * kRowStride + 1 + b];
                 devsum += (uint64_t)P.devices[s];
                 if (P.devices[s] < P.min_devices[m]) status |= MAASO_CAND_EMEMFIT;
@@ -57,38 +49,8 @@ __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c
             if (devsum > P.budget) status |= MAASO_CAND_EBUDGET;
         }
     }
-    // where it can go
-    int bg = -1, bt = -1;
-    uint32_t need = 0;  // room in the walking kernel
-    if (!status) {
-        if (threads_ok) {
-            // as many lanes per item as placements of this size fit the warp's pools
-            const uint32_t fit = n ? min(P.thread_pool_units / units, P.thread_hot_units / (2u * n)) : 32u;
-            const uint32_t lanes[9] = {32, 24, 16, 12, 8, 6, 4, 2, 1};
-            for (int i = 0; i < 9; i++)
-                if (fit >= lanes[i]) { bt = kThreadBucket0 + i; break; }
-        }
-        if (P.walk_bytes) {
-            const bool big = n > kWalkBig && !P.walk_long;
-            need = walk_region_bytes(P.n_models, n, slot_bytes, P.walk_long || queues ? kWalkLongKind : (big ? kWalkBigKind : kWalkUsual));
-            if (big) {
-                // (and all of the pool has to hold it if it is handed over)
-                if (max(need, walk_region_bytes(P.n_models, n, slot_bytes64, kWalkLongKind)) <= P.walk_bytes * (uint32_t)kWalkWarps) bt = kWalkBig0;
-            } else {
-                // one warp's part of the walking kernel's pool, or 2, 4, 8 of them (16 with 64-bit times)
-                const uint32_t part = P.walk_long ? P.walk_bytes : P.walk_usual;
-                for (uint32_t k = 0; k < (uint32_t)kWalkModes - 1u && bt < 0; k++)
-                    if (need <= (part << k)) bt = (P.walk_long ? kWalkLong0 : kWalkBucket0) + (int)k;
-                if (bt < 0 && P.walk_long && need <= part * 16u) bt = kWalkLong0 + 4;
-            }
-        }
-        if (P.mapping == MAASO_MAP_BLOCK) bg = n <= 2 ? 6 : (n <= 4 ? 7 : (n <= 8 ? 8 : kGenericBlockBucket));
-        else if (P.pack) bg = n <= 4 ? kPack4 : (n <= 8 ? kPack8 : -1);  // (what the pack kernel needs room for leaves the walking kernel room for all)
-        else if (groups_ok && n <= 32) bg = n <= 1 ? 0 : 32 - __clz((int)(n - 1));
-        // More than 32 instances outside the walking and the thread kernel: one warp per placement with the lane-group
-        // code.  (One block per placement only when the block mapping is asked for.)
-        else if (bt < 0 || (groups_ok && !P.walk_bytes)) bg = kWideBucket;
-    }
+    Home home = {-1, -1, 0u};
+    if (!status) home = route_home(P, size);
     if (P.dump_row) P.dump_row[c] = -1;
     const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
     for (uint32_t t = 0; t < n_traces; t++) {
@@ -104,8 +66,8 @@ __device__ __forceinline__ Place place_candidate(const EvalParams& P, uint32_t c
     const uint32_t bin = (kCostBins - 1) - min((uint32_t)(kCostBins - 1), sum_b / 8u);
     Place r;
     r.status = status;
-    r.code = bg >= 0 ? (((uint32_t)bg << 8) | bin) : kNowhere;
-    r.code2 = bt >= 0 ? (((uint32_t)bt << 8) | (bt == kWalkBig0 ? walk_big_bin(need) : bin)) : kNowhere;
+    r.code = home.group >= 0 ? (((uint32_t)home.group << 8) | bin) : kNowhere;
+    r.code2 = home.walk >= 0 ? (((uint32_t)home.walk << 8) | (home.walk == kWalkBig0 ? walk_big_bin(home.need) : bin)) : kNowhere;
     r.loaded = (uint64_t)P.demand_tok_s >= 2ull * supply;
     return r;
 }

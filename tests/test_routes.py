@@ -1,0 +1,49 @@
+"""Routing (csrc/route.cuh, compiled here without CUDA): whatever the tables, classes, models, sizes and batch caps, every valid
+placement goes to a kernel that its call launches.  A placement without one would keep its "not scored" record."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+OPTIMISTIC, FROZEN, MAXGAP, QUEUES = 1, 2, 4, 8
+AUTO, BLOCK, GROUP, THREAD = 0, 1, 2, 3
+
+
+@pytest.fixture(scope="module")
+def routes(tmp_path_factory):
+    lib = str(tmp_path_factory.mktemp("routes") / "libroutes.so")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC", "-o", lib, os.path.join(HERE, "route_host.cpp")])
+    lib = ctypes.CDLL(lib)
+    u32, u64 = ctypes.c_uint32, ctypes.c_uint64
+    lib.routes_unscored.restype = lib.routes_wide_from.restype = u32
+    lib.routes_unscored.argtypes = [u32, u32, u64, u32, u32, u32, ctypes.POINTER(u32)]
+    lib.routes_wide_from.argtypes = [u32, u32, u32, u32, u32, u64, u32, u32, u32]
+    return lib
+
+
+def _unscored(routes, flags, mapping, items, fits32=1, pool=0, hot=0):
+    first = (ctypes.c_uint32 * 5)()
+    n = routes.routes_unscored(flags, mapping, items, fits32, pool, hot, first)
+    return n, dict(zip(("rows", "models", "classes", "instances", "cap"), first)) if n else None
+
+
+@pytest.mark.parametrize("flags", [0, OPTIMISTIC, FROZEN, QUEUES])
+@pytest.mark.parametrize("fits32", [1, 0])
+@pytest.mark.parametrize("items", [1, 1000, 4096, 4097, 6000, 100_000, 10 ** 7])
+def test_every_placement_has_a_kernel(routes, flags, fits32, items):
+    assert _unscored(routes, flags, AUTO, items, fits32) == (0, None)
+
+
+@pytest.mark.parametrize("mapping", [BLOCK, GROUP])
+def test_every_placement_has_a_kernel_where_the_mapping_is_asked_for(routes, mapping):
+    assert _unscored(routes, 0, mapping, 1000) == (0, None)
+    assert _unscored(routes, MAXGAP, GROUP, 1000) == (0, None)
+
+
+@pytest.mark.parametrize("pool, hot", [(128 << 10, 10 << 10), (30 << 10, 7 << 10), (4096, 1536), (8192, 2048)])
+def test_every_placement_has_a_kernel_with_threads(routes, pool, hot):
+    """(The pools' default sizes, and small ones that hold few instances.)"""
+    assert _unscored(routes, 0, THREAD, 1000, 1, pool, hot) == (0, None)
+    assert _unscored(routes, 0, AUTO, 1000, 1, pool, hot) == (0, None)
