@@ -130,7 +130,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                 const uint32_t word = P.inst[lo + li], md = word & 0xFu, r = md * P.n_strategies + ((word >> 4) & 0xFFu);
                 in.tag = 1u << md;
                 in.B = (word >> 12) & 0xFFu;
-                in.row = L.steps + r * kWalkRow;
+                in.row = L.steps + r * kWalkRowRcp;
                 in.pre_base = (uint32_t)P.rows[r * kRowStride];
                 in.pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
                 in.stepB = w1(in.row + 8u * in.B);
@@ -393,7 +393,10 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_c
     if (P.bucket_count[kPack4] + P.bucket_count[kPack8] == 0) return;
     const WalkLayout L = pack_layout(P.n_rows, P.n_classes);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
-    for (uint32_t i = tid; i < P.n_rows * 65u; i += 32u * Warps) w2(L.steps + 8u * i) = walk_step_entry(P, i);
+    for (uint32_t i = tid; i < P.n_rows * 65u; i += 32u * Warps) {
+        const uint32_t s = walk_step(P, i);
+        w2(L.steps + 8u * i) = make_uint2(s, walk_rcp(s));
+    }
     for (uint32_t c = tid; c < P.n_classes; c += 32u * Warps) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u], le = e < 0 ? (int64_t)1 << 62 : e;
         w4(L.lims + 16u * c) = make_uint4(a < 0 ? 0xFFFFFFFFu : (uint32_t)a, b < 0 ? 0xFFFFFFFFu : (uint32_t)b, lo32(le), hi32(le));

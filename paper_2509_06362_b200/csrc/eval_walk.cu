@@ -7,13 +7,15 @@ template <int Warps>
 static cudaError_t launch_fixed_speed(const EvalParams& P, int grid, cudaStream_t stream) {
     const bool opt = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) != 0;
     if (P.flags & MAASO_FLAG_INSTANCE_QUEUES)
-        return opt ? launch_walk<true, 2, true, false, Warps>(P, grid, stream) : launch_walk<false, 2, true, false, Warps>(P, grid, stream);
-    return opt ? launch_walk<true, 1, false, false, Warps>(P, grid, stream) : launch_walk<false, 1, false, false, Warps>(P, grid, stream);
+        return opt ? launch_walk<true, 2, true, false, false, Warps>(P, grid, stream) : launch_walk<false, 2, true, false, false, Warps>(P, grid, stream);
+    return opt ? launch_walk<true, 1, false, false, false, Warps>(P, grid, stream) : launch_walk<false, 1, false, false, false, Warps>(P, grid, stream);
 }
 cudaError_t launch_eval_walk(const EvalParams& P, int grid, cudaStream_t stream) {
     if (P.flags & (MAASO_FLAG_ENGINE_FROZEN | MAASO_FLAG_INSTANCE_QUEUES))
         return P.walk_warps == (uint32_t)kWalkWarpsFew ? launch_fixed_speed<kWalkWarpsFew>(P, grid, stream) : launch_fixed_speed<kWalkWarps>(P, grid, stream);
-    return (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) ? launch_walk<true, 0, false, false>(P, grid, stream) : launch_walk<false, 0, false, false>(P, grid, stream);
+    const bool opt = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) != 0;
+    if (P.walk_rcp) return opt ? launch_walk<true, 0, false, false, true>(P, grid, stream) : launch_walk<false, 0, false, false, true>(P, grid, stream);
+    return opt ? launch_walk<true, 0, false, false, false>(P, grid, stream) : launch_walk<false, 0, false, false, false>(P, grid, stream);
 }
 
 }  // namespace maaso

@@ -44,7 +44,16 @@ constexpr uint32_t kPackWarps = 14u;              // of the packed kernel (launc
 constexpr int kWalkRing = 64;                     // ring entries per warp
 constexpr uint32_t kBlockShared = 227u * 1024u;   // shared memory of a block
 
-constexpr uint32_t kWalkRow = 65u * 8u;           // bytes of a decode-step row
+// Decode-step rows in shared memory: steps alone, or each with its reciprocal, which spares the rounds a division and takes twice
+// the room.  The engines that fix a request's speed never divide by a step: steps alone.  The others carry reciprocals up to so
+// many rows; beyond that the room is worth more (more placements fit one warp's part of the pool).  Measured, with and without:
+//   up to 32 instances, 32-bit times: 12,000 x 10,000 under load, 100 rows 1.73 and 1.84 ms, 120 1.68 and 1.69, 160 1.76 and 1.70,
+//     256 2.36 and 2.01; 4,000 x 8,000 lightly loaded, 120 rows 2.29 and 2.54, 160 3.22 and 2.24; some 20 instances each, 6,000 x
+//     8,000, 100 rows 4.02 and 4.04, 120 3.03 and 2.97, 160 2.88 and 2.66
+//   more than 32: 2,000 x 5,000, 50 rows 9.29 and 9.39, 60 9.63 and 8.56, 100 7.53 and 6.82
+//   64-bit times: 5 to 6 % better with, up to 100 rows.  The line there is where the pool still holds every placement.
+constexpr uint32_t kWalkRow = 65u * 4u, kWalkRowRcp = 65u * 8u;  // bytes of a row
+constexpr uint32_t kWalkRcpRows = 128u, kWalkRcpRowsBig = 52u, kWalkRcpRowsLong = 80u;
 constexpr uint32_t kWalkList = 33u * 32u + 128u;  // list of 32 requests and one behind it, what lanes without an instance read
 
 // One block of the walking kernel (walk_kernel.cuh): the completion rings, SLO limits, decode-step tables, the pool.
@@ -53,19 +62,19 @@ struct WalkLayout {
     uint32_t ring_b;  // 64-bit times: [warps][kWalkRing] {request, instance}
     uint32_t lims;    // [n_classes] {TTFT limit, TBT limit (all ones = none), end-to-end limit (64 bits, 2^62 = none)}
     uint32_t wide;    // 64-bit times: [n_classes] {TTFT limit (2^62 = none), TBT limit (negative = none)}
-    uint32_t steps;   // [n_rows][65] {decode step, 2^32 / step} by running count (walk_dynamic.cuh: exact
-                      // reciprocals); a count of 0: a step of 1, an idle clock
+    uint32_t steps;   // [n_rows][65] decode step by running count, `rcp`: {step, reciprocal}, which is 2^32 / step or (walk_dynamic.cuh)
+                      // an exact one; a count of 0: a step of 1, an idle clock
     uint32_t list;    // `list`: [warps][kWalkList], requests that need a round, and the dummy region (walk_dynamic.cuh)
     uint32_t pool;
 };
-MAASO_HD inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes, bool wide, uint32_t warps, bool list = false) {
+MAASO_HD inline WalkLayout walk_layout(uint32_t n_rows, uint32_t n_classes, bool wide, uint32_t warps, bool rcp, bool list = false) {
     WalkLayout l;
     l.ring = 0;
     l.ring_b = warps * (uint32_t)kWalkRing * 16u;
     l.lims = l.ring_b + (wide ? warps * (uint32_t)kWalkRing * 8u : 0u);
     l.wide = l.lims + n_classes * 16u;
     l.steps = l.wide + (wide ? n_classes * 16u : 0u);
-    l.list = (l.steps + n_rows * kWalkRow + 15u) & ~15u;
+    l.list = (l.steps + n_rows * (rcp ? kWalkRowRcp : kWalkRow) + 15u) & ~15u;
     l.pool = (l.list + (list ? warps * kWalkList : 0u) + 127u) & ~127u;
     return l;
 }
@@ -104,7 +113,7 @@ MAASO_HD inline uint32_t walk_big_bin(uint32_t need) {
 
 // Packed kernel (eval_pack.cu): a lane's block minima, free slots, keys; 16 bytes so that lanes start in different banks.
 constexpr uint32_t kPackLane = 32u + 64u + 256u + 16u;
-MAASO_HD inline WalkLayout pack_layout(uint32_t n_rows, uint32_t n_classes) { return walk_layout(n_rows, n_classes, false, kPackWarps); }
+MAASO_HD inline WalkLayout pack_layout(uint32_t n_rows, uint32_t n_classes) { return walk_layout(n_rows, n_classes, false, kPackWarps, true); }
 inline bool pack_fits(uint32_t n_rows, uint32_t n_classes) {
     return pack_layout(n_rows, n_classes).pool + 32u * kPackWarps * kPackLane <= kBlockShared;
 }
@@ -116,6 +125,8 @@ struct Route {
     uint32_t walk_bytes;     // walking kernel: bytes of shared memory one of 16 warps has for a placement, 0 = not used
     uint32_t walk_usual;     // the same for placements of up to 32 instances, with walk_warps warps
     uint32_t walk_warps;
+    uint32_t walk_rcp;       // decode-step rows of the walking kernel carry reciprocals: up to 32 instances and 32-bit times,
+    uint32_t walk_rcp_big;   // more instances or 64-bit times
     uint32_t walk_parts;     // queues: parts a placement is replayed in, 1 or the number of models
     uint32_t walk_long;      // the whole batch with 64-bit times
     uint32_t walk_all;       // MAASO_MAP_AUTO: the batch goes to the walking kernel whatever its load
@@ -133,7 +144,9 @@ inline void route_walk(Route& r, uint64_t items, uint32_t sm_count, bool fits32)
     const bool queues = (r.flags & MAASO_FLAG_INSTANCE_QUEUES) != 0;  // always with 64-bit times
     const bool fixed_speed = route_fixed_speed(r.flags);
     r.walk_long = fits32 || queues ? 0u : 1u;
-    r.walk_bytes = ((kBlockShared - walk_layout(r.n_rows, r.n_classes, true, kWalkWarps).pool) / kWalkWarps) & ~15u;
+    r.walk_rcp = !fixed_speed && r.n_rows <= kWalkRcpRows ? 1u : 0u;
+    r.walk_rcp_big = !fixed_speed && r.n_rows <= (r.walk_long ? kWalkRcpRowsLong : kWalkRcpRowsBig) ? 1u : 0u;
+    r.walk_bytes = ((kBlockShared - walk_layout(r.n_rows, r.n_classes, true, kWalkWarps, r.walk_rcp_big != 0).pool) / kWalkWarps) & ~15u;
     // With queues the models of a placement are independent of one another and can be replayed side by side, while the batch is
     // bound by its longest chains: every part scans the whole trace.  Whole and in parts: the paper's shape (three models),
     // 300 x 8,000 3.4 and 2.0 ms, 1,000 4.15 and 2.15, 5,000 7.9 and 5.7, 18,000 18.3 and 17.7, 2,000 x 17,000 9.25 and 5.35; three
@@ -141,7 +154,7 @@ inline void route_walk(Route& r, uint64_t items, uint32_t sm_count, bool fits32)
     // 15.5; at 16 a second 10,000 x 5,000 4.0 and 4.5.  The warps per block go by the parts (6,000 of them 7.2 ms with 12, 5.3 with 16).
     r.walk_parts = queues && items <= 3ull * sm_count * kWalkWarpsFew ? r.n_models : 1u;
     r.walk_warps = fixed_speed && items * r.walk_parts <= 3ull * sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
-    r.walk_usual = ((kBlockShared - walk_layout(r.n_rows, r.n_classes, queues, r.walk_warps, !fixed_speed).pool) / r.walk_warps) & ~15u;
+    r.walk_usual = ((kBlockShared - walk_layout(r.n_rows, r.n_classes, queues, r.walk_warps, r.walk_rcp != 0, !fixed_speed).pool) / r.walk_warps) & ~15u;
     // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,
     // which several placements of one warp share in the packed kernel; its steps take the same time however few placements
     // there are, so that the line lies where the walking kernel needs as long.  Measured on 4,000 requests, walking and packed:

@@ -12,7 +12,8 @@
 //   - the choice's key names the lane: one minimum and one comparison;
 //   - the usual path shares no value with the uncommon ones (what merged with them cost 30 instructions a round);
 //   - a wait is one operation on the winner's slots: the request takes over the slot that frees;
-//   - a step count is a high product and a shift (exact reciprocals), without a correction;
+//   - a step count is a high product and a shift (exact reciprocals), without a correction (large tables, whose rows have none: a
+//     division);
 //   - chunks that need no round are skipped in a loop of their own;
 //   - shared memory is addressed directly (5 % against references into the block's array);
 //   - lower bounds for the scan are written when a list is through, not on every round.
@@ -27,9 +28,7 @@ namespace maaso {
 
 // ceil(dt / s) = (2 (dt + s - 1) m >> 32) >> L with L = ceil(log2 s), m = ceil(2^(31 + L) / s) < 2^32: exact for dt + s - 1 <
 // 2^31 (m s - 2^(31 + L) < s <= 2^L; Granlund and Montgomery's division by an invariant).  A row's entry: {s << 5 | L, m}.
-__device__ __forceinline__ uint2 walk_exact_entry(const EvalParams& P, uint32_t i) {
-    const uint32_t r = i / 65u, w = i - 65u * r;
-    const uint32_t s = w ? max((uint32_t)P.rows[r * kRowStride + 1u + w], 1u) : 1u;
+__device__ __forceinline__ uint2 walk_exact_entry(uint32_t s) {
     const uint32_t sh = s > 1u ? 32u - (uint32_t)__clz((int)(s - 1u)) : 0u;
     return make_uint2((s << 5) | sh, (uint32_t)((((uint64_t)1 << (31u + sh)) + (s - 1u)) / s));
 }
@@ -72,8 +71,10 @@ __device__ __forceinline__ void st1(uint32_t a, uint32_t v) { asm volatile("st.s
 __device__ __forceinline__ void stb(uint32_t a, uint32_t v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void min_shared(uint32_t a, uint32_t v) { asm volatile("red.shared.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 
-template <bool Opt>
+// `Rcp`: the decode-step rows carry reciprocals.
+template <bool Opt, bool Rcp>
 struct WalkDynamic {
+    static constexpr uint32_t kEntry = Rcp ? 8u : 4u;
     using Limits = typename Walk<Opt, 0, false, false>::Limits;
     static constexpr int32_t kFar = kWalkFar;
     // A key: tier << 31 | (predicted first token - now, at most kOffMax) << 5 | lane.  From kOffMax on (a minute ahead) the
@@ -128,15 +129,15 @@ struct WalkDynamic {
                     bit = 1u << md;  // of its model; 0 from when it has left the horizon on: nothing is asked of it any more (see Walk)
                     place = e.y;
                     B = (e.x >> 12) & 0xFFu;
-                    row = L.steps + r * kWalkRow;
+                    row = L.steps + r * (Rcp ? kWalkRowRcp : kWalkRow);
                     pre_base = (uint32_t)P.rows[r * kRowStride];
                     pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
-                    stepB = ld1(row + 8u * B) >> 5;
+                    stepB = ld1(row + kEntry * B) >> 5;
                     // the smallest step a prediction can use: the step at the batch cap, or (optimistic estimate) at any
                     // level up to it
                     low_step = stepB;
                     if (Opt)
-                        for (uint32_t l = 1; l < B; l++) low_step = min(low_step, ld1(row + 8u * l) >> 5);
+                        for (uint32_t l = 1; l < B; l++) low_step = min(low_step, ld1(row + kEntry * l) >> 5);
                     min_shared(models + 16u * md, pre_base);
                     min_shared(models + 16u * md + 4u, low_step);
                     // per instance: earliest start, prefill base and slope, smallest prediction step
@@ -185,8 +186,12 @@ struct WalkDynamic {
                 c_in = v.z;
                 c_meta = v.w;
             };
+            auto entry = [&](uint32_t at) -> uint2 {
+                if constexpr (Rcp) return ld2(at);
+                else return make_uint2(ld1(at), 0u);
+            };
             auto peek = [&]() {
-                more = ld2(row + 8u * w + 8u);
+                more = entry(row + kEntry * w + kEntry);
                 top = ldb(area + 32u + w);  // (a full instance's is not looked at)
                 top_min = ld1(area + ((top >> 1) & 28u));
             };
@@ -209,7 +214,7 @@ struct WalkDynamic {
                     st1(keys + 4u * s, kKeyEmpty);
                     st1(mb, kKeyEmpty);
                     const uint4 k0 = ld4(kb), k1 = ld4(kb + 16u), m0 = ld4(area), m1 = ld4(area + 16u);
-                    const uint2 cur = ld2(row + 8u * w - 8u), run = ld2(pay + 8u * s);
+                    const uint2 cur = entry(row + kEntry * w - kEntry), run = ld2(pay + 8u * s);
                     const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                     const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
                     if (!stay) {
@@ -244,7 +249,8 @@ struct WalkDynamic {
             };
             // Decode steps until `dt` later; 2 (dt + step - 1) < 2^32.
             auto steps_of = [&](int32_t dt) -> uint32_t {
-                return __funnelshift_r(__umulhi(2u * ((uint32_t)dt + sw - 1u), rcp), 0u, step);
+                if constexpr (Rcp) return __funnelshift_r(__umulhi(2u * ((uint32_t)dt + sw - 1u), rcp), 0u, step);
+                else return ((uint32_t)dt + sw - 1u) / sw;
             };
             auto start = [&]() -> int32_t { return w == B ? tc : t; };
             // What is rare, out of the rounds' way.  Moves the epoch for request `src` of the chunk at `cb`, to the dispatcher's

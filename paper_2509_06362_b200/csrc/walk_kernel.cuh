@@ -42,6 +42,7 @@
 //           horizon in mid-trace and are handed over
 //   Big     more than 32 instances: lane l takes instances l, l + 32, ... one after the other (those of a model are
 //           neighbours, so a round looks at one or two of these strides); their state rests in shared memory
+//   Rcp     decode-step rows carry reciprocals (route.cuh: which tables' rows do)
 #pragma once
 #include <cstring>
 #include <type_traits>
@@ -90,10 +91,9 @@ __device__ __forceinline__ uint32_t walk_steps(int64_t dt, uint32_t s, uint32_t 
     return (d >> 32) == 0 ? walk_steps((int32_t)dt, s, rs) : (uint32_t)(d / s);
 }
 // Entry i of the decode-step rows in shared memory (WalkLayout::steps).
-__device__ __forceinline__ uint2 walk_step_entry(const EvalParams& P, uint32_t i) {
+__device__ __forceinline__ uint32_t walk_step(const EvalParams& P, uint32_t i) {
     const uint32_t r = i / 65u, w = i - 65u * r;
-    const uint32_t s = w ? max((uint32_t)P.rows[r * kRowStride + 1u + w], 1u) : 1u;
-    return make_uint2(s, walk_rcp(s));
+    return w ? max((uint32_t)P.rows[r * kRowStride + 1u + w], 1u) : 1u;
 }
 
 // Accounts the completion ring, one entry per lane and pass, into the lane's own sums in the region `base`:
@@ -264,7 +264,7 @@ struct WInst {
     uint32_t pay;  // of what its running requests must remember
 };
 
-template <bool Opt, int Eng, bool Wide, bool Big>
+template <bool Opt, int Eng, bool Wide, bool Big, bool Rcp = (Eng == 0)>
 struct Walk {
     using T = typename std::conditional<Wide, int64_t, int32_t>::type;
     using U = typename std::conditional<Wide, uint64_t, uint32_t>::type;
@@ -279,6 +279,7 @@ struct Walk {
     static constexpr uint32_t kBlock = Wide ? kWalkBlockLong : (Big ? kWalkBlockKeys : kWalkBlock);
     static constexpr WalkKind kKind = Wide ? kWalkLongKind : (Big ? kWalkBigKind : kWalkUsual);
     static constexpr uint32_t kRest = Wide ? 80u : 48u;
+    static constexpr uint32_t kEntry = Rcp ? 8u : 4u, kRow = Rcp ? kWalkRowRcp : kWalkRow;
 
     // A class's limits; does a first token `since` after the arrival, with `Sm1` more tokens of `step`, meet them?
     struct Limits {
@@ -319,7 +320,7 @@ struct Walk {
             u[3] = make_uint4(e.y, e.z, e.w, 0u);
         }
         memcpy(&in, u, sizeof(Inst));
-        if (!Wide && Opt) in.stepB = w1(in.row + 8u * in.B);
+        if (!Wide && Opt) in.stepB = w1(in.row + kEntry * in.B);
     }
 
     // One warp takes the placements of a bucket, one after the other.  `base`: its part of shared memory;
@@ -390,15 +391,15 @@ struct Walk {
                         in.tag = (1u << md) | (e.y << 16);
                         in.B = (e.x >> 12) & 0xFFu;
                         nblk = (in.B + 7u) >> 3;
-                        in.row = L.steps + r * kWalkRow;
+                        in.row = L.steps + r * kRow;
                         in.pre_base = (uint32_t)P.rows[r * kRowStride];
                         in.pre_q16 = (uint32_t)P.rows[r * kRowStride + 1];
-                        in.stepB = w1(in.row + 8u * in.B);
+                        in.stepB = w1(in.row + kEntry * in.B);
                         // the smallest step a prediction can use: the step at the batch cap, or (optimistic estimate) at any
                         // level up to it
                         uint32_t ms = in.stepB;
                         if (Opt)
-                            for (uint32_t w = 1; w < in.B; w++) ms = min(ms, w1(in.row + 8u * w));
+                            for (uint32_t w = 1; w < in.B; w++) ms = min(ms, w1(in.row + kEntry * w));
                         atomicMin(&w1(models + 16u * md), in.pre_base);
                         atomicMin(&w1(models + 16u * md + 4u), ms);
                         // per instance: earliest start, prefill base and slope, smallest prediction step
@@ -479,6 +480,11 @@ struct Walk {
                 c_in = v.z;
                 c_meta = v.w;
             };
+            // Entry of the instance's row: decode step and reciprocal, the latter computed when the level changes if rows have none.
+            auto entry = [&](uint32_t at) -> uint2 {
+                if constexpr (Rcp) return w2(at);
+                else return make_uint2(w1(at), 0u);
+            };
             auto is_due = [&](T upto) { return kFixed ? in.tb <= upto : in.tb < upto; };
             // when the instance could start a request
             auto start = [&]() -> T { return kFixed ? (in.w == in.B ? in.tb : now) : (in.w == in.B ? in.tb + (T)in.sw : in.t); };
@@ -486,7 +492,7 @@ struct Walk {
             auto next_end = [&](uint32_t left, bool busy, uint2 step) {
                 const uint32_t sw = step.x;
                 in.sw = sw;
-                in.rsw = step.y;
+                in.rsw = Rcp ? step.y : walk_rcp(sw);
                 if constexpr (Wide) {
                     in.tb = busy ? in.t + (int64_t)((uint64_t)left * sw) - (int64_t)sw : kFar;
                 } else {
@@ -531,7 +537,7 @@ struct Walk {
                             w1(k8) = kKeyEmpty;
                             w1(mb) = kKeyEmpty;
                             const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(in.area), m1 = w4(in.area + 16u);
-                            const uint2 step = w2(in.row + 8u * in.w - 8u);
+                            const uint2 step = entry(in.row + kEntry * in.w - kEntry);
                             uint2 run;  // first token, request; 64-bit times: first token
                             uint32_t rq = 0;
                             if constexpr (kAway) run = __ldcg(reinterpret_cast<const uint2*>(away + 2u * (k8 - L.pool)));
@@ -585,7 +591,7 @@ struct Walk {
             auto peek = [&]() {
                 if (!kFixed) {
                     top = walk_smem[in.area + 32u + in.w];
-                    more = w2(in.row + 8u * in.w + 8u);
+                    more = entry(in.row + kEntry * in.w + kEntry);
                 }
             };
             // One request's times into the ring (`e`: its entry).
@@ -615,7 +621,7 @@ struct Walk {
                         level -= (uint32_t)(__popc(__ballot_sync(kWFull, v[0] == tb)) + __popc(__ballot_sync(kWFull, v[1] == tb)));
                         first = in.tb + pre;
                     }
-                    const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? 8u * level : 0u) + 8u);
+                    const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? kEntry * level : 0u) + kEntry);
                     T fin = first + (T)span;
                     if (win) {
                         if constexpr (Wide) {
@@ -797,7 +803,7 @@ struct Walk {
                             // distributor prediction (Sec. IV-F steps 2-3)
                             const T t = start();
                             uint32_t sB = in.stepB;
-                            if (Opt && !full) sB = kFixed ? w1(in.row + 8u * in.w + 8u) : more.x;
+                            if (Opt && !full) sB = kFixed ? w1(in.row + kEntry * in.w + kEntry) : more.x;
                             const bool ok = elig && lim.met((U)(t + p - arrival), Sm1, sB);
                             // smallest (tier, predicted first token >= now >= 0), lowest instance among equals
                             const U k = ok ? (full ? kTier1 : (U)0) | (U)(t + p) : kNone;
@@ -904,7 +910,7 @@ namespace maaso {
 
 // `Warps`: 16, or 12 for a batch that 12 per SM can hold.  Mode k: the block's warps >> k at work, each with 2^k times one warp's part of the pool.  The first placements
 // are dealt out in order, over the SMs first; after that whoever is free takes the next.
-template <bool Opt, int Eng, bool Wide, bool Big, int Warps>
+template <bool Opt, int Eng, bool Wide, bool Big, int Warps, bool Rcp>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_constant__ EvalParams P) {
     constexpr bool kLong = Wide && Eng != 2;  // (queues: 64-bit times in the usual buckets)
     constexpr int kFirst = kLong ? kWalkLong0 : (Big ? kWalkBig0 : kWalkBucket0);
@@ -913,10 +919,13 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
     for (int mode = 0; mode < (Big && !kLong ? 1 : kWalkModes); mode++) any |= P.bucket_count[kFirst + mode];
     if (any == 0) return;
     constexpr bool kDynamic = Eng == 0 && !Wide && !Big;
-    const WalkLayout L = walk_layout(P.n_rows, P.n_classes, Wide, Warps, kDynamic);
+    const WalkLayout L = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Rcp, kDynamic);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
-    for (uint32_t i = tid; i < P.n_rows * 65u; i += (32 * Warps)) 
-        w2(L.steps + 8u * i) = kDynamic ? walk_exact_entry(P, i) : walk_step_entry(P, i);
+    for (uint32_t i = tid; i < P.n_rows * 65u; i += (32 * Warps)) {
+        const uint32_t s = walk_step(P, i);
+        if constexpr (!Rcp) w1(L.steps + 4u * i) = kDynamic ? s << 5 : s;
+        else w2(L.steps + 8u * i) = kDynamic ? walk_exact_entry(s) : make_uint2(s, walk_rcp(s));
+    }
     for (uint32_t c = tid; c < P.n_classes; c += (32 * Warps)) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u];
         const int64_t none = (int64_t)1 << 62, le = e < 0 ? none : e;
@@ -941,13 +950,13 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
             idx = __shfl_sync(kWFull, idx, 0);
         }
         if (warp < act)
-            Walk<Opt, Eng, Wide, Big>::bucket(P, L, kWalkBig0, L.pool + warp * part, idx, gridDim.x,
+            Walk<Opt, Eng, Wide, Big, Rcp>::bucket(P, L, kWalkBig0, L.pool + warp * part, idx, gridDim.x,
                                               reinterpret_cast<unsigned char*>(P.payload) + blockIdx.x * walk_big_scratch(pool));
     } else {
         for (int mode = kWalkModes - 1; mode >= 0; mode--) {
             if (P.bucket_count[kFirst + mode] == 0) continue;  // the same for the whole block
             const uint32_t act = (uint32_t)Warps >> mode, part = (kLong ? P.walk_bytes : P.walk_usual) << mode;
-            using Body = typename std::conditional<kDynamic, WalkDynamic<Opt>, Walk<Opt, Eng, Wide, Big>>::type;
+            using Body = typename std::conditional<kDynamic, WalkDynamic<Opt, Rcp>, Walk<Opt, Eng, Wide, Big, Rcp>>::type;
             if (warp < act)
                 Body::bucket(P, L, kFirst + mode, L.pool + warp * part, warp * gridDim.x + blockIdx.x,
                                                   act * gridDim.x, nullptr);
@@ -956,10 +965,10 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
     }
 }
 
-template <bool Opt, int Eng, bool Wide, bool Big, int Warps = kWalkWarps>
+template <bool Opt, int Eng, bool Wide, bool Big, bool Rcp, int Warps = kWalkWarps>
 static cudaError_t launch_walk(const EvalParams& P, int grid, cudaStream_t stream) {
-    auto kernel = eval_walk_kernel<Opt, Eng, Wide, Big, Warps>;
-    const size_t smem = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Eng == 0 && !Wide && !Big).pool + (Big || (Wide && Eng != 2) ? P.walk_bytes * kWalkWarps : P.walk_usual * Warps);
+    auto kernel = eval_walk_kernel<Opt, Eng, Wide, Big, Warps, Rcp>;
+    const size_t smem = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Rcp, Eng == 0 && !Wide && !Big).pool + (Big || (Wide && Eng != 2) ? P.walk_bytes * kWalkWarps : P.walk_usual * Warps);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<grid, (32 * Warps), smem, stream>>>(P);

@@ -46,6 +46,35 @@ def test_large_tables_and_full_caps(oracle_mod, rows, n_classes, n_models, flags
 
 
 @pytest.mark.parametrize("flags", [0, 1])
+@pytest.mark.parametrize("rows", [80, 81, 256])
+def test_large_tables_and_64_bit_times(oracle_mod, rows, flags):
+    import paper_2509_06362_b200 as m
+    rng = np.random.default_rng(rows)
+    prof = _tables(1, rows, rng)
+    off, inst = gen.candidates_from_lists([_placement(prof, n, cap, rng) for n in (1, 8, 32, 33, 128) for cap in (1, 64)])
+    tr, classes = _workload(400, 100.0, 1, 71, rng)
+    classes["e2e_us"] = np.where(classes["e2e_us"] < 0, 1 << 39, classes["e2e_us"])
+    want = _check(oracle_mod, m, prof, tr, classes, off, inst, flags)
+    assert (want["status"] == 0).all() and want["n_served"].max() > 200
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+@pytest.mark.parametrize("rows", [52, 53, 128, 129])
+def test_rows_with_and_without_reciprocals(oracle_mod, rows, flags):
+    """Either side of the lines from which on the rows carry no reciprocals: whatever a round divides by, steps of 1 us and of 2^24 - 1
+    and an idle instance's among them."""
+    import paper_2509_06362_b200 as m
+    rng = np.random.default_rng(rows)
+    prof = _tables(1, rows, rng)
+    prof["step_us"][0, 0], prof["step_us"][0, 1] = 1, (1 << 24) - 1
+    lists = [_placement(prof, n, cap, rng) for n in (1, 5, 32, 33, 70, 128) for cap in (1, 2, 9, 64)]
+    off, inst = gen.candidates_from_lists(lists + [[(0, 0, 64)], [(0, 1, 3), (0, 0, 2)], [(0, 1, 1)] * 40 + [(0, 0, 64)] * 40])
+    tr, classes = _workload(600, 60.0, 1, 4, rng)
+    want = _check(oracle_mod, m, prof, tr, classes, off, inst, flags)
+    assert (want["status"] == 0).all() and want["n_served"].max() > 300
+
+
+@pytest.mark.parametrize("flags", [0, 1])
 def test_full_caps_in_a_batch_that_packs(oracle_mod, flags):
     import paper_2509_06362_b200 as m
     rng = np.random.default_rng(9)

@@ -9,6 +9,7 @@ import pytest
 HERE = os.path.dirname(os.path.abspath(__file__))
 OPTIMISTIC, FROZEN, MAXGAP, QUEUES = 1, 2, 4, 8
 AUTO, BLOCK, GROUP, THREAD = 0, 1, 2, 3
+MAX_ROWS = 256
 
 
 @pytest.fixture(scope="module")
@@ -47,3 +48,18 @@ def test_every_placement_has_a_kernel_with_threads(routes, pool, hot):
     """(The pools' default sizes, and small ones that hold few instances.)"""
     assert _unscored(routes, 0, THREAD, 1000, 1, pool, hot) == (0, None)
     assert _unscored(routes, 0, AUTO, 1000, 1, pool, hot) == (0, None)
+
+
+@pytest.mark.parametrize("flags", [0, OPTIMISTIC, FROZEN, QUEUES])
+@pytest.mark.parametrize("items", [1000, 10 ** 6])
+def test_large_tables_leave_the_walking_kernel_its_room(routes, flags, items):
+    """The one-warp kernel, up to 592 MB of scratch, is launched for tables near the largest only, and there for placements near the
+    largest: 16 models of 10 strategies are none of those."""
+    for rows in range(1, MAX_ROWS + 1):
+        for classes in (4, 71):
+            first = routes.routes_wide_from(flags, AUTO, rows, 1, classes, items, 1, 0, 0)
+            if rows <= 176 or flags in (FROZEN, QUEUES):
+                assert first == 0, (rows, classes)
+            else:
+                assert first == 0 or first > 100, (rows, classes)
+    assert routes.routes_wide_from(flags, AUTO, 160, 16, 71, items, 1, 0, 0) == 0
