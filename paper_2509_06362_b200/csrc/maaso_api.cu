@@ -629,7 +629,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
             may_leave = may_leave || o.flags != 0 || (double)kWalkNowMax + 2.0 * ahead >= (double)kWalkHorizon;
         }
         may_leave = may_leave && !(o.flags & MAASO_FLAG_INSTANCE_QUEUES);
-        route_walk(P, (uint64_t)C * n_traces, (uint32_t)ctx->sm_count, fits);
+        route_walk(P, (uint64_t)C * n_traces, cands->n_inst * n_traces, (uint32_t)ctx->sm_count, fits);
     }
     const bool threads = o.mapping == MAASO_MAP_THREAD || (o.mapping == MAASO_MAP_AUTO && !variant && C >= ctx->thread_min_cand);
     P.thread_min_cand = threads ? ctx->thread_min_cand : 0u;

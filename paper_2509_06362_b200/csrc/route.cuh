@@ -139,8 +139,8 @@ MAASO_HD inline bool route_fixed_speed(uint32_t flags) { return (flags & (MAASO_
 MAASO_HD inline bool route_variant(uint32_t flags) { return route_fixed_speed(flags) || (flags & MAASO_FLAG_TBT_MAXGAP) != 0; }
 
 // The walking and the packed kernel's part of a call that the walking kernel runs: room, and who takes the batch.
-// `items`: placements times traces; `fits32`: 32-bit times hold the batch's tables and limits.
-inline void route_walk(Route& r, uint64_t items, uint32_t sm_count, bool fits32) {
+// `items`: placements times traces, `insts`: instances times traces; `fits32`: 32-bit times hold the batch's tables and limits.
+inline void route_walk(Route& r, uint64_t items, uint64_t insts, uint32_t sm_count, bool fits32) {
     const bool queues = (r.flags & MAASO_FLAG_INSTANCE_QUEUES) != 0;  // always with 64-bit times
     const bool fixed_speed = route_fixed_speed(r.flags);
     r.walk_long = fits32 || queues ? 0u : 1u;
@@ -148,11 +148,18 @@ inline void route_walk(Route& r, uint64_t items, uint32_t sm_count, bool fits32)
     r.walk_rcp_big = !fixed_speed && r.n_rows <= (r.walk_long ? kWalkRcpRowsLong : kWalkRcpRowsBig) ? 1u : 0u;
     r.walk_bytes = ((kBlockShared - walk_layout(r.n_rows, r.n_classes, true, kWalkWarps, r.walk_rcp_big != 0).pool) / kWalkWarps) & ~15u;
     // With queues the models of a placement are independent of one another and can be replayed side by side, while the batch is
-    // bound by its longest chains: every part scans the whole trace.  Whole and in parts: the paper's shape (three models),
-    // 300 x 8,000 3.4 and 2.0 ms, 1,000 4.15 and 2.15, 5,000 7.9 and 5.7, 18,000 18.3 and 17.7, 2,000 x 17,000 9.25 and 5.35; three
-    // models under load, 500 x 10,000 1.64 and 1.36, 2,000 2.40 and 1.86, 5,000 2.55 and 2.30, 10,000 3.2 and 4.1, 40,000 11.9 and
-    // 15.5; at 16 a second 10,000 x 5,000 4.0 and 4.5.  The warps per block go by the parts (6,000 of them 7.2 ms with 12, 5.3 with 16).
-    r.walk_parts = queues && items <= 3ull * sm_count * kWalkWarpsFew ? r.n_models : 1u;
+    // bound by its longest chains: every part scans the whole trace.  A placement has no more parts than instances, and what decides is
+    // the number of parts in all, up to twelve a warp, and that of placements, as few models gain less.  Whole and in parts (ms),
+    // lightly loaded and (after the semicolon) under load:
+    //   two models      4,000 x 6,000 6.9 and 5.7; 3.3 and 3.3    8,000 9.8 and 10.2; 3.7 and 3.8
+    //   three           1,000 3.6 and 1.7; 1.9 and 1.5            5,300 7.1 and 5.6; 2.7 and 2.8        16,000 14.8 and 15.4; 6.1 and 7.7
+    //   eight           1,330 3.8 and 1.4; 2.6 and 1.1            3,280 4.0 and 3.0; 2.5 and 2.2        5,300 5.2 and 4.6; 3.1 and 3.3
+    //     17 instances  1,330 3.9 and 2.2; 2.9 and 2.1            2,660 5.0 and 3.9; 2.8 and 3.4        5,300 8.3 and 7.4; 4.9 and 6.3
+    //   sixteen         1,330 2.6 and 1.1; 2.5 and 1.1            3,280 2.9 and 2.4; 2.5 and 2.3        5,300 3.9 and 3.7; 2.7 and 3.6
+    //     21 instances  1,330 8.5 and 7.1; 7.6 and 7.1            2,660 10.2 and 9.7; 8.0 and 9.3       5,300 12.8 and 13.2; 10.6 and 13.4
+    // (The paper's shape, 2,000 x 17,000: 9.25 and 5.35.)  The warps per block go by the parts (6,000 of them 7.2 ms with 12, 5.3 with 16).
+    const uint64_t parts = items * r.n_models < insts ? items * r.n_models : insts;
+    r.walk_parts = queues && items <= 3ull * sm_count * kWalkWarpsFew && parts <= 12ull * sm_count * kWalkWarpsFew ? r.n_models : 1u;
     r.walk_warps = fixed_speed && items * r.walk_parts <= 3ull * sm_count * kWalkWarpsFew ? kWalkWarpsFew : kWalkWarps;
     r.walk_usual = ((kBlockShared - walk_layout(r.n_rows, r.n_classes, queues, r.walk_warps, r.walk_rcp != 0, !fixed_speed).pool) / r.walk_warps) & ~15u;
     // Small batches walk whatever their load.  A large one that is not loaded is bound by the instructions of its rounds,

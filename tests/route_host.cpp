@@ -22,7 +22,7 @@ static Route make_route(uint32_t flags, uint32_t mapping, uint32_t rows, uint32_
     r.n_classes = classes;
     r.thread_pool_units = thread_pool / 16u;
     r.thread_hot_units = thread_hot / 16u;
-    if (mapping == MAASO_MAP_AUTO && !(flags & MAASO_FLAG_TBT_MAXGAP) && !thread_pool) route_walk(r, items, 148u, fits32);
+    if (mapping == MAASO_MAP_AUTO && !(flags & MAASO_FLAG_TBT_MAXGAP) && !thread_pool) route_walk(r, items, 8u * items, 148u, fits32);
     return r;
 }
 
@@ -58,4 +58,15 @@ extern "C" uint32_t routes_unscored(uint32_t flags, uint32_t mapping, uint64_t i
 extern "C" uint32_t routes_wide_from(uint32_t flags, uint32_t mapping, uint32_t rows, uint32_t models, uint32_t classes, uint64_t items, uint32_t fits32,
                                      uint32_t thread_pool, uint32_t thread_hot) {
     return route_launches(make_route(flags, mapping, rows, models, classes, items, fits32 != 0, thread_pool, thread_hot), 1u << 20, false).wide_from;
+}
+
+// Parts that a placement is replayed in with a queue in front of every instance.
+extern "C" uint32_t routes_parts(uint32_t models, uint64_t items, uint64_t insts) {
+    Route r = Route();
+    r.flags = MAASO_FLAG_INSTANCE_QUEUES;
+    r.n_rows = 10u * models;
+    r.n_models = models;
+    r.n_classes = 3;
+    route_walk(r, items, insts, 148u, true);
+    return r.walk_parts;
 }

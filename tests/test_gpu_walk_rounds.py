@@ -93,3 +93,19 @@ def test_queues_by_model(oracle_mod, n_models, flags):
     for k, t in enumerate(traces):
         assert_records_equal(got[k], oracle_mod.eval_placements(prof, t, classes, off, inst, 10 ** 6, mask, flags), f"trace {k}")
     c.close()
+
+
+@pytest.mark.parametrize("n", [1332, 1333])  # as many parts as there may be, and one placement more: all of them whole
+def test_queues_of_many_models(oracle_mod, n):
+    import paper_2509_06362_b200 as m
+    rng = np.random.default_rng(n)
+    W = gen.WMAX
+    prof = {"n_models": 16, "n_strategies": 1, "wmax": W, "devices": np.ones(1, dtype=np.int32), "min_devices": np.ones(16, dtype=np.int32),
+            "prefill_base_us": rng.integers(0, 3000, size=(16, 1)).astype(np.int32), "prefill_q16": np.full((16, 1), 9000, dtype=np.int32),
+            "step_us": rng.integers(5000, 30_000, size=(16, 1, W)).astype(np.int32)}
+    off, inst = gen.candidates_from_lists([[(int(k), 0, int(rng.choice([1, 3, 8]))) for k in rng.integers(0, 16, size=16)] for _ in range(n)])
+    tr = _requests(200, [0, 1000, 60_000], [1, 2, 100, 400], rng)
+    tr["model"] = rng.integers(0, 16, size=len(tr))
+    classes = gen.make_classes([(None, None, None), (600_000, 20_000, None), (None, None, 9_000_000)])
+    want = _check(oracle_mod, m, prof, tr, classes, off, inst, 8)
+    assert want["n_served"].max() > 50 and (want["n_rejected"] > 0).any()

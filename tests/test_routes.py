@@ -18,7 +18,8 @@ def routes(tmp_path_factory):
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC", "-o", lib, os.path.join(HERE, "route_host.cpp")])
     lib = ctypes.CDLL(lib)
     u32, u64 = ctypes.c_uint32, ctypes.c_uint64
-    lib.routes_unscored.restype = lib.routes_wide_from.restype = u32
+    lib.routes_unscored.restype = lib.routes_wide_from.restype = lib.routes_parts.restype = u32
+    lib.routes_parts.argtypes = [u32, u64, u64]
     lib.routes_unscored.argtypes = [u32, u32, u64, u32, u32, u32, ctypes.POINTER(u32)]
     lib.routes_wide_from.argtypes = [u32, u32, u32, u32, u32, u64, u32, u32, u32]
     return lib
@@ -63,3 +64,14 @@ def test_large_tables_leave_the_walking_kernel_its_room(routes, flags, items):
             else:
                 assert first == 0 or first > 100, (rows, classes)
     assert routes.routes_wide_from(flags, AUTO, 160, 16, 71, items, 1, 0, 0) == 0
+
+
+@pytest.mark.parametrize("models", [1, 2, 3, 8, 16])
+@pytest.mark.parametrize("size", [1, 5, 17, 128])
+def test_queues_are_replayed_in_parts_up_to_a_number_of_parts(routes, models, size):
+    """Every part scans the whole trace: their number is bounded, however many models there are."""
+    for items in (1, 100, 1000, 1330, 2000, 4000, 5328, 5329, 20_000):
+        parts = routes.routes_parts(models, items, items * size)
+        assert parts in (1, models)
+        in_all = items * min(models, size)
+        assert (parts == models) == (models == 1 or (items <= 3 * 148 * 12 and in_all <= 12 * 148 * 12)), (items, parts)
