@@ -26,13 +26,6 @@
 
 namespace maaso {
 
-// ceil(dt / s) = (2 (dt + s - 1) m >> 32) >> L with L = ceil(log2 s), m = ceil(2^(31 + L) / s) < 2^32: exact for dt + s - 1 <
-// 2^31 (m s - 2^(31 + L) < s <= 2^L; Granlund and Montgomery's division by an invariant).  A row's entry: {s << 5 | L, m}.
-__device__ __forceinline__ uint2 walk_exact_entry(uint32_t s) {
-    const uint32_t sh = s > 1u ? 32u - (uint32_t)__clz((int)(s - 1u)) : 0u;
-    return make_uint2((s << 5) | sh, (uint32_t)((((uint64_t)1 << (31u + sh)) + (s - 1u)) / s));
-}
-
 // A load that stays where it is written, ahead of what it is for (the compiler moves a plain one down to its use).
 __device__ __forceinline__ uint4 load_ahead(const uint4* p) {
     uint4 v;
@@ -249,7 +242,7 @@ struct WalkDynamic {
             };
             // Decode steps until `dt` later; 2 (dt + step - 1) < 2^32.
             auto steps_of = [&](int32_t dt) -> uint32_t {
-                if constexpr (Rcp) return __funnelshift_r(__umulhi(2u * ((uint32_t)dt + sw - 1u), rcp), 0u, step);
+                if constexpr (Rcp) return walk_exact_steps(dt, sw, step, rcp);
                 else return ((uint32_t)dt + sw - 1u) / sw;
             };
             auto start = [&]() -> int32_t { return w == B ? tc : t; };

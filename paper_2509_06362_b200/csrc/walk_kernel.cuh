@@ -46,6 +46,7 @@
 #pragma once
 #include <cstring>
 #include <type_traits>
+#include "steps.cuh"
 #include "walk.cuh"
 
 namespace maaso {
@@ -78,17 +79,6 @@ __device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_s
 __device__ __forceinline__ uint64_t warp_min(uint64_t v) {  // the smallest high half, the smallest low half that comes with it
     const uint32_t hi = (uint32_t)(v >> 32), mh = __reduce_min_sync(kWFull, hi);
     return ((uint64_t)mh << 32) | __reduce_min_sync(kWFull, hi == mh ? (uint32_t)v : 0xFFFFFFFFu);
-}
-// ceil(dt / s) for 0 <= dt < 2^31, s < 2^31, rs = (2^32 - 1) / s rounded down: the estimate is at most the quotient and less
-// than two below it, since rs > 2^32 / s - 1.
-__device__ __forceinline__ uint32_t walk_rcp(uint32_t s) { return 0xFFFFFFFFu / s; }
-__device__ __forceinline__ uint32_t walk_steps(int32_t dt, uint32_t s, uint32_t rs) {
-    const uint32_t d = (uint32_t)dt + s - 1u, q = __umulhi(d, rs);
-    return q + (d - q * s >= s ? 1u : 0u);
-}
-__device__ __forceinline__ uint32_t walk_steps(int64_t dt, uint32_t s, uint32_t rs) {
-    const uint64_t d = (uint64_t)dt + (s - 1u);
-    return (d >> 32) == 0 ? walk_steps((int32_t)dt, s, rs) : (uint32_t)(d / s);
 }
 // Entry i of the decode-step rows in shared memory (WalkLayout::steps).
 __device__ __forceinline__ uint32_t walk_step(const EvalParams& P, uint32_t i) {
@@ -924,7 +914,10 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
     for (uint32_t i = tid; i < P.n_rows * 65u; i += (32 * Warps)) {
         const uint32_t s = walk_step(P, i);
         if constexpr (!Rcp) w1(L.steps + 4u * i) = kDynamic ? s << 5 : s;
-        else w2(L.steps + 8u * i) = kDynamic ? walk_exact_entry(s) : make_uint2(s, walk_rcp(s));
+        else if constexpr (kDynamic) {
+            const ExactEntry e = walk_exact_entry(s);
+            w2(L.steps + 8u * i) = make_uint2(e.step, e.m);
+        } else w2(L.steps + 8u * i) = make_uint2(s, walk_rcp(s));
     }
     for (uint32_t c = tid; c < P.n_classes; c += (32 * Warps)) {
         const int64_t a = P.classes[3u * c], b = P.classes[3u * c + 1u], e = P.classes[3u * c + 2u];
