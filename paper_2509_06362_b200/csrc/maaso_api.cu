@@ -764,11 +764,11 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         for (uint32_t t = 0; t < n_traces; t++) inv += traces[t]->tok_rate > 0.0 ? 1.0 / traces[t]->tok_rate : 1.0;
         // Twice a placement's capacity is what the validation kernel calls loaded.  Against the packed kernel the walking kernel is the
         // better one from about its capacity on already, unless a batch of one model is larger than what the packed kernel's warps
-        // hold at once (six placements a warp on average; its steps take as long for fewer).  Measured on 4,000 requests, walking
+        // hold at once (14 warps per SM, six placements a warp on average; its steps take as long for fewer).  Measured on 4,000 requests, walking
         // and packed, between the two lines: one node 5,000 at 6 and 8 a second 2.5 and 4.5, 2.1 and 4.4 ms, 10,864 at 8 3.9 and 5.1,
         // 14,000 at 6 6.1 and 5.5, 20,000 at 6 and 8 8.5 and 6.1, 6.2 and 5.5; three models at 4 a second 24,576 7.4 and 10.0, 40,000
         // 11.5 and 15.0.  Below both: 10,864 at 6 a second 5.0 and 5.2, three models at 2 a second 24,576 10.9 and 11.3.
-        const bool early = L.pack && (ctx->n_models > 1 || (uint64_t)C * n_traces <= 7ull * kWalkWarpsFew * ctx->sm_count);
+        const bool early = L.pack && (ctx->n_models > 1 || (uint64_t)C * n_traces <= 6ull * kPackWarps * ctx->sm_count);
         const double d = n_traces / inv * (early ? 2.0 : 1.0);
         P.demand_tok_s = d >= 4.0e9 ? 4000000000u : (uint32_t)d;
     }

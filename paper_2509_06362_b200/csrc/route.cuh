@@ -168,11 +168,17 @@ inline void route_walk(Route& r, uint64_t items, uint64_t insts, uint32_t sm_cou
     //   one model     at 1 a second 3,000 placements 4.1 and 4.1 ms, 4,096 4.5 and 4.15, 5,000 5.5 and 4.3; at 2 a second 4,096 4.4
     //                 and 4.35, 5,000 4.5 and 4.5, 6,500 6.3 and 4.65; at 4 a second 6,500 4.4 and 4.6, 8,192 5.7 and 4.8
     //   three models  (a third of the lanes of a step at work) at 1 a second 12,288 7.6 and 8.5, 18,432 10.8 and 10.4; at 2 a second
-    //                 18,432 8.4 and 10.0, 40,000 16.9 and 17.2; at 4 a second 40,000 11.6 and 15.1 (and walking by its load)
+    //                 18,432 8.4 and 10.0, 40,000 16.9 and 17.2; at 4 a second 40,000 11.6 and 15.1 (and it walks by its load: eval_impl)
     // With the optimistic estimate one model at 2 a second 4,096 5.05 and 4.85, three 12,288 7.4 and 8.1, 24,576 13.7 and 12.4.
-    // With fixed speeds or queues the alternative is the lane-group kernel; measured before the walking kernel's bodies parted: fixed
-    // speeds equal at 6,200 and more, 9,100 and more with several models; queues at 3,600 to 7,300, with two models 4,900 to 10,100,
-    // with three 7,200 to 11,400 (so that for several models the line is late there).
+    // With fixed speeds or queues the alternative is the lane-group kernel, and the lines are early for one model and late for two.
+    // Walking (queues: in one piece) and lane groups, 4,000 requests:
+    //   fixed speeds    one model at 1 and 2 a second 4,096 7.4 and 9.9, 5.3 and 9.1; 6,144 8.2 and 10.0, 7.1 and 9.4; 8,192 10.6 and
+    //                   10.0, 8.4 and 9.3; two at 1 and 3 a second 6,144 6.6 and 7.9, 5.0 and 7.8; 9,000 9.0 and 8.2, 6.4 and 8.0;
+    //                   12,288 11.7 and 8.4, 8.2 and 8.4; three at 1 and 4 a second 18,432 11.7 and 15.0, 7.1 and 13.3; 30,000 18.5
+    //                   and 20.7, 10.9 and 19.1
+    //   queues          one 4,096 7.6 and 9.5, 5.6 and 8.6; 8,192 11.0 and 9.7, 8.9 and 8.7; two 6,144 7.3 and 7.7, 5.9 and 7.6;
+    //                   9,000 10.0 and 7.9, 8.4 and 7.9; 12,288 13.1 and 8.2, 10.7 and 8.2; three 9,216 8.7 and 8.7, 6.9 and 8.3;
+    //                   18,432 15.8 and 15.0, 12.7 and 14.1
     r.walk_all = items <= (r.n_models == 1 ? 4096u : 6144u * (uint64_t)r.n_models) ? 1u : 0u;
     r.pack = !r.walk_all && !r.walk_long && !route_variant(r.flags) && pack_fits(r.n_rows, r.n_classes) ? 1u : 0u;
 }

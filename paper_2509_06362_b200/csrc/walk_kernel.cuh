@@ -25,7 +25,7 @@
 // Measured (B200, whole calls with routing and top-k; lane-group, thread or one-warp kernel before): 143 placements x 500
 // requests 0.17 ms (0.56), one node's 10,864 x 10,000 4.6 ms (12.0), 2,000 x 17,000 of the paper's shape 6.4 to 6.6 ms (33.9), with
 // queues 5.3 ms (27.8), with fixed speeds 9.5 ms, three models, 100,000 x 100,000 under load 92.4 ms (135), 2,000 placements of 33
-// to 128 instances x 10,000 8.1 to 8.7 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
+// to 128 instances x 10,000 7.8 to 8.7 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
 // needs is therefore read from shared memory ahead of the choice, the uncommon outcomes share one branch, and tests of several
 // conditions are written without branches (& and | for && and ||).
 //
