@@ -50,7 +50,8 @@ constexpr uint32_t kBlockShared = 227u * 1024u;   // shared memory of a block
 //   up to 32 instances, 32-bit times: 12,000 x 10,000 under load, 100 rows 1.73 and 1.84 ms, 120 1.68 and 1.69, 160 1.76 and 1.70,
 //     256 2.36 and 2.01; 4,000 x 8,000 lightly loaded, 120 rows 2.29 and 2.54, 160 3.22 and 2.24; some 20 instances each, 6,000 x
 //     8,000, 100 rows 4.02 and 4.04, 120 3.03 and 2.97, 160 2.88 and 2.66
-//   more than 32: 2,000 x 5,000, 50 rows 9.29 and 9.39, 60 9.63 and 8.56, 100 7.53 and 6.82
+//   more than 32: 2,000 x 5,000, 50 rows 9.29 and 9.39, 60 9.63 and 8.56, 100 7.53 and 6.82 (a few hundred of them, which all run at
+//     once either way, 1 to 2 % better with)
 //   64-bit times: 5 to 6 % better with, up to 100 rows.  The line there is where the pool still holds every placement.
 constexpr uint32_t kWalkRow = 65u * 4u, kWalkRowRcp = 65u * 8u;  // bytes of a row
 constexpr uint32_t kWalkRcpRows = 128u, kWalkRcpRowsBig = 52u, kWalkRcpRowsLong = 80u;
