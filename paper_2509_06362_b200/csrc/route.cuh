@@ -266,7 +266,10 @@ inline Launches route_launches(const Route& r, uint64_t n_inst, bool may_leave) 
     l.wide_from = 0;
     for (uint32_t n = 1; n <= (uint32_t)MAASO_MAX_INSTANCES && n <= n_inst && !l.wide_from; n++) {
         PlacementSize s = {n, 0u, 0u, 0u};
-        for (uint32_t i = 0; i < n; i++) s.add(r, MAASO_WMAX);
+        s.add(r, MAASO_WMAX);
+        s.slots *= n;
+        s.slots64 *= n;
+        s.units *= n;
         if (route_home(r, s).group == kWideBucket) l.wide_from = n;
     }
     return l;
