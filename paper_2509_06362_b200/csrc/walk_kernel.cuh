@@ -898,8 +898,9 @@ struct Walk {
 #include "walk_dynamic.cuh"
 namespace maaso {
 
-// `Warps`: 16, or 12 for a batch that 12 per SM can hold.  Mode k: the block's warps >> k at work, each with 2^k times one warp's part of the pool.  The first placements
-// are dealt out in order, over the SMs first; after that whoever is free takes the next.
+// `Warps`: 16, or 12 for small batches under fixed speeds and queues (route.cuh).  Mode k: the block's warps >> k at work, each with
+// 2^k times one warp's part of the pool.  The first placements are dealt out in order, over the SMs first; after that whoever is
+// free takes the next.
 template <bool Opt, int Eng, bool Wide, bool Big, int Warps, bool Rcp>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_constant__ EvalParams P) {
     constexpr bool kLong = Wide && Eng != 2;  // (queues: 64-bit times in the usual buckets)

@@ -79,7 +79,7 @@ def test_three_models(oracle_mod, flags):
 
 @pytest.mark.parametrize("flags", [0, 1])
 @pytest.mark.parametrize("far", [False, True])
-@pytest.mark.parametrize("copies", [1, 3])  # 4,464 items: 12 warps per SM hold them at once; 13,392: 16 take several each
+@pytest.mark.parametrize("copies", [1, 3])  # 4,464 items: 12 warps per SM hold them at once; 13,392: 14 take several each
 def test_several_traces(oracle_mod, copies, far, flags):
     """Every item of the packed kernel exists once per trace: records, unserved requests and histograms go to the trace's own
     block, traces of other lengths (an empty one among them) end at other times, and a placement that leaves the horizon under
