@@ -370,7 +370,8 @@ MAASO_API int maaso_topk_noalloc(const maaso_result *results, uint64_t n_cand, u
 /* Optional device timing.  While enabled, maaso_eval_placements and maaso_topk record CUDA
  * events on the caller's stream around each kernel family; maaso_get_timing waits for the
  * events of the most recent calls and reports milliseconds (0 for a family that did not
- * run).  Off by default; costs a few event records per call when on. */
+ * run).  Off by default; costs a few event records per call when on, and kernels of different
+ * families that otherwise run side by side run one after the other. */
 typedef struct {
     float prep_ms;  /* validation, routing + bucket sort (+ dump buffer fill) */
     float group_ms; /* walking, packed and lane-group scoring kernels (up to 32 instances) */

@@ -176,6 +176,11 @@ __device__ __forceinline__ int64_t prefill_us(uint32_t base, uint32_t q16, uint3
     return (int64_t)base + (int64_t)(((uint64_t)q16 * in_tokens + 32768u) >> 16);
 }
 
+// A kernel lets the next one's blocks start where its own leave room; the next one, launched for it, waits for its end (a kernel
+// that is launched the usual way waits for nothing here).
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- mbarrier + 1-D bulk copy (TMA) -----------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -254,7 +259,8 @@ struct EvalParams : Route {
     maaso_result* out;
     uint32_t* bucket_count;  // [64]: candidates per bucket after planning, and the kCtr* counters
     uint32_t* bucket_list;   // [kNumBuckets][n_cand], each bucket sorted by decreasing cost estimate
-    uint32_t* work_ctr;      // [16]: next work item of the block kernels [1..4], of the thread buckets [5..13], of the wide kernel [14]
+    uint32_t* work_ctr;      // [16]: next work item of the packed kernel [0], of the block kernels [1..4], of the thread buckets [5..13], of the
+                             // wide kernel [14]; blocks of the walking kernel that have started [15]
     uint32_t* hist;          // [kHistRows][kCostBins]: candidates per cost bin by set, then write cursors
     uint32_t* code;          // [n_cand] lane-group / block bucket << 8 | cost bin, 0xFFFFFFFF if none
     uint32_t* code2;         // [n_cand] walking or thread bucket << 8 | cost bin, 0xFFFFFFFF if none
@@ -265,6 +271,7 @@ struct EvalParams : Route {
     uint32_t n_sm;
     uint32_t promote_pct;
     uint32_t* walk_ctr;      // [kWalkBuckets]: next placement of each walking bucket
+    uint32_t big_grid;       // blocks of the walking kernel for more than 32 instances; 0: none, or none beside the smaller placements
     long long wait_cycles;   // bound of every device-side wait
     uint32_t stall_test;     // test hook: never issue the trace copies
     int32_t* dump_row;       // [n_cand] or null

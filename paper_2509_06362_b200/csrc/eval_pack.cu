@@ -391,6 +391,7 @@ template <bool Opt, int Warps>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
     if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
     if (P.bucket_count[kPack4] + P.bucket_count[kPack8] == 0) return;
+    let_next_start();
     const WalkLayout L = pack_layout(P.n_rows, P.n_classes);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
     for (uint32_t i = tid; i < P.n_rows * 65u; i += 32u * Warps) {

@@ -6,9 +6,9 @@ namespace maaso {
 cudaError_t launch_eval_walk_long(const EvalParams& P, int grid, cudaStream_t stream) {
     const bool opt = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) != 0;
     if (P.flags & MAASO_FLAG_ENGINE_FROZEN)
-        return opt ? launch_walk<true, 1, true, true, false>(P, grid, stream) : launch_walk<false, 1, true, true, false>(P, grid, stream);
-    if (P.walk_rcp_big) return opt ? launch_walk<true, 0, true, true, true>(P, grid, stream) : launch_walk<false, 0, true, true, true>(P, grid, stream);
-    return opt ? launch_walk<true, 0, true, true, false>(P, grid, stream) : launch_walk<false, 0, true, true, false>(P, grid, stream);
+        return opt ? launch_walk<true, 1, true, true, false>(P, grid, false, stream) : launch_walk<false, 1, true, true, false>(P, grid, false, stream);
+    if (P.walk_rcp_big) return opt ? launch_walk<true, 0, true, true, true>(P, grid, false, stream) : launch_walk<false, 0, true, true, true>(P, grid, false, stream);
+    return opt ? launch_walk<true, 0, true, true, false>(P, grid, false, stream) : launch_walk<false, 0, true, true, false>(P, grid, false, stream);
 }
 
 }  // namespace maaso

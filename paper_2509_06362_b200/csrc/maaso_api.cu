@@ -23,7 +23,7 @@ cudaError_t launch_eval_thread(const EvalParams& P, int grid, uint32_t pool_byte
 int occupancy_eval_thread(const EvalParams& P, uint32_t pool_bytes, uint32_t hot_bytes, bool in_smem);
 size_t thread_scratch_per_warp(uint32_t pool_bytes);
 uint32_t thread_fixed_smem(uint32_t n_models, uint32_t n_rows);
-cudaError_t launch_eval_walk(const EvalParams& P, int grid, cudaStream_t stream);
+cudaError_t launch_eval_walk(const EvalParams& P, int grid, bool overlap, cudaStream_t stream);
 cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream);
 size_t pack_scratch(int grid);
 cudaError_t launch_eval_walk_big(const EvalParams& P, int grid, cudaStream_t stream);
@@ -688,6 +688,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         const uint64_t most = cands->n_inst / (kWalkBig + 1) * n_traces;
         grid_big = most < (uint64_t)ctx->sm_count ? (int)most : ctx->sm_count;
     }
+    P.big_grid = ctx->timing ? 0u : (uint32_t)grid_big;  // (timed: kernel families one after the other)
     const bool away = grid_big > 0 && !variant;  // its running requests are in global memory
     if (L.groups) {
         const int occ_g = occupancy_eval_group(P, tile, group_blocks, ctx->smem_per_sm);
@@ -793,8 +794,17 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "packed kernel launch");
     }
+    auto launch_big = [&]() {
+        EvalParams PB = P;
+        PB.payload = reinterpret_cast<Payload*>(sb + off_pay_b);
+        launches++;
+        return launch_eval_walk_big(PB, grid_big, stream);
+    };
+    if (P.big_grid) e = launch_big();
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     if (L.walk) {
-        e = launch_eval_walk(P, ctx->sm_count, stream);
+        // side by side with the larger placements, or with what is left of the packed ones
+        e = launch_eval_walk(P, ctx->sm_count, !ctx->timing && (P.big_grid || L.pack), stream);
         launches++;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     }
@@ -811,13 +821,8 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         if (e != cudaSuccess) return cuda_fail(ctx, e, "thread kernel launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[6], stream);
-    if (grid_big > 0) {
-        EvalParams PB = P;
-        PB.payload = reinterpret_cast<Payload*>(sb + off_pay_b);
-        e = launch_eval_walk_big(PB, grid_big, stream);
-        launches++;
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
-    }
+    if (grid_big > 0 && !P.big_grid) e = launch_big();
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "walking kernel launch");
     if (L.far) {
         e = launch_eval_walk_long(P, ctx->sm_count, stream);
         launches++;

@@ -898,17 +898,59 @@ struct Walk {
 #include "walk_dynamic.cuh"
 namespace maaso {
 
+// Warps of a block that replay placements of more than 32 instances side by side: the room that the list's first, its largest, needs
+// decides.
+__device__ __forceinline__ uint32_t walk_big_warps(const EvalParams& P, uint32_t warps) {
+    const uint32_t cand = P.bucket_list[(size_t)kWalkBig0 * P.n_cand];
+    return max(1u, min(warps, P.walk_bytes * kWalkWarps / ((256u - (P.code2[cand] & 0xFFu)) * kWalkStepBytes)));
+}
+
+// Blocks that replay the placements of more than 32 instances; the others go to the smaller ones, side by side with them (the kernel
+// for those is launched second and starts where this one leaves room).  As many as hold them all at once, and no fewer than
+// their share of the work, one of them counted as eight smaller ones (25 warp milliseconds alone and 40 in company, against 4, over 40,000
+// requests).  One kernel after the other, a few hundred of them among 30,000 ran three warps on each SM for 29 of 80 ms; side by side
+// 51 ms (73 -> 51 and 82 -> 51 over two draws).
+__device__ __forceinline__ uint32_t walk_big_blocks(const EvalParams& P) {
+    const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
+    const uint64_t big = (uint64_t)P.bucket_count[kWalkBig0] * n_traces;
+    if (P.big_grid == 0u || big == 0u) return 0u;
+    uint64_t small = 0;
+    for (int mode = 0; mode < kWalkModes; mode++) small += P.bucket_count[kWalkBucket0 + mode];
+    small *= (uint64_t)n_traces * P.walk_parts;
+    const uint32_t warps = walk_big_warps(P, (uint32_t)kWalkWarps);
+    const uint64_t once = (big + warps - 1u) / warps, share = (8u * big * P.big_grid + 8u * big + small - 1u) / (8u * big + small);
+    return (uint32_t)min(min((uint64_t)P.big_grid, big), max(once, share));
+}
+
 // `Warps`: 16, or 12 for small batches under fixed speeds and queues (route.cuh).  Mode k: the block's warps >> k at work, each with
-// 2^k times one warp's part of the pool.  The first placements are dealt out in order, over the SMs first; after that whoever is
-// free takes the next.
+// 2^k times one warp's part of the pool.  The first placements are dealt out in order, over the SMs first, but not to blocks that
+// start late; after that whoever is free takes the next.
 template <bool Opt, int Eng, bool Wide, bool Big, int Warps, bool Rcp>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_constant__ EvalParams P) {
     constexpr bool kLong = Wide && Eng != 2;  // (queues: 64-bit times in the usual buckets)
     constexpr int kFirst = kLong ? kWalkLong0 : (Big ? kWalkBig0 : kWalkBucket0);
-    if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
     uint32_t any = 0;
     for (int mode = 0; mode < (Big && !kLong ? 1 : kWalkModes); mode++) any |= P.bucket_count[kFirst + mode];
-    if (any == 0) return;
+    if (P.stall_test) any = 0;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
+    uint32_t blocks = gridDim.x, mine = blockIdx.x;  // blocks that the first placements are dealt out to, this one's number
+    if constexpr (Big && !kLong) {
+        blocks = min(gridDim.x, any * (P.n_traces > 1 ? P.n_traces : 1u));
+        if (P.big_grid) blocks = min(blocks, walk_big_blocks(P));
+        if (blockIdx.x >= blocks) return;
+        let_next_start();
+    } else {
+        const uint32_t others = !Big && any ? walk_big_blocks(P) : 0u;
+        if (others) {  // some blocks start late: numbers go by who starts first
+            if (threadIdx.x == 0) w1(0u) = atomicAdd(&P.work_ctr[15], 1u);  // (where the rings will be)
+            __syncthreads();
+            mine = w1(0u);
+            blocks -= min(blocks, others);
+        }
+        if (any == 0) {
+            wait_for_last();
+            return;
+        }
+    }
     constexpr bool kDynamic = Eng == 0 && !Wide && !Big;
     const WalkLayout L = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Rcp, kDynamic);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
@@ -935,41 +977,56 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
         // block's share of the list: the first blocks to start would take what others have the room for (tables of 100 rows, 500 x
         // 4,000 with and without that bound: fixed speeds 3.90 and 4.14 ms, queues 4.31 and 4.51).
         const uint32_t n = P.bucket_count[kWalkBig0];
-        if (blockIdx.x >= n * (P.n_traces > 1 ? P.n_traces : 1u)) return;
         const uint32_t cand = P.bucket_list[(size_t)kWalkBig0 * P.n_cand + blockIdx.x / (P.n_traces > 1 ? P.n_traces : 1u)];
         const uint32_t pool = P.walk_bytes * kWalkWarps, room = (256u - (P.code2[cand] & 0xFFu)) * kWalkStepBytes;
-        const uint32_t share = (n * (P.n_traces > 1 ? P.n_traces : 1u) + gridDim.x - 1u) / gridDim.x;
+        const uint32_t share = (n * (P.n_traces > 1 ? P.n_traces : 1u) + blocks - 1u) / blocks;
         const uint32_t act = max(1u, min(min((uint32_t)Warps, share), pool / room)), part = (pool / act) & ~127u;
         // (how many that is differs from block to block: the first warps start with what is theirs, the rest with whatever is next)
         uint32_t idx = blockIdx.x;
         if (warp > 0 && warp < act) {
-            if ((tid & 31u) == 0) idx = gridDim.x + atomicAdd(&P.walk_ctr[kWalkBig0 - kWalkBucket0], 1u);
+            if ((tid & 31u) == 0) idx = blocks + atomicAdd(&P.walk_ctr[kWalkBig0 - kWalkBucket0], 1u);
             idx = __shfl_sync(kWFull, idx, 0);
         }
         if (warp < act)
-            Walk<Opt, Eng, Wide, Big, Rcp>::bucket(P, L, kWalkBig0, L.pool + warp * part, idx, gridDim.x,
+            Walk<Opt, Eng, Wide, Big, Rcp>::bucket(P, L, kWalkBig0, L.pool + warp * part, idx, blocks,
                                               reinterpret_cast<unsigned char*>(P.payload) + blockIdx.x * walk_big_scratch(pool));
     } else {
         for (int mode = kWalkModes - 1; mode >= 0; mode--) {
             if (P.bucket_count[kFirst + mode] == 0) continue;  // the same for the whole block
             const uint32_t act = (uint32_t)Warps >> mode, part = (kLong ? P.walk_bytes : P.walk_usual) << mode;
             using Body = typename std::conditional<kDynamic, WalkDynamic<Opt, Rcp>, Walk<Opt, Eng, Wide, Big, Rcp>>::type;
-            if (warp < act)
-                Body::bucket(P, L, kFirst + mode, L.pool + warp * part, warp * gridDim.x + blockIdx.x,
-                                                  act * gridDim.x, nullptr);
+            if (warp < act) {
+                uint32_t idx = warp * blocks + mine;
+                if (mine >= blocks) {
+                    if ((tid & 31u) == 0) idx = act * blocks + atomicAdd(&P.walk_ctr[kFirst + mode - kWalkBucket0], 1u);
+                    idx = __shfl_sync(kWFull, idx, 0);
+                }
+                Body::bucket(P, L, kFirst + mode, L.pool + warp * part, idx, act * blocks, nullptr);
+            }
             if (mode) __syncthreads();
         }
+        wait_for_last();
     }
 }
 
 template <bool Opt, int Eng, bool Wide, bool Big, bool Rcp, int Warps = kWalkWarps>
-static cudaError_t launch_walk(const EvalParams& P, int grid, cudaStream_t stream) {
+static cudaError_t launch_walk(const EvalParams& P, int grid, bool overlap, cudaStream_t stream) {
     auto kernel = eval_walk_kernel<Opt, Eng, Wide, Big, Warps, Rcp>;
     const size_t smem = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Rcp, Eng == 0 && !Wide && !Big).pool + (Big || (Wide && Eng != 2) ? P.walk_bytes * kWalkWarps : P.walk_usual * Warps);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, (32 * Warps), smem, stream>>>(P);
-    return cudaGetLastError();
+    // `overlap`: its blocks may start before the kernel ahead of it has ended
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config = {};
+    config.gridDim = dim3((unsigned)grid);
+    config.blockDim = dim3(32u * Warps);
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = &attr;
+    config.numAttrs = overlap ? 1u : 0u;
+    return cudaLaunchKernelEx(&config, kernel, P);
 }
 
 }  // namespace maaso
