@@ -295,16 +295,19 @@ struct WalkDynamic {
                 const uint32_t first = __ballot_sync(kWFull, live);
                 if (Opt || first == 0u) return first;
                 // each instance of the model by itself: its start time at the latest look at it, its prefill of this
-                // request, its step
+                // request, its step; two at a time, as what one waits for is a chain of loads and products (30,000 x 30,000 under load
+                // 9.42 -> 9.15 ms, one node's first 148 1 % less)
                 bool ok = rel == kFar;
                 uint32_t j = live ? me.z : 0u;
                 const uint32_t j_end = live ? me.w : 0u;
-                while (__any_sync(kWFull, j < j_end && !ok)) {
-                    const uint4 e = ld4(j < j_end ? j : ents);  // (no branch)
+                do {
+                    const bool one = j < j_end, two = j + 16u < j_end;
+                    const uint4 e = ld4(one ? j : ents), f = ld4(two ? j + 16u : ents);  // (no branch)
                     const uint32_t since = (uint32_t)(max(at, (int32_t)e.x) - rel) + (uint32_t)Walk<Opt, 0, false, false>::prefill(e.y, e.z, c_in);
-                    ok = ok | ((j < j_end) & lim.met(since, Sm1, e.w));
-                    j += 16u;
-                }
+                    const uint32_t since2 = (uint32_t)(max(at, (int32_t)f.x) - rel) + (uint32_t)Walk<Opt, 0, false, false>::prefill(f.y, f.z, c_in);
+                    ok = ok | (one & lim.met(since, Sm1, e.w)) | (two & lim.met(since2, Sm1, f.w));
+                    j += 32u;
+                } while (__any_sync(kWFull, j < j_end && !ok));
                 return __ballot_sync(kWFull, live && ok);
             };
             auto report = [&](uint32_t served, uint32_t end) {
@@ -321,13 +324,21 @@ struct WalkDynamic {
                     if (side) report(0u, 32u);
                 }
                 if (cb >= n_req) break;
+                bool gone = false;  // (its rounds are over)
                 uint32_t from = 0, served = 0, end = 32u;  // `end`: where a failed placement stops
                 do {
                     // The list of requests that need a round, up to one that is out of the epoch's reach; what the keys need room
-                    // for (an end index is at most 2^16 beyond one before it).
-                    const uint32_t far = __ballot_sync(kWFull, max(now, rel) >= kWalkNowMax) & live;
-                    if (__any_sync(kWFull, (w > 0) & (K > kRelMax - (40u << 16)))) {
-                        if (w > 0) {
+                    // for (an end index is at most 2^16 beyond one before it), a placement that left the horizon: one vote for all that is
+                    // rare (under load 1.6 % less).
+                    const bool mine = ((live >> lane) & 1u) != 0u, beyond = mine & (max(now, rel) >= kWalkNowMax), high = (w > 0) & (K > kRelMax - (40u << 16));
+                    uint32_t far = 0;
+                    if (__any_sync(kWFull, beyond | high | (bit == 0u && lane < n_i))) {
+                        if (__any_sync(kWFull, bit == 0u && lane < n_i)) {
+                            gone = true;
+                            break;
+                        }
+                        far = __ballot_sync(kWFull, beyond);
+                        if (__any_sync(kWFull, high) && w > 0) {
                             const uint32_t d = K << 6;
                             for (uint32_t at = area; at < pay; at += at == area + 28u ? 68u : 4u) {  // block minima, keys
                                 const uint32_t k = ld1(at);
@@ -335,12 +346,12 @@ struct WalkDynamic {
                             }
                             if (kmin != kKeyEmpty) kmin -= d;
                             peek();
+                            K = 0;
                         }
-                        K = 0;
+                        if (far) live &= (far & (0u - far)) - 1u;
                     }
-                    if (far) live &= (far & (0u - far)) - 1u;
                     uint32_t n = (uint32_t)__popc(live);
-                    if ((live >> lane) & 1u) {
+                    if (((live >> lane) & 1u) != 0u) {
                         // {arrival, input tokens, model bit | lane << 16, keys below this take the usual path}
                         // {bound of the first token after the arrival, of the step, of the end + 1, output tokens - 1 | the factor of the step in
                         // the bound of the end << 16 (the same, 0 without a limit)}
@@ -533,7 +544,7 @@ struct WalkDynamic {
                     live = test(from);
                 } while (live);
                 if (side) report(served, end);
-                if (status || __any_sync(kWFull, lane < n_i && bit == 0u)) break;
+                if (gone | (status != 0u)) break;
             }
 
             // ---- through the trace: drain, account, write the record ------------------------------------------------
