@@ -245,6 +245,15 @@ struct EvalParams : Route {
     const uint64_t* trace_class_tot[kMaxTraces];  // [n_classes][2]: count, checksum sum
     uint32_t trace_n[kMaxTraces];
     const uint4* trace_reqs[kMaxTraces];  // walking kernel: the requests as loaded
+    // Walking kernel: the requests of the patient classes once more, in order, their indices, and for every 32 requests of the trace
+    // how many patient ones are ahead of them (null, 0: not kept).  Requests of the other classes (`impatient`: the set of those below
+    // 32) must start within `patience` us of their arrival; when the clock is `trace_lead` ahead it is worth leaving them out.
+    const uint4* trace_patient[kMaxTraces];
+    uint32_t trace_n_patient[kMaxTraces];
+    int32_t trace_lead[kMaxTraces];
+    int32_t patience;
+    uint32_t impatient;
+    uint32_t apart;  // they are looked at by themselves
     const uint64_t* rej_hash;  // [n_req] checksum term of "request r was rejected" (same for every candidate)
     const int32_t* rows;     // [n_rows][kRowStride]
     const int32_t* devices;

@@ -1,5 +1,6 @@
 // C ABI of the placement-scoring library: handles, validation, host<->device copies and
 // kernel launches.  Semantics of every entry point are documented in include/maaso.h.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -11,6 +12,7 @@
 
 namespace maaso {
 cudaError_t launch_prep(const EvalParams& P, const uint32_t* dump_idx, cudaStream_t stream, int* launches);
+cudaError_t launch_pick_patient(const uint4* reqs, const int64_t* classes, int64_t patience, const uint32_t* ahead, uint4* out, uint32_t* idx, uint32_t n);
 cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n);
 cudaError_t launch_scan_trace(const uint4* reqs, const int64_t* classes, uint4* scan, uint32_t n);
 size_t scan_trace_units(uint32_t n);
@@ -58,6 +60,9 @@ struct maaso_trace {
     uint4* d_cooked;  // prepared records for the lane-group kernel
     uint4* d_scan;    // scan records for the thread mapping
     uint64_t* d_class_tot;  // per class: number of requests, sum of their "rejected" checksum terms
+    uint4* d_patient;  // with what follows: EvalParams::trace_patient
+    uint32_t n_patient, impatient;
+    int32_t patience, lead;
     std::vector<int64_t> h_classes;  // host copy of the class table (several traces in one call must agree on it)
     uint64_t n;
     uint32_t n_classes;
@@ -401,6 +406,29 @@ MAASO_API int maaso_load_profile(maaso_ctx* ctx, const maaso_profile_desc* d) {
     return MAASO_OK;
 }
 
+// Classes by how long after its arrival a request can still meet its limits (no limit on the first token or the end: for good).
+// Where one group of them is at least eight times as patient as the rest, the trace keeps its requests apart as well
+// (EvalParams::trace_patient); returns the longest patience of the rest, or -1.
+static int64_t split_by_patience(const std::vector<int64_t>& cls) {
+    std::vector<int64_t> slack;
+    for (size_t k = 0; k < cls.size(); k += 3) {
+        int64_t s = cls[k] >= 0 ? cls[k] : INT64_MAX;
+        if (cls[k + 2] >= 0 && cls[k + 2] < s) s = cls[k + 2];
+        slack.push_back(s);
+    }
+    std::sort(slack.begin(), slack.end());
+    int64_t at = -1;
+    double most = 8.0;
+    for (size_t i = 0; i + 1 < slack.size(); i++) {
+        const double ratio = (double)slack[i + 1] / (double)std::max<int64_t>(slack[i], 1);
+        if (slack[i] < kWalkLimMax && ratio >= most) {
+            most = ratio;
+            at = slack[i];
+        }
+    }
+    return at;
+}
+
 MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64_t n, const maaso_slo_class* classes,
                      uint32_t n_classes, maaso_trace** out) {
     if (!ctx || !out) return MAASO_EINVAL;
@@ -443,8 +471,19 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     uint64_t tok_sum = 0;
     uint32_t max_in = 0, max_out = 0;
     std::vector<uint32_t> count((size_t)n_classes * MAASO_MAX_MODELS, 0);
+    const int64_t patience = split_by_patience(cls);
+    std::vector<uint32_t> patient(n_classes, 0), ahead;
+    uint32_t n_patient = 0, impatient = 0;
+    if (patience >= 0) {
+        ahead.resize(n / 32 + 1);
+        for (uint32_t k = 0; k < n_classes; k++) {
+            patient[k] = (cls[3 * k] < 0 || cls[3 * k] > patience) && (cls[3 * k + 2] < 0 || cls[3 * k + 2] > patience);
+            if (!patient[k] && k < 32) impatient |= 1u << k;
+        }
+    }
     for (uint64_t r = 0; r < n; r++) {
         const maaso_request& q = host[r];
+        if (patience >= 0 && r % 32 == 0) ahead[r / 32] = n_patient;
         if (q.arrival_us < prev || q.arrival_us > kArrMax)
             return fail(ctx, MAASO_EINVAL, "trace: arrivals must be non-negative, non-decreasing, below 2^50");
         prev = q.arrival_us;
@@ -456,6 +495,7 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         if (q.in_tokens > max_in) max_in = q.in_tokens;
         if (q.out_tokens > max_out) max_out = q.out_tokens;
         count[(size_t)q.cls * MAASO_MAX_MODELS + q.model]++;
+        n_patient += patient[q.cls];
         class_tot[(size_t)q.cls * 2] += 1;
         class_tot[(size_t)q.cls * 2 + 1] += host_rejected_hash((uint32_t)r);
     }
@@ -473,6 +513,12 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     {
         const double span_s = n > 1 ? (double)(host[n - 1].arrival_us - host[0].arrival_us) * 1e-6 : 0.0;
         t->tok_rate = span_s > 0.0 ? (double)tok_sum / span_s : 0.0;
+        // Apart from the others only if that leaves half of them out, and once 40 of them in a row are likely to be enough.
+        if ((uint64_t)n_patient * 2 > n || !t->small_limits) n_patient = 0;
+        t->n_patient = n_patient;
+        t->patience = (int32_t)std::max<int64_t>(patience, 0);
+        t->impatient = impatient;
+        t->lead = (int32_t)std::min(t->patience + 40e6 * span_s / (double)std::max<uint32_t>(n_patient, 1u), 2147483647.0);
     }
     t->h_classes = cls;
     // requests | prepared records | scan tiles | rejection hashes | per-class totals, SLO classes
@@ -483,6 +529,8 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     const size_t o_scan = off;   off = align_up(off + scan_trace_units((uint32_t)n) * 16, 256);
     const size_t o_hash = off;   off = align_up(off + n1 * 8, 256);
     const size_t o_small = off;  off = align_up(off + (class_tot.size() + cls.size()) * 8, 256);
+    const size_t o_ahead = off + (size_t)n_patient * 20;  // behind the patient requests and their indices
+    const size_t o_patient = off; off = align_up(n_patient ? o_ahead + ahead.size() * 4 : off, 256);
     cudaError_t e = cudaSuccess;
     if (ctx->spare && ctx->spare_bytes >= off && ctx->spare_bytes / 4 <= off) {
         t->mem = ctx->spare;
@@ -508,12 +556,19 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     t->d_rej_hash = reinterpret_cast<uint64_t*>(mem + o_hash);
     t->d_class_tot = reinterpret_cast<uint64_t*>(mem + o_small);
     t->d_classes = reinterpret_cast<int64_t*>(mem + o_small) + class_tot.size();
+    t->d_patient = reinterpret_cast<uint4*>(mem + o_patient);
     std::vector<int64_t> small(class_tot.begin(), class_tot.end());
     small.insert(small.end(), cls.begin(), cls.end());
     if (n) e = cudaMemcpyAsync(t->d_reqs, reqs, n * sizeof(maaso_request),
                                on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, cudaStreamLegacy);
     if (e == cudaSuccess) e = cudaMemcpyAsync(mem + o_small, small.data(), small.size() * 8, cudaMemcpyHostToDevice, cudaStreamLegacy);
     if (e == cudaSuccess) e = launch_cook_trace(t->d_reqs, t->d_classes, t->d_cooked, t->d_rej_hash, (uint32_t)n);
+    if (n_patient) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mem + o_ahead, ahead.data(), ahead.size() * 4, cudaMemcpyHostToDevice, cudaStreamLegacy);
+        if (e == cudaSuccess)
+            e = launch_pick_patient(t->d_reqs, t->d_classes, patience, reinterpret_cast<const uint32_t*>(mem + o_ahead), t->d_patient,
+                                    reinterpret_cast<uint32_t*>(t->d_patient + n_patient), (uint32_t)n);
+    }
     if (e == cudaSuccess) e = launch_scan_trace(t->d_reqs, t->d_classes, t->d_scan, (uint32_t)n);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
@@ -589,7 +644,16 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         P.trace_class_tot[t] = traces[t]->d_class_tot;
         P.trace_n[t] = (uint32_t)traces[t]->n;
         P.trace_reqs[t] = traces[t]->d_reqs;
+        P.trace_patient[t] = traces[t]->d_patient;
+        P.trace_n_patient[t] = traces[t]->n_patient;
+        P.trace_lead[t] = traces[t]->lead;
     }
+    P.patience = trace->patience;
+    P.impatient = trace->impatient;
+    // (not where every rejected request is to be written down)
+    P.apart = 0u;
+    if (!o.dump_n && !o.rejected_by_model)
+        for (uint32_t t = 0; t < n_traces; t++) P.apart |= traces[t]->n_patient;
     P.rows = ctx->d_rows;
     P.devices = ctx->d_devices;
     P.min_devices = ctx->d_min_devices;

@@ -273,6 +273,30 @@ __global__ void cook_trace_kernel(const uint4* reqs, const int64_t* classes, uin
     o[2] = make_uint4(lo(h), hi(h), (q.S - 1u) | (q.cls << 16) | (q.model << 24), 0u);
 }
 
+// The requests whose first token or end may come more than `patience` us after their arrival, in order, and their indices;
+// `ahead`: how many of them are ahead of each 32 requests.
+__global__ void pick_patient_kernel(const uint4* reqs, const int64_t* classes, int64_t patience, const uint32_t* ahead, uint4* out, uint32_t* idx,
+                                    uint32_t n) {
+    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    bool patient = false;
+    if (r < n) {
+        v = reqs[r];
+        const uint32_t cls = decode_request(v).cls;
+        const int64_t ttft = classes[cls * 3 + 0], e2e = classes[cls * 3 + 2];
+        patient = (ttft < 0 || ttft > patience) && (e2e < 0 || e2e > patience);
+    }
+    const uint32_t set = __ballot_sync(0xFFFFFFFFu, patient);
+    if (!patient) return;
+    const uint32_t at = ahead[r / 32u] + (uint32_t)__popc(set & ((1u << (r & 31u)) - 1u));
+    out[at] = v;
+    idx[at] = r;
+}
+cudaError_t launch_pick_patient(const uint4* reqs, const int64_t* classes, int64_t patience, const uint32_t* ahead, uint4* out, uint32_t* idx, uint32_t n) {
+    pick_patient_kernel<<<(n + 255) / 256, 256>>>(reqs, classes, patience, ahead, out, idx, n);
+    return cudaGetLastError();
+}
+
 // Scan tiles of the thread mapping.  Tile t (kScanTile requests) is a header followed by one
 // 16-byte record per request.
 //   record: {arrival - the tile's base arrival (all ones: does not fit 32 bits, look at the full record),

@@ -925,7 +925,7 @@ __device__ __forceinline__ uint32_t walk_big_blocks(const EvalParams& P) {
 // `Warps`: 16, or 12 for small batches under fixed speeds and queues (route.cuh).  Mode k: the block's warps >> k at work, each with
 // 2^k times one warp's part of the pool.  The first placements are dealt out in order, over the SMs first, but not to blocks that
 // start late; after that whoever is free takes the next.
-template <bool Opt, int Eng, bool Wide, bool Big, int Warps, bool Rcp>
+template <bool Opt, int Eng, bool Wide, bool Big, int Warps, bool Rcp, bool Apart>
 __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_constant__ EvalParams P) {
     constexpr bool kLong = Wide && Eng != 2;  // (queues: 64-bit times in the usual buckets)
     constexpr int kFirst = kLong ? kWalkLong0 : (Big ? kWalkBig0 : kWalkBucket0);
@@ -994,7 +994,7 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
         for (int mode = kWalkModes - 1; mode >= 0; mode--) {
             if (P.bucket_count[kFirst + mode] == 0) continue;  // the same for the whole block
             const uint32_t act = (uint32_t)Warps >> mode, part = (kLong ? P.walk_bytes : P.walk_usual) << mode;
-            using Body = typename std::conditional<kDynamic, WalkDynamic<Opt, Rcp>, Walk<Opt, Eng, Wide, Big, Rcp>>::type;
+            using Body = typename std::conditional<kDynamic, WalkDynamic<Opt, Rcp, Apart>, Walk<Opt, Eng, Wide, Big, Rcp>>::type;
             if (warp < act) {
                 uint32_t idx = warp * blocks + mine;
                 if (mine >= blocks) {
@@ -1009,9 +1009,9 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_walk_kernel(const __grid_c
     }
 }
 
-template <bool Opt, int Eng, bool Wide, bool Big, bool Rcp, int Warps = kWalkWarps>
+template <bool Opt, int Eng, bool Wide, bool Big, bool Rcp, int Warps = kWalkWarps, bool Apart = false>
 static cudaError_t launch_walk(const EvalParams& P, int grid, bool overlap, cudaStream_t stream) {
-    auto kernel = eval_walk_kernel<Opt, Eng, Wide, Big, Warps, Rcp>;
+    auto kernel = eval_walk_kernel<Opt, Eng, Wide, Big, Warps, Rcp, Apart>;
     const size_t smem = walk_layout(P.n_rows, P.n_classes, Wide, Warps, Rcp, Eng == 0 && !Wide && !Big).pool + (Big || (Wide && Eng != 2) ? P.walk_bytes * kWalkWarps : P.walk_usual * Warps);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
