@@ -23,8 +23,9 @@
 // Measured against the body that it replaced here (that of Walk): warp instructions of a round that admits 189 -> 135, with a
 // completion before 286 -> 214, with a wait 304 -> 171; 2,000 x 17,000 of the paper's shape 8.9 -> 6.4 ms, one node's 10,864 x
 // 10,000 6.4 -> 4.63, three models under load 12,000 x 30,000 4.51 -> 4.25, masked sub-clusters 9,000 x 12,000 18.3 -> 15.9.
-// Dropped: completions and admissions without a branch, lanes that have none writing to a dummy region (a lone warp as fast,
-// +5 % instructions); the accounting of completions inlined (+7 %).
+// Dropped: completions without a branch (a lone warp 1 % faster, in company up to 4 % slower: thirteen selections); the accounting of
+// completions inlined (+7 %); two requests of different models in one round (most rounds of a loaded placement wait, which makes
+// the second one's look stale: +2 to 15 %); levels by address and block minima by atomics (as fast).
 #pragma once
 
 namespace maaso {
@@ -66,6 +67,20 @@ __device__ __forceinline__ void st2(uint32_t a, const uint2& v) {
 __device__ __forceinline__ void st1(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void stb(uint32_t a, uint32_t v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void min_shared(uint32_t a, uint32_t v) { asm volatile("red.shared.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+
+__device__ __forceinline__ void st1_if(bool p, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void st4_if(bool p, uint32_t a, const uint4& v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}"
+                 ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void stb_if(bool p, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void st2_if(bool p, uint32_t a, const uint2& v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.shared.v2.u32 [%0], {%1, %2};\n\t}" ::"r"(a), "r"(v.x), "r"(v.y), "r"((uint32_t)p) : "memory");
+}
 
 // `Rcp`: the decode-step rows carry reciprocals.  `Apart`: patient requests are also looked at by themselves (EvalParams::trace_patient).
 template <bool Opt, bool Rcp, bool Apart>
@@ -455,22 +470,29 @@ struct WalkDynamic {
                         // smallest (tier, predicted first token >= now), lowest instance among equals
                         const uint32_t key = ok ? (min((uint32_t)(first - now), kOffMax) << 5) + (full ? lane + kTier1 : lane) : kNone;
                         const uint32_t best = __reduce_min_sync(kWFull, key);
+                        // "map": prefill at the step boundary (running decodes stall), then occupy a free slot.  Every lane computes what it
+                        // would leave and one takes it: without a branch that only one lane takes 3 to 6 % less (computed ahead of the
+                        // choice, while it is under way, 1 to 3 % less alone but 3 % more under load, where most rounds wait).
+                        auto admit = [&](bool win) {
+                            const uint32_t nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top, nmin = min(kmin, nk), n_sw = more.x >> 5;
+                            const uint64_t ahead = (uint64_t)((nmin >> 6) - nK) * n_sw;
+                            const uint32_t n_end = (uint32_t)ahead + (uint32_t)first;
+                            const bool n_in = ((uint32_t)(ahead >> 32) == 0u) & (max((uint32_t)ahead, n_end) <= (uint32_t)kWalkHorizon);
+                            st1_if(win, area + kWalkKeys + 4u * top, nk);
+                            st2_if(win, pay + 8u * top, make_uint2((uint32_t)first, req));
+                            st1_if(win, area + ((top >> 1) & 28u), min(top_min, nk));
+                            t = win ? first : t;
+                            K = win ? nK : K;
+                            kmin = win ? nmin : kmin;
+                            w = win ? w + 1u : w;
+                            step = win ? more.x : step;
+                            rcp = win ? more.y : rcp;
+                            sw = win ? n_sw : sw;
+                            tc = win ? (int32_t)n_end : tc;
+                            bit = win & !n_in ? 0u : bit;
+                        };
                         if (best < usual) {
-                            // "map": prefill at the step boundary (running decodes stall), then occupy a free slot
-                            if (key == best) {
-                                const uint32_t nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
-                                st1(area + kWalkKeys + 4u * top, nk);
-                                st2(pay + 8u * top, make_uint2((uint32_t)first, req));
-                                st1(area + ((top >> 1) & 28u), min(top_min, nk));
-                                t = first;
-                                K = nK;
-                                kmin = min(kmin, nk);
-                                w++;
-                                step = more.x;
-                                rcp = more.y;
-                                sw = step >> 5;
-                                next_end(true);
-                            }
+                            admit(key == best);
                             peek();
                         } else if (best == kNone) {
                             // overflow protection: nobody can meet the deadline.  What the scan went by is out of date: once more
@@ -508,26 +530,30 @@ struct WalkDynamic {
                                 // With the worst-case estimate the next round cannot choose differently: at that time the winner has
                                 // a free slot with the same predicted first token, and no other instance's prediction can have become
                                 // earlier or feasible.  So it is only counted, and the request takes the slot over.
-                                bool twin = false;
-                                if (win) {
-                                    const uint32_t s = kmin & 63u, keys = area + kWalkKeys, kb = keys + 4u * (s & 56u), mb = area + ((s >> 1) & 28u);
-                                    st1(keys + 4u * s, kKeyEmpty);
-                                    st1(mb, kKeyEmpty);
+                                bool twin;
+                                {  // (without a branch, as above, 1 to 2 % less; the other lanes look at their first slot)
+                                    const uint32_t s = win ? kmin & 63u : 0u, keys = area + kWalkKeys, kb = keys + 4u * (s & 56u), mb = area + ((s >> 1) & 28u);
+                                    st1_if(win, keys + 4u * s, kKeyEmpty);
+                                    st1_if(win, mb, kKeyEmpty);
                                     const uint4 k0 = ld4(kb), k1 = ld4(kb + 16u), m0 = ld4(area), m1 = ld4(area + 16u);
                                     const uint2 run = ld2(pay + 8u * s);
                                     const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                                     const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
                                     const uint32_t bmin = min8(kv), others = min(bmin, min8(mv));
-                                    K = kmin >> 6;
-                                    const uint32_t nk = ((K + Sm1) << 6) | s;
-                                    st4(ring + 16u * ring_n, make_uint4((uint32_t)t0, run.x, run.y, place));
-                                    st1(keys + 4u * s, nk);
-                                    st2(pay + 8u * s, make_uint2((uint32_t)first, req));
-                                    st1(mb, min(bmin, nk));
-                                    t = first;
-                                    kmin = min(others, nk);
-                                    next_end(true);
-                                    twin = (others >> 6) == K;
+                                    const uint32_t nK = kmin >> 6, nk = ((nK + Sm1) << 6) | s, nmin = min(others, nk);
+                                    st4_if(win, ring + 16u * ring_n, make_uint4((uint32_t)t0, run.x, run.y, place));
+                                    st1_if(win, keys + 4u * s, nk);
+                                    st2_if(win, pay + 8u * s, make_uint2((uint32_t)first, req));
+                                    st1_if(win, mb, min(bmin, nk));
+                                    const uint64_t ahead = (uint64_t)((nmin >> 6) - nK) * sw;
+                                    const uint32_t n_end = (uint32_t)ahead + (uint32_t)first;
+                                    const bool n_in = ((uint32_t)(ahead >> 32) == 0u) & (max((uint32_t)ahead, n_end) <= (uint32_t)kWalkHorizon);
+                                    K = win ? nK : K;
+                                    t = win ? first : t;
+                                    kmin = win ? nmin : kmin;
+                                    tc = win ? (int32_t)n_end : tc;
+                                    bit = win & !n_in ? 0u : bit;
+                                    twin = win & ((others >> 6) == nK);
                                 }
                                 if (++ring_n >= kRoom) flush();
                                 uint32_t tm = __ballot_sync(kWFull, twin | (now >= kWalkNowMax));
@@ -553,20 +579,7 @@ struct WalkDynamic {
                                 }
                                 if (++ring_n >= kRoom) flush();
                             } else {  // (as above)
-                                if (win) {
-                                    const uint32_t nK = w > 0u ? K : 0u, nk = ((nK + Sm1) << 6) | top;
-                                    st1(area + kWalkKeys + 4u * top, nk);
-                                    st2(pay + 8u * top, make_uint2((uint32_t)first, req));
-                                    st1(area + ((top >> 1) & 28u), min(top_min, nk));
-                                    t = first;
-                                    K = nK;
-                                    kmin = min(kmin, nk);
-                                    w++;
-                                    step = more.x;
-                                    rcp = more.y;
-                                    sw = step >> 5;
-                                    next_end(true);
-                                }
+                                admit(win);
                                 peek();
                             }
                         }
