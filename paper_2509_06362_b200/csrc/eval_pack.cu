@@ -101,7 +101,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
     const uint32_t n8 = (P.bucket_count[kPack8] + 3u) / 4u, n4 = (P.bucket_count[kPack4] + 7u) / 8u;
     const uint32_t total = (n8 + n4) * n_traces;
-    const uint32_t area = L.pool + threadIdx.x * kPackLane, keys = area + 96u;
+    const uint32_t area = L.pool + threadIdx.x * kPackLane, keys = area + 96u, smem = smem_addr(walk_smem);
     unsigned char* const scratch = reinterpret_cast<unsigned char*>(P.payload) + ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * kPackScratch;
     uint2* const pay = reinterpret_cast<uint2*>(scratch);
     const bool use_mask = P.class_mask != nullptr && P.n_classes <= 32;
@@ -214,6 +214,11 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
             take_chunk(nxt);
             nxt = __ldg(reqs + min(cb + 32u + lane, n_req - 1u));
             const uint32_t n_chunk = min(32u, n_req - cb);
+            // what the keys need room for: an end index is at most 2^16 beyond one before it
+            if (__any_sync(kWFull, (in.w > 0) & (in.K > kPackRelMax - (40u << 16))) && in.w > 0) {
+                in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K << 7, in.kmin);
+                in.K = 0;
+            }
             for (uint32_t i = 0; i < n_chunk; i++) {
                 int32_t arrival = __shfl_sync(kWFull, rel, (int)i);
                 const uint32_t in_tok = __shfl_sync(kWFull, c_in, (int)i), meta = __shfl_sync(kWFull, c_meta, (int)i);
@@ -307,22 +312,23 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                     } else {
                         // The entry taken now is the slot's last but one: copies of earlier steps have to be through, this step's not.
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
-                        if (win) {
-                            in.t += pre;
-                            if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
-                            if (in.K + Sm1 > kPackRelMax) {
-                                in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K << 7, in.kmin);
-                                in.K = 0;
-                            }
-                            const uint32_t nk = ((in.K + Sm1) << 7) | top;
-                            w1(keys + 4u * (top & 63u)) = nk;
-                            pay[top] = make_uint2((uint32_t)in.t, cb + i);
-                            const uint32_t mb = area + ((top >> 1) & 28u);
-                            w1(mb) = min(w1(mb), nk);
-                            in.kmin = min(in.kmin, nk);
-                            in.w++;
-                            next_end((in.kmin >> 7) - in.K, true, more);
-                        }
+                        // (without a branch: every lane computes what it would leave, the winners take it: one node's 10,864 x 5,000
+                        // 6.6 -> 6.5 ms, with 12 warps 6.3 -> 6.2; three models, 40,000 x 3,000 13.8 -> 13.5)
+                        const uint32_t nK = in.w > 0 ? in.K : 0u, nk = ((nK + Sm1) << 7) | top, nmin = min(in.kmin, nk);  // (no live end index: the counter restarts)
+                        const int32_t nt = in.t + pre;
+                        const uint64_t tc = (uint64_t)((nmin >> 7) - nK) * more.x + (uint32_t)nt;
+                        st1_if(win, smem + keys + 4u * (top & 63u), nk);
+                        if (win) pay[top] = make_uint2((uint32_t)nt, cb + i);
+                        const uint32_t mb = smem + area + ((top >> 1) & 28u);
+                        st1_if(win, mb, min(ld1(mb), nk));
+                        in.t = win ? nt : in.t;
+                        in.K = win ? nK : in.K;
+                        in.kmin = win ? nmin : in.kmin;
+                        in.w = win ? in.w + 1u : in.w;
+                        in.sw = win ? more.x : in.sw;
+                        in.rsw = win ? more.y : in.rsw;
+                        in.tb = win ? (int32_t)((uint32_t)tc - more.x) : in.tb;
+                        bad = bad | (win & (tc > (uint64_t)kWalkHorizon));
                     }
                     if (!Opt) break;
                     act = again;
@@ -415,15 +421,15 @@ static cudaError_t launch_pack(const EvalParams& P, int grid, cudaStream_t strea
     kernel<<<grid, 32 * Warps, smem, stream>>>(P);
     return cudaGetLastError();
 }
-// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which take 152 to
-// 156 registers there and spill nothing (14 warps: 88 to 100 bytes).  14 and not 16 for the rest: their shared memory fits a
+// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which take 156 to
+// 158 registers there and spill nothing (14 warps: 92 to 100 bytes).  14 and not 16 for the rest: their shared memory fits a
 // partition that leaves 60 KB of L1 instead of 28 (16 rates, 10,864 x 2,500: 29.5 and 31.7 ms, optimistic estimate 32.0 and 33.5).
-// Measured, 12 and 14 warps: one node's 10,864 x 4,000 under 1, 2 and 4 traces 5.0 and 5.2, 7.7 and 8.0, 13.6 and 13.2, 16 traces x
-// 2,500 30.9 and 29.5; three models at 1 a second, 20,000 x 4,000 11.8 and 11.3, 40,000 20.8 and 19.4.  So the line is where it must
-// lie for several models and early for one, which 12 warps serve better up to about 25,000 placements.
+// Measured, 12 and 14 warps, optimistic estimate: one node's 10,864 x 4,000 under 2 traces 8.3 and 8.9, 4 traces x 10,000 35.7 and 34.7;
+// worst-case estimate 10,864 x 5,000 6.2 and 6.5, 3 traces x 4,000 10.9 and 10.6; three models, 40,000 x 3,000 14.5 and 13.5, at 1 a
+// second 20,000 x 4,000 11.8 and 11.3.  So the line is at two such waves with one model and at one with several.
 cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
     const uint64_t placements = (uint64_t)P.n_cand * (P.n_traces > 1 ? P.n_traces : 1u);
-    return placements <= 6ull * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kPackWarps>(P, grid, stream);
+    return placements <= (P.n_models == 1 ? 14ull : 6ull) * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kPackWarps>(P, grid, stream);
 }
 
 }  // namespace maaso
