@@ -68,20 +68,6 @@ __device__ __forceinline__ void st1(uint32_t a, uint32_t v) { asm volatile("st.s
 __device__ __forceinline__ void stb(uint32_t a, uint32_t v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void min_shared(uint32_t a, uint32_t v) { asm volatile("red.shared.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 
-__device__ __forceinline__ void st1_if(bool p, uint32_t a, uint32_t v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void st4_if(bool p, uint32_t a, const uint4& v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}"
-                 ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void stb_if(bool p, uint32_t a, uint32_t v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void st2_if(bool p, uint32_t a, const uint2& v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.shared.v2.u32 [%0], {%1, %2};\n\t}" ::"r"(a), "r"(v.x), "r"(v.y), "r"((uint32_t)p) : "memory");
-}
-
 // `Rcp`: the decode-step rows carry reciprocals.  `Apart`: patient requests are also looked at by themselves (EvalParams::trace_patient).
 template <bool Opt, bool Rcp, bool Apart>
 struct WalkDynamic {

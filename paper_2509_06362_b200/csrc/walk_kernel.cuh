@@ -23,11 +23,15 @@
 // the shortest round (walk_dynamic.cuh).  `Walk` here is the body of all the others.
 //
 // Measured (B200, whole calls with routing and top-k; lane-group, thread or one-warp kernel before): 143 placements x 500
-// requests 0.17 ms (0.56), one node's 10,864 x 10,000 4.6 ms (12.0), 2,000 x 17,000 of the paper's shape 6.4 to 6.6 ms (33.9), with
-// queues 5.3 ms (27.8), with fixed speeds 9.5 ms, three models, 100,000 x 100,000 under load 92.4 ms (135), 2,000 placements of 33
-// to 128 instances x 10,000 7.8 to 8.7 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
+// requests 0.15 ms (0.56), one node's 10,864 x 10,000 4.2 ms (12.0), 2,000 x 17,000 of the paper's shape 6.0 to 6.2 ms (33.9), with
+// queues 5.2 ms (27.8), three models, 100,000 x 100,000 under load 52 ms (135), 2,000 placements of 33 to 128 instances x
+// 10,000 6.7 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
 // needs is therefore read from shared memory ahead of the choice, the uncommon outcomes share one branch, and tests of several
 // conditions are written without branches (& and | for && and ||).
+// What some of the lanes do, an admission or an instance's state out of and into shared memory, all lanes compute, with
+// predicated stores and selections: parting the lanes and joining them again took longer than the work (2,000 placements of 33 to 128
+// instances x 10,000 8.40 -> 6.75 ms, 500 with fixed speeds 7.54 -> 6.02; masked sub-clusters, 9,000 x 12,000 9.03 -> 7.74).
+// Completions are left in a branch (without it 2 % slower to 2 % faster).
 //
 // The block's pool of shared memory is split evenly among its warps.  Placements beyond one warp's part run
 // first, with half, a quarter, ... of the warps at work and twice, four times, ... the room for each (kWalkModes);
@@ -79,6 +83,20 @@ __device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_s
 __device__ __forceinline__ uint64_t warp_min(uint64_t v) {  // the smallest high half, the smallest low half that comes with it
     const uint32_t hi = (uint32_t)(v >> 32), mh = __reduce_min_sync(kWFull, hi);
     return ((uint64_t)mh << 32) | __reduce_min_sync(kWFull, hi == mh ? (uint32_t)v : 0xFFFFFFFFu);
+}
+// Stores of the lanes for which `p` holds, to shared memory by its own addresses, without a branch.
+__device__ __forceinline__ void st1_if(bool p, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void st4_if(bool p, uint32_t a, const uint4& v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}"
+                 ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void stb_if(bool p, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void st2_if(bool p, uint32_t a, const uint2& v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.shared.v2.u32 [%0], {%1, %2};\n\t}" ::"r"(a), "r"(v.x), "r"(v.y), "r"((uint32_t)p) : "memory");
 }
 // Entry i of the decode-step rows in shared memory (WalkLayout::steps).
 __device__ __forceinline__ uint32_t walk_step(const EvalParams& P, uint32_t i) {
@@ -301,6 +319,13 @@ struct Walk {
         for (uint32_t k = 0; k < kRest / 16u; k++)
             if (all || k < (Wide ? 3u : 2u)) w4(rest + 16u * (k * n_i + j)) = u[k];
     }
+    // What a round changes, of the lanes for which `p` holds.
+    static __device__ __forceinline__ void put_if(bool p, uint32_t rest, uint32_t n_i, uint32_t j, const Inst& in) {
+        uint4 u[(sizeof(Inst) + 15) / 16];
+        memcpy(u, &in, sizeof(Inst));
+#pragma unroll
+        for (uint32_t k = 0; k < (Wide ? 3u : 2u); k++) st4_if(p, smem_addr(walk_smem) + rest + 16u * (k * n_i + j), u[k]);
+    }
     static __device__ __forceinline__ void get(uint32_t rest, uint32_t ents, uint32_t n_i, uint32_t j, Inst& in) {
         uint4 u[(sizeof(Inst) + 15) / 16];
 #pragma unroll
@@ -318,6 +343,7 @@ struct Walk {
     static __device__ __forceinline__ void bucket(const EvalParams& P, const WalkLayout& L, int bucket, uint32_t base,
                                                   uint32_t static_idx, uint32_t static_total, unsigned char* away) {
         constexpr uint32_t kCap = (uint32_t)kWalkRing;
+        const uint32_t smem = smem_addr(walk_smem);
         const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
         const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
         // With a queue in front of every instance the dispatcher never waits, and requests of one model leave no trace on the
@@ -644,6 +670,31 @@ struct Walk {
                         record(ring_n, in.t, in.t, req);
                     }
                     ring_n++;
+                } else if constexpr (!Wide) {
+                    // (without a branch: every lane computes what it would leave, the winner takes it)
+                    uint32_t nK = in.w > 0 ? in.K : 0u;  // no live end index: the counter restarts
+                    if (win && nK + Sm1 > kRelMax) {
+                        in.kmin = walk_rebase(in.area, in.keys, (in.B + 7u) >> 3, nK << 6, in.kmin);
+                        nK = 0;
+                    }
+                    const uint32_t nk = ((nK + Sm1) << 6) | top, nmin = min(in.kmin, nk), k8 = in.keys + 4u * top, mb = in.area + ((top >> 1) & 28u);
+                    const T nt = in.t + pre;
+                    const uint64_t tc = (uint64_t)((nmin >> 6) - nK) * more.x + (uint32_t)nt;
+                    st1_if(win, smem + k8, nk);
+                    st1_if(win, smem + mb, min(w1(mb), nk));
+                    if constexpr (kAway) {
+                        if (win) __stcg(reinterpret_cast<uint2*>(away + 2u * (k8 - L.pool)), make_uint2((uint32_t)nt, req));
+                    } else {
+                        st2_if(win, smem + in.pay + 8u * top, make_uint2((uint32_t)nt, req));
+                    }
+                    in.t = win ? nt : in.t;
+                    in.K = win ? nK : in.K;
+                    in.kmin = win ? nmin : in.kmin;
+                    in.w = win ? in.w + 1u : in.w;
+                    in.sw = win ? more.x : in.sw;
+                    in.rsw = win ? (Rcp ? more.y : walk_rcp(more.x)) : in.rsw;
+                    in.tb = win ? (T)((uint32_t)tc - more.x) : in.tb;
+                    bad = bad | (win & (tc > (uint64_t)kWalkHorizon));
                 } else if (win) {
                     const uint32_t slot = top;
                     in.t += pre;
@@ -780,8 +831,8 @@ struct Walk {
                         uint32_t at = lane;  // the instance behind `key`
                         for (uint32_t s = j_lo; s < j_hi; s += 32u) {
                             if (Big) {
-                                if (s + lane < n_i) get(rest, ents, n_i, s + lane, in);
-                                else in.tag = 0;
+                                get(rest, ents, n_i, min(s + lane, n_i - 1u), in);  // (no branch)
+                                in.tag = s + lane < n_i ? in.tag : 0u;
                             }
                             elig = (((in.tag >> model) & 1u) != 0u) & !bad;
                             const T p = prefill(in.pre_base, in.pre_q16, in_tok);
@@ -798,15 +849,13 @@ struct Walk {
                             // smallest (tier, predicted first token >= now >= 0), lowest instance among equals
                             const U k = ok ? (full ? kTier1 : (U)0) | (U)(t + p) : kNone;
                             if (Big) {
-                                if (elig) {
-                                    put(rest, n_i, s + lane, in, false);
-                                    lb = min(lb, t + (T)in.pre_base);
-                                }
+                                put_if(elig, rest, n_i, s + lane, in);
+                                lb = elig ? min(lb, t + (T)in.pre_base) : lb;
                                 if (k < key) { key = k; t0 = t; pre = p; at = s + lane; }
                             } else {
                                 key = k; t0 = t; pre = p;
                             }
-                            if (Big && elig && !Wide) w1(ents + 16u * (s + lane)) = (uint32_t)t;
+                            if (Big && !Wide) st1_if(elig, smem + ents + 16u * (s + lane), (uint32_t)t);
                         }
                         const U best = warp_min(key);
                         again = false;
@@ -814,11 +863,9 @@ struct Walk {
                         if (Big && best != kNone) {
                             const uint32_t lowest = __reduce_min_sync(kWFull, key == best ? at : 0xFFFFFFFFu);
                             wl = (int)(lowest & 31u);
-                            if ((int)lane == wl) {
-                                at = lowest;
-                                get(rest, ents, n_i, at, in);
-                                peek();
-                            }
+                            at = (int)lane == wl ? lowest : min(lane, n_i - 1u);  // (no branch)
+                            get(rest, ents, n_i, at, in);
+                            peek();
                         }
                         const bool win = (int)lane == wl;
                         bool go = true, queued = false;
@@ -852,9 +899,9 @@ struct Walk {
                         }
                         if (go) {
                             admit(win, wl, req, Sm1, pre, queued);
-                            if (Big && win) {
-                                if (!Wide) w1(ents + 16u * at) = (uint32_t)start();
-                                put(rest, n_i, at, in, false);
+                            if (Big) {
+                                if (!Wide) st1_if(win, smem + ents + 16u * at, (uint32_t)start());
+                                put_if(win, rest, n_i, at, in);
                             }
                         }
                         if (!Big && elig) wt<T>(Wide ? rest + 8u * lane : ent) = start();
