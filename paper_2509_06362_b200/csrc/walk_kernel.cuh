@@ -283,6 +283,9 @@ struct Walk {
     static constexpr U kTier1 = (U)1 << (8 * sizeof(U) - 1);
     static constexpr U kNone = ~(U)0;
     static constexpr uint32_t kKeyBytes = kFixed ? (uint32_t)sizeof(T) : 4u;
+    // Queues: times are below 2^58 (see the admission), so that a key has room for the lane (5 % less than a vote and a search
+    // for the winner's bit)
+    static constexpr bool kLaneKey = Eng == 2 && Wide && !Big;
     static constexpr bool kAway = Big && !Wide && !kFixed;  // running requests' data in global memory
     static constexpr uint32_t kBlock = Wide ? kWalkBlockLong : (Big ? kWalkBlockKeys : kWalkBlock);
     static constexpr WalkKind kKind = Wide ? kWalkLongKind : (Big ? kWalkBigKind : kWalkUsual);
@@ -619,6 +622,14 @@ struct Walk {
                     w4(ring + e * 16u) = make_uint4((uint32_t)fin, (uint32_t)first, req, in.tag >> 16);
                 }
             };
+            auto record_if = [&](bool p, uint32_t e, T fin, T first, uint32_t req) {
+                if constexpr (Wide) {
+                    st4_if(p, smem + ring + e * 16u, make_uint4(lo32(fin), hi32(fin), lo32(first), hi32(first)));
+                    st2_if(p, smem + ring_b + e * 8u, make_uint2(req, in.tag >> 16));
+                } else {
+                    st4_if(p, smem + ring + e * 16u, make_uint4((uint32_t)fin, (uint32_t)first, req, in.tag >> 16));
+                }
+            };
             // "map": prefill at the step boundary (running decodes stall), then occupy a free slot.  With fixed speeds the slot
             // is busy until the finish time, and `queued` takes over the slot that frees first; an instance's finish times
             // are in falling order, the winner's (lane `wl`) are moved by all lanes.  All lanes call it.
@@ -639,14 +650,9 @@ struct Walk {
                     }
                     const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? kEntry * level : 0u) + kEntry);
                     T fin = first + (T)span;
-                    if (win) {
-                        if constexpr (Wide) {
-                            if (((uint64_t)fin >> 57) != 0) status = MAASO_CAND_ELOOP;  // beyond what the engine takes
-                        } else {
-                            bad = bad || span > (uint64_t)kWalkHorizon || fin > (T)kWalkHorizon;
-                        }
-                        record(ring_n, fin, first, req);
-                    }
+                    if constexpr (Wide) status = win & (((uint64_t)fin >> 57) != 0) ? (uint32_t)MAASO_CAND_ELOOP : status;  // beyond what the engine takes
+                    else bad = bad | (win & ((span > (uint64_t)kWalkHorizon) | (fin > (T)kWalkHorizon)));
+                    record_if(win, ring_n, fin, first, req);
                     ring_n++;
                     fin = wshfl(fin, wl);
                     uint32_t pos = n;
@@ -657,10 +663,9 @@ struct Walk {
                     }
                     if (lane == 0) wt<T>(a + kKeyBytes * pos) = fin;
                     __syncwarp();
-                    if (win) {
-                        in.w = n + 1u;
-                        in.tb = wt<T>(a + kKeyBytes * n);
-                    }
+                    const T next_free = wt<T>(a + kKeyBytes * n);
+                    in.w = win ? n + 1u : in.w;
+                    in.tb = win ? next_free : in.tb;
                 } else if (Sm1 == 0u) {  // done at the end of its prefill, never occupies a slot
                     if (ring_n + 1u > kCap) flush();
                     if (win) {
@@ -847,7 +852,7 @@ struct Walk {
                             if (Opt && !full) sB = kFixed ? w1(in.row + kEntry * in.w + kEntry) : more.x;
                             const bool ok = elig && lim.met((U)(t + p - arrival), Sm1, sB);
                             // smallest (tier, predicted first token >= now >= 0), lowest instance among equals
-                            const U k = ok ? (full ? kTier1 : (U)0) | (U)(t + p) : kNone;
+                            const U k = !ok ? kNone : (full ? kTier1 : (U)0) | (kLaneKey ? (U)(t + p) << 5 | lane : (U)(t + p));
                             if (Big) {
                                 put_if(elig, rest, n_i, s + lane, in);
                                 lb = elig ? min(lb, t + (T)in.pre_base) : lb;
@@ -859,7 +864,9 @@ struct Walk {
                         }
                         const U best = warp_min(key);
                         again = false;
-                        int wl = __ffs((int)__ballot_sync(kWFull, key == best)) - 1;  // the winner's lane
+                        int wl;  // the winner's lane
+                        if constexpr (kLaneKey) wl = (int)((uint32_t)best & 31u);
+                        else wl = __ffs((int)__ballot_sync(kWFull, key == best)) - 1;
                         if (Big && best != kNone) {
                             const uint32_t lowest = __reduce_min_sync(kWFull, key == best ? at : 0xFFFFFFFFu);
                             wl = (int)(lowest & 31u);
