@@ -736,7 +736,8 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         pay_thread = ((size_t)grid_t * (thread_scratch_per_warp(thread_pool) + (ctx->thread_arena_kb > 0 ? thread_pool : 0)) +
                       sizeof(Payload) - 1) / sizeof(Payload);
     }
-    const Launches L = route_launches(P, cands->n_inst, may_leave);
+    // (an instance takes a device at least: beyond the budget no placement is valid)
+    const Launches L = route_launches(P, cands->n_inst < cands->budget ? cands->n_inst : cands->budget, may_leave);
     // Blocks per SM of the lane-group kernel.  A batch that three blocks per SM can hold in one
     // wave is bound by its longest dependent chains, which run faster with fewer warps sharing a
     // scheduler; a larger batch is bound by instruction issue and wants all four.  Lanes needed

@@ -253,6 +253,7 @@ struct Launches {
     bool groups, pack, walk, big, far, threads, blocks;
     uint32_t wide_from;  // one-warp kernel: the fewest instances of a placement that it takes; 0: it is not launched
 };
+// `n_inst`: the most instances that a valid placement of the call can have.
 inline Launches route_launches(const Route& r, uint64_t n_inst, bool may_leave) {
     Launches l;
     l.groups = route_groups(r);
