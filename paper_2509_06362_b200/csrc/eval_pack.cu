@@ -91,7 +91,10 @@ __device__ __forceinline__ void copy_run(uint32_t entry, const uint2* run) {
 // One warp takes work items, one after the other: 32 / G placements of the bucket whose groups have G lanes, the largest
 // placements first.  (One numbering for both buckets: starting on each from the same warps would have some replay an item
 // of each in a row where there is one item for each warp.)
-template <bool Opt>
+// `Straight`: completions and admissions without a branch; every lane computes what it would leave, those concerned take it.  Where the
+// longest items decide, that is better (one node's 10,864 x 5,000 with 12 warps 6.28 -> 6.03 ms), over many waves of items the
+// instructions count (16 rates x 10,864 x 10,000 121.2 and 122.1 ms, worst-case estimate 112.5 and 113.2).
+template <bool Opt, bool Straight>
 static __device__ __forceinline__ void pack_items(const EvalParams& P, const WalkLayout& L, uint32_t idx, uint32_t static_total) {
     using W = Walk<Opt, 0, false, false>;
     using Limits = typename W::Limits;
@@ -175,7 +178,36 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
             while (dm) {
                 const uint32_t adds = (uint32_t)__popc(dm & gmask);
                 if (__any_sync(kWFull, ring_n + adds > cap)) flush();
-                if (due) {
+                if constexpr (Straight) {
+                    // (the other lanes look at their first slot)
+                    const uint32_t run = due ? in.kmin & 127u : 0u, slot = run & 63u, kb = keys + ((slot >> 3) << 5), mb = area + ((slot >> 3) << 2);
+                    const uint32_t e = ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below));
+                    if (due) copy_run(e, pay + run);
+                    st1_if(due, smem + keys + (slot << 2), kKeyEmpty);
+                    st1_if(due, smem + mb, kKeyEmpty);
+                    const uint4 k0 = w4(kb), k1 = w4(kb + 16u), m0 = w4(area), m1 = w4(area + 16u);
+                    const uint2 step = w2(in.row + 8u * in.w - 8u);
+                    const int32_t nt = in.tb + (int32_t)in.sw;
+                    const uint32_t nK = in.kmin >> 7, nw = in.w - 1u;
+                    stb_if(due, smem + area + 32u + nw, run ^ 64u);
+                    st2_if(due, smem + e + 8u, make_uint2((uint32_t)nt, li));
+                    const uint32_t kv[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                    const uint32_t mv[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                    const uint32_t bmin = min8(kv), nmin = min(bmin, min8(mv)), left = (nmin >> 7) - nK;
+                    st1_if(due, smem + mb, bmin);
+                    const bool busy = nw > 0u;
+                    const uint64_t tc = (uint64_t)left * step.x + (uint32_t)nt;
+                    const int32_t ntb = busy ? (int32_t)((uint32_t)tc - step.x) : kFar;
+                    in.t = due ? nt : in.t;
+                    in.K = due ? nK : in.K;
+                    in.w = due ? nw : in.w;
+                    in.kmin = due ? nmin : in.kmin;
+                    in.tb = due ? ntb : in.tb;
+                    in.sw = due ? step.x : in.sw;
+                    in.rsw = due ? step.y : in.rsw;
+                    bad = bad | (due & busy & (tc > (uint64_t)kWalkHorizon));
+                    due = due & busy & ((left == 0u) | (ntb < upto)) & !bad;
+                } else if (due) {
                     const uint32_t slot = in.kmin & 63u, run = in.kmin & 127u, kb = keys + ((slot >> 3) << 5);
                     const uint32_t e = ring + 16u * (ring_n + (uint32_t)__popc(dm & gmask & below));
                     copy_run(e, pay + run);
@@ -214,8 +246,8 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
             take_chunk(nxt);
             nxt = __ldg(reqs + min(cb + 32u + lane, n_req - 1u));
             const uint32_t n_chunk = min(32u, n_req - cb);
-            // what the keys need room for: an end index is at most 2^16 beyond one before it
-            if (__any_sync(kWFull, (in.w > 0) & (in.K > kPackRelMax - (40u << 16))) && in.w > 0) {
+            // what the keys need room for: an end index is at most 2^16 beyond one before it (else one request at a time)
+            if (Straight && __any_sync(kWFull, (in.w > 0) & (in.K > kPackRelMax - (40u << 16))) && in.w > 0) {
                 in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K << 7, in.kmin);
                 in.K = 0;
             }
@@ -312,23 +344,38 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
                     } else {
                         // The entry taken now is the slot's last but one: copies of earlier steps have to be through, this step's not.
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
-                        // (without a branch: every lane computes what it would leave, the winners take it: one node's 10,864 x 5,000
-                        // 6.6 -> 6.5 ms, with 12 warps 6.3 -> 6.2; three models, 40,000 x 3,000 13.8 -> 13.5)
-                        const uint32_t nK = in.w > 0 ? in.K : 0u, nk = ((nK + Sm1) << 7) | top, nmin = min(in.kmin, nk);  // (no live end index: the counter restarts)
-                        const int32_t nt = in.t + pre;
-                        const uint64_t tc = (uint64_t)((nmin >> 7) - nK) * more.x + (uint32_t)nt;
-                        st1_if(win, smem + keys + 4u * (top & 63u), nk);
-                        if (win) pay[top] = make_uint2((uint32_t)nt, cb + i);
-                        const uint32_t mb = smem + area + ((top >> 1) & 28u);
-                        st1_if(win, mb, min(ld1(mb), nk));
-                        in.t = win ? nt : in.t;
-                        in.K = win ? nK : in.K;
-                        in.kmin = win ? nmin : in.kmin;
-                        in.w = win ? in.w + 1u : in.w;
-                        in.sw = win ? more.x : in.sw;
-                        in.rsw = win ? more.y : in.rsw;
-                        in.tb = win ? (int32_t)((uint32_t)tc - more.x) : in.tb;
-                        bad = bad | (win & (tc > (uint64_t)kWalkHorizon));
+                        if constexpr (Straight) {
+                            const uint32_t nK = in.w > 0 ? in.K : 0u, nk = ((nK + Sm1) << 7) | top, nmin = min(in.kmin, nk);  // (no live end index: the counter restarts)
+                            const int32_t nt = in.t + pre;
+                            const uint64_t tc = (uint64_t)((nmin >> 7) - nK) * more.x + (uint32_t)nt;
+                            st1_if(win, smem + keys + 4u * (top & 63u), nk);
+                            if (win) pay[top] = make_uint2((uint32_t)nt, cb + i);
+                            const uint32_t mb = smem + area + ((top >> 1) & 28u);
+                            st1_if(win, mb, min(ld1(mb), nk));
+                            in.t = win ? nt : in.t;
+                            in.K = win ? nK : in.K;
+                            in.kmin = win ? nmin : in.kmin;
+                            in.w = win ? in.w + 1u : in.w;
+                            in.sw = win ? more.x : in.sw;
+                            in.rsw = win ? more.y : in.rsw;
+                            in.tb = win ? (int32_t)((uint32_t)tc - more.x) : in.tb;
+                            bad = bad | (win & (tc > (uint64_t)kWalkHorizon));
+                        } else if (win) {
+                            in.t += pre;
+                            if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
+                            if (in.K + Sm1 > kPackRelMax) {
+                                in.kmin = walk_rebase(area, keys, (in.B + 7u) >> 3, in.K << 7, in.kmin);
+                                in.K = 0;
+                            }
+                            const uint32_t nk = ((in.K + Sm1) << 7) | top;
+                            w1(keys + 4u * (top & 63u)) = nk;
+                            pay[top] = make_uint2((uint32_t)in.t, cb + i);
+                            const uint32_t mb = area + ((top >> 1) & 28u);
+                            w1(mb) = min(w1(mb), nk);
+                            in.kmin = min(in.kmin, nk);
+                            in.w++;
+                            next_end((in.kmin >> 7) - in.K, true, more);
+                        }
                     }
                     if (!Opt) break;
                     act = again;
@@ -409,7 +456,7 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_c
         w4(L.lims + 16u * c) = make_uint4(a < 0 ? 0xFFFFFFFFu : (uint32_t)a, b < 0 ? 0xFFFFFFFFu : (uint32_t)b, lo32(le), hi32(le));
     }
     __syncthreads();
-    pack_items<Opt>(P, L, warp * gridDim.x + blockIdx.x, gridDim.x * Warps);
+    pack_items<Opt, Warps == kWalkWarpsFew>(P, L, warp * gridDim.x + blockIdx.x, gridDim.x * Warps);
 }
 
 template <int Warps>
