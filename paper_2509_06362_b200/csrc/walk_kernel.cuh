@@ -283,7 +283,7 @@ struct Walk {
     static constexpr U kTier1 = (U)1 << (8 * sizeof(U) - 1);
     static constexpr U kNone = ~(U)0;
     static constexpr uint32_t kKeyBytes = kFixed ? (uint32_t)sizeof(T) : 4u;
-    // Queues: times are below 2^58 (see the admission), so that a key has room for the lane (5 % less than a vote and a search
+    // Queues: times are below 2^58 (see the admission), so that a key has room for the lane (3 % less than a vote and a search
     // for the winner's bit)
     static constexpr bool kLaneKey = Eng == 2 && Wide && !Big;
     static constexpr bool kAway = Big && !Wide && !kFixed;  // running requests' data in global memory
