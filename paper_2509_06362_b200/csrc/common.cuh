@@ -229,6 +229,15 @@ __device__ __forceinline__ void bulk_load(void* dst_smem, const void* src_gmem, 
 }
 
 // Everything a scoring kernel needs, passed by value.
+// The list of a trace's patient requests (EvalParams::trace_patient) while the trace is prepared.
+struct PatientList {
+    int64_t patience;
+    uint4* reqs;       // the requests, in order
+    uint32_t* idx;     // their indices
+    uint32_t* ahead;   // [n / 32 + 1] how many are ahead of each 32 requests of the trace
+    uint32_t* counts;  // [tiles] how many are in each tile; null: no list
+};
+
 struct EvalParams : Route {
     const uint4* reqs;
     uint32_t n_req;

@@ -12,9 +12,8 @@
 
 namespace maaso {
 cudaError_t launch_prep(const EvalParams& P, const uint32_t* dump_idx, cudaStream_t stream, int* launches);
-cudaError_t launch_pick_patient(const uint4* reqs, const int64_t* classes, int64_t patience, const uint32_t* ahead, uint4* out, uint32_t* idx, uint32_t n);
-cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n);
-cudaError_t launch_scan_trace(const uint4* reqs, const int64_t* classes, uint4* scan, uint32_t n);
+cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* cooked, uint64_t* rej_hash, uint4* scan, const PatientList& list, uint32_t n);
+uint32_t scan_trace_tiles(uint32_t n);
 size_t scan_trace_units(uint32_t n);
 cudaError_t launch_eval_group(const EvalParams& P, int grid, int tile_recs, int blocks_per_sm, int smem_per_sm,
                               cudaStream_t stream);
@@ -471,19 +470,8 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     uint64_t tok_sum = 0;
     uint32_t max_in = 0, max_out = 0;
     std::vector<uint32_t> count((size_t)n_classes * MAASO_MAX_MODELS, 0);
-    const int64_t patience = split_by_patience(cls);
-    std::vector<uint32_t> patient(n_classes, 0), ahead;
-    uint32_t n_patient = 0, impatient = 0;
-    if (patience >= 0) {
-        ahead.resize(n / 32 + 1);
-        for (uint32_t k = 0; k < n_classes; k++) {
-            patient[k] = (cls[3 * k] < 0 || cls[3 * k] > patience) && (cls[3 * k + 2] < 0 || cls[3 * k + 2] > patience);
-            if (!patient[k] && k < 32) impatient |= 1u << k;
-        }
-    }
     for (uint64_t r = 0; r < n; r++) {
         const maaso_request& q = host[r];
-        if (patience >= 0 && r % 32 == 0) ahead[r / 32] = n_patient;
         if (q.arrival_us < prev || q.arrival_us > kArrMax)
             return fail(ctx, MAASO_EINVAL, "trace: arrivals must be non-negative, non-decreasing, below 2^50");
         prev = q.arrival_us;
@@ -495,9 +483,14 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
         if (q.in_tokens > max_in) max_in = q.in_tokens;
         if (q.out_tokens > max_out) max_out = q.out_tokens;
         count[(size_t)q.cls * MAASO_MAX_MODELS + q.model]++;
-        n_patient += patient[q.cls];
         class_tot[(size_t)q.cls * 2] += 1;
         class_tot[(size_t)q.cls * 2 + 1] += host_rejected_hash((uint32_t)r);
+    }
+    const int64_t patience = split_by_patience(cls);
+    uint32_t n_patient = 0, impatient = 0;
+    for (uint32_t k = 0; k < n_classes && patience >= 0; k++) {
+        if ((cls[3 * k] < 0 || cls[3 * k] > patience) && (cls[3 * k + 2] < 0 || cls[3 * k + 2] > patience)) n_patient += (uint32_t)class_tot[2 * k];
+        else if (k < 32) impatient |= 1u << k;
     }
     maaso_trace* t = new (std::nothrow) maaso_trace();
     if (!t) return MAASO_ENOMEM;
@@ -529,8 +522,8 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     const size_t o_scan = off;   off = align_up(off + scan_trace_units((uint32_t)n) * 16, 256);
     const size_t o_hash = off;   off = align_up(off + n1 * 8, 256);
     const size_t o_small = off;  off = align_up(off + (class_tot.size() + cls.size()) * 8, 256);
-    const size_t o_ahead = off + (size_t)n_patient * 20;  // behind the patient requests and their indices
-    const size_t o_patient = off; off = align_up(n_patient ? o_ahead + ahead.size() * 4 : off, 256);
+    // the patient requests, their indices, how many are ahead of each 32 requests, how many are in each tile
+    const size_t o_patient = off; off = align_up(off + (n_patient ? (size_t)n_patient * 20 + (n / 32 + 1 + scan_trace_tiles((uint32_t)n)) * 4 : 0), 256);
     cudaError_t e = cudaSuccess;
     if (ctx->spare && ctx->spare_bytes >= off && ctx->spare_bytes / 4 <= off) {
         t->mem = ctx->spare;
@@ -562,14 +555,10 @@ MAASO_API int maaso_load_trace(maaso_ctx* ctx, const maaso_request* reqs, uint64
     if (n) e = cudaMemcpyAsync(t->d_reqs, reqs, n * sizeof(maaso_request),
                                on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, cudaStreamLegacy);
     if (e == cudaSuccess) e = cudaMemcpyAsync(mem + o_small, small.data(), small.size() * 8, cudaMemcpyHostToDevice, cudaStreamLegacy);
-    if (e == cudaSuccess) e = launch_cook_trace(t->d_reqs, t->d_classes, t->d_cooked, t->d_rej_hash, (uint32_t)n);
-    if (n_patient) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(mem + o_ahead, ahead.data(), ahead.size() * 4, cudaMemcpyHostToDevice, cudaStreamLegacy);
-        if (e == cudaSuccess)
-            e = launch_pick_patient(t->d_reqs, t->d_classes, patience, reinterpret_cast<const uint32_t*>(mem + o_ahead), t->d_patient,
-                                    reinterpret_cast<uint32_t*>(t->d_patient + n_patient), (uint32_t)n);
-    }
-    if (e == cudaSuccess) e = launch_scan_trace(t->d_reqs, t->d_classes, t->d_scan, (uint32_t)n);
+    PatientList list = {patience, t->d_patient, reinterpret_cast<uint32_t*>(t->d_patient + n_patient), nullptr, nullptr};
+    list.ahead = list.idx + n_patient;
+    if (n_patient) list.counts = list.ahead + n / 32 + 1;
+    if (e == cudaSuccess) e = launch_cook_trace(t->d_reqs, t->d_classes, t->d_cooked, t->d_rej_hash, t->d_scan, list, (uint32_t)n);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         cudaFree(t->mem);

@@ -252,49 +252,39 @@ __global__ void dump_fill_kernel(int64_t* finish, int64_t* first, int32_t* inst,
     }
 }
 
-// The checksum term of a rejected request depends on the request alone: computed once per trace, with the
-// prepared record.
-// Prepared trace records for the lane-group kernel (layout: common.cuh).
-__global__ void cook_trace_kernel(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const Request q = decode_request(reqs[r]);
-    const int64_t l_ttft = classes[q.cls * 3 + 0], l_tbt = classes[q.cls * 3 + 1], l_e2e = classes[q.cls * 3 + 2];
-    const int64_t dl_ttft = l_ttft < 0 ? INT64_MAX : q.arrival + l_ttft;
-    const int64_t dl_e2e = l_e2e < 0 ? INT64_MAX : q.arrival + l_e2e;
-    const uint32_t tbt32 = (l_tbt < 0 || l_tbt > 0xFFFFFFFFll) ? 0xFFFFFFFFu : (uint32_t)l_tbt;
-    const uint64_t h = rejected_hash(r);
-    rej_hash[r] = h;
-    auto lo = [](uint64_t v) { return (uint32_t)v; };
-    auto hi = [](uint64_t v) { return (uint32_t)(v >> 32); };
-    uint4* o = out + (size_t)r * kCookedWords;
-    o[0] = make_uint4(lo((uint64_t)q.arrival), hi((uint64_t)q.arrival), lo((uint64_t)dl_ttft), hi((uint64_t)dl_ttft));
-    o[1] = make_uint4(lo((uint64_t)dl_e2e), hi((uint64_t)dl_e2e), q.in_tokens, tbt32);
-    o[2] = make_uint4(lo(h), hi(h), (q.S - 1u) | (q.cls << 16) | (q.model << 24), 0u);
+// A class whose requests may get their first token and their end more than `patience` us after their arrival.
+__device__ __forceinline__ bool is_patient(const int64_t* classes, uint32_t cls, int64_t patience) {
+    const int64_t ttft = classes[cls * 3 + 0], e2e = classes[cls * 3 + 2];
+    return (ttft < 0 || ttft > patience) && (e2e < 0 || e2e > patience);
 }
 
-// The requests whose first token or end may come more than `patience` us after their arrival, in order, and their indices;
-// `ahead`: how many of them are ahead of each 32 requests.
-__global__ void pick_patient_kernel(const uint4* reqs, const int64_t* classes, int64_t patience, const uint32_t* ahead, uint4* out, uint32_t* idx,
-                                    uint32_t n) {
+// The checksum term of a rejected request depends on the request alone: computed once per trace, with the
+// prepared record.
+// Prepared trace records for the lane-group kernel (layout: common.cuh), and how many of a tile's requests are patient ones
+// (kScanTile threads).
+__global__ void cook_trace_kernel(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n, PatientList list) {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
     bool patient = false;
     if (r < n) {
-        v = reqs[r];
-        const uint32_t cls = decode_request(v).cls;
-        const int64_t ttft = classes[cls * 3 + 0], e2e = classes[cls * 3 + 2];
-        patient = (ttft < 0 || ttft > patience) && (e2e < 0 || e2e > patience);
+        const Request q = decode_request(reqs[r]);
+        const int64_t l_ttft = classes[q.cls * 3 + 0], l_tbt = classes[q.cls * 3 + 1], l_e2e = classes[q.cls * 3 + 2];
+        const int64_t dl_ttft = l_ttft < 0 ? INT64_MAX : q.arrival + l_ttft;
+        const int64_t dl_e2e = l_e2e < 0 ? INT64_MAX : q.arrival + l_e2e;
+        const uint32_t tbt32 = (l_tbt < 0 || l_tbt > 0xFFFFFFFFll) ? 0xFFFFFFFFu : (uint32_t)l_tbt;
+        const uint64_t h = rejected_hash(r);
+        rej_hash[r] = h;
+        auto lo = [](uint64_t v) { return (uint32_t)v; };
+        auto hi = [](uint64_t v) { return (uint32_t)(v >> 32); };
+        uint4* o = out + (size_t)r * kCookedWords;
+        o[0] = make_uint4(lo((uint64_t)q.arrival), hi((uint64_t)q.arrival), lo((uint64_t)dl_ttft), hi((uint64_t)dl_ttft));
+        o[1] = make_uint4(lo((uint64_t)dl_e2e), hi((uint64_t)dl_e2e), q.in_tokens, tbt32);
+        o[2] = make_uint4(lo(h), hi(h), (q.S - 1u) | (q.cls << 16) | (q.model << 24), 0u);
+        patient = is_patient(classes, q.cls, list.patience);
     }
-    const uint32_t set = __ballot_sync(0xFFFFFFFFu, patient);
-    if (!patient) return;
-    const uint32_t at = ahead[r / 32u] + (uint32_t)__popc(set & ((1u << (r & 31u)) - 1u));
-    out[at] = v;
-    idx[at] = r;
-}
-cudaError_t launch_pick_patient(const uint4* reqs, const int64_t* classes, int64_t patience, const uint32_t* ahead, uint4* out, uint32_t* idx, uint32_t n) {
-    pick_patient_kernel<<<(n + 255) / 256, 256>>>(reqs, classes, patience, ahead, out, idx, n);
-    return cudaGetLastError();
+    if (list.counts) {
+        const int k = __syncthreads_count(patient);
+        if (threadIdx.x == 0) list.counts[blockIdx.x] = (uint32_t)k;
+    }
 }
 
 // Scan tiles of the thread mapping.  Tile t (kScanTile requests) is a header followed by one
@@ -310,7 +300,10 @@ cudaError_t launch_pick_patient(const uint4* reqs, const int64_t* classes, int64
 //   unit 4: base arrival (int64) = arrival of the tile's first request;
 //   units 5..20: per class slot a 256-bit map of the tile's requests of that class;
 //   units 21..36: the same per model (models 7 and up share slot 7).
-__global__ void scan_trace_kernel(const uint4* reqs, const int64_t* classes, uint4* scan, uint32_t n) {
+// And the tile's part of the list of patient requests: here and not on the host or in a kernel of its own, as loading a trace is bound
+// by the host's pass over the requests and by the number of copies and launches (with all three 0.037, 0.069 and 0.387 ms for 500, 10,000
+// and 100,000 requests, this way 0.032, 0.061 and 0.343, without a list 0.030, 0.061 and 0.342).
+__global__ void scan_trace_kernel(const uint4* reqs, const int64_t* classes, uint4* scan, uint32_t n, PatientList list) {
     const uint32_t tile = blockIdx.x, t = threadIdx.x;  // kScanTile threads
     __shared__ int64_t thr[8];
     if (t < 8) thr[t] = INT64_MIN;
@@ -319,8 +312,12 @@ __global__ void scan_trace_kernel(const uint4* reqs, const int64_t* classes, uin
     uint4* const base = scan + (size_t)tile * (kScanTile + kScanHdrUnits);
     const int64_t base_arrival = decode_request(reqs[tile * kScanTile]).arrival;
     uint32_t cslot = 0xFFu, mslot = 0xFFu;
+    uint4 raw = make_uint4(0u, 0u, 0u, 0u);
+    bool patient = false;
     if (r < n) {
-        const Request q = decode_request(reqs[r]);
+        raw = reqs[r];
+        const Request q = decode_request(raw);
+        patient = is_patient(classes, q.cls, list.patience);
         const int64_t l_ttft = classes[q.cls * 3 + 0], l_e2e = classes[q.cls * 3 + 2];
         const uint32_t t32 = (l_ttft < 0 || l_ttft >= 0xFFFFFFFFll) ? 0xFFFFFFFFu : (uint32_t)l_ttft;
         const uint32_t e32 = (l_e2e < 0 || l_e2e >= 0xFFFFFFFFll) ? 0xFFFFFFFFu : (uint32_t)l_e2e;
@@ -348,17 +345,34 @@ __global__ void scan_trace_kernel(const uint4* reqs, const int64_t* classes, uin
     }
     if (t == 4) base[kScanHdrBase] = make_uint4((uint32_t)base_arrival, (uint32_t)((uint64_t)base_arrival >> 32), 0u, 0u);
     if (t >= 5 && t < 8) base[kScanHdrUnits - 3 + (t - 5)] = make_uint4(0u, 0u, 0u, 0u);  // padding units 37..39
+    if (list.counts) {
+        __shared__ uint32_t before[kScanTile / 32], own[kScanTile / 32];
+        uint32_t at = 0;  // patient requests ahead of this one: those of earlier tiles, of earlier warps, of earlier lanes
+        for (uint32_t i = t; i < tile; i += kScanTile) at += list.counts[i];
+        at = __reduce_add_sync(0xFFFFFFFFu, at);
+        const uint32_t set = __ballot_sync(0xFFFFFFFFu, patient), lane = t & 31u;
+        if (lane == 0) before[t >> 5] = at, own[t >> 5] = (uint32_t)__popc(set);
+        __syncthreads();
+        at = 0;
+        for (uint32_t v = 0; v < kScanTile / 32; v++) at += before[v] + (v < t >> 5 ? own[v] : 0u);
+        if (lane == 0 && r < n) list.ahead[r / 32u] = at;
+        if (patient) {
+            at += (uint32_t)__popc(set & ((1u << lane) - 1u));
+            list.reqs[at] = raw;
+            list.idx[at] = r;
+        }
+    }
 }
 size_t scan_trace_units(uint32_t n) {
     const size_t tiles = ((size_t)n + kScanTile - 1) / kScanTile;
     return (tiles ? tiles : 1) * (kScanTile + kScanHdrUnits);
 }
-cudaError_t launch_scan_trace(const uint4* reqs, const int64_t* classes, uint4* scan, uint32_t n) {
-    if (n) scan_trace_kernel<<<(n + kScanTile - 1) / kScanTile, kScanTile>>>(reqs, classes, scan, n);
-    return cudaGetLastError();
-}
-cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* out, uint64_t* rej_hash, uint32_t n) {
-    if (n) cook_trace_kernel<<<(n + 255) / 256, 256>>>(reqs, classes, out, rej_hash, n);
+uint32_t scan_trace_tiles(uint32_t n) { return (uint32_t)(((uint64_t)n + kScanTile - 1) / kScanTile); }
+// Everything that is prepared of a trace, on the legacy stream.
+cudaError_t launch_cook_trace(const uint4* reqs, const int64_t* classes, uint4* cooked, uint64_t* rej_hash, uint4* scan, const PatientList& list, uint32_t n) {
+    if (n == 0) return cudaSuccess;
+    cook_trace_kernel<<<scan_trace_tiles(n), kScanTile>>>(reqs, classes, cooked, rej_hash, n, list);
+    scan_trace_kernel<<<scan_trace_tiles(n), kScanTile>>>(reqs, classes, scan, n, list);
     return cudaGetLastError();
 }
 
