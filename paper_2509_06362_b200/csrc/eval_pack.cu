@@ -88,6 +88,12 @@ __device__ __forceinline__ void copy_run(uint32_t entry, const uint2* run) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(entry + smem_addr(walk_smem)), "l"(run) : "memory");
 }
 
+// Work items of a batch: of groups of eight lanes, of all.
+__device__ __forceinline__ uint32_t pack_items8(const EvalParams& P) { return (P.bucket_count[kPack8] + 3u) / 4u; }
+__device__ __forceinline__ uint32_t pack_total(const EvalParams& P) {
+    return (pack_items8(P) + (P.bucket_count[kPack4] + 7u) / 8u) * (P.n_traces > 1 ? P.n_traces : 1u);
+}
+
 // One warp takes work items, one after the other: 32 / G placements of the bucket whose groups have G lanes, the largest
 // placements first.  (One numbering for both buckets: starting on each from the same warps would have some replay an item
 // of each in a row where there is one item for each warp.)
@@ -102,8 +108,7 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     constexpr uint32_t kTier1 = 1u << 31, kNone = ~0u;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, below = (1u << lane) - 1u;
     const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
-    const uint32_t n8 = (P.bucket_count[kPack8] + 3u) / 4u, n4 = (P.bucket_count[kPack4] + 7u) / 8u;
-    const uint32_t total = (n8 + n4) * n_traces;
+    const uint32_t n8 = pack_items8(P), total = pack_total(P);
     const uint32_t area = L.pool + threadIdx.x * kPackLane, keys = area + 96u, smem = smem_addr(walk_smem);
     unsigned char* const scratch = reinterpret_cast<unsigned char*>(P.payload) + ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * kPackScratch;
     uint2* const pay = reinterpret_cast<uint2*>(scratch);
@@ -439,11 +444,21 @@ static __device__ __forceinline__ void pack_items(const EvalParams& P, const Wal
     }
 }
 
-// `Warps`: 14 with 128 registers each, or 12 with room for 168 (launch_eval_pack).
+// Do 12 warps per SM serve so many items better than 14 (of `grid` SMs)?  See launch_eval_pack.
+constexpr uint32_t kPackFewWaves = 2u, kPackFewAgain = 16u;
+__device__ __forceinline__ bool pack_few(uint32_t items, uint32_t grid) {
+    const uint32_t wave = kWalkWarpsFew * grid;
+    return items <= wave || (items > kPackFewAgain * grid && items <= kPackFewWaves * wave);
+}
+
+// `Warps`: 14 with 128 registers each, or 12 with room for 168.  `one_of_two`: both are launched, and the number of items decides which
+// of them replays the batch (launch_eval_pack).
 template <bool Opt, int Warps>
-__global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P) {
+__global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_constant__ EvalParams P, bool one_of_two) {
     if (P.stall_test) return;  // test hook: nothing is scored, every valid candidate keeps its "not scored" mark
-    if (P.bucket_count[kPack4] + P.bucket_count[kPack8] == 0) return;
+    const uint32_t items = pack_total(P);
+    if (items == 0) return;
+    if (one_of_two && pack_few(items, gridDim.x) != (Warps == kWalkWarpsFew)) return;
     let_next_start();
     const WalkLayout L = pack_layout(P.n_rows, P.n_classes);
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
@@ -460,23 +475,33 @@ __global__ void __launch_bounds__(32 * Warps, 1) eval_pack_kernel(const __grid_c
 }
 
 template <int Warps>
-static cudaError_t launch_pack(const EvalParams& P, int grid, cudaStream_t stream) {
+static cudaError_t launch_pack(const EvalParams& P, int grid, bool one_of_two, cudaStream_t stream, int* launches) {
     const size_t smem = pack_layout(P.n_rows, P.n_classes).pool + 32u * Warps * kPackLane;
     auto kernel = (P.flags & MAASO_FLAG_PRED_OPTIMISTIC) ? eval_pack_kernel<true, Warps> : eval_pack_kernel<false, Warps>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, 32 * Warps, smem, stream>>>(P);
+    kernel<<<grid, 32 * Warps, smem, stream>>>(P, one_of_two);
+    ++*launches;
     return cudaGetLastError();
 }
-// A batch that 12 warps per SM hold at once (six placements a warp on average) is bound by its longest items, which take 156 to
-// 158 registers there and spill nothing (14 warps: 92 to 100 bytes).  14 and not 16 for the rest: their shared memory fits a
-// partition that leaves 60 KB of L1 instead of 28 (16 rates, 10,864 x 2,500: 29.5 and 31.7 ms, optimistic estimate 32.0 and 33.5).
-// Measured, 12 and 14 warps, optimistic estimate: one node's 10,864 x 4,000 under 2 traces 8.3 and 8.9, 4 traces x 10,000 35.7 and 34.7;
-// worst-case estimate 10,864 x 5,000 6.2 and 6.5, 3 traces x 4,000 10.9 and 10.6; three models, 40,000 x 3,000 14.5 and 13.5, at 1 a
-// second 20,000 x 4,000 11.8 and 11.3.  So the line is at two such waves with one model and at one with several.
-cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream) {
-    const uint64_t placements = (uint64_t)P.n_cand * (P.n_traces > 1 ? P.n_traces : 1u);
-    return placements <= (P.n_models == 1 ? 14ull : 6ull) * kWalkWarpsFew * (uint64_t)grid ? launch_pack<kWalkWarpsFew>(P, grid, stream) : launch_pack<kPackWarps>(P, grid, stream);
+// A batch whose items 12 warps per SM hold at once is bound by its longest items, which take 154 to 158 registers there and spill
+// nothing (14 warps: 88 to 100 bytes).  14 and not 16 for the rest: their shared memory fits a partition that leaves 60 KB of L1
+// instead of 28 (16 rates, 10,864 x 2,500: 29.5 and 31.7 ms, optimistic estimate 32.0 and 33.5).  With more items 12 take a second
+// wave that 14 do not need, or hardly; from 16 items per SM on both take two, which 12 run faster; the third wave again is better shared
+// by 14, and beyond it neither is better throughout (0.92 to 1.14 of the time).  One model on one node, 2,500 requests at 1 a second, 12
+// and 14 warps: 1,497 items (10,000 placements; 12 warps on each of 148 SMs hold 1,776) 2.94 and 3.25 ms, 1,646 3.00 and 3.23, 1,797
+// 3.95 and 3.37, 1,945 4.65 and 3.48, 2,094 4.78 and 4.35, 2,318 4.83 and 5.17, 2,540 4.88 and 5.49, 3,243 5.61 and 5.75, 3,510 5.71 and
+// 6.16, 3,731 7.18 and 6.34, 4,026 7.52 and 6.60; the optimistic estimate and two traces within 2 % of these ratios; two models, 12,800 x
+// 3,000 (one wave) 3.50 and 3.88, 16,000 (in the second) 5.07 and 4.60, 24,000 6.24 and 6.73.
+// An item is four to eight placements, and how many items a batch has is known on the device alone: where the placements leave it
+// open, both kernels are launched and one of them returns at once.  (14 first: the shorter batches' tail is what the walking
+// kernel, which is launched next, starts beside.)
+cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream, int* launches) {
+    const uint64_t placements = (uint64_t)P.n_cand * (P.n_traces > 1 ? P.n_traces : 1u), wave = (uint64_t)kWalkWarpsFew * (uint64_t)grid;
+    if (placements > 8 * kPackFewWaves * wave) return launch_pack<kPackWarps>(P, grid, false, stream, launches);
+    const bool both = placements > 4 * wave;
+    const cudaError_t e = both ? launch_pack<kPackWarps>(P, grid, true, stream, launches) : cudaSuccess;
+    return e != cudaSuccess ? e : launch_pack<kWalkWarpsFew>(P, grid, both, stream, launches);
 }
 
 }  // namespace maaso

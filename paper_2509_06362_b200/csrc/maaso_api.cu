@@ -25,7 +25,7 @@ int occupancy_eval_thread(const EvalParams& P, uint32_t pool_bytes, uint32_t hot
 size_t thread_scratch_per_warp(uint32_t pool_bytes);
 uint32_t thread_fixed_smem(uint32_t n_models, uint32_t n_rows);
 cudaError_t launch_eval_walk(const EvalParams& P, int grid, bool overlap, cudaStream_t stream);
-cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream);
+cudaError_t launch_eval_pack(const EvalParams& P, int grid, cudaStream_t stream, int* launches);
 size_t pack_scratch(int grid);
 cudaError_t launch_eval_walk_big(const EvalParams& P, int grid, cudaStream_t stream);
 cudaError_t launch_eval_walk_long(const EvalParams& P, int grid, cudaStream_t stream);
@@ -844,8 +844,7 @@ static int eval_impl(maaso_ctx* ctx, const maaso_trace* const* traces, uint32_t 
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel launch");
     }
     if (L.pack) {
-        e = launch_eval_pack(P, ctx->sm_count, stream);
-        launches++;
+        e = launch_eval_pack(P, ctx->sm_count, stream, &launches);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "packed kernel launch");
     }
     auto launch_big = [&]() {
