@@ -253,7 +253,7 @@ struct WalkDynamic {
             // What is rare, out of the rounds' way.  Moves the epoch for request `src` of the chunk at `cb` of `arr`, to the dispatcher's
             // clock (or to the request's arrival, if that is later): what happens before it is simulated, everything else is
             // measured from there on.
-            auto move_epoch = [&](const uint4* arr, uint32_t n_arr, uint32_t cb, uint32_t src) {
+            auto move_epoch = [&](const uint4* arr, uint32_t n_arr, uint32_t cb, uint32_t src, bool patient, int32_t& mark) {
                 const uint4 v = __ldg(arr + cb + src);
                 const int64_t to = max(epoch + now, i64_of(v.x, v.y));
                 const int32_t up = to - epoch >= (int64_t)kFar ? kFar : (int32_t)(to - epoch);  // (cut off only if all is idle by then)
@@ -280,6 +280,7 @@ struct WalkDynamic {
                 flush();
                 epoch = to;
                 now = 0;
+                if (Apart && !patient) mark = 0;
                 take_chunk(__ldg(arr + min(cb + lane, n_arr - 1u)));
                 __syncwarp();
             };
@@ -291,7 +292,8 @@ struct WalkDynamic {
             const uint32_t* const pat_idx = reinterpret_cast<const uint32_t*>(pats + n_pat);
             const bool only_pat = Apart && n_pat && use_mask && (cmask & P.impatient) == 0u;
             const uint4* arr = reqs;
-            uint32_t cb = 0, n_arr = n_req, first_lane = 0, resume = 0;
+            uint32_t cb = 0, n_arr = n_req, first_lane = 0;
+            int32_t mark = 0;  // while the list is read: where the trace goes on; else the dispatcher's clock before which it is not turned to again
             bool apart = false;
             auto counted = [&]() { return cb + lane < n_arr && ((cmask >> ((c_meta >> 16) & 31u)) & 1u); };
             auto turn_to = [&](bool patient, uint32_t at) {
@@ -302,8 +304,16 @@ struct WalkDynamic {
                 first_lane = patient ? 0u : at & 31u;
                 nxt = __ldg(arr + min(cb + lane, n_arr - 1u));
             };
-            // Behind the last patient request that has been looked at.
-            auto leave = [&]() { turn_to(false, max(resume, cb ? __ldg(pat_idx + min(cb, n_pat) - 1u) + 1u : 0u)); };
+            // Goes on behind the last patient request that has been looked at.  The list's next 32 reach so far that they and what is between
+            // them are worth the turn once the clock is the others' patience beyond the last of them; behind its end it never is.  (Turning after
+            // every chunk in vain, 30,000 requests, 10,000 placements: all patient ones in the first tenth 8.0 instead of 7.5 ms, one in 1,000 after
+            // that 7.9 instead of 7.3.)
+            auto leave = [&]() {
+                const int32_t reach = cb < n_pat ? __reduce_max_sync(kWFull, rel) : kFar;
+                const uint32_t to = max((uint32_t)mark, cb ? __ldg(pat_idx + min(cb, n_pat) - 1u) + 1u : 0u);
+                mark = reach >= kWalkNowMax ? kFar : reach + P.patience;
+                turn_to(false, to);
+            };
             // Which of the chunk's requests from lane `from` on may need the distributor.
             auto test = [&](uint32_t from) -> uint32_t {
                 const uint32_t Sm1 = (c_meta & 0xFFFFu) - 1u, model = c_meta >> 24;
@@ -346,8 +356,8 @@ struct WalkDynamic {
                     live = test(Apart ? first_lane : 0u);
                     if (live) break;
                     if (Apart) {
-                        if (!apart && n_pat && first_lane == 0u && !__any_sync(kWFull, rel >= now - P.trace_lead[tr])) {
-                            resume = cb + 32u;
+                        if (!apart && n_pat && first_lane == 0u && now >= mark && !__any_sync(kWFull, rel >= now - P.trace_lead[tr])) {
+                            mark = (int32_t)(cb + 32u);
                             turn_to(true, __ldg(pat_idx + n_pat + cb / 32u));
                             cb -= 32u;
                         }
@@ -357,7 +367,7 @@ struct WalkDynamic {
                     }
                 }
                 if (live == 0u) {
-                    if (!(Apart && apart)) break;
+                    if (!(Apart && apart) || only_pat) break;
                     leave();
                     cb -= 32u;
                     continue;
@@ -578,7 +588,7 @@ struct WalkDynamic {
                     served |= live & (from < 32u ? (1u << from) - 1u : ~0u) & ~rejected;
                     __syncwarp();
                     if (status) break;
-                    if (move) move_epoch(arr, n_arr, cb, from);
+                    if (move) move_epoch(arr, n_arr, cb, from, apart, mark);
                     else if (from >= 32u) break;
                     live = test(from);
                 } while (live);
