@@ -960,20 +960,15 @@ __device__ __forceinline__ uint32_t walk_big_warps(const EvalParams& P, uint32_t
 }
 
 // Blocks that replay the placements of more than 32 instances; the others go to the smaller ones, side by side with them (the kernel
-// for those is launched second and starts where this one leaves room).  As many as hold them all at once, and no fewer than
-// their share of the work, one of them counted as eight smaller ones (25 warp milliseconds alone and 40 in company, against 4, over 40,000
-// requests).  One kernel after the other, a few hundred of them among 30,000 ran three warps on each SM for 29 of 80 ms; side by side
-// 51 ms (73 -> 51 and 82 -> 51 over two draws).
+// for those is launched second and starts where this one leaves room).  One kernel after the other, a few hundred of the larger ones
+// among 30,000 ran three warps on each SM for 29 of 80 ms; side by side 51 ms (73 -> 51 and 82 -> 51 over two draws).
 __device__ __forceinline__ uint32_t walk_big_blocks(const EvalParams& P) {
     const uint32_t n_traces = P.n_traces > 1 ? P.n_traces : 1u;
     const uint64_t big = (uint64_t)P.bucket_count[kWalkBig0] * n_traces;
     if (P.big_grid == 0u || big == 0u) return 0u;
     uint64_t small = 0;
     for (int mode = 0; mode < kWalkModes; mode++) small += P.bucket_count[kWalkBucket0 + mode];
-    small *= (uint64_t)n_traces * P.walk_parts;
-    const uint32_t warps = walk_big_warps(P, (uint32_t)kWalkWarps);
-    const uint64_t once = (big + warps - 1u) / warps, share = (8u * big * P.big_grid + 8u * big + small - 1u) / (8u * big + small);
-    return (uint32_t)min(min((uint64_t)P.big_grid, big), max(once, share));
+    return walk_big_share(big, small * n_traces, walk_big_warps(P, (uint32_t)kWalkWarps), P.big_grid);
 }
 
 // `Warps`: 16, or 12 for small batches under fixed speeds and queues (route.cuh).  Mode k: the block's warps >> k at work, each with
