@@ -700,7 +700,7 @@ struct Walk {
                     in.rsw = win ? (Rcp ? more.y : walk_rcp(more.x)) : in.rsw;
                     in.tb = win ? (T)((uint32_t)tc - more.x) : in.tb;
                     bad = bad | (win & (tc > (uint64_t)kWalkHorizon));
-                } else if (win) {
+                } else if (win) {  // 64-bit times
                     const uint32_t slot = top;
                     in.t += pre;
                     if (in.w == 0) in.K = 0;  // no live end index: the counter restarts
@@ -709,16 +709,9 @@ struct Walk {
                         in.K = 0;
                     }
                     const uint32_t nk = ((in.K + Sm1) << 6) | slot;
-                    const uint32_t k8 = in.keys + 4u * slot;
-                    w1(k8) = nk;
-                    if constexpr (kAway) {
-                        __stcg(reinterpret_cast<uint2*>(away + 2u * (k8 - L.pool)), make_uint2((uint32_t)in.t, req));
-                    } else if constexpr (!Wide) {
-                        w2(in.pay + 8u * slot) = make_uint2((uint32_t)in.t, req);
-                    } else {
-                        w1(in.pay + 4u * slot) = req;
-                        w2(firsts() + 8u * slot) = make_uint2(lo32(in.t), hi32(in.t));
-                    }
+                    w1(in.keys + 4u * slot) = nk;
+                    w1(in.pay + 4u * slot) = req;
+                    w2(firsts() + 8u * slot) = make_uint2(lo32(in.t), hi32(in.t));
                     atomicMin(&w1(in.area + ((slot >> 3) << 2)), nk);
                     in.kmin = min(in.kmin, nk);
                     in.w++;
