@@ -23,9 +23,9 @@
 // the shortest round (walk_dynamic.cuh).  `Walk` here is the body of all the others.
 //
 // Measured (B200, whole calls with routing and top-k; lane-group, thread or one-warp kernel before): 143 placements x 500
-// requests 0.15 ms (0.56), one node's 10,864 x 10,000 4.2 ms (12.0), 2,000 x 17,000 of the paper's shape 6.0 to 6.2 ms (33.9), with
-// queues 5.2 ms (27.8), three models, 100,000 x 100,000 under load 52 ms (135), 2,000 placements of 33 to 128 instances x
-// 10,000 6.7 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
+// requests 0.14 ms (0.56), one node's 10,864 x 10,000 4.2 ms (12.0), 2,000 x 17,000 of the paper's shape 5.9 to 6.4 ms (33.9), with
+// queues 5.3 ms (27.8), three models, 100,000 x 100,000 under load 52 ms (135), 2,000 placements of 33 to 128 instances x
+// 10,000 6.3 to 7.4 ms (13.8).  Nearly all instructions of a round depend on one another: what the next step
 // needs is therefore read from shared memory ahead of the choice, the uncommon outcomes share one branch, and tests of several
 // conditions are written without branches (& and | for && and ||).
 // What some of the lanes do, an admission or an instance's state out of and into shared memory, all lanes compute, with
