@@ -30,7 +30,8 @@
 // conditions are written without branches (& and | for && and ||).
 // What some of the lanes do, an admission or an instance's state out of and into shared memory, all lanes compute, with
 // predicated stores and selections: parting the lanes and joining them again took longer than the work (2,000 placements of 33 to 128
-// instances x 10,000 8.40 -> 6.75 ms, 500 with fixed speeds 7.54 -> 6.02; masked sub-clusters, 9,000 x 12,000 9.03 -> 7.74).
+// instances x 10,000 8.40 -> 6.75 ms, 500 with fixed speeds 7.54 -> 6.02; masked sub-clusters, 9,000 x 12,000 9.03 -> 7.74; kStraight says
+// where not).
 // Completions are left in a branch (without it 2 % slower to 2 % faster).
 //
 // The block's pool of shared memory is split evenly among its warps.  Placements beyond one warp's part run
@@ -283,6 +284,9 @@ struct Walk {
     static constexpr U kTier1 = (U)1 << (8 * sizeof(U) - 1);
     static constexpr U kNone = ~(U)0;
     static constexpr uint32_t kKeyBytes = kFixed ? (uint32_t)sizeof(T) : 4u;
+    // Fixed speeds and queues, a winner's ring entry and next free slot: without a branch, but for up to 32 instances with 32-bit times, which
+    // that makes 1 % slower on average (three models, 12,000 x 6,000 at 400 a second 1.14 and 1.16 ms, the paper's shape up to 2.8 %).
+    static constexpr bool kStraight = Wide || Big;
     // Queues: times are below 2^58 (see the admission), so that a key has room for the lane (3 % less than a vote and a search
     // for the winner's bit)
     static constexpr bool kLaneKey = Eng == 2 && Wide && !Big;
@@ -650,9 +654,14 @@ struct Walk {
                     }
                     const uint64_t span = (uint64_t)Sm1 * w1(in.row + (win ? kEntry * level : 0u) + kEntry);
                     T fin = first + (T)span;
-                    if constexpr (Wide) status = win & (((uint64_t)fin >> 57) != 0) ? (uint32_t)MAASO_CAND_ELOOP : status;  // beyond what the engine takes
-                    else bad = bad | (win & ((span > (uint64_t)kWalkHorizon) | (fin > (T)kWalkHorizon)));
-                    record_if(win, ring_n, fin, first, req);
+                    if constexpr (kStraight) {
+                        if constexpr (Wide) status = win & (((uint64_t)fin >> 57) != 0) ? (uint32_t)MAASO_CAND_ELOOP : status;  // beyond what the engine takes
+                        else bad = bad | (win & ((span > (uint64_t)kWalkHorizon) | (fin > (T)kWalkHorizon)));
+                        record_if(win, ring_n, fin, first, req);
+                    } else if (win) {
+                        bad = bad || span > (uint64_t)kWalkHorizon || fin > (T)kWalkHorizon;
+                        record(ring_n, fin, first, req);
+                    }
                     ring_n++;
                     fin = wshfl(fin, wl);
                     uint32_t pos = n;
@@ -663,9 +672,14 @@ struct Walk {
                     }
                     if (lane == 0) wt<T>(a + kKeyBytes * pos) = fin;
                     __syncwarp();
-                    const T next_free = wt<T>(a + kKeyBytes * n);
-                    in.w = win ? n + 1u : in.w;
-                    in.tb = win ? next_free : in.tb;
+                    if constexpr (kStraight) {
+                        const T next_free = wt<T>(a + kKeyBytes * n);
+                        in.w = win ? n + 1u : in.w;
+                        in.tb = win ? next_free : in.tb;
+                    } else if (win) {
+                        in.w = n + 1u;
+                        in.tb = wt<T>(a + kKeyBytes * n);
+                    }
                 } else if (Sm1 == 0u) {  // done at the end of its prefill, never occupies a slot
                     if (ring_n + 1u > kCap) flush();
                     if (win) {
